@@ -146,7 +146,7 @@ int infaas_catalog_load(const infaas_variant *rows, uint32_t n_variants, uint32_
   if (n_tasks == 0 || n_tasks > 65535u) return INFAAS_E_BAD_TASK;
   if (n_variants == 0 || n_variants > INFAAS_MAX_VARIANTS) return INFAAS_E_TOO_LARGE;
 
-  // ---- validate and bucket by task (stable: ascending id inside a task) ----
+  // ---- validate and bucket by task ----
   std::vector<uint32_t> task_off(n_tasks + 1, 0);
   uint32_t acc_min = 10000, acc_max = 0, lat_min = 0xFFFFFFFFu;
   for (uint32_t v = 0; v < n_variants; ++v) {
@@ -177,19 +177,10 @@ int infaas_catalog_load(const infaas_variant *rows, uint32_t n_variants, uint32_
     reg_off[t + 1] = (uint32_t)region_bytes;
   }
 
-  std::vector<uint32_t> h_lat(n_variants), h_cost(n_variants), h_id(n_variants), h_queued(n_variants),
-      slot_of_id(n_variants);
-  std::vector<uint16_t> h_batch(n_variants), h_acc(n_variants), h_arch(n_variants);
-  std::vector<unsigned long long> h_qps(n_variants);
+  std::vector<uint32_t> members(n_variants);                       // each task's ids, ascending
   {
     std::vector<uint32_t> cursor(task_off.begin(), task_off.end() - 1);
-    for (uint32_t v = 0; v < n_variants; ++v) {
-      const infaas_variant &r = rows[v];
-      const uint32_t s = cursor[r.task]++;
-      h_lat[s] = r.lat_us; h_batch[s] = r.batch; h_acc[s] = r.acc_bp; h_cost[s] = r.cost;
-      h_id[s] = v; h_queued[s] = r.queued; slot_of_id[v] = s; h_arch[s] = r.arch;
-      h_qps[s] = 1000000000ull * r.batch / r.lat_us;     // floor(10^9 * batch / lat_us)
-    }
+    for (uint32_t v = 0; v < n_variants; ++v) members[cursor[rows[v].task]++] = v;
   }
 
   infaas_catalog *c = new (std::nothrow) infaas_catalog();
@@ -218,17 +209,23 @@ int infaas_catalog_load(const infaas_variant *rows, uint32_t n_variants, uint32_
   const size_t o_lat = carve((size_t)n_variants * 4), o_batch = carve((size_t)n_variants * 2);
   const size_t o_acc = carve((size_t)n_variants * 2), o_cost = carve((size_t)n_variants * 4);
   const size_t o_id = carve((size_t)n_variants * 4), o_queued = carve((size_t)n_variants * 4);
+  const size_t o_order = carve((size_t)n_variants * 4), o_cost_run = carve((size_t)n_variants * 4);
+  const size_t o_class = carve((size_t)n_variants * 2), o_class_acc = carve((size_t)n_variants * 2);
+  const size_t o_n_class = carve((size_t)n_tasks * 4);
   const size_t o_pred = carve((size_t)n_variants * 4), o_served = carve((size_t)n_variants * 8);
   const size_t o_count = carve((size_t)n_variants * 4);
   const size_t o_state = carve((size_t)n_variants), o_load_lat = carve((size_t)n_variants * 4);
   const size_t o_inst = carve((size_t)n_variants * 4), o_arch = carve((size_t)n_variants * 2);
   const size_t o_task_slo = carve((size_t)n_tasks * 4), o_qps = carve((size_t)n_variants * 8);
+  const size_t o_slot_of_id = carve((size_t)n_variants * 4);
   const size_t o_hw = carve((size_t)n_variants), o_worker_of = carve((size_t)n_variants * 4);
   const size_t o_best_inst = carve((size_t)n_variants * 8), o_best_hw = carve(256 * 8);
   const size_t o_regions = carve((size_t)region_bytes);
   const size_t o_flen = carve((size_t)n_tasks * 4), o_slow = carve(((size_t)n_tasks + n_extra) * 16);
   const size_t o_seg_base = carve((n_tasks + 1) * 4), o_xhdr = carve((size_t)n_extra * 16 + 16);
-  const size_t o_image = carve((size_t)worst_image), o_hdr = carve(16);
+  // (the rows and members are uploaded into the image's space: the first rebuild comes after the layout)
+  const size_t up_rows = round_up((size_t)n_variants * sizeof(infaas_variant), 256), up_bytes = up_rows + (size_t)n_variants * 4;
+  const size_t o_image = carve((size_t)worst_image > up_bytes ? (size_t)worst_image : up_bytes), o_hdr = carve(16);
   const size_t o_counters = carve(24), o_rebuild = carve(32), o_err = carve(4), o_seen = carve(4);
 
 #define LOAD_TRY(expr)                                                     \
@@ -247,20 +244,7 @@ int infaas_catalog_load(const infaas_variant *rows, uint32_t n_variants, uint32_
   LOAD_TRY(cudaMemcpy(base + o_task_off, task_off.data(), (n_tasks + 1) * 4, cudaMemcpyHostToDevice));
   LOAD_TRY(cudaMemcpy(base + o_reg_off, reg_off.data(), (n_tasks + 1) * 4, cudaMemcpyHostToDevice));
   LOAD_TRY(cudaMemcpy(base + o_seg_base, seg_base.data(), (n_tasks + 1) * 4, cudaMemcpyHostToDevice));
-  LOAD_TRY(cudaMemcpy(base + o_lat, h_lat.data(), (size_t)n_variants * 4, cudaMemcpyHostToDevice));
-  LOAD_TRY(cudaMemcpy(base + o_batch, h_batch.data(), (size_t)n_variants * 2, cudaMemcpyHostToDevice));
-  LOAD_TRY(cudaMemcpy(base + o_acc, h_acc.data(), (size_t)n_variants * 2, cudaMemcpyHostToDevice));
-  LOAD_TRY(cudaMemcpy(base + o_cost, h_cost.data(), (size_t)n_variants * 4, cudaMemcpyHostToDevice));
-  LOAD_TRY(cudaMemcpy(base + o_id, h_id.data(), (size_t)n_variants * 4, cudaMemcpyHostToDevice));
-  LOAD_TRY(cudaMemcpy(base + o_queued, h_queued.data(), (size_t)n_variants * 4, cudaMemcpyHostToDevice));
-  LOAD_TRY(cudaMemcpy(base + o_arch, h_arch.data(), (size_t)n_variants * 2, cudaMemcpyHostToDevice));
-  LOAD_TRY(cudaMemcpy(base + o_qps, h_qps.data(), (size_t)n_variants * 8, cudaMemcpyHostToDevice));
   c->s_qps = reinterpret_cast<unsigned long long *>(base + o_qps);
-  {
-    std::vector<unsigned char> h_hw(n_variants);
-    for (uint32_t v = 0; v < n_variants; ++v) h_hw[v] = rows[v].hw;
-    LOAD_TRY(cudaMemcpy(base + o_hw, h_hw.data(), n_variants, cudaMemcpyHostToDevice));
-  }
   c->hw_by_id = base + o_hw;
   c->worker_of = reinterpret_cast<uint32_t *>(base + o_worker_of);
   c->best_inst = reinterpret_cast<unsigned long long *>(base + o_best_inst);
@@ -280,6 +264,11 @@ int infaas_catalog_load(const infaas_variant *rows, uint32_t n_variants, uint32_
   d.s_acc = reinterpret_cast<const uint16_t *>(base + o_acc);
   d.s_cost = reinterpret_cast<const uint32_t *>(base + o_cost);
   d.s_id = reinterpret_cast<const uint32_t *>(base + o_id);
+  d.s_order = reinterpret_cast<const uint32_t *>(base + o_order);
+  d.s_cost_run = reinterpret_cast<const uint32_t *>(base + o_cost_run);
+  d.s_class = reinterpret_cast<const uint16_t *>(base + o_class);
+  d.class_acc = reinterpret_cast<const uint16_t *>(base + o_class_acc);
+  d.n_class = reinterpret_cast<const uint32_t *>(base + o_n_class);
   d.s_queued = reinterpret_cast<uint32_t *>(base + o_queued);
   d.s_pred = reinterpret_cast<uint32_t *>(base + o_pred);
   d.s_served = reinterpret_cast<unsigned long long *>(base + o_served);
@@ -302,12 +291,32 @@ int infaas_catalog_load(const infaas_variant *rows, uint32_t n_variants, uint32_
   d.alloc_ctr = reinterpret_cast<unsigned long long *>(base + o_rebuild);
   d.err = reinterpret_cast<uint32_t *>(base + o_err);
   d.slo_seen = reinterpret_cast<uint32_t *>(base + o_seen);
-  c->slot_of_id.swap(slot_of_id);
   c->task_off.swap(task_off);
   c->reg_off.swap(reg_off);
   c->worst_image_bytes = (uint32_t)worst_image;
 
+  {
+    LOAD_TRY(cudaMemcpy(d.image, rows, (size_t)n_variants * sizeof(infaas_variant), cudaMemcpyHostToDevice));
+    LOAD_TRY(cudaMemcpy(d.image + up_rows, members.data(), (size_t)n_variants * 4, cudaMemcpyHostToDevice));
+    infaas::CatalogLayout o{};
+    o.rows = reinterpret_cast<const infaas_variant *>(d.image);
+    o.members = reinterpret_cast<const uint32_t *>(d.image + up_rows);
+    o.task_off = d.task_off;
+    o.s_lat = const_cast<uint32_t *>(d.s_lat); o.s_cost = const_cast<uint32_t *>(d.s_cost);
+    o.s_id = const_cast<uint32_t *>(d.s_id); o.s_queued = d.s_queued;
+    o.s_order = const_cast<uint32_t *>(d.s_order); o.s_cost_run = const_cast<uint32_t *>(d.s_cost_run);
+    o.n_class = const_cast<uint32_t *>(d.n_class);
+    o.slot_of_id = reinterpret_cast<uint32_t *>(base + o_slot_of_id);
+    o.s_batch = const_cast<uint16_t *>(d.s_batch); o.s_acc = const_cast<uint16_t *>(d.s_acc);
+    o.s_arch = c->s_arch; o.s_class = const_cast<uint16_t *>(d.s_class);
+    o.class_acc = const_cast<uint16_t *>(d.class_acc);
+    o.s_qps = c->s_qps; o.hw_by_id = c->hw_by_id;
+    LOAD_TRY(infaas::launch_layout(o, n_tasks, max_task, nullptr));
+    c->slot_of_id.resize(n_variants);
+    LOAD_TRY(cudaMemcpy(c->slot_of_id.data(), o.slot_of_id, (size_t)n_variants * 4, cudaMemcpyDeviceToHost));
+  }
   LOAD_TRY(infaas::prepare_select_kernel());
+  LOAD_TRY(infaas::prepare_tally_kernel());
   LOAD_TRY(infaas::prepare_rebuild_kernel());
   LOAD_TRY(infaas::launch_rebuild(d, /*advance_queues=*/false, 0, nullptr));
   LOAD_TRY(cudaDeviceSynchronize());

@@ -67,8 +67,7 @@ namespace infaas {
 //
 // Per task in global memory (`regions`): keys u64[V] (pred_lat | acc_bp << 32, scan order,
 // F used; for Inactive entries the latency includes the loading latency) and ids u32[V], for
-// lists without an index and for inspection; then local u16[V], the entries' indices inside
-// the task, which the next rebuild uses as its first filter.
+// lists without an index and for inspection.
 // ---------------------------------------------------------------------------------------
 constexpr uint32_t INDEX_MAX_F = 248;
 constexpr uint32_t SLO_BUCKETS = 256;
@@ -148,7 +147,7 @@ inline __host__ __device__ uint32_t block_capacity(uint32_t V, uint32_t nbw) {
   const uint32_t F = V < INDEX_MAX_F ? V : INDEX_MAX_F;
   return block_layout(F, F, F, nbw).bytes;
 }
-inline __host__ __device__ uint32_t region_capacity(uint32_t V) { return round_up_u32(14u * V, 64u); }
+inline __host__ __device__ uint32_t region_capacity(uint32_t V) { return round_up_u32(12u * V, 64u); }
 
 // Slow-path parameters of a list segment (one uint4 each, global memory; a task's first
 // segment at index task, further segments at n_tasks + their index).
@@ -157,8 +156,11 @@ inline __host__ __device__ uint32_t region_capacity(uint32_t V) { return round_u
 // Header of a further segment (xhdr, global memory):
 //   x = t2_off   y = Ka + 1   z = image offset of its bitmap   w = 0
 // ---------------------------------------------------------------------------------------
-// Device catalog.  "Slot" order: variants bucketed by task, ascending id inside a task;
-// task t owns slots task_off[t] .. task_off[t+1]-1 and all s_* arrays are indexed by slot.
+// Device catalog.  "Slot" order: variants bucketed by task, inside a task by (cost, 10000-acc,
+// id); task t owns slots task_off[t] .. task_off[t+1]-1 and all s_* arrays are indexed by slot.
+// A variant's local index is its slot less the task's first.  Cost and accuracy never change, so
+// everything about the list order that does not hang on the predicted latency is laid down here
+// once: s_order, s_cost_run, s_class and class_acc below.
 // ---------------------------------------------------------------------------------------
 struct DeviceCatalog {
   uint32_t n_variants;
@@ -172,6 +174,12 @@ struct DeviceCatalog {
   const uint16_t *s_acc;
   const uint32_t *s_cost;
   const uint32_t *s_id;
+  const uint32_t *s_order;     // position in (10000-acc, local) order (13 bits) | first local index of the
+                               // same (cost, acc) << 13 (13 bits) | bit 31: others share (cost, acc)
+  const uint32_t *s_cost_run;  // local indices of equal cost: first | (last + 1) << 16
+  const uint16_t *s_class;     // rank of the accuracy among the task's distinct ones, 0 = highest
+  const uint16_t *class_acc;   // accuracy of class k of task t at [task_off[t] + k]
+  const uint32_t *n_class;     // [n_tasks] distinct accuracies
   uint32_t *s_queued;
   uint32_t *s_pred;
   unsigned long long *s_served;
@@ -200,6 +208,18 @@ struct DeviceCatalog {
   uint32_t *slo_seen;            // OR of all SLOs the selection kernel has read
 };
 
+// What the layout kernel reads (rows by id; members = each task's ids in ascending order) and the
+// arrays it fills (see DeviceCatalog; s_arch, s_qps = floor(10^9 * batch / lat_us) are the
+// autoscaler's, hw_by_id the worker choice's, slot_of_id the host's).
+struct CatalogLayout {
+  const infaas_variant *rows;
+  const uint32_t *members, *task_off;
+  uint32_t *s_lat, *s_cost, *s_id, *s_queued, *s_order, *s_cost_run, *n_class, *slot_of_id;
+  uint16_t *s_batch, *s_acc, *s_arch, *s_class, *class_acc;
+  unsigned long long *s_qps;
+  unsigned char *hw_by_id;
+};
+
 // Device error codes stored in DeviceCatalog::err.
 enum : uint32_t {
   DEV_ERR_NONE = 0,
@@ -209,14 +229,16 @@ enum : uint32_t {
 // Largest dynamic shared memory the selection kernel may be given (227 KB per CTA on
 // sm_100, minus its static shared memory).
 constexpr uint32_t SELECT_MAX_SMEM = 227u * 1024u - 256u;
-// Sort buffers of the rebuild kernel: 13 bytes per padded entry.
-constexpr uint32_t REBUILD_MAX_SMEM = INFAAS_MAX_TASK_VARIANTS * 13u;
+// Shared memory of the rebuild kernel per variant of the largest task.
+constexpr uint32_t REBUILD_ROW_SMEM = 22u;
 
 // Once per device, with that device current: raise the kernels' shared-memory limits.
 cudaError_t prepare_select_kernel();
+cudaError_t prepare_tally_kernel();
 cudaError_t prepare_rebuild_kernel();
 
 // Launchers (host).  All are asynchronous on `stream` and allocate nothing.
+cudaError_t launch_layout(const CatalogLayout &o, uint32_t n_tasks, uint32_t max_task_variants, cudaStream_t stream);
 cudaError_t launch_rebuild(const DeviceCatalog &c, bool advance_queues, uint32_t window_us,
                            cudaStream_t stream);
 cudaError_t launch_tally(const DeviceCatalog &c, const uint32_t *d_decision, uint64_t n,

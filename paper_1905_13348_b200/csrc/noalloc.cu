@@ -42,9 +42,9 @@ extern "C" int infaas_tally_static(const uint32_t *d_decision, uint64_t n, uint3
     if (!g_scratch_addr[cuda_device]) {
       void *p = nullptr;
       int sms = 0;
-      // (the tally kernels' shared-memory limit is a per-device attribute, set here too)
+      // (the tally kernel's shared-memory limit is a per-device attribute, set here too)
       if ((e = cudaGetSymbolAddress(&p, g_tally_scratch)) != cudaSuccess ||
-          (e = infaas::prepare_rebuild_kernel()) != cudaSuccess ||
+          (e = infaas::prepare_tally_kernel()) != cudaSuccess ||
           (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, cuda_device)) != cudaSuccess) {
         rc = infaas::record_cuda_error(e);
       } else if (!p || sms <= 0) {

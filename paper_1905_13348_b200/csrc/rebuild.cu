@@ -1,0 +1,719 @@
+// Queue recursion, predicted latency and the per-task scan lists with their rank index.
+//
+// Section 4 of the paper says a loaded variant's latency is not its profiled one.  Here each
+// variant's queue is advanced by one window of tallied decisions, its load-adjusted latency is
+// recomputed, and every task's list of non-dominated variants is rebuilt in (cost, pred_lat,
+// -acc, id) order (rebuild kernel).  On a state-aware catalog the same step moves the variants'
+// life-cycle states with the load (Section 4, state machine) and builds the Active and the
+// Inactive list of every task.
+#include "common.cuh"
+
+namespace infaas {
+
+namespace {
+
+constexpr uint32_t NONE = 0xFFFFFFFFu;
+constexpr uint32_t REBUILD_THREADS = 1024;
+constexpr uint32_t REBUILD_WARPS = REBUILD_THREADS / 32;
+
+// IEEE-754 pattern of a u32 converted to float toward zero: a monotone, roughly logarithmic
+// code.  The selection kernel derives the same bucket from it.
+__device__ __forceinline__ uint32_t float_bits(uint32_t x) { return __float_as_uint(__uint2float_rz(x)); }
+// Smallest u32 whose float_bits is >= pattern (pattern below that of 2^32).
+__device__ __forceinline__ uint32_t float_bits_floor(uint32_t pattern) {
+  return __float2uint_ru(__uint_as_float(pattern));
+}
+constexpr uint32_t BITS_OF_2_POW_32 = 0x4F800000u;
+
+// Coarse grid of the prune: at most GRID x GRID cells (row = run of local indices, column = run
+// of positions in accuracy order), one word of padding per row.
+constexpr uint32_t GRID = 64, GRID_PITCH = GRID + 1;
+
+// Shared memory used while building the index of one list segment.
+struct IndexScratch {
+  uint32_t pred[256], ids[256];     // the segment in scan order; latencies behind its end are NONE
+  uint32_t sorted[256];             // its latencies ascending (equal ones in scan order)
+  uint32_t ent[256];                // same order: accuracy rank << 16 | last of its latency << 8 | position
+  uint32_t Pd[256];                 // distinct latencies
+  uint32_t bcnt[256], bthr[256];    // per SLO bucket: distinct latencies inside it, one of them
+  uint32_t wbits[MAX_ACC_WORDS];    // per bitmap word: the accuracies present
+  // per latency rank: the most accurate entry (acc << 16 | 0xFFFF - position, 0 = none); per
+  // accuracy rank: the fastest entry (pred << 32 | position, ~0 = none); then their running
+  // maximum / minimum
+  uint32_t rankA[256], bestA[257];
+  unsigned long long rankB[256], bestB[257];
+  uint16_t acc[256];
+  unsigned char wpre[MAX_ACC_WORDS];         // accuracies present in the words before
+  unsigned char at[256], rank[256];          // sorted order: position, latency rank
+  unsigned char ord_start[257], stair[256];  // per latency rank: stair entries before it; holds one
+  unsigned char part[REBUILD_WARPS * 32];    // rank table: first position per column of a run of entries
+  uint32_t ks, ka, base;
+};
+
+// Fixed part of the image for a task without index (also entry n_tasks): a header word,
+// records and a bitmap that make every query of the task read "none".  All threads.
+__device__ __forceinline__ void write_dummy_task(const DeviceCatalog &c, uint32_t t) {
+  const uint32_t T = c.n_tasks;
+  if (threadIdx.x == 0) reinterpret_cast<uint32_t *>(c.image + IMAGE_HDR_OFFSET)[t] = DUMMY_HEADER;
+  uint32_t *rec = reinterpret_cast<uint32_t *>(c.image + image_rec_offset(T) + t * REC_STRIDE);
+  for (uint32_t j = threadIdx.x; j < SLO_BUCKETS; j += blockDim.x) rec[j] = 0u;
+  uint32_t *bm = reinterpret_cast<uint32_t *>(c.image + image_bitmap_offset(T) + t * bitmap_stride(c.nbw));
+  for (uint32_t j = threadIdx.x; j < c.nbw; j += blockDim.x) bm[j] = 0u;
+}
+
+// Bucket scale of the SLO records: S (16..23) and bmin such that SLO_BUCKETS - 1 buckets of
+// 2^S float patterns cover everything from the catalog's smallest profiled latency up to the
+// largest SLO asked for so far (as a bit mask: every SLO seen is <= cap).
+__device__ __forceinline__ void bucket_scale(const DeviceCatalog &c, uint32_t &Sh, uint32_t &bmin) {
+  uint32_t cap = *c.slo_seen | SLO_CAP_FLOOR_US;
+  cap |= cap >> 1; cap |= cap >> 2; cap |= cap >> 4; cap |= cap >> 8; cap |= cap >> 16;
+  const uint32_t clo = c.lat_code_lo;
+  const uint32_t chi = max(clo, __float_as_uint(__uint2float_rz(cap)) >> 16);
+  uint32_t sh = 0;
+  while ((chi >> sh) - (clo >> sh) > SLO_BUCKETS - 2) ++sh;
+  bmin = clo >> sh;
+  Sh = 16u + sh;
+}
+
+// Sum / OR over the aligned group of 8 lanes this lane belongs to.
+__device__ __forceinline__ uint32_t group8_add(uint32_t v) {
+  v += __shfl_xor_sync(0xFFFFFFFFu, v, 1);
+  v += __shfl_xor_sync(0xFFFFFFFFu, v, 2);
+  v += __shfl_xor_sync(0xFFFFFFFFu, v, 4);
+  return v;
+}
+__device__ __forceinline__ uint32_t group8_or(uint32_t v) {
+  v |= __shfl_xor_sync(0xFFFFFFFFu, v, 1);
+  v |= __shfl_xor_sync(0xFFFFFFFFu, v, 2);
+  v |= __shfl_xor_sync(0xFFFFFFFFu, v, 4);
+  return v;
+}
+
+// Inclusive scans over the lanes of a warp.
+__device__ __forceinline__ uint32_t warp_scan_add(uint32_t x) {
+  const uint32_t lane = threadIdx.x & 31u;
+#pragma unroll
+  for (uint32_t o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+    if (lane >= o) x += y;
+  }
+  return x;
+}
+// (shfl_up leaves the lanes without a source unchanged: minimum and maximum need no guard)
+template <class T>
+__device__ __forceinline__ T warp_scan_min(T x) {
+#pragma unroll
+  for (uint32_t o = 1; o < 32; o <<= 1) x = min(x, __shfl_up_sync(0xFFFFFFFFu, x, o));
+  return x;
+}
+__device__ __forceinline__ uint32_t warp_scan_max(uint32_t x) {
+#pragma unroll
+  for (uint32_t o = 1; o < 32; o <<= 1) x = max(x, __shfl_up_sync(0xFFFFFFFFu, x, o));
+  return x;
+}
+
+// One atomic per allocation places a block in the image and, on a CTA's last allocation
+// (`done`), counts the CTA as finished with the cursor.  The CTA that is counted last knows the
+// final image size: it publishes it for the kernels that follow and clears the counter for the
+// next rebuild.  One thread only, in two halves so that the atomic's round trip can overlap other
+// work: place_block_issue returns the counter's old value, place_block_finish (same arguments)
+// the block's offset behind the fixed part of the image.
+__device__ __forceinline__ unsigned long long place_block_issue(const DeviceCatalog &c, uint32_t bytes, bool done) {
+  return atomicAdd(c.alloc_ctr, ((unsigned long long)(done ? 1u : 0u) << 32) | bytes);
+}
+__device__ __forceinline__ uint32_t place_block_finish(const DeviceCatalog &c, unsigned long long old,
+                                                       uint32_t bytes, bool done) {
+  if (done && (uint32_t)(old >> 32) == gridDim.x - 1u) {
+    c.image_hdr[0] = image_var_offset(c.n_tasks, c.nbw) + (uint32_t)old + bytes;
+    *c.alloc_ctr = 0ull;
+  }
+  return (uint32_t)old;
+}
+
+// Clears what build_index accumulates into (all threads; a barrier must follow).
+__device__ __forceinline__ void clear_scratch(IndexScratch &S) {
+  for (uint32_t i = threadIdx.x; i < 256u; i += REBUILD_THREADS) {
+    S.pred[i] = NONE; S.bcnt[i] = 0u; S.rankA[i] = 0u; S.rankB[i] = ~0ull;
+  }
+  for (uint32_t i = threadIdx.x; i < MAX_ACC_WORDS; i += REBUILD_THREADS) S.wbits[i] = 0u;
+}
+
+// Builds the exact index of a list segment of F <= INDEX_MAX_F entries (layout in common.cuh) into
+// a block of the image obtained from the block cursor.  S.pred / S.acc / S.ids hold the segment
+// in scan order, the accumulators are clear.  Returns false (all threads) if it cannot be
+// indexed: its block lies beyond the image's capacity or beyond what the header's offset field
+// addresses.
+// `xi`: NONE for the task's first segment (header word, SLO records and bitmap go into the
+// fixed part of the image), else the index of this further segment (header to xhdr[xi], bitmap
+// into the block, no records: only the slow path comes here).  `next`: 1 + index of the task's
+// next segment, 0 if this is the last (the CTA's last allocation, then).
+//
+// The chain is bound by latency (barriers and shared-memory round trips), so it has few steps:
+// one pair loop (latency order), accuracy ranks straight from the bitmap, and the rank table as a
+// running minimum down its columns -- F steps per column, cut into runs of entries so that all
+// warps work, instead of F bits per cell.
+__device__ bool build_index(const DeviceCatalog &c, uint32_t t, uint32_t F, IndexScratch &S, uint32_t xi,
+                            uint32_t next) {
+  const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+  constexpr uint32_t B = REBUILD_THREADS;
+  const bool first = xi == NONE;
+  const uint32_t acc_lo = c.acc_lo, nbw = c.nbw;      // the catalog's accuracy window
+
+  // 1. latency order by counting smaller (latency, position), 8 lanes per entry, 4 entries per
+  // load; the accuracies' bits
+  for (uint32_t p0 = 0; p0 < F; p0 += B / 8u) {        // uniform trip count
+    const uint32_t p = p0 + (tid >> 3), sub = tid & 7u;
+    uint32_t cnt = 0, pp = 0;
+    if (p < F) {
+      pp = S.pred[p];
+      for (uint32_t q = 4u * sub; q < F; q += 32u) {
+        const uint4 v = *reinterpret_cast<const uint4 *>(&S.pred[q]);
+        cnt += (uint32_t)(v.x < pp) | ((uint32_t)(v.x == pp) & (uint32_t)(q < p));
+        cnt += (uint32_t)(v.y < pp) | ((uint32_t)(v.y == pp) & (uint32_t)(q + 1u < p));
+        cnt += (uint32_t)(v.z < pp) | ((uint32_t)(v.z == pp) & (uint32_t)(q + 2u < p));
+        cnt += (uint32_t)(v.w < pp) | ((uint32_t)(v.w == pp) & (uint32_t)(q + 3u < p));
+      }
+    }
+    cnt = group8_add(cnt);
+    if (p < F && sub == 0u) {
+      S.sorted[cnt] = pp;
+      S.at[cnt] = (unsigned char)p;
+      const uint32_t x = S.acc[p] - acc_lo, xw = x / ACC_WORD_BITS;
+      atomicOr(&S.wbits[xw], 1u << (x - xw * ACC_WORD_BITS));
+    }
+  }
+  uint32_t bmin, Sh;                                   // SLO buckets
+  bucket_scale(c, Sh, bmin);
+  __syncthreads();
+
+  // 2. dense latency ranks (warps 0-7, one sorted entry per thread), running popcounts of the
+  // accuracy bitmap (warps 8 and up, one word per thread)
+  if (warp < 8u) {
+    const uint32_t i = tid;
+    uint32_t before = 0;
+    for (uint32_t w = 0; w < warp && 32u * w < F; ++w) {
+      const uint32_t x = 32u * w + lane;
+      before += __popc(__ballot_sync(0xFFFFFFFFu, x < F && (x == 0u || S.sorted[x] != S.sorted[x - 1u])));
+    }
+    const bool fresh = i < F && (i == 0u || S.sorted[i] != S.sorted[i - 1u]);
+    const unsigned m = __ballot_sync(0xFFFFFFFFu, fresh);
+    if (i < F) {
+      const uint32_t r = before + __popc(m & ((2u << lane) - 1u)) - 1u;
+      S.rank[i] = (unsigned char)r;
+      if (fresh) {
+        const uint32_t v = S.sorted[i];
+        S.Pd[r] = v;
+        // larger latencies than the largest SLO asked for so far share bucket 255
+        const uint32_t b = min(max(float_bits(v) >> Sh, bmin) - bmin, SLO_BUCKETS - 1u);
+        atomicAdd(&S.bcnt[b], 1u);
+        S.bthr[b] = v;                                 // read only where it is the bucket's only one
+      }
+      if (i == F - 1u) S.ks = r + 1u;
+    }
+  } else {
+    for (uint32_t w0 = 32u * (warp - 8u); w0 < nbw; w0 += B - 256u) {     // uniform per warp
+      uint32_t below = 0;
+      for (uint32_t x = lane; x < w0; x += 32u) below += __popc(S.wbits[x]);
+      below = __reduce_add_sync(0xFFFFFFFFu, below);
+      const uint32_t w = w0 + lane, pc = w < nbw ? __popc(S.wbits[w]) : 0u;
+      const uint32_t incl = below + warp_scan_add(pc);
+      if (w < nbw) S.wpre[w] = (unsigned char)(incl - pc);
+      if (w == nbw - 1u) S.ka = incl;
+    }
+  }
+  __syncthreads();
+  const uint32_t Ks = S.ks, Ka = S.ka, width = Ka + 1u;
+  const BlockLayout BL = block_layout(F, Ks, Ka, first ? 0u : nbw);
+  const SlowLayout SL = slow_layout(F, Ks, Ka);
+
+  // 3. the block's place in the image (the atomic is in flight until step 4 ends); the sorted
+  // entries with their accuracy ranks, and the best entry per rank; SLO records
+  unsigned long long placed = 0;
+  if (tid == B - 1u) placed = place_block_issue(c, BL.bytes, next == 0u);
+  if (tid < F) {
+    const uint32_t p = S.at[tid], r = S.rank[tid], acc = S.acc[p];
+    const uint32_t x = acc - acc_lo, xw = x / ACC_WORD_BITS;
+    const uint32_t ra = S.wpre[xw] + __popc(S.wbits[xw] & ((1u << (x - xw * ACC_WORD_BITS)) - 1u));
+    const uint32_t last = tid == F - 1u || S.rank[tid + 1u] != r;
+    S.ent[tid] = (ra << 16) | (last << 8) | p;
+    atomicMax(&S.rankA[r], (acc << 16) | (0xFFFFu - p));                            // most accurate, first position
+    atomicMin(&S.rankB[ra], ((unsigned long long)S.sorted[tid] << 32) | p);         // fastest, first position
+  }
+  if (first && tid >= B / 2u && tid < B / 2u + SLO_BUCKETS) {
+    // one bucket per thread; lb = latencies in lower buckets
+    uint32_t *rec = reinterpret_cast<uint32_t *>(c.image + image_rec_offset(c.n_tasks) + t * REC_STRIDE);
+    const uint32_t j = tid - B / 2u;
+    uint32_t below = 0;
+    for (uint32_t i = lane; i < (j & ~31u); i += 32u) below += S.bcnt[i];
+    below = __reduce_add_sync(0xFFFFFFFFu, below);
+    const uint32_t cnt = S.bcnt[j], thr = S.bthr[j];
+    const uint32_t lb = below + warp_scan_add(cnt) - cnt;
+    const uint32_t lo = j ? float_bits_floor((bmin + j) << Sh) : 0u;
+    const uint32_t nxt = (bmin + j + 1u) << Sh;
+    const uint32_t hi = (j == SLO_BUCKETS - 1u || nxt >= BITS_OF_2_POW_32) ? NONE : float_bits_floor(nxt) - 1u;
+    uint32_t r = (Ks + 1u) << 24;                                // exact slow path
+    if (cnt == 0u) {
+      r = lb << 24;
+    } else if (cnt == 1u && (lo >> 24) == (hi >> 24)) {
+      r = thr <= lo ? (lb + 1u) << 24 : (lb << 24) | (0x00FFFFFFu - ((thr - 1u) & 0x00FFFFFFu));
+    }
+    rec[j] = r;
+  }
+  __syncthreads();
+
+  // 4. rank table, first half.  T2[r][k] = smallest position among the entries whose latency rank
+  // is < r and whose accuracy rank is >= k: a running minimum over the entries in latency order.
+  // A thread takes one column and one run of entries: here the run's minimum.
+  const uint32_t cols = (width + 31u) >> 5, runs = REBUILD_WARPS / cols;      // warps side by side; at least 4 runs
+  const uint32_t run_len = ((F + runs - 1u) / runs + 3u) & ~3u;
+  const uint32_t run = warp / cols, col = (warp - run * cols) * 32u + lane;
+  const uint32_t i0 = min(F, run * run_len), i1 = run < runs ? min(F, i0 + run_len) : i0;
+  const uint32_t col_key = col << 16;
+  if (i0 < i1) {
+    uint32_t v = 0xFFu;
+#pragma unroll 4
+    for (uint32_t i = i0; i < i1; ++i) {
+      const uint32_t e = S.ent[i];
+      if (e >= col_key) v = min(v, e & 0xFFu);
+    }
+    S.part[run * cols * 32u + col] = (unsigned char)v;
+  }
+  // what the nearest-miss search reads, as running aggregates over the ranks: bestA[r] over
+  // latency ranks < r (and with it the stair entries: those more accurate than everything
+  // faster), bestB[k] over accuracy ranks >= k, ord_start[r] = stair entries with latency rank < r
+  if (warp == 0u) {
+    uint32_t carry = 0, stairs = 0;
+    for (uint32_t c0 = 0; c0 <= Ks; c0 += 32u) {
+      const uint32_t i = c0 + lane, x = i < Ks ? S.rankA[i] : 0u;
+      const uint32_t incl = max(warp_scan_max(x), carry);
+      const uint32_t up = __shfl_up_sync(0xFFFFFFFFu, incl, 1), before = lane ? up : carry;
+      const bool st = i < Ks && (before == 0u || (x >> 16) > (before >> 16));
+      const unsigned m = __ballot_sync(0xFFFFFFFFu, st);
+      if (i <= Ks) {
+        S.bestA[i] = before;
+        S.ord_start[i] = (unsigned char)(stairs + __popc(m & ((1u << lane) - 1u)));
+      }
+      if (i < Ks) S.stair[i] = st;
+      stairs += __popc(m);
+      carry = __shfl_sync(0xFFFFFFFFu, incl, 31);
+    }
+  } else if (warp == 1u) {
+    unsigned long long carry = ~0ull;
+    if (lane == 0u) S.bestB[Ka] = ~0ull;
+    for (uint32_t c0 = 0; c0 < Ka; c0 += 32u) {              // from the top down
+      const uint32_t q = c0 + lane;
+      const unsigned long long x = min(warp_scan_min(q < Ka ? S.rankB[Ka - 1u - q] : ~0ull), carry);
+      if (q < Ka) S.bestB[Ka - 1u - q] = x;
+      carry = __shfl_sync(0xFFFFFFFFu, x, 31);
+    }
+  }
+  if (tid == B - 1u) {
+    uint32_t base = image_var_offset(c.n_tasks, nbw) + place_block_finish(c, placed, BL.bytes, next == 0u);
+    if (base + BL.bytes > c.image_capacity || base + BL.t2 >= IMAGE_T2_LIMIT) base = NONE;
+    S.base = base;
+  }
+  __syncthreads();
+  const uint32_t base = S.base;
+  if (base == NONE) return false;
+  unsigned char *blk = c.image + base;
+  unsigned char *slow = blk + BL.slow;
+
+  // 5. rank table, second half: each run starts from the minimum of the runs before it and writes a
+  // row after the last entry of every latency
+  unsigned char *T2 = blk + BL.t2;
+  if (i0 < i1 && col < width) {
+    uint32_t v = F;
+    for (uint32_t w = 0; w < run; ++w) v = min(v, (uint32_t)S.part[w * cols * 32u + col]);
+    if (run == 0u) T2[col] = (unsigned char)F;                   // nothing is fast enough
+    unsigned char *row = T2 + (S.rank[i0] + 1u) * width + col;
+#pragma unroll 4
+    for (uint32_t i = i0; i < i1; ++i) {
+      const uint32_t e = S.ent[i];
+      if (e >= col_key) v = min(v, e & 0xFFu);
+      if (e & 0x100u) { *row = (unsigned char)v; row += width; }
+    }
+    if (i1 == F) *row = (unsigned char)F;                        // row Ks + 1: the slow path's
+  }
+
+  // the small tables, each by a range of warps of its own: [lo, lo + n) of the CTA's threads run
+  // `body(x)` for x = 0 .. count - 1
+  auto share = [&](uint32_t lo, uint32_t n, uint32_t count, auto body) {
+    if (tid >= lo && tid < lo + n)
+      for (uint32_t x = tid - lo; x < count; x += n) body(x);
+  };
+  uint32_t *bitmap = first ? reinterpret_cast<uint32_t *>(c.image + image_bitmap_offset(c.n_tasks) + t * bitmap_stride(nbw))
+                           : reinterpret_cast<uint32_t *>(blk + BL.bitmap);
+  share(0, B / 4u, nbw, [&](uint32_t w) { bitmap[w] = ((uint32_t)S.wpre[w] << 24) | S.wbits[w]; });
+  uint32_t *bestA = reinterpret_cast<uint32_t *>(slow + SL.bestA);
+  uint2 *walk = reinterpret_cast<uint2 *>(slow + SL.walk);      // the stair entries, ascending latency
+  share(B / 4u, B / 4u, Ks + 1u, [&](uint32_t r) {               // position 0xFF stands for "none"
+    const uint32_t v = S.bestA[r], o = S.ord_start[r];
+    bestA[r] = v ? (v >> 16) | ((0xFFFFu - (v & 0xFFFFu)) << 16) : 0xFFu << 16;
+    slow[SL.ordStart + r] = (unsigned char)o;
+    if (r < Ks && S.stair[r]) {
+      const uint32_t a = S.rankA[r];
+      walk[o] = make_uint2(S.Pd[r], (a >> 16) | ((0xFFFFu - (a & 0xFFFFu)) << 16));
+    }
+    if (r == Ks) {
+      const uint32_t nxt = next;
+      c.slow[first ? t : c.n_tasks + xi] = make_uint4(base + BL.slow, F | (Ks << 8) | (Ka << 16), 0u, o | (nxt << 8));
+    }
+  });
+  uint2 *bestB = reinterpret_cast<uint2 *>(slow + SL.bestB);
+  share(B / 2u, B / 4u, Ka + 1u, [&](uint32_t k) {
+    const unsigned long long v = S.bestB[k];
+    bestB[k] = v == ~0ull ? make_uint2(0u, 0xFFu) : make_uint2((uint32_t)(v >> 32), (uint32_t)v);
+  });
+  uint32_t *ids_end = reinterpret_cast<uint32_t *>(blk + BL.t2);   // ids, reversed; slot F holds PENDING
+  uint32_t *Pd_g = reinterpret_cast<uint32_t *>(slow + SL.Pd);
+  share(3u * B / 4u, B / 4u, F + 1u, [&](uint32_t p) {
+    ids_end[-1 - (int)p] = p < F ? S.ids[p] : PENDING;
+    if (p < Ks) Pd_g[p] = S.Pd[p];
+  });
+  if (tid == 0u) {
+    if (first) reinterpret_cast<uint32_t *>(c.image + IMAGE_HDR_OFFSET)[t] = (base + BL.t2) | (width << 24);
+    else c.xhdr[xi] = make_uint4(base + BL.t2, width, base + BL.bitmap, 0u);
+  }
+  return true;
+}
+
+// What the queue recursion reads of one variant.
+struct Row {
+  uint32_t lat, batch, queued, id, order, count, state, load_lat;
+  unsigned long long served;
+};
+__device__ __forceinline__ Row load_row(const DeviceCatalog &c, uint32_t slot, bool advance) {
+  Row r;
+  r.lat = c.s_lat[slot];
+  r.batch = c.s_batch[slot];
+  r.queued = c.s_queued[slot];
+  r.order = c.s_order[slot];
+  r.id = 0; r.count = 0; r.served = 0; r.state = INFAAS_STATE_ACTIVE; r.load_lat = 0;
+  if (c.stateful) { r.state = c.s_state[slot]; r.load_lat = c.s_load_lat[slot]; }
+  if (advance) {
+    r.id = c.s_id[slot];
+    r.served = c.s_served[slot];
+    r.count = c.count_by_id[r.id];
+  }
+  return r;
+}
+// Queue recursion and states; returns the predicted latency and leaves the new state in r.state.
+__device__ __forceinline__ uint32_t advance_row(const DeviceCatalog &c, uint32_t slot, Row &r, bool advance,
+                                                uint32_t window_us) {
+  uint32_t queued = r.queued;
+  if (advance) {
+    unsigned long long arrived = (unsigned long long)queued + r.count;
+    if (arrived > NONE) arrived = NONE;
+    unsigned long long drain = (unsigned long long)window_us * r.batch / r.lat;
+    if (drain > NONE) drain = NONE;
+    queued = arrived > drain ? (uint32_t)(arrived - drain) : 0u;
+    c.s_served[slot] = r.served + r.count;
+    c.s_queued[slot] = queued;
+    c.count_by_id[r.id] = 0;        // not right behind its load: a store to an address whose load is
+                                    // still in flight holds up everything behind it (measured: 4 us)
+    if (c.stateful) {
+      // loaded by its first queries; at peak throughput while a backlog remains
+      if (r.state == INFAAS_STATE_INACTIVE && r.count > 0) r.state = INFAAS_STATE_ACTIVE;
+      if (r.state == INFAAS_STATE_ACTIVE || r.state == INFAAS_STATE_OVERLOADED)
+        r.state = queued > 0 ? INFAAS_STATE_OVERLOADED : INFAAS_STATE_ACTIVE;
+      c.s_state[slot] = (unsigned char)r.state;
+    }
+  }
+  const unsigned long long p = (unsigned long long)r.lat + (unsigned long long)queued * r.lat / r.batch;
+  const uint32_t pred = p > NONE ? NONE : (uint32_t)p;
+  c.s_pred[slot] = pred;
+  return pred;
+}
+
+// One CTA per task.
+//
+// List of the Active variants (all variants of a catalog without states).  Slots are in (cost,
+// 10000-acc, id) order, so with `order` = position in (10000-acc, local) order a variant q before
+// p in both orders with pred_q <= pred_p dominates p, and the only other way to be dominated is a
+// faster variant of the same cost and accuracy.  The two orders never change, only pred does, so
+// nothing is sorted: pred is reduced into a grid of at most 64 x 64 cells (runs of local indices
+// x runs of positions in accuracy order); after a running minimum along rows and columns, the cell
+// diagonally before p's tells whether something in a strictly earlier row and column dominates it.
+// What passes (a few more than survive) is compared with the entries of its own row and column
+// only.  Survivors of equal cost are a staircase (later in accuracy order = faster), so list
+// positions follow from counting survivors: those before the run of equal cost, then the run
+// backwards.
+//
+// List of the Inactive variants: ordered by (eff, 10000-acc, id) with eff in place of cost and
+// pred; at most the fastest variant (lowest id) of every distinct accuracy is on it, if it is
+// faster than everything more accurate, and the list runs from the lowest accuracy up.
+//
+// Bound by the latency of its chain of barriers, shared-memory round trips and the loads at its
+// start; measured on one B200: 64 tasks x 256 variants, lists of up to 100 entries: 10.8 us (22.9
+// with pair loops over variants and survivors), 128 x 512: 12.2 us (33.8), 4 x 4096 on a trade-off
+// surface, lists of up to 505 entries: 52 us (340 with a sort and a scan of the sorted entries).
+__global__ void __launch_bounds__(REBUILD_THREADS)
+rebuild_kernel(DeviceCatalog c, int advance, uint32_t window_us) {
+  extern __shared__ __align__(16) unsigned char dyn[];
+  constexpr uint32_t KEEP_WORDS = INFAAS_MAX_TASK_VARIANTS / 32;
+  constexpr uint32_t POOL = sizeof(IndexScratch) > GRID * GRID_PITCH * 4 ? sizeof(IndexScratch) : GRID * GRID_PITCH * 4;
+  __shared__ __align__(16) unsigned char pool[POOL];              // the grid, then the index scratch
+  __shared__ uint32_t keep[KEEP_WORDS + 1], keep_pre[KEEP_WORDS + 1];
+  __shared__ unsigned long long warp_min[REBUILD_WARPS];
+  __shared__ uint32_t warp_cnt[REBUILD_WARPS];
+  __shared__ uint32_t n_cand;
+  uint32_t *grid = reinterpret_cast<uint32_t *>(pool);
+  IndexScratch &S = *reinterpret_cast<IndexScratch *>(pool);
+  constexpr uint32_t B = REBUILD_THREADS;
+
+  const uint32_t t = blockIdx.x, tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+  const uint32_t base = c.task_off[t], V = c.task_off[t + 1] - base;
+  // shared memory per variant (REBUILD_ROW_SMEM bytes)
+  uint2 *by_local = reinterpret_cast<uint2 *>(dyn);               // (pred, accuracy position); position 0xFFFF: not listed
+  uint2 *by_acc = by_local + V;                                    // accuracy order: (pred, local); local 0xFFFF: not listed
+  uint32_t *run_min = reinterpret_cast<uint32_t *>(by_acc + V);   // at the first of each (cost, accuracy): smallest pred
+  uint16_t *cand = reinterpret_cast<uint16_t *>(run_min + V);     // entries the grid lets through
+
+  unsigned char *region = c.regions + c.reg_off[t];
+  unsigned long long *keys_g = reinterpret_cast<unsigned long long *>(region);
+  uint32_t *ids_g = reinterpret_cast<uint32_t *>(region + 8u * V);
+
+  // 1. queue recursion, states, predicted latencies; coarse grid.  Each thread's first variant
+  // stays in registers.
+  Row r0;
+  uint32_t acc0 = 0, run0 = 0, pred0 = 0;
+  if (tid < V) {
+    r0 = load_row(c, base + tid, advance);
+    acc0 = c.s_acc[base + tid];
+    run0 = c.s_cost_run[base + tid];
+    if (!advance) r0.id = c.s_id[base + tid];
+  }
+  uint32_t cs = 4;                                                 // log2 of the rows' and columns' run length
+  while (V > (GRID << cs)) ++cs;
+  const uint32_t ng = (V + (1u << cs) - 1u) >> cs;
+  for (uint32_t i = tid; i < ng * GRID_PITCH; i += B) grid[i] = NONE;
+  for (uint32_t i = tid; i < V; i += B) run_min[i] = NONE;
+  for (uint32_t i = tid; i <= KEEP_WORDS; i += B) keep[i] = 0u;
+  if (tid == 0u) n_cand = 0u;
+  __syncthreads();
+  for (uint32_t i = tid; i < V; i += B) {
+    Row r = i == tid ? r0 : load_row(c, base + i, advance);
+    const uint32_t pred = advance_row(c, base + i, r, advance, window_us);
+    const uint32_t pos = r.order & 0x1FFFu;
+    if (r.state == INFAAS_STATE_ACTIVE) {
+      by_local[i] = make_uint2(pred, pos);
+      by_acc[pos] = make_uint2(pred, i);
+      // NONE stands for "no entry" in the grid: a saturated latency counts as one less there
+      atomicMin(&grid[(i >> cs) * GRID_PITCH + (pos >> cs)], min(pred, NONE - 1u));
+      if (r.order >> 31) atomicMin(&run_min[(r.order >> 13) & 0x1FFFu], pred);
+    } else {
+      by_local[i] = make_uint2(NONE, 0xFFFFu);
+      by_acc[pos] = make_uint2(NONE, 0xFFFFu);
+    }
+    if (i == tid) { pred0 = pred; r0.state = r.state; }
+  }
+  __syncthreads();
+  // 2. running minimum along the rows, then down the columns (GRID = two values per lane)
+  for (uint32_t y = warp; y < ng; y += REBUILD_WARPS) {
+    uint32_t *row = grid + y * GRID_PITCH;
+    const uint32_t x0 = warp_scan_min(lane < ng ? row[lane] : NONE);
+    if (lane < ng) row[lane] = x0;
+    if (ng > 32u) {
+      const uint32_t carry = __shfl_sync(0xFFFFFFFFu, x0, 31);
+      const uint32_t x1 = min(warp_scan_min(lane + 32u < ng ? row[lane + 32u] : NONE), carry);
+      if (lane + 32u < ng) row[lane + 32u] = x1;
+    }
+  }
+  __syncthreads();
+  for (uint32_t x = warp; x < ng; x += REBUILD_WARPS) {
+    uint32_t *col = grid + x;
+    const uint32_t x0 = warp_scan_min(lane < ng ? col[lane * GRID_PITCH] : NONE);
+    if (lane < ng) col[lane * GRID_PITCH] = x0;
+    if (ng > 32u) {
+      const uint32_t carry = __shfl_sync(0xFFFFFFFFu, x0, 31);
+      const uint32_t x1 = min(warp_scan_min(lane + 32u < ng ? col[(lane + 32u) * GRID_PITCH] : NONE), carry);
+      if (lane + 32u < ng) col[(lane + 32u) * GRID_PITCH] = x1;
+    }
+  }
+  __syncthreads();
+  // 3. what the grid lets through ...
+  for (uint32_t i0 = 0; i0 < V; i0 += B) {
+    const uint32_t i = i0 + tid;
+    bool pass = false;
+    if (i < V) {
+      const uint2 a = by_local[i];
+      if (a.y != 0xFFFFu) {
+        const uint32_t y = i >> cs, x = a.y >> cs;
+        const uint32_t g = y && x ? grid[(y - 1u) * GRID_PITCH + x - 1u] : NONE;
+        const uint32_t order = i0 ? c.s_order[base + i] : r0.order;
+        // (a latency of NONE - 1 cannot be told from a saturated one in the grid: step 4 looks at all)
+        pass = g > min(a.x, NONE - 1u) || (a.x == NONE - 1u && g == NONE - 1u);
+        if (order >> 31) pass = pass && a.x <= run_min[(order >> 13) & 0x1FFFu];
+      }
+    }
+    const unsigned m = __ballot_sync(0xFFFFFFFFu, pass);
+    uint32_t at = 0;
+    if (m && lane == 0u) at = atomicAdd(&n_cand, (uint32_t)__popc(m));
+    at = __shfl_sync(0xFFFFFFFFu, at, 0);
+    if (pass) cand[at + __popc(m & ((1u << lane) - 1u))] = (uint16_t)i;
+  }
+  __syncthreads();
+  // 4. ... against its own row and column of the grid, 8 lanes per entry
+  const uint32_t nc = n_cand;
+  for (uint32_t x0 = 0; x0 < nc; x0 += B / 8u) {
+    const uint32_t x = x0 + (tid >> 3), sub = tid & 7u;
+    uint32_t dom = 0, p = 0;
+    if (x < nc) {
+      p = cand[x];
+      const uint2 a = by_local[p];
+      const uint32_t lo = a.x == NONE - 1u ? 0u : (p >> cs) << cs;
+      for (uint32_t q = lo + sub; q < p; q += 8u) {
+        const uint2 b = by_local[q];
+        dom |= (uint32_t)(b.x <= a.x) & (uint32_t)(b.y < a.y);
+      }
+      for (uint32_t j = ((a.y >> cs) << cs) + sub; j < a.y; j += 8u) {
+        const uint2 b = by_acc[j];
+        dom |= (uint32_t)(b.x <= a.x) & (uint32_t)(b.y < p);
+      }
+    }
+    dom = group8_or(dom);
+    if (x < nc && sub == 0u && !dom) atomicOr(&keep[p >> 5], 1u << (p & 31u));
+  }
+  __syncthreads();
+  // 5. survivors before each word of the bit set (warp 0); scratch of the next steps
+  const uint32_t n_words = (V + 31u) >> 5;
+  if (warp == 0u) {
+    uint32_t carry = 0;
+    for (uint32_t w0 = 0; w0 <= n_words; w0 += 32u) {
+      const uint32_t w = w0 + lane, pc = w < n_words ? __popc(keep[w]) : 0u;
+      const uint32_t incl = carry + warp_scan_add(pc);
+      if (w <= n_words) keep_pre[w] = incl - pc;
+      carry = __shfl_sync(0xFFFFFFFFu, incl, 31);
+    }
+  }
+  clear_scratch(S);                                                // the grid is not needed any more
+  unsigned long long *class_best = reinterpret_cast<unsigned long long *>(by_acc);   // nor is by_acc
+  const uint32_t n_class = c.stateful ? c.n_class[t] : 0u;
+  for (uint32_t k = tid; k < n_class; k += B) class_best[k] = ~0ull;
+  __syncthreads();
+  // 6. the list into the task's region, its first segment also into the index scratch
+  auto emit = [&](uint32_t pos, uint32_t pred, uint32_t acc, uint32_t id) {
+    keys_g[pos] = ((unsigned long long)acc << 32) | pred;
+    ids_g[pos] = id;
+    if (pos < INDEX_MAX_F) { S.ids[pos] = id; S.pred[pos] = pred; S.acc[pos] = (uint16_t)acc; }
+  };
+  auto before = [&](uint32_t i) { return keep_pre[i >> 5] + __popc(keep[i >> 5] & ((1u << (i & 31u)) - 1u)); };
+  for (uint32_t i = tid; i < V; i += B) {
+    if (!((keep[i >> 5] >> (i & 31u)) & 1u)) continue;
+    const bool reg = i == tid;
+    const uint32_t run = reg ? run0 : c.s_cost_run[base + i];
+    const uint32_t pos = before(run & 0xFFFFu) + before(run >> 16) - 1u - before(i);
+    emit(pos, reg ? pred0 : by_local[i].x, reg ? acc0 : c.s_acc[base + i], reg ? r0.id : c.s_id[base + i]);
+  }
+  uint32_t F = keep_pre[n_words];
+  if (c.stateful) {
+    for (uint32_t i = tid; i < V; i += B) {
+      const uint32_t st = i == tid ? r0.state : c.s_state[base + i];
+      if (st != INFAAS_STATE_INACTIVE) continue;
+      const unsigned long long e = (unsigned long long)(i == tid ? pred0 : c.s_pred[base + i]) +
+                                   (i == tid ? r0.load_lat : c.s_load_lat[base + i]);
+      const uint32_t eff = e > NONE ? NONE : (uint32_t)e;
+      atomicMin(&class_best[c.s_class[base + i]], ((unsigned long long)eff << 32) | (i == tid ? r0.id : c.s_id[base + i]));
+    }
+    __syncthreads();
+    // each thread takes consecutive classes: running minimum from the highest accuracy down,
+    // survivors, their number
+    const uint32_t per = (n_class + B - 1u) / B, k0 = min(n_class, tid * per), k1 = min(n_class, k0 + per);
+    unsigned long long mine = ~0ull;
+    for (uint32_t k = k0; k < k1; ++k) mine = min(mine, class_best[k]);
+    const unsigned long long incl = warp_scan_min(mine);
+    if (lane == 31u) warp_min[warp] = incl;
+    __syncthreads();
+    unsigned long long best = __shfl_up_sync(0xFFFFFFFFu, incl, 1);
+    if (lane == 0u) best = ~0ull;
+    for (uint32_t w = 0; w < warp; ++w) best = min(best, warp_min[w]);
+    // on the list: faster than every more accurate variant (equally fast ones are dominated)
+    auto listed = [](unsigned long long x, unsigned long long ahead) {
+      return x != ~0ull && (ahead == ~0ull || (uint32_t)(x >> 32) < (uint32_t)(ahead >> 32));
+    };
+    uint32_t n = 0;
+    unsigned long long ahead = best;
+    for (uint32_t k = k0; k < k1; ++k) {
+      n += listed(class_best[k], ahead);
+      ahead = min(ahead, class_best[k]);
+    }
+    const uint32_t n_incl = warp_scan_add(n);
+    if (lane == 31u) warp_cnt[warp] = n_incl;
+    __syncthreads();
+    uint32_t ahead_n = n_incl - n, total = 0;
+    for (uint32_t w = 0; w < REBUILD_WARPS; ++w) {
+      ahead_n += w < warp ? warp_cnt[w] : 0u;
+      total += warp_cnt[w];
+    }
+    ahead = best;
+    for (uint32_t k = k0; k < k1; ++k) {
+      const unsigned long long x = class_best[k];
+      if (listed(x, ahead)) { emit(F + total - 1u - ahead_n, (uint32_t)(x >> 32), c.class_acc[base + k], (uint32_t)x); ++ahead_n; }
+      ahead = min(ahead, x);
+    }
+    F += total;
+  }
+  __syncthreads();
+  bool indexed = F > 0;
+  bool counted = false;                       // has this CTA made its last allocation?
+  // index the list -- the two lists of a state-aware catalog count as one, the Inactive entries
+  // behind the Active ones: "first position that meets both requirements, else the smallest
+  // distance at the lowest position" is all the index knows about order -- segment by segment
+  // (INDEX_MAX_F positions each; almost always one)
+  if (indexed) {
+    const uint32_t nseg = (F + INDEX_MAX_F - 1u) / INDEX_MAX_F, x0 = c.seg_base[t];
+    for (uint32_t sg = 0; sg < nseg && indexed; ++sg) {
+      const uint32_t off = sg * INDEX_MAX_F, Fseg = min(INDEX_MAX_F, F - off);
+      if (sg) {                                   // later segments: back from the task's region
+        __syncthreads();
+        clear_scratch(S);
+        __syncthreads();
+        for (uint32_t i = tid; i < Fseg; i += B) {
+          const unsigned long long e = keys_g[off + i];
+          S.ids[i] = ids_g[off + i]; S.pred[i] = (uint32_t)e; S.acc[i] = (uint16_t)(e >> 32);
+        }
+        __syncthreads();
+      }
+      indexed = build_index(c, t, Fseg, S, sg ? x0 + sg - 1u : NONE, sg + 1u < nseg ? x0 + sg + 1u : 0u);
+      counted = sg + 1u == nseg;
+    }
+  }
+  if (!counted && tid == 0u) place_block_finish(c, place_block_issue(c, 0u, true), 0u, true);   // nothing (more) to place
+  if (!indexed) {
+    // no index: every query of this task reads "none"
+    write_dummy_task(c, t);
+    if (tid == 0u) c.slow[t] = make_uint4(0u, 0u, F == 0 ? TASK_FLAG_INVALID : TASK_FLAG_NOT_INDEXED, 0u);
+  }
+  if (t == 0u) {
+    // entry n_tasks (queries whose task is out of range), the dummy block, and the bucket scale
+    // every CTA has used, for the selection kernel
+    write_dummy_task(c, c.n_tasks);
+    if (tid < IMAGE_DUMMY_BYTES / 4u) reinterpret_cast<uint32_t *>(c.image)[tid] = tid == 3u ? PENDING : 0u;
+    if (tid == 0u) {
+      uint32_t Sh, bmin;
+      bucket_scale(c, Sh, bmin);
+      c.image_hdr[1] = (127u - Sh) << 23;
+      c.image_hdr[2] = __float_as_uint(-(float)bmin);
+    }
+  }
+  if (tid == 0u) c.f_len[t] = F;
+}
+
+// The block sizes the thread ranges above rely on.
+static_assert(REBUILD_THREADS == 1024 && SLO_BUCKETS == 256 && INDEX_MAX_F < 256, "thread ranges of build_index");
+
+}  // namespace
+
+cudaError_t prepare_rebuild_kernel() {
+  return cudaFuncSetAttribute(rebuild_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)(INFAAS_MAX_TASK_VARIANTS * REBUILD_ROW_SMEM));
+}
+
+cudaError_t launch_rebuild(const DeviceCatalog &c, bool advance_queues, uint32_t window_us,
+                           cudaStream_t stream) {
+  const size_t smem = (size_t)c.max_task_variants * REBUILD_ROW_SMEM;
+  rebuild_kernel<<<c.n_tasks, REBUILD_THREADS, smem, stream>>>(c, advance_queues ? 1 : 0, window_us);
+  return cudaGetLastError();
+}
+
+}  // namespace infaas

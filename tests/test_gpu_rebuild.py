@@ -1,0 +1,71 @@
+"""GPU parity of the list rebuild at the sizes where its grid, its per-thread rows and its index
+segments have edges: lists against the oracle's, decisions and load state through a few windows."""
+import numpy as np
+import pytest
+
+from oracle import OracleCatalog
+from paper_1905_13348_b200 import workloads as W
+from tests.helpers import rows_from
+from tests.test_gpu_parity import assert_state_equal, run_both
+from tests.test_gpu_stateful import _states, run_stateful
+
+pytestmark = pytest.mark.gpu
+
+# rows and columns of the grid hold 16 variants up to 1024 variants, 32 up to 2048 and so on; a
+# thread has one variant up to 1024; 8192 is the limit
+SIZES = [1, 15, 17, 31, 33, 255, 257, 512, 1023, 1025, 2049, 8192]
+
+
+def _workload(V, kind, n=6000, window=1999):
+    rng = np.random.default_rng([V, len(kind)])
+    sizes = [V, 0, max(1, V // 3)]
+    task = np.repeat(np.arange(3), sizes)
+    N = task.size
+    lat = np.exp(rng.uniform(np.log(500.0), np.log(2e6), N)).astype(np.int64)
+    batch = rng.choice([1, 2, 7, 64, 65535], N)
+    if kind == "ties":                    # few costs, accuracies and latencies: runs of equal (cost, accuracy)
+        cost, acc = rng.integers(1, 4, N), 7000 + 30 * rng.integers(0, 5, N)
+        lat = rng.choice([1000, 4000, 20_000, 20_001], N)
+        queued = rng.choice([0, 0, 5], N)
+    elif kind == "one":                   # a single cost and accuracy
+        cost, acc, queued = np.full(N, 9), np.full(N, 8000), rng.integers(0, 3, N)
+    elif kind == "saturated":             # predicted latencies of 2^32-2 and 2^32-1 among ordinary ones
+        cost, acc = rng.integers(1, 500, N), rng.integers(0, 10001, N)
+        pick = rng.random(N)
+        lat = np.where(pick < 0.4, 2**32 - 2, np.where(pick < 0.8, 2**32 - 1, lat))
+        queued = rng.choice([0, 0, 0, 2**32 - 1], N)
+    else:                                 # a trade-off: long lists
+        cost = (4e7 / lat**0.6 * np.exp(0.2 * rng.standard_normal(N))).astype(np.int64) + 1
+        acc = np.clip(3000 + 900 * np.log10(lat) + 150 * rng.standard_normal(N), 0, 10000).astype(np.int64)
+        queued = np.zeros(N, np.int64)
+    rows = rows_from(task, batch, lat, acc, cost, queued)
+    rows = rows[rng.permutation(N)].copy()
+    q_task = rng.choice([0, 0, 0, 1, 2, 3], n).astype(np.uint16)
+    q_slo = np.exp(rng.uniform(np.log(300.0), np.log(4.2e9), n)).astype(np.uint64).clip(0, 2**32 - 1).astype(np.uint32)
+    q_slo[::97] = 2**32 - 2
+    q_acc = rng.choice(np.concatenate([rows["acc_bp"], [0, 9999]]), n).astype(np.uint16)
+    return W.Workload(f"{kind}{V}", 3, rows, q_task, q_slo, q_acc, window, 3_000, "edges of the rebuild")
+
+
+@pytest.mark.parametrize("kind", ["ties", "one", "saturated", "tradeoff"])
+@pytest.mark.parametrize("V", SIZES)
+def test_lists_and_decisions_at_the_edges(V, kind):
+    import paper_1905_13348_b200 as P
+    w = _workload(V, kind)
+    cat, o = P.infaas_catalog_load(w.rows, w.n_tasks), OracleCatalog(w.rows, w.n_tasks)
+    try:
+        assert_state_equal(cat, o)
+        for t in range(w.n_tasks):
+            assert np.array_equal(P.infaas_catalog_get_frontier(cat, t), o.frontier(t)), t
+    finally:
+        cat.free()
+    run_both(w)
+
+
+@pytest.mark.parametrize("kind", ["ties", "saturated", "tradeoff"])
+@pytest.mark.parametrize("V", [17, 257, 1025, 8192])
+def test_two_lists_at_the_edges(V, kind):
+    w = _workload(V, kind)
+    rng = np.random.default_rng(V)
+    load = rng.choice(np.array([0, 1, 5000, 2**32 - 1], np.uint32), w.n_variants)
+    run_stateful(w, _states(rng, w.n_variants, (0.45, 0.45, 0.05, 0.05)), load)
