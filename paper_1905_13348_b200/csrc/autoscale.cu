@@ -59,6 +59,8 @@ autoscale_kernel(DeviceCatalog c, const uint32_t *s_inst, const uint16_t *s_arch
   __shared__ uint32_t s_r;                       // slot of the running variant, ~0 if none
   const uint32_t t = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t lo = c.task_off[t], hi = c.task_off[t + 1];
+  chain_wait();
+  chain_next();
 
   // load served, capacity of what runs, and which running variant served most (ties: lower id)
   unsigned long long served = 0, cap = 0, key = 0;
@@ -149,9 +151,8 @@ cudaError_t launch_autoscale(const DeviceCatalog &c, const uint32_t *s_inst, con
                              const unsigned long long *s_qps, const uint32_t *task_slo, uint32_t window_us, uint32_t slack_pct,
                              uint32_t lambda_milli, uint32_t *d_variant, uint32_t *d_delta,
                              cudaStream_t stream) {
-  autoscale_kernel<<<c.n_tasks, AUTOSCALE_THREADS, 0, stream>>>(c, s_inst, s_arch, s_qps, task_slo, window_us, slack_pct,
-                                                                lambda_milli, d_variant, d_delta);
-  return cudaGetLastError();
+  return launch_chained(autoscale_kernel, c.n_tasks, AUTOSCALE_THREADS, 0, stream, c, s_inst, s_arch, s_qps, task_slo,
+                        window_us, slack_pct, lambda_milli, d_variant, d_delta);
 }
 
 }  // namespace infaas

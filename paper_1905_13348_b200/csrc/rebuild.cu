@@ -382,20 +382,24 @@ struct Row {
   uint32_t lat, batch, queued, id, order, count, state, load_lat;
   unsigned long long served;
 };
-__device__ __forceinline__ Row load_row(const DeviceCatalog &c, uint32_t slot, bool advance) {
+// ... what no kernel writes
+__device__ __forceinline__ Row load_fixed(const DeviceCatalog &c, uint32_t slot) {
   Row r;
   r.lat = c.s_lat[slot];
   r.batch = c.s_batch[slot];
-  r.queued = c.s_queued[slot];
   r.order = c.s_order[slot];
-  r.id = 0; r.count = 0; r.served = 0; r.state = INFAAS_STATE_ACTIVE; r.load_lat = 0;
+  r.id = c.s_id[slot];
+  return r;
+}
+// ... and the rest
+__device__ __forceinline__ void load_load(const DeviceCatalog &c, uint32_t slot, bool advance, Row &r) {
+  r.queued = c.s_queued[slot];
+  r.count = 0; r.served = 0; r.state = INFAAS_STATE_ACTIVE; r.load_lat = 0;
   if (c.stateful) { r.state = c.s_state[slot]; r.load_lat = c.s_load_lat[slot]; }
   if (advance) {
-    r.id = c.s_id[slot];
-    r.served = c.s_served[slot];
     r.count = c.count_by_id[r.id];
+    r.served = c.s_served[slot];
   }
-  return r;
 }
 // Queue recursion and states; returns the predicted latency and leaves the new state in r.state.
 __device__ __forceinline__ uint32_t advance_row(const DeviceCatalog &c, uint32_t slot, Row &r, bool advance,
@@ -478,11 +482,13 @@ rebuild_kernel(DeviceCatalog c, int advance, uint32_t window_us) {
   Row r0;
   uint32_t acc0 = 0, run0 = 0, pred0 = 0;
   if (tid < V) {
-    r0 = load_row(c, base + tid, advance);
+    r0 = load_fixed(c, base + tid);
     acc0 = c.s_acc[base + tid];
     run0 = c.s_cost_run[base + tid];
-    if (!advance) r0.id = c.s_id[base + tid];
   }
+  chain_wait();
+  chain_next();
+  if (tid < V) load_load(c, base + tid, advance, r0);
   uint32_t cs = 4;                                                 // log2 of the rows' and columns' run length
   while (V > (GRID << cs)) ++cs;
   const uint32_t ng = (V + (1u << cs) - 1u) >> cs;
@@ -492,7 +498,11 @@ rebuild_kernel(DeviceCatalog c, int advance, uint32_t window_us) {
   if (tid == 0u) n_cand = 0u;
   __syncthreads();
   for (uint32_t i = tid; i < V; i += B) {
-    Row r = i == tid ? r0 : load_row(c, base + i, advance);
+    Row r = r0;
+    if (i != tid) {
+      r = load_fixed(c, base + i);
+      load_load(c, base + i, advance, r);
+    }
     const uint32_t pred = advance_row(c, base + i, r, advance, window_us);
     const uint32_t pos = r.order & 0x1FFFu;
     if (r.state == INFAAS_STATE_ACTIVE) {
@@ -712,8 +722,7 @@ cudaError_t prepare_rebuild_kernel() {
 cudaError_t launch_rebuild(const DeviceCatalog &c, bool advance_queues, uint32_t window_us,
                            cudaStream_t stream) {
   const size_t smem = (size_t)c.max_task_variants * REBUILD_ROW_SMEM;
-  rebuild_kernel<<<c.n_tasks, REBUILD_THREADS, smem, stream>>>(c, advance_queues ? 1 : 0, window_us);
-  return cudaGetLastError();
+  return launch_chained(rebuild_kernel, c.n_tasks, REBUILD_THREADS, smem, stream, c, advance_queues ? 1 : 0, window_us);
 }
 
 }  // namespace infaas

@@ -457,6 +457,8 @@ select_kernel(DeviceCatalog c, uint32_t stage_bytes, Queries q, uint64_t n, uint
   const uint64_t q0 = (uint64_t)blockIdx.x * per_cta;
   if (q0 >= n) return;
   const uint32_t span = (uint32_t)min(n - q0, per_cta);     // <= MAX_SPAN (checked by the launcher)
+  chain_wait();
+  chain_next();
   // Everything the kernel has to wait for before its first decision starts at once: the staging
   // of `stage_bytes` (what the host planned for: the reserved room or the image buffer, whichever
   // is smaller -- the bytes behind the live image are never looked at), the words the last rebuild
@@ -518,11 +520,8 @@ cudaError_t launch_select(const DeviceCatalog &c, const uint16_t *d_task, const 
   if (grid > 0x7FFFFFFFull) return cudaErrorInvalidValue;
   Queries q{d_task, d_slo, d_min_acc, d_decision};
   const uint32_t stage_bytes = (image_smem < c.image_capacity ? image_smem : c.image_capacity) & ~15u;
-  if (tally)
-    select_kernel<true><<<(uint32_t)grid, SELECT_THREADS, image_smem + PARK_BYTES, stream>>>(c, stage_bytes, q, n, per_cta);
-  else
-    select_kernel<false><<<(uint32_t)grid, SELECT_THREADS, image_smem + PARK_BYTES, stream>>>(c, stage_bytes, q, n, per_cta);
-  return cudaGetLastError();
+  return launch_chained(tally ? select_kernel<true> : select_kernel<false>, (uint32_t)grid, SELECT_THREADS,
+                        image_smem + PARK_BYTES, stream, c, stage_bytes, q, n, per_cta);
 }
 
 }  // namespace infaas

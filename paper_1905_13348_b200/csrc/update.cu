@@ -34,6 +34,8 @@ tally_kernel(const uint32_t *__restrict__ decision, uint64_t n, uint32_t n_varia
   __shared__ uint32_t blk[3];
   if (threadIdx.x < 3) blk[threadIdx.x] = 0;
   __syncthreads();
+  chain_wait();
+  chain_next();
   uint32_t n_feas = 0, n_nofeas = 0, n_inval = 0;
   const uint64_t n4 = n >> 2;
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
@@ -86,6 +88,8 @@ tally_smem_kernel(const uint32_t *__restrict__ decision, uint64_t n, uint32_t n_
   for (uint32_t i = threadIdx.x; i < my_bins; i += blockDim.x) hist[i] = 0;
   if (threadIdx.x < 3) blk[threadIdx.x] = 0;
   __syncthreads();
+  chain_wait();
+  chain_next();
   // per decision: one shared-memory atomic and two counters; invalid
   // decisions are what remains of the total
   uint32_t n_feas = 0, n_nofeas = 0, n_seen = 0;
@@ -137,6 +141,7 @@ tally_smem_kernel(const uint32_t *__restrict__ decision, uint64_t n, uint32_t n_
 
 constexpr uint32_t TALLY_SMEM_MAX_VARIANTS = 49152;   // 192 KB of bins
 constexpr uint32_t TALLY_SMEM_MAX_PARTS = 8;           // beyond this many id ranges: global atomics
+constexpr size_t TALLY_SMEM_ALONE = 116 * 1024;
 constexpr uint64_t TALLY_SMEM_MIN_N = 1u << 18;        // below this the zero/flush passes cost more than they save
 
 cudaError_t launch_tally(const DeviceCatalog &c, const uint32_t *d_decision, uint64_t n,
@@ -145,21 +150,22 @@ cudaError_t launch_tally(const DeviceCatalog &c, const uint32_t *d_decision, uin
   const uint32_t parts = (c.n_variants + TALLY_SMEM_MAX_VARIANTS - 1) / TALLY_SMEM_MAX_VARIANTS;
   if (n >= TALLY_SMEM_MIN_N && parts <= TALLY_SMEM_MAX_PARTS) {
     const uint32_t bins = ((c.n_variants + parts - 1) / parts + 3u) & ~3u;
-    const size_t smem = (size_t)(bins + 32) * 4;                 // 32 spare bins
+    size_t smem = (size_t)(bins + 32) * 4;                       // 32 spare bins
+    // more than half of an SM's shared memory: launched while the selection kernel drains, two CTAs
+    // on the SMs that finish first would leave others idle (+5 us on 2^24 decisions)
+    if (smem < TALLY_SMEM_ALONE) smem = TALLY_SMEM_ALONE;
     // one CTA of 1024 threads per SM: half as many histograms to clear and flush as two of 512
     uint64_t want = ((n >> 2) + TALLY_SMEM_THREADS * 8 - 1) / (TALLY_SMEM_THREADS * 8);
     uint64_t shares = (uint64_t)sm_count / parts;              // CTAs per id range
     if (shares > want) shares = want;
     if (shares < 1) shares = 1;
-    tally_smem_kernel<<<(uint32_t)(shares * parts), TALLY_SMEM_THREADS, smem, stream>>>(
-        d_decision, n, c.n_variants, bins, parts, c.count_by_id, c.counters);
-    return cudaGetLastError();
+    return launch_chained(tally_smem_kernel, (uint32_t)(shares * parts), TALLY_SMEM_THREADS, smem, stream, d_decision, n,
+                          c.n_variants, bins, parts, c.count_by_id, c.counters);
   }
   uint64_t want = ((n >> 2) + 255) / 256;
   const uint64_t most = (uint64_t)sm_count * 8;
   uint32_t grid = (uint32_t)(want < 1 ? 1 : (want > most ? most : want));
-  tally_kernel<<<grid, 256, 0, stream>>>(d_decision, n, c.n_variants, c.count_by_id, c.counters);
-  return cudaGetLastError();
+  return launch_chained(tally_kernel, grid, 256, 0, stream, d_decision, n, c.n_variants, c.count_by_id, c.counters);
 }
 
 cudaError_t prepare_tally_kernel() {

@@ -51,6 +51,8 @@ __device__ __forceinline__ uint32_t worker_for(uint32_t d, uint32_t n_variants, 
 __global__ void __launch_bounds__(256)
 assign_workers_kernel(const uint32_t *__restrict__ decision, uint64_t n, uint32_t n_variants,
                       const uint32_t *__restrict__ worker_of, uint32_t *__restrict__ worker) {
+  chain_wait();
+  chain_next();
   const uint64_t n4 = n >> 2, stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += stride) {
     const uint4 d = __ldcs(reinterpret_cast<const uint4 *>(decision) + i);
@@ -94,8 +96,7 @@ cudaError_t launch_assign_workers(const uint32_t *d_decision, uint64_t n, uint32
   uint64_t want = ((n >> 2) + 255) / 256;
   const uint64_t cap = (uint64_t)sm_count * 8;
   const uint32_t grid = (uint32_t)(want < 1 ? 1 : (want > cap ? cap : want));
-  assign_workers_kernel<<<grid, 256, 0, stream>>>(d_decision, n, n_variants, worker_of, d_worker);
-  return cudaGetLastError();
+  return launch_chained(assign_workers_kernel, grid, 256, 0, stream, d_decision, n, n_variants, worker_of, d_worker);
 }
 
 }  // namespace infaas
