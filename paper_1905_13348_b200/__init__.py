@@ -18,5 +18,6 @@ _BINDING = ("infaas_catalog_load", "infaas_select_batch", "infaas_load_update",
 def __getattr__(name):
     if name in _BINDING:
         from . import binding
-        return getattr(binding, name)
+        value = globals()[name] = getattr(binding, name)      # the next look-up finds it here
+        return value
     raise AttributeError(name)

@@ -94,22 +94,45 @@ def _check(code: int, where: str) -> None:
         raise InfaasError(code, where)
 
 
+# What the per-call path needs of torch, looked up once: element types by width, and how to get the
+# current stream's pointer (a call that issues one kernel took 11 us on the host, 5 of them here).
+_widths: dict = {}
+_raw_stream = _current_device = None
+
+
+def _init_torch() -> None:
+    global _raw_stream, _current_device
+    import torch
+    torch.cuda.init()                       # the raw getters below assume it (and it refuses a forked child)
+    _raw_stream, _current_device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+
+
+def _forget_torch() -> None:
+    global _raw_stream
+    _raw_stream = None
+
+
+os.register_at_fork(after_in_child=_forget_torch)
+
+
 def _dev_ptr(t, dtype_name: str):
     """Device pointer of a contiguous torch CUDA tensor of the given integer width."""
-    import torch
-    widths = {"u16": (torch.int16, torch.uint16), "u32": (torch.int32, torch.uint32)}
     if t is None:
         return None
-    if not t.is_cuda or not t.is_contiguous() or t.dtype not in widths[dtype_name]:
+    if not _widths:
+        import torch
+        _widths.update(u16=frozenset((torch.int16, torch.uint16)), u32=frozenset((torch.int32, torch.uint32)))
+    if not t.is_cuda or not t.is_contiguous() or t.dtype not in _widths[dtype_name]:
         raise TypeError(f"expected a contiguous CUDA tensor of {dtype_name}, got {t.dtype} on {t.device}")
     return t.data_ptr()
 
 
 def _stream_ptr(stream):
-    import torch
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is None:
+        _init_torch()
+    return _raw_stream(_current_device())
 
 
 class Catalog:
