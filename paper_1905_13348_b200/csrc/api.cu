@@ -1,6 +1,7 @@
 // C ABI of the library (declared in include/infaas.h): handle management, validation,
 // the host side of the catalog packer, and the calls that launch the kernels.
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <string>
 #include <vector>
@@ -14,7 +15,7 @@ struct infaas_catalog {
   int sm_count = 0;
   DeviceCatalog d{};
   void *arena = nullptr;                 // one device allocation holds every array
-  std::vector<uint32_t> slot_of_id;      // host copy, for get_state
+  uint32_t *slot_of_id = nullptr;        // device, by variant id
   std::vector<uint32_t> task_off, reg_off;
   uint32_t select_smem = 0;              // shared memory reserved for the staged image
   uint32_t worst_image_bytes = 0;        // image size if every block had its largest size
@@ -27,6 +28,13 @@ struct infaas_catalog {
   uint32_t *worker_of = nullptr;         // worker per variant id
   unsigned long long *best_inst = nullptr, *best_hw = nullptr;   // scratch of the table build
   bool workers_ready = false;
+  // The calls that exchange tables with the host pass them through one buffer on either side, kept
+  // with the catalog; they synchronise their stream before they return, so one at a time may use it.
+  std::mutex table_lock;
+  unsigned char *table = nullptr;        // in the arena, or table_grown
+  size_t table_bytes = 0;
+  void *table_grown = nullptr;
+  std::vector<unsigned char> h_table;
 };
 
 namespace {
@@ -86,18 +94,55 @@ inline uint32_t float_bits_rz(uint32_t x) {
   return ((e + 127u) << 23) | mant;
 }
 
-// Re-reads the image size from the device and decides how much shared memory the selection
-// kernel asks for: all of it while the image fits (it may grow or shrink between two such
-// refreshes without a change of plan), none for the image if it does not -- the kernel
-// then reads it from global memory and the space is worth more as L1 cache.
-int refresh_select_plan(infaas_catalog *c, cudaStream_t stream) {
-  uint32_t hdr[1] = {0};
-  CUDA_TRY(cudaMemcpyAsync(hdr, c->d.image_hdr, sizeof(hdr), cudaMemcpyDeviceToHost, stream));
-  CUDA_TRY(cudaStreamSynchronize(stream));
+// Decides how much shared memory the selection kernel asks for: all of it while the image fits
+// (it may grow or shrink between two such looks at its size without a change of plan), none for
+// the image if it does not -- the kernel then reads it from global memory and the space is worth
+// more as L1 cache.
+void plan_select(infaas_catalog *c, uint32_t image_bytes) {
   const uint32_t room = infaas::select_image_smem(infaas::SELECT_MAX_SMEM);
-  c->select_smem = hdr[0] <= room ? room : 0u;
+  c->select_smem = image_bytes <= room ? room : 0u;
+}
+int refresh_select_plan(infaas_catalog *c, cudaStream_t stream) {
+  uint32_t image_bytes = 0;
+  CUDA_TRY(cudaMemcpyAsync(&image_bytes, c->d.image_hdr, 4, cudaMemcpyDeviceToHost, stream));
+  CUDA_TRY(cudaStreamSynchronize(stream));
+  plan_select(c, image_bytes);
   return INFAAS_OK;
 }
+
+// Room for `bytes` in the table buffer of the device (table_lock held).
+int reserve_table(infaas_catalog *c, size_t bytes) {
+  if (bytes <= c->table_bytes) return INFAAS_OK;
+  void *p = nullptr;
+  CUDA_TRY(cudaMalloc(&p, bytes));
+  (void)cudaFree(c->table_grown);
+  c->table_grown = p;
+  c->table = static_cast<unsigned char *>(p);
+  c->table_bytes = bytes;
+  return INFAAS_OK;
+}
+
+// Host tables put side by side and sent to the device in one copy.
+struct Upload {
+  infaas_catalog *c;
+  size_t bytes = 0;
+  explicit Upload(infaas_catalog *cat) : c(cat) {}
+  // Appends a table; returns its offset in the device's buffer.
+  size_t add(const void *src, size_t n) {
+    const size_t off = bytes;
+    bytes = round_up(off + n, 16);
+    if (c->h_table.size() < bytes) c->h_table.resize(bytes);
+    if (n) memcpy(c->h_table.data() + off, src, n);
+    return off;
+  }
+  int send(cudaStream_t s) {
+    const int rc = reserve_table(c, bytes);
+    if (rc != INFAAS_OK) return rc;
+    CUDA_TRY(cudaMemcpyAsync(c->table, c->h_table.data(), bytes, cudaMemcpyHostToDevice, s));
+    return INFAAS_OK;
+  }
+  const uint32_t *u32(size_t off) const { return reinterpret_cast<const uint32_t *>(c->table + off); }
+};
 
 }  // namespace
 
@@ -219,6 +264,9 @@ int infaas_catalog_load(const infaas_variant *rows, uint32_t n_variants, uint32_
   const size_t o_task_slo = carve((size_t)n_tasks * 4), o_qps = carve((size_t)n_variants * 8);
   const size_t o_slot_of_id = carve((size_t)n_variants * 4);
   const size_t o_hw = carve((size_t)n_variants), o_worker_of = carve((size_t)n_variants * 4);
+  // tables of the host calls: the load state (16 B per variant), or instances and workers of about
+  // two per variant (a larger table gets a buffer of its own)
+  const size_t table_bytes = (size_t)n_variants * 32 + (size_t)n_tasks * 4 + 32768, o_table = carve(table_bytes);
   const size_t o_best_inst = carve((size_t)n_variants * 8), o_best_hw = carve(256 * 8);
   const size_t o_regions = carve((size_t)region_bytes);
   const size_t o_flen = carve((size_t)n_tasks * 4), o_slow = carve(((size_t)n_tasks + n_extra) * 16);
@@ -246,6 +294,9 @@ int infaas_catalog_load(const infaas_variant *rows, uint32_t n_variants, uint32_
   LOAD_TRY(cudaMemcpy(base + o_seg_base, seg_base.data(), (n_tasks + 1) * 4, cudaMemcpyHostToDevice));
   c->s_qps = reinterpret_cast<unsigned long long *>(base + o_qps);
   c->hw_by_id = base + o_hw;
+  c->slot_of_id = reinterpret_cast<uint32_t *>(base + o_slot_of_id);
+  c->table = base + o_table;
+  c->table_bytes = table_bytes;
   c->worker_of = reinterpret_cast<uint32_t *>(base + o_worker_of);
   c->best_inst = reinterpret_cast<unsigned long long *>(base + o_best_inst);
   c->best_hw = reinterpret_cast<unsigned long long *>(base + o_best_hw);
@@ -306,14 +357,12 @@ int infaas_catalog_load(const infaas_variant *rows, uint32_t n_variants, uint32_
     o.s_id = const_cast<uint32_t *>(d.s_id); o.s_queued = d.s_queued;
     o.s_order = const_cast<uint32_t *>(d.s_order); o.s_cost_run = const_cast<uint32_t *>(d.s_cost_run);
     o.n_class = const_cast<uint32_t *>(d.n_class);
-    o.slot_of_id = reinterpret_cast<uint32_t *>(base + o_slot_of_id);
+    o.slot_of_id = c->slot_of_id;
     o.s_batch = const_cast<uint16_t *>(d.s_batch); o.s_acc = const_cast<uint16_t *>(d.s_acc);
     o.s_arch = c->s_arch; o.s_class = const_cast<uint16_t *>(d.s_class);
     o.class_acc = const_cast<uint16_t *>(d.class_acc);
     o.s_qps = c->s_qps; o.hw_by_id = c->hw_by_id;
     LOAD_TRY(infaas::launch_layout(o, n_tasks, max_task, nullptr));
-    c->slot_of_id.resize(n_variants);
-    LOAD_TRY(cudaMemcpy(c->slot_of_id.data(), o.slot_of_id, (size_t)n_variants * 4, cudaMemcpyDeviceToHost));
   }
   LOAD_TRY(infaas::prepare_select_kernel());
   LOAD_TRY(infaas::prepare_tally_kernel());
@@ -410,18 +459,16 @@ int infaas_catalog_set_states(infaas_catalog *c, const uint8_t *h_state, const u
   DeviceScope scope(c->device);
   if (scope.status != cudaSuccess) return cuda_fail(scope.status);
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-  std::vector<unsigned char> st(nv);
-  std::vector<uint32_t> ll(nv, 0u);
-  for (uint32_t v = 0; v < nv; ++v) {
-    st[c->slot_of_id[v]] = h_state[v];
-    if (h_load_lat_us) ll[c->slot_of_id[v]] = h_load_lat_us[v];
-  }
-  CUDA_TRY(cudaMemcpyAsync(c->d.s_state, st.data(), nv, cudaMemcpyHostToDevice, s));
-  CUDA_TRY(cudaMemcpyAsync(const_cast<uint32_t *>(c->d.s_load_lat), ll.data(), (size_t)nv * 4,
-                           cudaMemcpyHostToDevice, s));
+  std::lock_guard<std::mutex> lock(c->table_lock);
+  Upload up(c);
+  const size_t o_state = up.add(h_state, nv);
+  const size_t o_load = h_load_lat_us ? up.add(h_load_lat_us, (size_t)nv * 4) : 0;
+  const int rc = up.send(s);
+  if (rc != INFAAS_OK) return rc;
+  CUDA_TRY(infaas::launch_scatter(c->d, h_load_lat_us ? up.u32(o_load) : nullptr, const_cast<uint32_t *>(c->d.s_load_lat),
+                                  c->table + o_state, nullptr, nullptr, s));
   c->d.stateful = 1;
   CUDA_TRY(infaas::launch_rebuild(c->d, /*advance_queues=*/false, 0, s));
-  CUDA_TRY(cudaStreamSynchronize(s));     // the host copies above go out of scope
   return refresh_select_plan(c, s);
 }
 
@@ -430,11 +477,10 @@ int infaas_catalog_get_states(infaas_catalog *c, uint8_t *h_state, void *cuda_st
   DeviceScope scope(c->device);
   if (scope.status != cudaSuccess) return cuda_fail(scope.status);
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-  const uint32_t nv = c->d.n_variants;
-  std::vector<unsigned char> st(nv);
-  CUDA_TRY(cudaMemcpyAsync(st.data(), c->d.s_state, nv, cudaMemcpyDeviceToHost, s));
+  std::lock_guard<std::mutex> lock(c->table_lock);
+  CUDA_TRY(infaas::launch_states(c->d, c->slot_of_id, c->table, s));
+  CUDA_TRY(cudaMemcpyAsync(h_state, c->table, c->d.n_variants, cudaMemcpyDeviceToHost, s));
   CUDA_TRY(cudaStreamSynchronize(s));
-  for (uint32_t v = 0; v < nv; ++v) h_state[v] = st[c->slot_of_id[v]];
   return INFAAS_OK;
 }
 
@@ -445,10 +491,12 @@ int infaas_autoscale_config(infaas_catalog *c, const uint32_t *h_instances, cons
   if (scope.status != cudaSuccess) return cuda_fail(scope.status);
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   const uint32_t nv = c->d.n_variants;
-  std::vector<uint32_t> inst(nv);
-  for (uint32_t v = 0; v < nv; ++v) inst[c->slot_of_id[v]] = h_instances[v];
-  CUDA_TRY(cudaMemcpyAsync(c->s_inst, inst.data(), (size_t)nv * 4, cudaMemcpyHostToDevice, s));
-  CUDA_TRY(cudaMemcpyAsync(c->task_slo, h_task_slo_us, (size_t)c->d.n_tasks * 4, cudaMemcpyHostToDevice, s));
+  std::lock_guard<std::mutex> lock(c->table_lock);
+  Upload up(c);
+  const size_t o_inst = up.add(h_instances, (size_t)nv * 4), o_slo = up.add(h_task_slo_us, (size_t)c->d.n_tasks * 4);
+  const int rc = up.send(s);
+  if (rc != INFAAS_OK) return rc;
+  CUDA_TRY(infaas::launch_scatter(c->d, up.u32(o_inst), c->s_inst, nullptr, up.u32(o_slo), c->task_slo, s));
   CUDA_TRY(cudaStreamSynchronize(s));
   c->autoscale_ready = true;
   return INFAAS_OK;
@@ -474,28 +522,16 @@ int infaas_workers_config(infaas_catalog *c, const uint32_t *h_inst_variant, con
   DeviceScope scope(c->device);
   if (scope.status != cudaSuccess) return cuda_fail(scope.status);
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-  // one temporary buffer: three u32 arrays of n_inst, one u32 array and one u8 array of n_workers
-  const size_t ib = round_up((size_t)n_inst * 4, 256), wb = round_up((size_t)n_workers * 4, 256);
-  unsigned char *tmp = nullptr;
-  CUDA_TRY(cudaMalloc(&tmp, 3 * ib + 2 * wb + 256));
-  uint32_t *d_iv = reinterpret_cast<uint32_t *>(tmp), *d_iw = reinterpret_cast<uint32_t *>(tmp + ib),
-           *d_il = reinterpret_cast<uint32_t *>(tmp + 2 * ib), *d_wu = reinterpret_cast<uint32_t *>(tmp + 3 * ib);
-  unsigned char *d_wh = tmp + 3 * ib + wb;
-  cudaError_t e = cudaSuccess;
-  auto up = [&](void *dst, const void *src, size_t bytes) {
-    if (e == cudaSuccess && bytes) e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, s);
-  };
-  up(d_iv, h_inst_variant, (size_t)n_inst * 4);
-  up(d_iw, h_inst_worker, (size_t)n_inst * 4);
-  up(d_il, h_inst_load, (size_t)n_inst * 4);
-  up(d_wu, h_worker_util, (size_t)n_workers * 4);
-  up(d_wh, h_worker_hw, (size_t)n_workers);
-  if (e == cudaSuccess)
-    e = infaas::launch_workers_build(c->d.n_variants, c->hw_by_id, d_iv, d_iw, d_il, n_inst, d_wh, d_wu, n_workers,
-                                     c->best_inst, c->best_hw, c->worker_of, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  (void)cudaFree(tmp);
-  if (e != cudaSuccess) return cuda_fail(e);
+  std::lock_guard<std::mutex> lock(c->table_lock);
+  Upload up(c);
+  const size_t o_iv = up.add(h_inst_variant, (size_t)n_inst * 4), o_iw = up.add(h_inst_worker, (size_t)n_inst * 4),
+               o_il = up.add(h_inst_load, (size_t)n_inst * 4), o_wu = up.add(h_worker_util, (size_t)n_workers * 4),
+               o_wh = up.add(h_worker_hw, (size_t)n_workers);
+  const int rc = up.bytes ? up.send(s) : INFAAS_OK;
+  if (rc != INFAAS_OK) return rc;
+  CUDA_TRY(infaas::launch_workers_build(c->d.n_variants, c->hw_by_id, up.u32(o_iv), up.u32(o_iw), up.u32(o_il), n_inst,
+                                        c->table + o_wh, up.u32(o_wu), n_workers, c->best_inst, c->best_hw, c->worker_of, s));
+  CUDA_TRY(cudaStreamSynchronize(s));
   c->workers_ready = true;
   return INFAAS_OK;
 }
@@ -520,39 +556,28 @@ int infaas_catalog_get_state(infaas_catalog *c, uint32_t *h_queued, uint32_t *h_
   DeviceScope scope(c->device);
   if (scope.status != cudaSuccess) return cuda_fail(scope.status);
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-  const uint32_t nv = c->d.n_variants;
-  std::vector<uint32_t> tmp32;
-  std::vector<unsigned long long> tmp64;
-  if (h_queued) {
-    tmp32.resize(nv);
-    CUDA_TRY(cudaMemcpyAsync(tmp32.data(), c->d.s_queued, (size_t)nv * 4, cudaMemcpyDeviceToHost, s));
-    CUDA_TRY(cudaStreamSynchronize(s));
-    for (uint32_t v = 0; v < nv; ++v) h_queued[v] = tmp32[c->slot_of_id[v]];
-  }
-  if (h_pred_lat_us) {
-    tmp32.resize(nv);
-    CUDA_TRY(cudaMemcpyAsync(tmp32.data(), c->d.s_pred, (size_t)nv * 4, cudaMemcpyDeviceToHost, s));
-    CUDA_TRY(cudaStreamSynchronize(s));
-    for (uint32_t v = 0; v < nv; ++v) h_pred_lat_us[v] = tmp32[c->slot_of_id[v]];
-  }
-  if (h_served_total) {
-    tmp64.resize(nv);
-    CUDA_TRY(cudaMemcpyAsync(tmp64.data(), c->d.s_served, (size_t)nv * 8, cudaMemcpyDeviceToHost, s));
-    CUDA_TRY(cudaStreamSynchronize(s));
-    for (uint32_t v = 0; v < nv; ++v) h_served_total[v] = tmp64[c->slot_of_id[v]];
-  }
-  if (h_counters) {
-    unsigned long long k[3];
-    CUDA_TRY(cudaMemcpyAsync(k, c->d.counters, sizeof(k), cudaMemcpyDeviceToHost, s));
-    CUDA_TRY(cudaStreamSynchronize(s));
-    for (int i = 0; i < 3; ++i) h_counters[i] = k[i];
-  }
-  uint32_t err = 0;
-  CUDA_TRY(cudaMemcpyAsync(&err, c->d.err, 4, cudaMemcpyDeviceToHost, s));
+  const size_t nv = c->d.n_variants;
+  // [tail][served][queued][pred], by id; copied as far as it is asked for
+  const size_t o_served = round_up(sizeof(infaas::LoadStateTail), 256), o_queued = o_served + nv * 8, o_pred = o_queued + nv * 4;
+  const size_t bytes = h_pred_lat_us ? o_pred + nv * 4 : h_queued ? o_pred : h_served_total ? o_queued : o_served;
+  std::lock_guard<std::mutex> lock(c->table_lock);
+  CUDA_TRY(infaas::launch_load_state(c->d, c->slot_of_id, reinterpret_cast<infaas::LoadStateTail *>(c->table),
+                                     reinterpret_cast<unsigned long long *>(c->table + o_served),
+                                     reinterpret_cast<uint32_t *>(c->table + o_queued),
+                                     reinterpret_cast<uint32_t *>(c->table + o_pred), s));
+  if (c->h_table.size() < bytes) c->h_table.resize(bytes);
+  CUDA_TRY(cudaMemcpyAsync(c->h_table.data(), c->table, bytes, cudaMemcpyDeviceToHost, s));
   CUDA_TRY(cudaStreamSynchronize(s));
-  int rc = refresh_select_plan(c, s);
-  if (rc != INFAAS_OK) return rc;
-  if (err != infaas::DEV_ERR_NONE) {
+  const unsigned char *h = c->h_table.data();
+  infaas::LoadStateTail tail;
+  memcpy(&tail, h, sizeof(tail));
+  if (h_served_total) memcpy(h_served_total, h + o_served, nv * 8);
+  if (h_queued) memcpy(h_queued, h + o_queued, nv * 4);
+  if (h_pred_lat_us) memcpy(h_pred_lat_us, h + o_pred, nv * 4);
+  if (h_counters)
+    for (int i = 0; i < 3; ++i) h_counters[i] = tail.counters[i];
+  plan_select(c, tail.image_bytes);
+  if (tail.err != infaas::DEV_ERR_NONE) {
     CUDA_TRY(cudaMemsetAsync(c->d.err, 0, 4, s));
     CUDA_TRY(cudaStreamSynchronize(s));
     return INFAAS_E_DEVICE;
@@ -613,6 +638,7 @@ void infaas_catalog_free(infaas_catalog *c) {
   if (c->arena) {
     DeviceScope scope(c->device);
     (void)cudaFree(c->arena);
+    (void)cudaFree(c->table_grown);
   }
   delete c;
 }

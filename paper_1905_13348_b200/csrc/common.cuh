@@ -288,6 +288,20 @@ cudaError_t launch_autoscale(const DeviceCatalog &c, const uint32_t *s_inst, con
                              uint32_t lambda_milli, uint32_t *d_variant, uint32_t *d_delta,
                              cudaStream_t stream);
 
+// Tables ordered by variant id, from and to the per-slot arrays.
+struct LoadStateTail {
+  unsigned long long counters[3];
+  uint32_t err, image_bytes;
+};
+cudaError_t launch_load_state(const DeviceCatalog &c, const uint32_t *slot_of_id, LoadStateTail *tail,
+                              unsigned long long *served, uint32_t *queued, uint32_t *pred, cudaStream_t stream);
+cudaError_t launch_states(const DeviceCatalog &c, const uint32_t *slot_of_id, unsigned char *state, cudaStream_t stream);
+// s_value[slot] = value_by_id[id] (0 without a table); with state_by_id also the states; with by_task
+// also task_value[t] = by_task[t].
+cudaError_t launch_scatter(const DeviceCatalog &c, const uint32_t *value_by_id, uint32_t *s_value,
+                           const unsigned char *state_by_id, const uint32_t *by_task, uint32_t *task_value,
+                           cudaStream_t stream);
+
 // Worker choice.  Build: one worker per variant from the instance table {variant, worker, load}
 // and the worker table {hardware code, utilisation} (device arrays); best_inst [n_variants] and
 // best_hw [256] are scratch.  Assign: worker[q] = worker_of[decision[q]] for decisions below

@@ -14,6 +14,8 @@ constexpr unsigned long long NO_KEY = ~0ull;
 __global__ void workers_reset_kernel(unsigned long long *best_inst, uint32_t n_variants,
                                      unsigned long long *best_hw) {
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+  chain_wait();
+  chain_next();
   if (i < n_variants) best_inst[i] = NO_KEY;
   if (i < 256u) best_hw[i] = NO_KEY;
 }
@@ -26,6 +28,8 @@ __global__ void workers_scan_kernel(const uint32_t *inst_variant, const uint32_t
                                     uint32_t n_workers, unsigned long long *best_inst,
                                     unsigned long long *best_hw) {
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+  chain_wait();
+  chain_next();
   if (i < n_inst) {
     const uint32_t v = inst_variant[i], w = inst_worker[i];
     if (v < n_variants && w < n_workers) atomicMin(best_inst + v, ((unsigned long long)inst_load[i] << 32) | w);
@@ -37,6 +41,8 @@ __global__ void workers_final_kernel(uint32_t n_variants, const unsigned char *h
                                      const unsigned long long *best_inst, const unsigned long long *best_hw,
                                      uint32_t *worker_of) {
   const uint32_t v = blockIdx.x * blockDim.x + threadIdx.x;
+  chain_wait();
+  chain_next();
   if (v >= n_variants) return;
   unsigned long long k = best_inst[v];
   if (k == NO_KEY) k = best_hw[hw_by_id[v]];
@@ -79,14 +85,15 @@ cudaError_t launch_workers_build(uint32_t n_variants, const unsigned char *hw_by
                                  uint32_t *worker_of, cudaStream_t stream) {
   const uint32_t B = 256;
   const uint32_t m = n_variants > 256u ? n_variants : 256u;
-  workers_reset_kernel<<<(m + B - 1) / B, B, 0, stream>>>(best_inst, n_variants, best_hw);
+  cudaError_t e = launch_chained(workers_reset_kernel, (m + B - 1) / B, B, 0, stream, best_inst, n_variants, best_hw);
   const uint32_t k = n_inst > n_workers ? n_inst : n_workers;
-  if (k)
-    workers_scan_kernel<<<(k + B - 1) / B, B, 0, stream>>>(inst_variant, inst_worker, inst_load, n_inst, n_variants,
-                                                           worker_hw, worker_util, n_workers, best_inst, best_hw);
-  workers_final_kernel<<<(n_variants + B - 1) / B, B, 0, stream>>>(n_variants, hw_by_id, best_inst, best_hw,
-                                                                   worker_of);
-  return cudaGetLastError();
+  if (e == cudaSuccess && k)
+    e = launch_chained(workers_scan_kernel, (k + B - 1) / B, B, 0, stream, inst_variant, inst_worker, inst_load, n_inst,
+                       n_variants, worker_hw, worker_util, n_workers, best_inst, best_hw);
+  if (e == cudaSuccess)
+    e = launch_chained(workers_final_kernel, (n_variants + B - 1) / B, B, 0, stream, n_variants, hw_by_id, best_inst,
+                       best_hw, worker_of);
+  return e;
 }
 
 cudaError_t launch_assign_workers(const uint32_t *d_decision, uint64_t n, uint32_t n_variants,

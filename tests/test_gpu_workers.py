@@ -78,3 +78,30 @@ def test_assign_before_config_is_an_error():
         assert e.value.code == -11
     finally:
         cat.free()
+
+
+def test_tables_larger_than_the_catalogs_own_buffer():
+    """The host tables pass through a buffer sized by the catalog: an instance table far larger than
+    the catalog gets one of its own, and the calls after it still work."""
+    import paper_1905_13348_b200 as P
+    import torch
+    from oracle import OracleCatalog
+    rng = np.random.default_rng(77)
+    w = W.make("C1", n_queries=1000)
+    cat, o = P.infaas_catalog_load(w.rows, w.n_tasks), OracleCatalog(w.rows, w.n_tasks)
+    want_dec = o.select(w.task, w.slo_us, w.min_acc_bp, 4)
+    dec = torch.from_numpy(want_dec.view(np.int32)).cuda()
+    out = torch.empty_like(dec)
+    for n_inst, n_workers in ((3, 5), (50_021, 9_001), (0, 0), (120_000, 20_000), (7, 3)):
+        iv = rng.integers(0, w.n_variants, n_inst).astype(np.uint32)
+        iw = rng.integers(0, max(1, n_workers), n_inst).astype(np.uint32)
+        il = rng.integers(0, 9, n_inst).astype(np.uint32)
+        hw = rng.integers(0, 4, n_workers).astype(np.uint8)
+        ut = rng.integers(0, 9, n_workers).astype(np.uint32)
+        P.infaas_workers_config(cat, iv, iw, il, hw, ut)
+        P.infaas_assign_workers(cat, dec, out)
+        want = assign_workers(w.rows, iv, iw, il, hw, ut, want_dec)
+        assert np.array_equal(out.cpu().numpy().view(np.uint32), want), (n_inst, n_workers)
+        st = P.infaas_catalog_get_state(cat)
+        assert np.array_equal(st["queued"], o.queued) and np.array_equal(st["pred_lat_us"], o.pred_lat())
+    cat.free()
