@@ -38,14 +38,12 @@ struct IndexScratch {
   uint32_t bcnt[256], bthr[256];    // per SLO bucket: distinct latencies inside it, one of them
   uint32_t wbits[MAX_ACC_WORDS];    // per bitmap word: the accuracies present
   // per latency rank: the most accurate entry (acc << 16 | 0xFFFF - position, 0 = none); per
-  // accuracy rank: the fastest entry (pred << 32 | position, ~0 = none); then their running
-  // maximum / minimum
-  uint32_t rankA[256], bestA[257];
-  unsigned long long rankB[256], bestB[257];
+  // accuracy rank: the fastest entry (its index in latency order, NONE = none)
+  uint32_t rankA[256], rankB[256];
   uint16_t acc[256];
   unsigned char wpre[MAX_ACC_WORDS];         // accuracies present in the words before
   unsigned char at[256], rank[256];          // sorted order: position, latency rank
-  unsigned char ord_start[257], stair[256];  // per latency rank: stair entries before it; holds one
+  unsigned char stair[256];                  // latency rank holds a stair entry
   unsigned char part[REBUILD_WARPS * 32];    // rank table: first position per column of a run of entries
   uint32_t ks, ka, base;
 };
@@ -56,36 +54,33 @@ __device__ __forceinline__ void write_dummy_task(const DeviceCatalog &c, uint32_
   const uint32_t T = c.n_tasks;
   if (threadIdx.x == 0) reinterpret_cast<uint32_t *>(c.image + IMAGE_HDR_OFFSET)[t] = DUMMY_HEADER;
   uint32_t *rec = reinterpret_cast<uint32_t *>(c.image + image_rec_offset(T) + t * REC_STRIDE);
+#pragma unroll 1
   for (uint32_t j = threadIdx.x; j < SLO_BUCKETS; j += blockDim.x) rec[j] = 0u;
   uint32_t *bm = reinterpret_cast<uint32_t *>(c.image + image_bitmap_offset(T) + t * bitmap_stride(c.nbw));
+#pragma unroll 1
   for (uint32_t j = threadIdx.x; j < c.nbw; j += blockDim.x) bm[j] = 0u;
 }
 
 // Bucket scale of the SLO records: S (16..23) and bmin such that SLO_BUCKETS - 1 buckets of
 // 2^S float patterns cover everything from the catalog's smallest profiled latency up to the
 // largest SLO asked for so far (as a bit mask: every SLO seen is <= cap).
-__device__ __forceinline__ void bucket_scale(const DeviceCatalog &c, uint32_t &Sh, uint32_t &bmin) {
-  uint32_t cap = *c.slo_seen | SLO_CAP_FLOOR_US;
+__device__ __forceinline__ void bucket_scale(const DeviceCatalog &c, uint32_t slo_seen, uint32_t &Sh, uint32_t &bmin) {
+  uint32_t cap = slo_seen | SLO_CAP_FLOOR_US;
   cap |= cap >> 1; cap |= cap >> 2; cap |= cap >> 4; cap |= cap >> 8; cap |= cap >> 16;
   const uint32_t clo = c.lat_code_lo;
   const uint32_t chi = max(clo, __float_as_uint(__uint2float_rz(cap)) >> 16);
   uint32_t sh = 0;
+#pragma unroll 1
   while ((chi >> sh) - (clo >> sh) > SLO_BUCKETS - 2) ++sh;
   bmin = clo >> sh;
   Sh = 16u + sh;
 }
 
-// Sum / OR over the aligned group of 8 lanes this lane belongs to.
+// Sum over the aligned group of 8 lanes this lane belongs to.
 __device__ __forceinline__ uint32_t group8_add(uint32_t v) {
   v += __shfl_xor_sync(0xFFFFFFFFu, v, 1);
   v += __shfl_xor_sync(0xFFFFFFFFu, v, 2);
   v += __shfl_xor_sync(0xFFFFFFFFu, v, 4);
-  return v;
-}
-__device__ __forceinline__ uint32_t group8_or(uint32_t v) {
-  v |= __shfl_xor_sync(0xFFFFFFFFu, v, 1);
-  v |= __shfl_xor_sync(0xFFFFFFFFu, v, 2);
-  v |= __shfl_xor_sync(0xFFFFFFFFu, v, 4);
   return v;
 }
 
@@ -111,6 +106,11 @@ __device__ __forceinline__ uint32_t warp_scan_max(uint32_t x) {
   for (uint32_t o = 1; o < 32; o <<= 1) x = max(x, __shfl_up_sync(0xFFFFFFFFu, x, o));
   return x;
 }
+// Exclusive: the lanes before this one (`none` in lane 0).
+__device__ __forceinline__ uint32_t lanes_before(uint32_t incl, uint32_t none) {
+  const uint32_t up = __shfl_up_sync(0xFFFFFFFFu, incl, 1);
+  return threadIdx.x & 31u ? up : none;
+}
 
 // One atomic per allocation places a block in the image and, on a CTA's last allocation
 // (`done`), counts the CTA as finished with the cursor.  The CTA that is counted last knows the
@@ -132,9 +132,11 @@ __device__ __forceinline__ uint32_t place_block_finish(const DeviceCatalog &c, u
 
 // Clears what build_index accumulates into (all threads; a barrier must follow).
 __device__ __forceinline__ void clear_scratch(IndexScratch &S) {
+#pragma unroll 1
   for (uint32_t i = threadIdx.x; i < 256u; i += REBUILD_THREADS) {
-    S.pred[i] = NONE; S.bcnt[i] = 0u; S.rankA[i] = 0u; S.rankB[i] = ~0ull;
+    S.pred[i] = NONE; S.bcnt[i] = 0u; S.rankA[i] = 0u; S.rankB[i] = NONE; S.stair[i] = 0;
   }
+#pragma unroll 1
   for (uint32_t i = threadIdx.x; i < MAX_ACC_WORDS; i += REBUILD_THREADS) S.wbits[i] = 0u;
 }
 
@@ -153,26 +155,29 @@ __device__ __forceinline__ void clear_scratch(IndexScratch &S) {
 // running minimum down its columns -- F steps per column, cut into runs of entries so that all
 // warps work, instead of F bits per cell.
 __device__ bool build_index(const DeviceCatalog &c, uint32_t t, uint32_t F, IndexScratch &S, uint32_t xi,
-                            uint32_t next) {
+                            uint32_t next, uint32_t Sh, uint32_t bmin) {
   const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
   constexpr uint32_t B = REBUILD_THREADS;
   const bool first = xi == NONE;
   const uint32_t acc_lo = c.acc_lo, nbw = c.nbw;      // the catalog's accuracy window
 
-  // 1. latency order by counting smaller (latency, position), 8 lanes per entry, 4 entries per
+  // 1. latency order: entry p comes behind the entries before it in the list that are not slower and
+  // those after it that are faster (latencies are at least 1).  8 lanes per entry, 4 entries per
   // load; the accuracies' bits
+#pragma unroll 1
   for (uint32_t p0 = 0; p0 < F; p0 += B / 8u) {        // uniform trip count
-    const uint32_t p = p0 + (tid >> 3), sub = tid & 7u;
+    const uint32_t p = p0 + (tid >> 3), sub = tid & 7u, own = p & ~3u;
     uint32_t cnt = 0, pp = 0;
     if (p < F) {
       pp = S.pred[p];
+#pragma unroll 2
       for (uint32_t q = 4u * sub; q < F; q += 32u) {
         const uint4 v = *reinterpret_cast<const uint4 *>(&S.pred[q]);
-        cnt += (uint32_t)(v.x < pp) | ((uint32_t)(v.x == pp) & (uint32_t)(q < p));
-        cnt += (uint32_t)(v.y < pp) | ((uint32_t)(v.y == pp) & (uint32_t)(q + 1u < p));
-        cnt += (uint32_t)(v.z < pp) | ((uint32_t)(v.z == pp) & (uint32_t)(q + 2u < p));
-        cnt += (uint32_t)(v.w < pp) | ((uint32_t)(v.w == pp) & (uint32_t)(q + 3u < p));
+        const uint32_t lim = pp - (uint32_t)(q >= own);
+        cnt += (uint32_t)(v.x <= lim) + (uint32_t)(v.y <= lim) + (uint32_t)(v.z <= lim) + (uint32_t)(v.w <= lim);
       }
+      // equal latencies in front of p inside its own four
+      if (sub < (p & 3u)) cnt += S.pred[own + sub] == pp;
     }
     cnt = group8_add(cnt);
     if (p < F && sub == 0u) {
@@ -182,8 +187,6 @@ __device__ bool build_index(const DeviceCatalog &c, uint32_t t, uint32_t F, Inde
       atomicOr(&S.wbits[xw], 1u << (x - xw * ACC_WORD_BITS));
     }
   }
-  uint32_t bmin, Sh;                                   // SLO buckets
-  bucket_scale(c, Sh, bmin);
   __syncthreads();
 
   // 2. dense latency ranks (warps 0-7, one sorted entry per thread), running popcounts of the
@@ -191,6 +194,7 @@ __device__ bool build_index(const DeviceCatalog &c, uint32_t t, uint32_t F, Inde
   if (warp < 8u) {
     const uint32_t i = tid;
     uint32_t before = 0;
+#pragma unroll 1
     for (uint32_t w = 0; w < warp && 32u * w < F; ++w) {
       const uint32_t x = 32u * w + lane;
       before += __popc(__ballot_sync(0xFFFFFFFFu, x < F && (x == 0u || S.sorted[x] != S.sorted[x - 1u])));
@@ -211,8 +215,10 @@ __device__ bool build_index(const DeviceCatalog &c, uint32_t t, uint32_t F, Inde
       if (i == F - 1u) S.ks = r + 1u;
     }
   } else {
+#pragma unroll 1
     for (uint32_t w0 = 32u * (warp - 8u); w0 < nbw; w0 += B - 256u) {     // uniform per warp
       uint32_t below = 0;
+#pragma unroll 1
       for (uint32_t x = lane; x < w0; x += 32u) below += __popc(S.wbits[x]);
       below = __reduce_add_sync(0xFFFFFFFFu, below);
       const uint32_t w = w0 + lane, pc = w < nbw ? __popc(S.wbits[w]) : 0u;
@@ -237,13 +243,14 @@ __device__ bool build_index(const DeviceCatalog &c, uint32_t t, uint32_t F, Inde
     const uint32_t last = tid == F - 1u || S.rank[tid + 1u] != r;
     S.ent[tid] = (ra << 16) | (last << 8) | p;
     atomicMax(&S.rankA[r], (acc << 16) | (0xFFFFu - p));                            // most accurate, first position
-    atomicMin(&S.rankB[ra], ((unsigned long long)S.sorted[tid] << 32) | p);         // fastest, first position
+    atomicMin(&S.rankB[ra], tid);                                                   // fastest, first position
   }
   if (first && tid >= B / 2u && tid < B / 2u + SLO_BUCKETS) {
     // one bucket per thread; lb = latencies in lower buckets
     uint32_t *rec = reinterpret_cast<uint32_t *>(c.image + image_rec_offset(c.n_tasks) + t * REC_STRIDE);
     const uint32_t j = tid - B / 2u;
     uint32_t below = 0;
+#pragma unroll 1
     for (uint32_t i = lane; i < (j & ~31u); i += 32u) below += S.bcnt[i];
     below = __reduce_add_sync(0xFFFFFFFFu, below);
     const uint32_t cnt = S.bcnt[j], thr = S.bthr[j];
@@ -265,7 +272,7 @@ __device__ bool build_index(const DeviceCatalog &c, uint32_t t, uint32_t F, Inde
   // is < r and whose accuracy rank is >= k: a running minimum over the entries in latency order.
   // A thread takes one column and one run of entries: here the run's minimum.
   const uint32_t cols = (width + 31u) >> 5, runs = REBUILD_WARPS / cols;      // warps side by side; at least 4 runs
-  const uint32_t run_len = ((F + runs - 1u) / runs + 3u) & ~3u;
+  const uint32_t run_len = max(8u, ((F + runs - 1u) / runs + 3u) & ~3u);
   const uint32_t run = warp / cols, col = (warp - run * cols) * 32u + lane;
   const uint32_t i0 = min(F, run * run_len), i1 = run < runs ? min(F, i0 + run_len) : i0;
   const uint32_t col_key = col << 16;
@@ -278,34 +285,18 @@ __device__ bool build_index(const DeviceCatalog &c, uint32_t t, uint32_t F, Inde
     }
     S.part[run * cols * 32u + col] = (unsigned char)v;
   }
-  // what the nearest-miss search reads, as running aggregates over the ranks: bestA[r] over
-  // latency ranks < r (and with it the stair entries: those more accurate than everything
-  // faster), bestB[k] over accuracy ranks >= k, ord_start[r] = stair entries with latency rank < r
-  if (warp == 0u) {
-    uint32_t carry = 0, stairs = 0;
-    for (uint32_t c0 = 0; c0 <= Ks; c0 += 32u) {
-      const uint32_t i = c0 + lane, x = i < Ks ? S.rankA[i] : 0u;
-      const uint32_t incl = max(warp_scan_max(x), carry);
-      const uint32_t up = __shfl_up_sync(0xFFFFFFFFu, incl, 1), before = lane ? up : carry;
-      const bool st = i < Ks && (before == 0u || (x >> 16) > (before >> 16));
-      const unsigned m = __ballot_sync(0xFFFFFFFFu, st);
-      if (i <= Ks) {
-        S.bestA[i] = before;
-        S.ord_start[i] = (unsigned char)(stairs + __popc(m & ((1u << lane) - 1u)));
-      }
-      if (i < Ks) S.stair[i] = st;
-      stairs += __popc(m);
-      carry = __shfl_sync(0xFFFFFFFFu, incl, 31);
-    }
-  } else if (warp == 1u) {
-    unsigned long long carry = ~0ull;
-    if (lane == 0u) S.bestB[Ka] = ~0ull;
-    for (uint32_t c0 = 0; c0 < Ka; c0 += 32u) {              // from the top down
-      const uint32_t q = c0 + lane;
-      const unsigned long long x = min(warp_scan_min(q < Ka ? S.rankB[Ka - 1u - q] : ~0ull), carry);
-      if (q < Ka) S.bestB[Ka - 1u - q] = x;
-      carry = __shfl_sync(0xFFFFFFFFu, x, 31);
-    }
+  // stair entries: those more accurate than everything faster (one per latency at most); 32 latency
+  // ranks per warp
+  uint32_t best_a = 0;                                            // latency ranks < this thread's
+  if (32u * warp <= Ks) {
+    const uint32_t r = tid;
+    uint32_t below = 0;
+#pragma unroll 1
+    for (uint32_t i = lane; i < 32u * warp; i += 32u) below = max(below, S.rankA[i]);
+    below = __reduce_max_sync(0xFFFFFFFFu, below);
+    const uint32_t x = r < Ks ? S.rankA[r] : 0u;
+    best_a = max(below, lanes_before(warp_scan_max(x), 0u));
+    if (r < Ks) S.stair[r] = best_a == 0u || (x >> 16) > (best_a >> 16);
   }
   if (tid == B - 1u) {
     uint32_t base = image_var_offset(c.n_tasks, nbw) + place_block_finish(c, placed, BL.bytes, next == 0u);
@@ -323,6 +314,7 @@ __device__ bool build_index(const DeviceCatalog &c, uint32_t t, uint32_t F, Inde
   unsigned char *T2 = blk + BL.t2;
   if (i0 < i1 && col < width) {
     uint32_t v = F;
+#pragma unroll 4
     for (uint32_t w = 0; w < run; ++w) v = min(v, (uint32_t)S.part[w * cols * 32u + col]);
     if (run == 0u) T2[col] = (unsigned char)F;                   // nothing is fast enough
     unsigned char *row = T2 + (S.rank[i0] + 1u) * width + col;
@@ -339,31 +331,45 @@ __device__ bool build_index(const DeviceCatalog &c, uint32_t t, uint32_t F, Inde
   // `body(x)` for x = 0 .. count - 1
   auto share = [&](uint32_t lo, uint32_t n, uint32_t count, auto body) {
     if (tid >= lo && tid < lo + n)
+#pragma unroll 1
       for (uint32_t x = tid - lo; x < count; x += n) body(x);
   };
   uint32_t *bitmap = first ? reinterpret_cast<uint32_t *>(c.image + image_bitmap_offset(c.n_tasks) + t * bitmap_stride(nbw))
                            : reinterpret_cast<uint32_t *>(blk + BL.bitmap);
   share(0, B / 4u, nbw, [&](uint32_t w) { bitmap[w] = ((uint32_t)S.wpre[w] << 24) | S.wbits[w]; });
-  uint32_t *bestA = reinterpret_cast<uint32_t *>(slow + SL.bestA);
-  uint2 *walk = reinterpret_cast<uint2 *>(slow + SL.walk);      // the stair entries, ascending latency
-  share(B / 4u, B / 4u, Ks + 1u, [&](uint32_t r) {               // position 0xFF stands for "none"
-    const uint32_t v = S.bestA[r], o = S.ord_start[r];
-    bestA[r] = v ? (v >> 16) | ((0xFFFFu - (v & 0xFFFFu)) << 16) : 0xFFu << 16;
-    slow[SL.ordStart + r] = (unsigned char)o;
-    if (r < Ks && S.stair[r]) {
+  // what the nearest-miss search reads: bestA[r] over latency ranks < r, the stair entries in
+  // ascending latency, ordStart[r] = stair entries with latency rank < r (the warps of step 4);
+  // position 0xFF stands for "none"
+  if (32u * warp <= Ks) {
+    const uint32_t r = tid;
+    uint32_t before = 0;
+#pragma unroll 1
+    for (uint32_t i = lane; i < 32u * warp; i += 32u) before += __popc(__ballot_sync(0xFFFFFFFFu, S.stair[i]));
+    const bool st = r < Ks && S.stair[r];
+    const uint32_t o = before + __popc(__ballot_sync(0xFFFFFFFFu, st) & ((1u << lane) - 1u));
+    if (r <= Ks) {
+      reinterpret_cast<uint32_t *>(slow + SL.bestA)[r] =
+          best_a ? (best_a >> 16) | ((0xFFFFu - (best_a & 0xFFFFu)) << 16) : 0xFFu << 16;
+      slow[SL.ordStart + r] = (unsigned char)o;
+    }
+    if (st) {
       const uint32_t a = S.rankA[r];
-      walk[o] = make_uint2(S.Pd[r], (a >> 16) | ((0xFFFFu - (a & 0xFFFFu)) << 16));
+      reinterpret_cast<uint2 *>(slow + SL.walk)[o] = make_uint2(S.Pd[r], (a >> 16) | ((0xFFFFu - (a & 0xFFFFu)) << 16));
     }
-    if (r == Ks) {
-      const uint32_t nxt = next;
-      c.slow[first ? t : c.n_tasks + xi] = make_uint4(base + BL.slow, F | (Ks << 8) | (Ka << 16), 0u, o | (nxt << 8));
-    }
-  });
-  uint2 *bestB = reinterpret_cast<uint2 *>(slow + SL.bestB);
-  share(B / 2u, B / 4u, Ka + 1u, [&](uint32_t k) {
-    const unsigned long long v = S.bestB[k];
-    bestB[k] = v == ~0ull ? make_uint2(0u, 0xFFu) : make_uint2((uint32_t)(v >> 32), (uint32_t)v);
-  });
+    if (r == Ks)
+      c.slow[first ? t : c.n_tasks + xi] = make_uint4(base + BL.slow, F | (Ks << 8) | (Ka << 16), 0u, o | (next << 8));
+  }
+  // bestB[k] over accuracy ranks >= k, 32 ranks from the top down per warp
+  if (warp >= 8u && warp < 16u && 32u * (warp - 8u) <= Ka) {
+    const uint32_t q0 = 32u * (warp - 8u), q = q0 + lane;        // q-th value of bestB from the top; bestB[Ka] is none
+    uint32_t above = NONE;
+#pragma unroll 1
+    for (uint32_t i = lane; i < q0; i += 32u) above = min(above, S.rankB[Ka - 1u - i]);
+    above = __reduce_min_sync(0xFFFFFFFFu, above);
+    const uint32_t i = min(above, lanes_before(warp_scan_min(q < Ka ? S.rankB[Ka - 1u - q] : NONE), NONE));
+    if (q <= Ka)
+      reinterpret_cast<uint2 *>(slow + SL.bestB)[Ka - q] = i == NONE ? make_uint2(0u, 0xFFu) : make_uint2(S.sorted[i], S.at[i]);
+  }
   uint32_t *ids_end = reinterpret_cast<uint32_t *>(blk + BL.t2);   // ids, reversed; slot F holds PENDING
   uint32_t *Pd_g = reinterpret_cast<uint32_t *>(slow + SL.Pd);
   share(3u * B / 4u, B / 4u, F + 1u, [&](uint32_t p) {
@@ -379,16 +385,18 @@ __device__ bool build_index(const DeviceCatalog &c, uint32_t t, uint32_t F, Inde
 
 // What the queue recursion reads of one variant.
 struct Row {
-  uint32_t lat, batch, queued, id, order, count, state, load_lat;
+  uint32_t lat, batch, queued, id, order, count, state, load_lat, drain;
   unsigned long long served;
 };
 // ... what no kernel writes
-__device__ __forceinline__ Row load_fixed(const DeviceCatalog &c, uint32_t slot) {
+__device__ __forceinline__ Row load_fixed(const DeviceCatalog &c, uint32_t slot, uint32_t window_us) {
   Row r;
   r.lat = c.s_lat[slot];
   r.batch = c.s_batch[slot];
   r.order = c.s_order[slot];
   r.id = c.s_id[slot];
+  const unsigned long long drain = (unsigned long long)window_us * r.batch / r.lat;   // queries served per window
+  r.drain = drain > NONE ? NONE : (uint32_t)drain;
   return r;
 }
 // ... and the rest
@@ -402,19 +410,14 @@ __device__ __forceinline__ void load_load(const DeviceCatalog &c, uint32_t slot,
   }
 }
 // Queue recursion and states; returns the predicted latency and leaves the new state in r.state.
-__device__ __forceinline__ uint32_t advance_row(const DeviceCatalog &c, uint32_t slot, Row &r, bool advance,
-                                                uint32_t window_us) {
+__device__ __forceinline__ uint32_t advance_row(const DeviceCatalog &c, uint32_t slot, Row &r, bool advance) {
   uint32_t queued = r.queued;
   if (advance) {
     unsigned long long arrived = (unsigned long long)queued + r.count;
     if (arrived > NONE) arrived = NONE;
-    unsigned long long drain = (unsigned long long)window_us * r.batch / r.lat;
-    if (drain > NONE) drain = NONE;
-    queued = arrived > drain ? (uint32_t)(arrived - drain) : 0u;
+    queued = arrived > r.drain ? (uint32_t)arrived - r.drain : 0u;
     c.s_served[slot] = r.served + r.count;
     c.s_queued[slot] = queued;
-    c.count_by_id[r.id] = 0;        // not right behind its load: a store to an address whose load is
-                                    // still in flight holds up everything behind it (measured: 4 us)
     if (c.stateful) {
       // loaded by its first queries; at peak throughput while a backlog remains
       if (r.state == INFAAS_STATE_INACTIVE && r.count > 0) r.state = INFAAS_STATE_ACTIVE;
@@ -423,7 +426,11 @@ __device__ __forceinline__ uint32_t advance_row(const DeviceCatalog &c, uint32_t
       c.s_state[slot] = (unsigned char)r.state;
     }
   }
-  const unsigned long long p = (unsigned long long)r.lat + (unsigned long long)queued * r.lat / r.batch;
+  unsigned long long p = r.lat;
+  if (queued) {                     // batch sizes are mostly powers of two
+    const unsigned long long w = (unsigned long long)queued * r.lat;
+    p += r.batch & (r.batch - 1u) ? w / r.batch : w >> (31 - __clz((int)r.batch));
+  }
   const uint32_t pred = p > NONE ? NONE : (uint32_t)p;
   c.s_pred[slot] = pred;
   return pred;
@@ -447,22 +454,24 @@ __device__ __forceinline__ uint32_t advance_row(const DeviceCatalog &c, uint32_t
 // pred; at most the fastest variant (lowest id) of every distinct accuracy is on it, if it is
 // faster than everything more accurate, and the list runs from the lowest accuracy up.
 //
-// Bound by the latency of its chain of barriers, shared-memory round trips and the loads at its
-// start; measured on one B200: 64 tasks x 256 variants, lists of up to 100 entries: 10.8 us (22.9
-// with pair loops over variants and survivors), 128 x 512: 12.2 us (33.8), 4 x 4096 on a trade-off
-// surface, lists of up to 505 entries: 52 us (340 with a sort and a scan of the sorted entries).
+// Bound by the latency of its chain of barriers and shared-memory round trips, and by fetching its
+// code: every line of it runs about once per launch, and with the compiler's unrolling (116 KB of
+// code) 40 % of the stalls were for instructions.  So the loops are not unrolled (47 KB) except the
+// few that run long.  Measured on one B200, in GPU clock cycles after the previous kernel's end: 64
+// tasks x 256 variants, lists of up to 100 entries: 16 K (18 K unrolled), 128 x 512: 19 K (22 K), 4 x
+// 4096 on a trade-off surface, lists of up to 505 entries: 77 K (90 K), two lists per task: 17 K
+// (23 K).  512 threads instead of 1024: short lists 5 % faster, lists of 100 entries 5 % slower.
 __global__ void __launch_bounds__(REBUILD_THREADS)
 rebuild_kernel(DeviceCatalog c, int advance, uint32_t window_us) {
   extern __shared__ __align__(16) unsigned char dyn[];
   constexpr uint32_t KEEP_WORDS = INFAAS_MAX_TASK_VARIANTS / 32;
-  constexpr uint32_t POOL = sizeof(IndexScratch) > GRID * GRID_PITCH * 4 ? sizeof(IndexScratch) : GRID * GRID_PITCH * 4;
-  __shared__ __align__(16) unsigned char pool[POOL];              // the grid, then the index scratch
-  __shared__ uint32_t keep[KEEP_WORDS + 1], keep_pre[KEEP_WORDS + 1];
+  __shared__ uint32_t grid[GRID * GRID_PITCH];
+  __shared__ __align__(16) IndexScratch S;
+  __shared__ uint32_t keep[KEEP_WORDS + 1], keep_pre[KEEP_WORDS + 1];   // bit sets: survivors, by local index ...
+  __shared__ uint32_t passed_local[KEEP_WORDS], passed_acc[KEEP_WORDS];   // ... what the grid lets through, both orders
   __shared__ unsigned long long warp_min[REBUILD_WARPS];
   __shared__ uint32_t warp_cnt[REBUILD_WARPS];
-  __shared__ uint32_t n_cand;
-  uint32_t *grid = reinterpret_cast<uint32_t *>(pool);
-  IndexScratch &S = *reinterpret_cast<IndexScratch *>(pool);
+  __shared__ uint32_t n_cand, n_inactive;
   constexpr uint32_t B = REBUILD_THREADS;
 
   const uint32_t t = blockIdx.x, tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
@@ -478,32 +487,36 @@ rebuild_kernel(DeviceCatalog c, int advance, uint32_t window_us) {
   uint32_t *ids_g = reinterpret_cast<uint32_t *>(region + 8u * V);
 
   // 1. queue recursion, states, predicted latencies; coarse grid.  Each thread's first variant
-  // stays in registers.
+  // stays in registers.  Before chain_wait: only what no kernel writes, and clearing.
   Row r0;
-  uint32_t acc0 = 0, run0 = 0, pred0 = 0;
+  uint32_t acc0 = 0, run0 = 0, class0 = 0, pred0 = 0;
   if (tid < V) {
-    r0 = load_fixed(c, base + tid);
+    r0 = load_fixed(c, base + tid, window_us);
     acc0 = c.s_acc[base + tid];
     run0 = c.s_cost_run[base + tid];
+    if (c.stateful) class0 = c.s_class[base + tid];
   }
-  chain_wait();
-  chain_next();
-  if (tid < V) load_load(c, base + tid, advance, r0);
   uint32_t cs = 4;                                                 // log2 of the rows' and columns' run length
+#pragma unroll 1
   while (V > (GRID << cs)) ++cs;
   const uint32_t ng = (V + (1u << cs) - 1u) >> cs;
+#pragma unroll 1
   for (uint32_t i = tid; i < ng * GRID_PITCH; i += B) grid[i] = NONE;
+#pragma unroll 1
   for (uint32_t i = tid; i < V; i += B) run_min[i] = NONE;
-  for (uint32_t i = tid; i <= KEEP_WORDS; i += B) keep[i] = 0u;
-  if (tid == 0u) n_cand = 0u;
+#pragma unroll 1
+  for (uint32_t i = tid; i <= KEEP_WORDS; i += B) { keep[i] = 0u; if (i < KEEP_WORDS) passed_acc[i] = 0u; }
+  clear_scratch(S);
+  if (tid == 0u) { n_cand = 0u; n_inactive = 0u; }
   __syncthreads();
-  for (uint32_t i = tid; i < V; i += B) {
-    Row r = r0;
-    if (i != tid) {
-      r = load_fixed(c, base + i);
-      load_load(c, base + i, advance, r);
-    }
-    const uint32_t pred = advance_row(c, base + i, r, advance, window_us);
+  chain_wait();
+  chain_next();
+  const uint32_t slo_seen = *c.slo_seen;
+  Row r = r0;
+#pragma unroll 1
+  for (uint32_t i = tid; i < V;) {
+    load_load(c, base + i, advance, r);
+    const uint32_t pred = advance_row(c, base + i, r, advance);
     const uint32_t pos = r.order & 0x1FFFu;
     if (r.state == INFAAS_STATE_ACTIVE) {
       by_local[i] = make_uint2(pred, pos);
@@ -515,10 +528,15 @@ rebuild_kernel(DeviceCatalog c, int advance, uint32_t window_us) {
       by_local[i] = make_uint2(NONE, 0xFFFFu);
       by_acc[pos] = make_uint2(NONE, 0xFFFFu);
     }
-    if (i == tid) { pred0 = pred; r0.state = r.state; }
+    if (i == tid) { pred0 = pred; r0.state = r.state; r0.load_lat = r.load_lat; }
+    i += B;
+    if (i < V) r = load_fixed(c, base + i, window_us);
   }
+  uint32_t bmin, Sh;                                               // SLO buckets
+  bucket_scale(c, slo_seen, Sh, bmin);
   __syncthreads();
   // 2. running minimum along the rows, then down the columns (GRID = two values per lane)
+#pragma unroll 1
   for (uint32_t y = warp; y < ng; y += REBUILD_WARPS) {
     uint32_t *row = grid + y * GRID_PITCH;
     const uint32_t x0 = warp_scan_min(lane < ng ? row[lane] : NONE);
@@ -530,6 +548,7 @@ rebuild_kernel(DeviceCatalog c, int advance, uint32_t window_us) {
     }
   }
   __syncthreads();
+#pragma unroll 1
   for (uint32_t x = warp; x < ng; x += REBUILD_WARPS) {
     uint32_t *col = grid + x;
     const uint32_t x0 = warp_scan_min(lane < ng ? col[lane * GRID_PITCH] : NONE);
@@ -542,6 +561,7 @@ rebuild_kernel(DeviceCatalog c, int advance, uint32_t window_us) {
   }
   __syncthreads();
   // 3. what the grid lets through ...
+#pragma unroll 1
   for (uint32_t i0 = 0; i0 < V; i0 += B) {
     const uint32_t i = i0 + tid;
     bool pass = false;
@@ -560,35 +580,52 @@ rebuild_kernel(DeviceCatalog c, int advance, uint32_t window_us) {
     uint32_t at = 0;
     if (m && lane == 0u) at = atomicAdd(&n_cand, (uint32_t)__popc(m));
     at = __shfl_sync(0xFFFFFFFFu, at, 0);
-    if (pass) cand[at + __popc(m & ((1u << lane) - 1u))] = (uint16_t)i;
+    if (lane == 0u && i < V) passed_local[i >> 5] = m;
+    if (pass) {
+      cand[at + __popc(m & ((1u << lane) - 1u))] = (uint16_t)i;
+      const uint32_t pos = by_local[i].y;
+      atomicOr(&passed_acc[pos >> 5], 1u << (pos & 31u));
+    }
   }
   __syncthreads();
-  // 4. ... against its own row and column of the grid, 8 lanes per entry
+  // 4. ... against the entries before it in its own row and column of the grid that were let through
+  // too (dominance is transitive and what is dominated by nothing is let through): one lane for
+  // the row, one for the column
   const uint32_t nc = n_cand;
-  for (uint32_t x0 = 0; x0 < nc; x0 += B / 8u) {
-    const uint32_t x = x0 + (tid >> 3), sub = tid & 7u;
+#pragma unroll 1
+  for (uint32_t x0 = 0; x0 < nc; x0 += B / 2u) {
+    const uint32_t x = x0 + (tid >> 1);
     uint32_t dom = 0, p = 0;
     if (x < nc) {
       p = cand[x];
       const uint2 a = by_local[p];
-      const uint32_t lo = a.x == NONE - 1u ? 0u : (p >> cs) << cs;
-      for (uint32_t q = lo + sub; q < p; q += 8u) {
-        const uint2 b = by_local[q];
-        dom |= (uint32_t)(b.x <= a.x) & (uint32_t)(b.y < a.y);
-      }
-      for (uint32_t j = ((a.y >> cs) << cs) + sub; j < a.y; j += 8u) {
-        const uint2 b = by_acc[j];
-        dom |= (uint32_t)(b.x <= a.x) & (uint32_t)(b.y < p);
+      const bool row = !(tid & 1u);
+      const uint2 *v = row ? by_local : by_acc;
+      const uint32_t *bits = row ? passed_local : passed_acc;
+      const uint32_t hi = row ? p : a.y, limit = row ? a.y : p;
+      const uint32_t lo = row && a.x == NONE - 1u ? 0u : (hi >> cs) << cs;
+#pragma unroll 1
+      for (uint32_t w = lo >> 5; w <= hi >> 5 && !dom; ++w) {
+        uint32_t m = bits[w];
+        if (w == lo >> 5) m &= ~0u << (lo & 31u);
+        if (w == hi >> 5) m &= (1u << (hi & 31u)) - 1u;
+#pragma unroll 1
+        while (m && !dom) {
+          const uint2 b = v[32u * w + (uint32_t)__ffs(m) - 1u];
+          m &= m - 1u;
+          dom = (uint32_t)(b.x <= a.x) & (uint32_t)(b.y < limit);
+        }
       }
     }
-    dom = group8_or(dom);
-    if (x < nc && sub == 0u && !dom) atomicOr(&keep[p >> 5], 1u << (p & 31u));
+    dom |= __shfl_xor_sync(0xFFFFFFFFu, dom, 1);
+    if (x < nc && !(tid & 1u) && !dom) atomicOr(&keep[p >> 5], 1u << (p & 31u));
   }
   __syncthreads();
-  // 5. survivors before each word of the bit set (warp 0); scratch of the next steps
+  // 5. survivors before each word of the bit set (warp 0)
   const uint32_t n_words = (V + 31u) >> 5;
   if (warp == 0u) {
     uint32_t carry = 0;
+#pragma unroll 1
     for (uint32_t w0 = 0; w0 <= n_words; w0 += 32u) {
       const uint32_t w = w0 + lane, pc = w < n_words ? __popc(keep[w]) : 0u;
       const uint32_t incl = carry + warp_scan_add(pc);
@@ -596,10 +633,10 @@ rebuild_kernel(DeviceCatalog c, int advance, uint32_t window_us) {
       carry = __shfl_sync(0xFFFFFFFFu, incl, 31);
     }
   }
-  clear_scratch(S);                                                // the grid is not needed any more
-  unsigned long long *class_best = reinterpret_cast<unsigned long long *>(by_acc);   // nor is by_acc
   const uint32_t n_class = c.stateful ? c.n_class[t] : 0u;
-  for (uint32_t k = tid; k < n_class; k += B) class_best[k] = ~0ull;
+  uint32_t *class_eff = reinterpret_cast<uint32_t *>(by_acc), *class_id = class_eff + n_class;   // by_acc is not needed any more
+#pragma unroll 1
+  for (uint32_t k = tid; k < n_class; k += B) { class_eff[k] = NONE; class_id[k] = NONE; }
   __syncthreads();
   // 6. the list into the task's region, its first segment also into the index scratch
   auto emit = [&](uint32_t pos, uint32_t pred, uint32_t acc, uint32_t id) {
@@ -608,6 +645,7 @@ rebuild_kernel(DeviceCatalog c, int advance, uint32_t window_us) {
     if (pos < INDEX_MAX_F) { S.ids[pos] = id; S.pred[pos] = pred; S.acc[pos] = (uint16_t)acc; }
   };
   auto before = [&](uint32_t i) { return keep_pre[i >> 5] + __popc(keep[i >> 5] & ((1u << (i & 31u)) - 1u)); };
+#pragma unroll 1
   for (uint32_t i = tid; i < V; i += B) {
     if (!((keep[i >> 5] >> (i & 31u)) & 1u)) continue;
     const bool reg = i == tid;
@@ -615,53 +653,83 @@ rebuild_kernel(DeviceCatalog c, int advance, uint32_t window_us) {
     const uint32_t pos = before(run & 0xFFFFu) + before(run >> 16) - 1u - before(i);
     emit(pos, reg ? pred0 : by_local[i].x, reg ? acc0 : c.s_acc[base + i], reg ? r0.id : c.s_id[base + i]);
   }
+  // the counts are cleared here, far behind their loads: a store to a line whose load is still in flight
+  // holds up everything behind it (4 us a launch when the store came right behind)
+  if (advance)
+#pragma unroll 1
+    for (uint32_t i = tid; i < V; i += B) c.count_by_id[i == tid ? r0.id : c.s_id[base + i]] = 0u;
   uint32_t F = keep_pre[n_words];
   if (c.stateful) {
-    for (uint32_t i = tid; i < V; i += B) {
-      const uint32_t st = i == tid ? r0.state : c.s_state[base + i];
-      if (st != INFAAS_STATE_INACTIVE) continue;
+    // the fastest Inactive variant of every accuracy class: its latency, then the lowest id with it
+    auto eff_of = [&](uint32_t i) {
       const unsigned long long e = (unsigned long long)(i == tid ? pred0 : c.s_pred[base + i]) +
                                    (i == tid ? r0.load_lat : c.s_load_lat[base + i]);
-      const uint32_t eff = e > NONE ? NONE : (uint32_t)e;
-      atomicMin(&class_best[c.s_class[base + i]], ((unsigned long long)eff << 32) | (i == tid ? r0.id : c.s_id[base + i]));
-    }
-    __syncthreads();
-    // each thread takes consecutive classes: running minimum from the highest accuracy down,
-    // survivors, their number
-    const uint32_t per = (n_class + B - 1u) / B, k0 = min(n_class, tid * per), k1 = min(n_class, k0 + per);
-    unsigned long long mine = ~0ull;
-    for (uint32_t k = k0; k < k1; ++k) mine = min(mine, class_best[k]);
-    const unsigned long long incl = warp_scan_min(mine);
-    if (lane == 31u) warp_min[warp] = incl;
-    __syncthreads();
-    unsigned long long best = __shfl_up_sync(0xFFFFFFFFu, incl, 1);
-    if (lane == 0u) best = ~0ull;
-    for (uint32_t w = 0; w < warp; ++w) best = min(best, warp_min[w]);
-    // on the list: faster than every more accurate variant (equally fast ones are dominated)
-    auto listed = [](unsigned long long x, unsigned long long ahead) {
-      return x != ~0ull && (ahead == ~0ull || (uint32_t)(x >> 32) < (uint32_t)(ahead >> 32));
+      return e > NONE ? NONE : (uint32_t)e;
     };
+    auto inactive = [&](uint32_t i) { return (i == tid ? r0.state : c.s_state[base + i]) == INFAAS_STATE_INACTIVE; };
+    auto class_of = [&](uint32_t i) { return i == tid ? class0 : c.s_class[base + i]; };
+#pragma unroll 1
+    for (uint32_t i = tid; i < V; i += B)
+      if (inactive(i)) atomicMin(&class_eff[class_of(i)], eff_of(i));
+    __syncthreads();
+#pragma unroll 1
+    for (uint32_t i = tid; i < V; i += B)
+      if (inactive(i) && class_eff[class_of(i)] == eff_of(i)) atomicMin(&class_id[class_of(i)], i == tid ? r0.id : c.s_id[base + i]);
+    __syncthreads();
+    // each thread takes consecutive classes (one, up to 1024 of them): running minimum from the
+    // highest accuracy down, survivors, their number.  A class without entry counts as 2^32.
+    const uint32_t per = max(1u, (n_class + B - 1u) / B), k0 = min(n_class, tid * per), k1 = min(n_class, k0 + per);
+    const uint32_t used = (n_class + 32u * per - 1u) / (32u * per);        // warps that have classes
+    auto eff_at = [&](uint32_t k) { return class_id[k] == NONE ? 1ull << 32 : (unsigned long long)class_eff[k]; };
+    unsigned long long mine = 1ull << 32;
+#pragma unroll 1
+    for (uint32_t k = k0; k < k1; ++k) mine = min(mine, eff_at(k));
+    unsigned long long best = 1ull << 32;
+    if (warp < used) {
+      const unsigned long long incl = warp_scan_min(mine);
+      if (lane == 31u) warp_min[warp] = incl;
+      best = __shfl_up_sync(0xFFFFFFFFu, incl, 1);
+      if (lane == 0u) best = 1ull << 32;
+    }
+    if (used > 1u) {
+      __syncthreads();
+#pragma unroll 1
+      for (uint32_t w = 0; w < min(warp, used); ++w) best = min(best, warp_min[w]);
+    }
+    // on the list: faster than every more accurate variant (equally fast ones are dominated)
     uint32_t n = 0;
     unsigned long long ahead = best;
+#pragma unroll 1
     for (uint32_t k = k0; k < k1; ++k) {
-      n += listed(class_best[k], ahead);
-      ahead = min(ahead, class_best[k]);
+      const unsigned long long x = eff_at(k);
+      n += x < ahead;
+      ahead = min(ahead, x);
     }
     const uint32_t n_incl = warp_scan_add(n);
     if (lane == 31u) warp_cnt[warp] = n_incl;
+    if (used > 1u) __syncthreads();
+    if (warp < used) {
+      uint32_t before_n = n_incl - n, total = 0;
+      if (used > 1u) {
+#pragma unroll 1
+        for (uint32_t w = 0; w < used; ++w) {
+          before_n += w < warp ? warp_cnt[w] : 0u;
+          total += warp_cnt[w];
+        }
+      } else {
+        total = __shfl_sync(0xFFFFFFFFu, n_incl, 31);
+      }
+      if (tid == 0u) n_inactive = total;
+      ahead = best;
+#pragma unroll 1
+      for (uint32_t k = k0; k < k1; ++k) {
+        const unsigned long long x = eff_at(k);
+        if (x < ahead) { emit(F + total - 1u - before_n, (uint32_t)x, c.class_acc[base + k], class_id[k]); ++before_n; }
+        ahead = min(ahead, x);
+      }
+    }
     __syncthreads();
-    uint32_t ahead_n = n_incl - n, total = 0;
-    for (uint32_t w = 0; w < REBUILD_WARPS; ++w) {
-      ahead_n += w < warp ? warp_cnt[w] : 0u;
-      total += warp_cnt[w];
-    }
-    ahead = best;
-    for (uint32_t k = k0; k < k1; ++k) {
-      const unsigned long long x = class_best[k];
-      if (listed(x, ahead)) { emit(F + total - 1u - ahead_n, (uint32_t)(x >> 32), c.class_acc[base + k], (uint32_t)x); ++ahead_n; }
-      ahead = min(ahead, x);
-    }
-    F += total;
+    F += n_inactive;
   }
   __syncthreads();
   bool indexed = F > 0;
@@ -672,19 +740,21 @@ rebuild_kernel(DeviceCatalog c, int advance, uint32_t window_us) {
   // (INDEX_MAX_F positions each; almost always one)
   if (indexed) {
     const uint32_t nseg = (F + INDEX_MAX_F - 1u) / INDEX_MAX_F, x0 = c.seg_base[t];
+#pragma unroll 1
     for (uint32_t sg = 0; sg < nseg && indexed; ++sg) {
       const uint32_t off = sg * INDEX_MAX_F, Fseg = min(INDEX_MAX_F, F - off);
       if (sg) {                                   // later segments: back from the task's region
         __syncthreads();
         clear_scratch(S);
         __syncthreads();
+#pragma unroll 1
         for (uint32_t i = tid; i < Fseg; i += B) {
           const unsigned long long e = keys_g[off + i];
           S.ids[i] = ids_g[off + i]; S.pred[i] = (uint32_t)e; S.acc[i] = (uint16_t)(e >> 32);
         }
         __syncthreads();
       }
-      indexed = build_index(c, t, Fseg, S, sg ? x0 + sg - 1u : NONE, sg + 1u < nseg ? x0 + sg + 1u : 0u);
+      indexed = build_index(c, t, Fseg, S, sg ? x0 + sg - 1u : NONE, sg + 1u < nseg ? x0 + sg + 1u : 0u, Sh, bmin);
       counted = sg + 1u == nseg;
     }
   }
@@ -695,22 +765,22 @@ rebuild_kernel(DeviceCatalog c, int advance, uint32_t window_us) {
     if (tid == 0u) c.slow[t] = make_uint4(0u, 0u, F == 0 ? TASK_FLAG_INVALID : TASK_FLAG_NOT_INDEXED, 0u);
   }
   if (t == 0u) {
-    // entry n_tasks (queries whose task is out of range), the dummy block, and the bucket scale
-    // every CTA has used, for the selection kernel
-    write_dummy_task(c, c.n_tasks);
-    if (tid < IMAGE_DUMMY_BYTES / 4u) reinterpret_cast<uint32_t *>(c.image)[tid] = tid == 3u ? PENDING : 0u;
+    // the bucket scale every CTA has used, for the selection kernel; at load time also entry n_tasks
+    // (queries whose task is out of range) and the dummy block, which never change
     if (tid == 0u) {
-      uint32_t Sh, bmin;
-      bucket_scale(c, Sh, bmin);
       c.image_hdr[1] = (127u - Sh) << 23;
       c.image_hdr[2] = __float_as_uint(-(float)bmin);
+    }
+    if (!advance) {
+      write_dummy_task(c, c.n_tasks);
+      if (tid < IMAGE_DUMMY_BYTES / 4u) reinterpret_cast<uint32_t *>(c.image)[tid] = tid == 3u ? PENDING : 0u;
     }
   }
   if (tid == 0u) c.f_len[t] = F;
 }
 
 // The block sizes the thread ranges above rely on.
-static_assert(REBUILD_THREADS == 1024 && SLO_BUCKETS == 256 && INDEX_MAX_F < 256, "thread ranges of build_index");
+static_assert(REBUILD_THREADS >= 512 && SLO_BUCKETS == 256 && INDEX_MAX_F < 256, "thread ranges of build_index");
 
 }  // namespace
 
