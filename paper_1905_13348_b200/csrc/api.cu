@@ -18,6 +18,7 @@ struct infaas_catalog {
   uint32_t *slot_of_id = nullptr;        // device, by variant id
   std::vector<uint32_t> task_off, reg_off;
   uint32_t select_smem = 0;              // shared memory reserved for the staged image
+  uint32_t image_seen = 0;               // size of the image when the host last looked
   uint32_t worst_image_bytes = 0;        // image size if every block had its largest size
   uint32_t *s_inst = nullptr;            // running instances per slot (Model-Autoscaler)
   uint16_t *s_arch = nullptr;            // architecture code per slot
@@ -101,6 +102,7 @@ inline uint32_t float_bits_rz(uint32_t x) {
 void plan_select(infaas_catalog *c, uint32_t image_bytes) {
   const uint32_t room = infaas::select_image_smem(infaas::SELECT_MAX_SMEM);
   c->select_smem = image_bytes <= room ? room : 0u;
+  c->image_seen = image_bytes;
 }
 int refresh_select_plan(infaas_catalog *c, cudaStream_t stream) {
   uint32_t image_bytes = 0;
@@ -237,7 +239,7 @@ int infaas_catalog_load(const infaas_variant *rows, uint32_t n_variants, uint32_
   // ---- one arena, carved into 256-byte aligned arrays ----
   // lists longer than the index supports are cut into segments; every segment but a task's
   // first needs a header and parameters outside the image
-  uint64_t worst_image = infaas::image_var_offset(n_tasks, nbw);
+  uint64_t worst_image = infaas::image_var_offset(n_tasks, infaas::buckets_for(n_tasks, max_task), nbw);
   std::vector<uint32_t> seg_base(n_tasks + 1, 0);
   for (uint32_t t = 0; t < n_tasks; ++t) {
     const uint32_t V = task_off[t + 1] - task_off[t];
@@ -335,6 +337,7 @@ int infaas_catalog_load(const infaas_variant *rows, uint32_t n_variants, uint32_
   d.image = base + o_image;
   d.image_capacity = (uint32_t)worst_image;
   d.image_hdr = reinterpret_cast<uint32_t *>(base + o_hdr);
+  d.n_buckets = infaas::buckets_for(n_tasks, max_task);
   d.acc_lo = acc_lo;
   d.nbw = nbw;
   d.lat_code_lo = float_bits_rz(lat_min) >> 16;
@@ -387,7 +390,7 @@ int infaas_select_batch(infaas_catalog *c, const uint16_t *d_task, const uint32_
   DeviceScope scope(c->device);
   if (scope.status != cudaSuccess) return cuda_fail(scope.status);
   CUDA_TRY(infaas::launch_select(c->d, d_task, d_slo_us, d_min_acc_bp, n, d_decision, c->sm_count,
-                                 c->select_smem, /*tally=*/false, static_cast<cudaStream_t>(cuda_stream)));
+                                 c->select_smem, c->image_seen, /*tally=*/false, static_cast<cudaStream_t>(cuda_stream)));
   return INFAAS_OK;
 }
 
@@ -408,7 +411,7 @@ int infaas_select_update(infaas_catalog *c, const uint16_t *d_task, const uint32
   if (scope.status != cudaSuccess) return cuda_fail(scope.status);
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   CUDA_TRY(infaas::launch_select(c->d, d_task, d_slo_us, d_min_acc_bp, n, d_decision, c->sm_count,
-                                 c->select_smem, /*tally=*/true, s));
+                                 c->select_smem, c->image_seen, /*tally=*/true, s));
   CUDA_TRY(infaas::launch_rebuild(c->d, /*advance_queues=*/true, window_us, s));
   return INFAAS_OK;
 }

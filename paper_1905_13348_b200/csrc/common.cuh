@@ -30,8 +30,8 @@ namespace infaas {
 //   T2[r][k] = first position whose pred_lat is among the r smallest values and whose
 //              acc_bp is not among the k smallest values, or F if there is none.
 //
-// r comes from one record of a table of SLO_BUCKETS records per task.  The bucket of an
-// SLO is  j = clamp((bits(slo) >> S) - bmin, 0, 255)  with bits(x) = the IEEE-754 pattern
+// r comes from one record of a table of n_buckets records per task.  The bucket of an
+// SLO is  j = clamp((bits(slo) >> S) - bmin, 0, n_buckets - 1)  with bits(x) = the IEEE-754 pattern
 // of x converted to float toward zero (a monotone, roughly logarithmic code) and one S = 16..23
 // and bmin for the whole catalog.  A record is  R << 24 | C  and
 // r = (record + (slo & 0xFFFFFF)) >> 24:
@@ -39,11 +39,12 @@ namespace infaas {
 //   - one latency `thr` inside it, and all SLOs of the bucket agree in their top byte:
 //     R = rank below, C = 0xFFFFFF - ((thr - 1) & 0xFFFFFF), so the add carries into R
 //     exactly when slo >= thr;
-//   - otherwise R = Ks + 1, C = 0: row Ks + 1 of T2 holds only F, which sends the query to
-//     the exact slow path.
+//   - otherwise R = Ks + 1, C = rank below | latencies inside << 8: rows Ks + 1 and Ks + 2 (the add
+//     may carry) of T2 hold only F, which sends the query to the exact slow path; that finds the
+//     rank among the latencies the record names.
 // The buckets run from the smallest profiled latency of the catalog (a predicted latency is
 // never below it) up to the largest SLO any batch has asked for so far (kept as a bit mask,
-// at least SLO_CAP_FLOOR_US); larger latencies share bucket 255.  The rebuild kernel derives
+// at least SLO_CAP_FLOOR_US); larger latencies share the last bucket.  The rebuild kernel derives
 // S and bmin from these two and publishes them beside the image size.
 // k comes from a bitmap over accuracy values with running popcounts (24 bitmap bits and an
 // 8-bit prefix count per word), exact at one basis point.  Every bitmap covers the same
@@ -55,13 +56,13 @@ namespace infaas {
 //          "none" and goes to the slow path)
 //   hdr    (n_tasks + 1) u32, one per task: t2_off | (Ka + 1) << 24; entry n_tasks serves
 //          queries whose task is out of range; padded to 128 bytes
-//   rec    (n_tasks + 1) x SLO_BUCKETS u32 records, REC_STRIDE bytes apart
+//   rec    (n_tasks + 1) x (n_buckets + 1) u32 records (the last one twice), rec_stride(n_buckets) bytes apart
 //   bitmap (n_tasks + 1) x nbw u32: the accuracy bitmaps of the tasks' first segments,
 //          bitmap_stride(nbw) bytes apart
 //   var    per-segment blocks, each 16-byte aligned:
 //          ids   u32[F + 1] in REVERSE order: ids[p] sits at t2_off - 4 - 4p, and the slot
 //                of p = F holds PENDING -- the fast path needs no compare for "none"
-//          T2    u8[(Ks + 2) * (Ka + 1)]  at t2_off (a multiple of 4)
+//          T2    u8[(Ks + 3) * (Ka + 1)]  at t2_off (a multiple of 4)
 //          bitmap u32[nbw]  (further segments only)
 //          slow-path tables (SlowLayout below)
 //
@@ -70,7 +71,7 @@ namespace infaas {
 // lists without an index and for inspection.
 // ---------------------------------------------------------------------------------------
 constexpr uint32_t INDEX_MAX_F = 248;
-constexpr uint32_t SLO_BUCKETS = 256;
+constexpr uint32_t MIN_BUCKETS = 256, MAX_BUCKETS = 2048;
 constexpr uint32_t ACC_WORD_BITS = 24;
 constexpr uint32_t MAX_ACC_WORDS = 420;          // accuracies 0 .. 10000 need at most 417 + 1 words
 constexpr uint32_t IMAGE_T2_LIMIT = 1u << 24;    // t2_off is a 24-bit field
@@ -85,18 +86,28 @@ inline __host__ __device__ uint32_t round_up_u32(uint32_t x, uint32_t a) { retur
 // A task's records and its bitmap start an odd number of words after the previous task's, so
 // that the tasks' hot entries (the same buckets, the lowest bitmap word) fall into different
 // shared-memory banks.
-constexpr uint32_t REC_STRIDE = 4u * (SLO_BUCKETS + 1u);   // bytes from one task's records to the next's
+inline __host__ __device__ uint32_t rec_stride(uint32_t nb) { return 4u * (nb + 1u); }   // bytes from one task's records to the next's
+// SLO buckets per task: 256, more for tasks of more than 256 variants while all records together stay
+// within 48 KB (up to 23 tasks).  Long lists have several latencies per bucket, and every query of
+// such a bucket takes the slow path: 2^22 queries on 4 x 4096 variants (lists of up to 320 entries)
+// take 84 us with 256 buckets and 51 us with 2048; with 2048 for lists of 40 entries the rebuild only
+// takes 1 us longer.
+inline __host__ __device__ uint32_t buckets_for(uint32_t n_tasks, uint32_t max_task_variants) {
+  uint32_t nb = MIN_BUCKETS;
+  while (nb < MAX_BUCKETS && nb < max_task_variants && rec_stride(2u * nb) * (n_tasks + 1u) <= 48u * 1024u) nb *= 2u;
+  return nb;
+}
 inline __host__ __device__ uint32_t bitmap_stride(uint32_t nbw) { return 4u * (nbw | 1u); }   // same, bitmaps
 constexpr uint32_t IMAGE_DUMMY_BYTES = 64u;               // the dummy block opens the image
 constexpr uint32_t IMAGE_HDR_OFFSET = IMAGE_DUMMY_BYTES;  // the task words follow it
 inline __host__ __device__ uint32_t image_rec_offset(uint32_t n_tasks) {
   return round_up_u32(IMAGE_HDR_OFFSET + 4u * (n_tasks + 1u), 128u);
 }
-inline __host__ __device__ uint32_t image_bitmap_offset(uint32_t n_tasks) {
-  return image_rec_offset(n_tasks) + REC_STRIDE * (n_tasks + 1u);
+inline __host__ __device__ uint32_t image_bitmap_offset(uint32_t n_tasks, uint32_t nb) {
+  return image_rec_offset(n_tasks) + rec_stride(nb) * (n_tasks + 1u);
 }
-inline __host__ __device__ uint32_t image_var_offset(uint32_t n_tasks, uint32_t nbw) {
-  return round_up_u32(image_bitmap_offset(n_tasks) + bitmap_stride(nbw) * (n_tasks + 1u), 64u);
+inline __host__ __device__ uint32_t image_var_offset(uint32_t n_tasks, uint32_t nb, uint32_t nbw) {
+  return round_up_u32(image_bitmap_offset(n_tasks, nb) + bitmap_stride(nbw) * (n_tasks + 1u), 64u);
 }
 // The task word of a task without index (and of entry n_tasks): T2 is the one zero byte at
 // offset 16 of the dummy block with row width 0, the id slot of position 0 below it holds
@@ -137,7 +148,7 @@ struct BlockLayout {
 inline __host__ __device__ BlockLayout block_layout(uint32_t F, uint32_t Ks, uint32_t Ka, uint32_t nbw) {
   BlockLayout B;
   B.t2 = 4u * (F + 1u);
-  B.bitmap = round_up_u32(B.t2 + (Ks + 2u) * (Ka + 1u), 4u);
+  B.bitmap = round_up_u32(B.t2 + (Ks + 3u) * (Ka + 1u), 4u);
   B.slow = round_up_u32(B.bitmap + 4u * nbw, 8u);
   B.bytes = round_up_u32(B.slow + slow_layout(F, Ks, Ka).bytes, 16u);
   return B;
@@ -198,6 +209,7 @@ struct DeviceCatalog {
   uint32_t image_capacity;
   uint32_t *image_hdr;       // published by the rebuild kernel: [0] bytes of the image, [1] the bucket
                              // scale 2^-S and [2] -bmin, both as float patterns
+  uint32_t n_buckets;        // SLO buckets per task
   uint32_t acc_lo, nbw;      // accuracy window of every bitmap: acc_lo (multiple of 24) .. acc_lo + 24 nbw - 1
   uint32_t lat_code_lo;      // bits(smallest profiled latency) >> 16: where the SLO buckets start
 
@@ -271,14 +283,18 @@ cudaError_t launch_tally(const DeviceCatalog &c, const uint32_t *d_decision, uin
 uint32_t select_image_smem(uint32_t image_smem);
 // `image_smem`: bytes of dynamic shared memory reserved for the staged image (multiple of
 // 16).  If the image is larger at run time the kernel reads it from global memory instead.
+// `image_seen`: bytes of the image when the host last looked.
 // `tally`: the kernel also adds the decisions to the pending per-variant counts and the
 // catalog's counters (what launch_tally would do with them).
 // Returns cudaErrorInvalidValue if n is too large for the launch geometry.
 cudaError_t launch_select(const DeviceCatalog &c, const uint16_t *d_task, const uint32_t *d_slo,
                           const uint16_t *d_min_acc, uint64_t n, uint32_t *d_decision,
-                          int sm_count, uint32_t image_smem, bool tally, cudaStream_t stream);
-// Batches below this size are tallied by the selection kernel itself in infaas_select_update.
-constexpr uint64_t FUSED_TALLY_MAX_N = 1u << 18;
+                          int sm_count, uint32_t image_smem, uint32_t image_seen, bool tally, cudaStream_t stream);
+// Batches below this size are tallied by the selection kernel itself in infaas_select_update.  A window
+// (select, tally, rebuild) with the fused / the separate tally, us: 64 tasks x 256 variants, 131,072
+// queries 16.9 / 20.0, 200,000: 19.4 / 21.2, 262,143: 21.6 / 22.1; 4 x 132 (few, hot variants), 131,072:
+// 20.3 / 20.1, 262,143: 27.0 / 20.6; 128 x 512, 160,000: 18.1 / 22.2, 262,143: 22.4 / 24.1.
+constexpr uint64_t FUSED_TALLY_MAX_N = 192 * 1024;
 
 // Scaling-up step of the Model-Autoscaler for every task, from the pending per-variant
 // counts; s_inst / s_arch / s_qps (floor(10^9 * batch / lat_us)) are per slot, task_slo per

@@ -16,10 +16,10 @@ constexpr uint32_t NONE = 0xFFFFFFFFu;
 constexpr uint32_t REBUILD_THREADS = 1024;
 constexpr uint32_t REBUILD_WARPS = REBUILD_THREADS / 32;
 
-// IEEE-754 pattern of a u32 converted to float toward zero: a monotone, roughly logarithmic
-// code.  The selection kernel derives the same bucket from it.
+// The code of a latency or SLO: the IEEE-754 pattern of x converted to float toward zero, monotone and
+// roughly logarithmic; the selection kernel derives the same bucket from it.
 __device__ __forceinline__ uint32_t float_bits(uint32_t x) { return __float_as_uint(__uint2float_rz(x)); }
-// Smallest u32 whose float_bits is >= pattern (pattern below that of 2^32).
+// Smallest u32 whose code is >= pattern (2^32 - 1 for patterns of 2^32 and above).
 __device__ __forceinline__ uint32_t float_bits_floor(uint32_t pattern) {
   return __float2uint_ru(__uint_as_float(pattern));
 }
@@ -35,7 +35,7 @@ struct IndexScratch {
   uint32_t sorted[256];             // its latencies ascending (equal ones in scan order)
   uint32_t ent[256];                // same order: accuracy rank << 16 | last of its latency << 8 | position
   uint32_t Pd[256];                 // distinct latencies
-  uint32_t bcnt[256], bthr[256];    // per SLO bucket: distinct latencies inside it, one of them
+  uint32_t bcnt[MAX_BUCKETS];       // how many of them per SLO bucket
   uint32_t wbits[MAX_ACC_WORDS];    // per bitmap word: the accuracies present
   // per latency rank: the most accurate entry (acc << 16 | 0xFFFF - position, 0 = none); per
   // accuracy rank: the fastest entry (its index in latency order, NONE = none)
@@ -53,15 +53,15 @@ struct IndexScratch {
 __device__ __forceinline__ void write_dummy_task(const DeviceCatalog &c, uint32_t t) {
   const uint32_t T = c.n_tasks;
   if (threadIdx.x == 0) reinterpret_cast<uint32_t *>(c.image + IMAGE_HDR_OFFSET)[t] = DUMMY_HEADER;
-  uint32_t *rec = reinterpret_cast<uint32_t *>(c.image + image_rec_offset(T) + t * REC_STRIDE);
+  uint32_t *rec = reinterpret_cast<uint32_t *>(c.image + image_rec_offset(T) + t * rec_stride(c.n_buckets));
 #pragma unroll 1
-  for (uint32_t j = threadIdx.x; j < SLO_BUCKETS; j += blockDim.x) rec[j] = 0u;
-  uint32_t *bm = reinterpret_cast<uint32_t *>(c.image + image_bitmap_offset(T) + t * bitmap_stride(c.nbw));
+  for (uint32_t j = threadIdx.x; j <= c.n_buckets; j += blockDim.x) rec[j] = 0u;
+  uint32_t *bm = reinterpret_cast<uint32_t *>(c.image + image_bitmap_offset(T, c.n_buckets) + t * bitmap_stride(c.nbw));
 #pragma unroll 1
   for (uint32_t j = threadIdx.x; j < c.nbw; j += blockDim.x) bm[j] = 0u;
 }
 
-// Bucket scale of the SLO records: S (16..23) and bmin such that SLO_BUCKETS - 1 buckets of
+// Bucket scale of the SLO records: S (16..23) and bmin such that n_buckets - 1 buckets of
 // 2^S float patterns cover everything from the catalog's smallest profiled latency up to the
 // largest SLO asked for so far (as a bit mask: every SLO seen is <= cap).
 __device__ __forceinline__ void bucket_scale(const DeviceCatalog &c, uint32_t slo_seen, uint32_t &Sh, uint32_t &bmin) {
@@ -71,7 +71,7 @@ __device__ __forceinline__ void bucket_scale(const DeviceCatalog &c, uint32_t sl
   const uint32_t chi = max(clo, __float_as_uint(__uint2float_rz(cap)) >> 16);
   uint32_t sh = 0;
 #pragma unroll 1
-  while ((chi >> sh) - (clo >> sh) > SLO_BUCKETS - 2) ++sh;
+  while ((chi >> sh) - (clo >> sh) > c.n_buckets - 2u) ++sh;
   bmin = clo >> sh;
   Sh = 16u + sh;
 }
@@ -124,18 +124,20 @@ __device__ __forceinline__ unsigned long long place_block_issue(const DeviceCata
 __device__ __forceinline__ uint32_t place_block_finish(const DeviceCatalog &c, unsigned long long old,
                                                        uint32_t bytes, bool done) {
   if (done && (uint32_t)(old >> 32) == gridDim.x - 1u) {
-    c.image_hdr[0] = image_var_offset(c.n_tasks, c.nbw) + (uint32_t)old + bytes;
+    c.image_hdr[0] = image_var_offset(c.n_tasks, c.n_buckets, c.nbw) + (uint32_t)old + bytes;
     *c.alloc_ctr = 0ull;
   }
   return (uint32_t)old;
 }
 
 // Clears what build_index accumulates into (all threads; a barrier must follow).
-__device__ __forceinline__ void clear_scratch(IndexScratch &S) {
+__device__ __forceinline__ void clear_scratch(IndexScratch &S, uint32_t n_buckets) {
 #pragma unroll 1
   for (uint32_t i = threadIdx.x; i < 256u; i += REBUILD_THREADS) {
-    S.pred[i] = NONE; S.bcnt[i] = 0u; S.rankA[i] = 0u; S.rankB[i] = NONE; S.stair[i] = 0;
+    S.pred[i] = NONE; S.rankA[i] = 0u; S.rankB[i] = NONE; S.stair[i] = 0;
   }
+#pragma unroll 1
+  for (uint32_t i = threadIdx.x; i < n_buckets; i += REBUILD_THREADS) S.bcnt[i] = 0u;
 #pragma unroll 1
   for (uint32_t i = threadIdx.x; i < MAX_ACC_WORDS; i += REBUILD_THREADS) S.wbits[i] = 0u;
 }
@@ -207,10 +209,8 @@ __device__ bool build_index(const DeviceCatalog &c, uint32_t t, uint32_t F, Inde
       if (fresh) {
         const uint32_t v = S.sorted[i];
         S.Pd[r] = v;
-        // larger latencies than the largest SLO asked for so far share bucket 255
-        const uint32_t b = min(max(float_bits(v) >> Sh, bmin) - bmin, SLO_BUCKETS - 1u);
-        atomicAdd(&S.bcnt[b], 1u);
-        S.bthr[b] = v;                                 // read only where it is the bucket's only one
+        // larger latencies than the largest SLO asked for so far share the last bucket
+        atomicAdd(&S.bcnt[min(max(float_bits(v) >> Sh, bmin) - bmin, c.n_buckets - 1u)], 1u);
       }
       if (i == F - 1u) S.ks = r + 1u;
     }
@@ -245,26 +245,31 @@ __device__ bool build_index(const DeviceCatalog &c, uint32_t t, uint32_t F, Inde
     atomicMax(&S.rankA[r], (acc << 16) | (0xFFFFu - p));                            // most accurate, first position
     atomicMin(&S.rankB[ra], tid);                                                   // fastest, first position
   }
-  if (first && tid >= B / 2u && tid < B / 2u + SLO_BUCKETS) {
-    // one bucket per thread; lb = latencies in lower buckets
-    uint32_t *rec = reinterpret_cast<uint32_t *>(c.image + image_rec_offset(c.n_tasks) + t * REC_STRIDE);
-    const uint32_t j = tid - B / 2u;
-    uint32_t below = 0;
+  if (first) {
+    // SLO records, 32 neighbouring buckets per warp and trip; below = latencies in lower buckets
+    const uint32_t nb = c.n_buckets;
+    uint32_t *rec = reinterpret_cast<uint32_t *>(c.image + image_rec_offset(c.n_tasks) + t * rec_stride(nb));
 #pragma unroll 1
-    for (uint32_t i = lane; i < (j & ~31u); i += 32u) below += S.bcnt[i];
-    below = __reduce_add_sync(0xFFFFFFFFu, below);
-    const uint32_t cnt = S.bcnt[j], thr = S.bthr[j];
-    const uint32_t lb = below + warp_scan_add(cnt) - cnt;
-    const uint32_t lo = j ? float_bits_floor((bmin + j) << Sh) : 0u;
-    const uint32_t nxt = (bmin + j + 1u) << Sh;
-    const uint32_t hi = (j == SLO_BUCKETS - 1u || nxt >= BITS_OF_2_POW_32) ? NONE : float_bits_floor(nxt) - 1u;
-    uint32_t r = (Ks + 1u) << 24;                                // exact slow path
-    if (cnt == 0u) {
-      r = lb << 24;
-    } else if (cnt == 1u && (lo >> 24) == (hi >> 24)) {
-      r = thr <= lo ? (lb + 1u) << 24 : (lb << 24) | (0x00FFFFFFu - ((thr - 1u) & 0x00FFFFFFu));
+    for (uint32_t j = (tid + B / 2u) % B; j < nb; j += B) {        // (not the first warps: they are busy above)
+      uint32_t below = 0;
+#pragma unroll 4
+      for (uint32_t i = lane; i < (j & ~31u); i += 32u) below += S.bcnt[i];
+      below = __reduce_add_sync(0xFFFFFFFFu, below);
+      const uint32_t cnt = S.bcnt[j];
+      below += warp_scan_add(cnt) - cnt;
+      const uint32_t lo = j ? float_bits_floor((bmin + j) << Sh) : 0u;
+      const uint32_t nxt = (bmin + j + 1u) << Sh;
+      const uint32_t hi = (j == nb - 1u || nxt >= BITS_OF_2_POW_32) ? NONE : float_bits_floor(nxt) - 1u;
+      uint32_t r = ((Ks + 1u) << 24) | (cnt << 8) | below;          // exact slow path
+      if (cnt == 0u) {
+        r = below << 24;
+      } else if (cnt == 1u && (lo >> 24) == (hi >> 24)) {
+        const uint32_t thr = S.Pd[below];
+        r = thr <= lo ? (below + 1u) << 24 : (below << 24) | (0x00FFFFFFu - ((thr - 1u) & 0x00FFFFFFu));
+      }
+      rec[j] = r;
+      if (j == nb - 1u) rec[nb] = r;                               // what an SLO beyond the last bucket reads
     }
-    rec[j] = r;
   }
   __syncthreads();
 
@@ -299,7 +304,7 @@ __device__ bool build_index(const DeviceCatalog &c, uint32_t t, uint32_t F, Inde
     if (r < Ks) S.stair[r] = best_a == 0u || (x >> 16) > (best_a >> 16);
   }
   if (tid == B - 1u) {
-    uint32_t base = image_var_offset(c.n_tasks, nbw) + place_block_finish(c, placed, BL.bytes, next == 0u);
+    uint32_t base = image_var_offset(c.n_tasks, c.n_buckets, nbw) + place_block_finish(c, placed, BL.bytes, next == 0u);
     if (base + BL.bytes > c.image_capacity || base + BL.t2 >= IMAGE_T2_LIMIT) base = NONE;
     S.base = base;
   }
@@ -324,7 +329,7 @@ __device__ bool build_index(const DeviceCatalog &c, uint32_t t, uint32_t F, Inde
       if (e >= col_key) v = min(v, e & 0xFFu);
       if (e & 0x100u) { *row = (unsigned char)v; row += width; }
     }
-    if (i1 == F) *row = (unsigned char)F;                        // row Ks + 1: the slow path's
+    if (i1 == F) { row[0] = (unsigned char)F; row[width] = (unsigned char)F; }   // rows Ks + 1, Ks + 2: the slow path's
   }
 
   // the small tables, each by a range of warps of its own: [lo, lo + n) of the CTA's threads run
@@ -334,7 +339,7 @@ __device__ bool build_index(const DeviceCatalog &c, uint32_t t, uint32_t F, Inde
 #pragma unroll 1
       for (uint32_t x = tid - lo; x < count; x += n) body(x);
   };
-  uint32_t *bitmap = first ? reinterpret_cast<uint32_t *>(c.image + image_bitmap_offset(c.n_tasks) + t * bitmap_stride(nbw))
+  uint32_t *bitmap = first ? reinterpret_cast<uint32_t *>(c.image + image_bitmap_offset(c.n_tasks, c.n_buckets) + t * bitmap_stride(nbw))
                            : reinterpret_cast<uint32_t *>(blk + BL.bitmap);
   share(0, B / 4u, nbw, [&](uint32_t w) { bitmap[w] = ((uint32_t)S.wpre[w] << 24) | S.wbits[w]; });
   // what the nearest-miss search reads: bestA[r] over latency ranks < r, the stair entries in
@@ -506,7 +511,7 @@ rebuild_kernel(DeviceCatalog c, int advance, uint32_t window_us) {
   for (uint32_t i = tid; i < V; i += B) run_min[i] = NONE;
 #pragma unroll 1
   for (uint32_t i = tid; i <= KEEP_WORDS; i += B) { keep[i] = 0u; if (i < KEEP_WORDS) passed_acc[i] = 0u; }
-  clear_scratch(S);
+  clear_scratch(S, c.n_buckets);
   if (tid == 0u) { n_cand = 0u; n_inactive = 0u; }
   __syncthreads();
   chain_wait();
@@ -745,7 +750,7 @@ rebuild_kernel(DeviceCatalog c, int advance, uint32_t window_us) {
       const uint32_t off = sg * INDEX_MAX_F, Fseg = min(INDEX_MAX_F, F - off);
       if (sg) {                                   // later segments: back from the task's region
         __syncthreads();
-        clear_scratch(S);
+        clear_scratch(S, c.n_buckets);
         __syncthreads();
 #pragma unroll 1
         for (uint32_t i = tid; i < Fseg; i += B) {
@@ -780,7 +785,7 @@ rebuild_kernel(DeviceCatalog c, int advance, uint32_t window_us) {
 }
 
 // The block sizes the thread ranges above rely on.
-static_assert(REBUILD_THREADS >= 512 && SLO_BUCKETS == 256 && INDEX_MAX_F < 256, "thread ranges of build_index");
+static_assert(REBUILD_THREADS >= 512 && INDEX_MAX_F < 254, "thread ranges of build_index");
 
 }  // namespace
 

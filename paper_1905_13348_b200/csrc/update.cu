@@ -142,13 +142,20 @@ tally_smem_kernel(const uint32_t *__restrict__ decision, uint64_t n, uint32_t n_
 constexpr uint32_t TALLY_SMEM_MAX_VARIANTS = 49152;   // 192 KB of bins
 constexpr uint32_t TALLY_SMEM_MAX_PARTS = 8;           // beyond this many id ranges: global atomics
 constexpr size_t TALLY_SMEM_ALONE = 116 * 1024;
-constexpr uint64_t TALLY_SMEM_MIN_N = 1u << 18;        // below this the zero/flush passes cost more than they save
+// Below this size the clear and flush passes over the bins cost more than the shared-memory atomics
+// save.  A window with the shared-memory / the global tally, us: 528 variants, 98,000 queries 18.0 /
+// 20.6; 6,000 variants, 65,536: 18.8 / 17.4, 131,072: 19.0 / 19.5; 16,384 variants, 98,000: 20.0 / 18.5,
+// 160,000: 20.0 / 20.6; 65,536 variants, 131,072: 22.7 / 21.0, 200,000: 23.5 / 27.1.
+inline uint64_t tally_smem_min_n(uint32_t n_variants) {
+  const uint64_t n = 65536 + 10ull * n_variants;
+  return n < 163840 ? n : 163840;
+}
 
 cudaError_t launch_tally(const DeviceCatalog &c, const uint32_t *d_decision, uint64_t n,
                          int sm_count, cudaStream_t stream) {
   if (n == 0) return cudaSuccess;
   const uint32_t parts = (c.n_variants + TALLY_SMEM_MAX_VARIANTS - 1) / TALLY_SMEM_MAX_VARIANTS;
-  if (n >= TALLY_SMEM_MIN_N && parts <= TALLY_SMEM_MAX_PARTS) {
+  if (n >= tally_smem_min_n(c.n_variants) && parts <= TALLY_SMEM_MAX_PARTS) {
     const uint32_t bins = ((c.n_variants + parts - 1) / parts + 3u) & ~3u;
     size_t smem = (size_t)(bins + 32) * 4;                       // 32 spare bins
     // more than half of an SM's shared memory: launched while the selection kernel drains, two CTAs
