@@ -338,6 +338,10 @@ int infaas_catalog_load(const infaas_variant *rows, uint32_t n_variants, uint32_
   d.image_capacity = (uint32_t)worst_image;
   d.image_hdr = reinterpret_cast<uint32_t *>(base + o_hdr);
   d.n_buckets = infaas::buckets_for(n_tasks, max_task);
+  // several CTAs per task where lists can span several segments, the SMs are idle, and no block can lie
+  // out of reach of the task word (the CTAs of a task could not agree on an index then)
+  const bool spread = max_task > 1024 && worst_image < infaas::IMAGE_T2_LIMIT && 4ull * n_tasks <= (uint64_t)c->sm_count;
+  d.rebuild_ctas = spread ? 4 : 1;
   d.acc_lo = acc_lo;
   d.nbw = nbw;
   d.lat_code_lo = float_bits_rz(lat_min) >> 16;

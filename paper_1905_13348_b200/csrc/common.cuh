@@ -210,6 +210,7 @@ struct DeviceCatalog {
   uint32_t *image_hdr;       // published by the rebuild kernel: [0] bytes of the image, [1] the bucket
                              // scale 2^-S and [2] -bmin, both as float patterns
   uint32_t n_buckets;        // SLO buckets per task
+  uint32_t rebuild_ctas;     // CTAs per task of the rebuild kernel (1 or 4)
   uint32_t acc_lo, nbw;      // accuracy window of every bitmap: acc_lo (multiple of 24) .. acc_lo + 24 nbw - 1
   uint32_t lat_code_lo;      // bits(smallest profiled latency) >> 16: where the SLO buckets start
 
@@ -258,19 +259,27 @@ cudaError_t prepare_rebuild_kernel();
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 template <class... P, class... A>
-inline cudaError_t launch_chained(void (*kernel)(P...), uint32_t grid, uint32_t block, size_t smem, cudaStream_t stream,
-                                  A... args) {
-  cudaLaunchAttribute attr{};
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
+inline cudaError_t launch_chained_cluster(void (*kernel)(P...), uint32_t grid, uint32_t cluster, uint32_t block, size_t smem,
+                                          cudaStream_t stream, A... args) {
+  cudaLaunchAttribute attr[2] = {};
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cluster;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(block);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+template <class... P, class... A>
+inline cudaError_t launch_chained(void (*kernel)(P...), uint32_t grid, uint32_t block, size_t smem, cudaStream_t stream,
+                                  A... args) {
+  return launch_chained_cluster(kernel, grid, 1, block, smem, stream, args...);
 }
 
 // Launchers (host).  All are asynchronous on `stream` and allocate nothing.

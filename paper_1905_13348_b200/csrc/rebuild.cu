@@ -150,14 +150,14 @@ __device__ __forceinline__ void clear_scratch(IndexScratch &S, uint32_t n_bucket
 // `xi`: NONE for the task's first segment (header word, SLO records and bitmap go into the
 // fixed part of the image), else the index of this further segment (header to xhdr[xi], bitmap
 // into the block, no records: only the slow path comes here).  `next`: 1 + index of the task's
-// next segment, 0 if this is the last (the CTA's last allocation, then).
+// next segment, 0 if this is the last.  `done`: the CTA's last allocation.
 //
 // The chain is bound by latency (barriers and shared-memory round trips), so it has few steps:
 // one pair loop (latency order), accuracy ranks straight from the bitmap, and the rank table as a
 // running minimum down its columns -- F steps per column, cut into runs of entries so that all
 // warps work, instead of F bits per cell.
 __device__ bool build_index(const DeviceCatalog &c, uint32_t t, uint32_t F, IndexScratch &S, uint32_t xi,
-                            uint32_t next, uint32_t Sh, uint32_t bmin) {
+                            uint32_t next, bool done, uint32_t Sh, uint32_t bmin) {
   const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
   constexpr uint32_t B = REBUILD_THREADS;
   const bool first = xi == NONE;
@@ -235,7 +235,7 @@ __device__ bool build_index(const DeviceCatalog &c, uint32_t t, uint32_t F, Inde
   // 3. the block's place in the image (the atomic is in flight until step 4 ends); the sorted
   // entries with their accuracy ranks, and the best entry per rank; SLO records
   unsigned long long placed = 0;
-  if (tid == B - 1u) placed = place_block_issue(c, BL.bytes, next == 0u);
+  if (tid == B - 1u) placed = place_block_issue(c, BL.bytes, done);
   if (tid < F) {
     const uint32_t p = S.at[tid], r = S.rank[tid], acc = S.acc[p];
     const uint32_t x = acc - acc_lo, xw = x / ACC_WORD_BITS;
@@ -304,7 +304,7 @@ __device__ bool build_index(const DeviceCatalog &c, uint32_t t, uint32_t F, Inde
     if (r < Ks) S.stair[r] = best_a == 0u || (x >> 16) > (best_a >> 16);
   }
   if (tid == B - 1u) {
-    uint32_t base = image_var_offset(c.n_tasks, c.n_buckets, nbw) + place_block_finish(c, placed, BL.bytes, next == 0u);
+    uint32_t base = image_var_offset(c.n_tasks, c.n_buckets, nbw) + place_block_finish(c, placed, BL.bytes, done);
     if (base + BL.bytes > c.image_capacity || base + BL.t2 >= IMAGE_T2_LIMIT) base = NONE;
     S.base = base;
   }
@@ -441,7 +441,9 @@ __device__ __forceinline__ uint32_t advance_row(const DeviceCatalog &c, uint32_t
   return pred;
 }
 
-// One CTA per task.
+// Queue recursion, prune and list of one task (all threads of one CTA): the list goes into the
+// task's region, its first segment also into S, which is cleared here.  Contains chain_wait.  Returns
+// the list's length.
 //
 // List of the Active variants (all variants of a catalog without states).  Slots are in (cost,
 // 10000-acc, id) order, so with `order` = position in (10000-acc, local) order a variant q before
@@ -458,20 +460,10 @@ __device__ __forceinline__ uint32_t advance_row(const DeviceCatalog &c, uint32_t
 // List of the Inactive variants: ordered by (eff, 10000-acc, id) with eff in place of cost and
 // pred; at most the fastest variant (lowest id) of every distinct accuracy is on it, if it is
 // faster than everything more accurate, and the list runs from the lowest accuracy up.
-//
-// Bound by the latency of its chain of barriers and shared-memory round trips, and by fetching its
-// code: every line of it runs about once per launch, and with the compiler's unrolling (116 KB of
-// code) 40 % of the stalls were for instructions.  So the loops are not unrolled (47 KB) except the
-// few that run long.  Measured on one B200, in GPU clock cycles after the previous kernel's end: 64
-// tasks x 256 variants, lists of up to 100 entries: 16 K (18 K unrolled), 128 x 512: 19 K (22 K), 4 x
-// 4096 on a trade-off surface, lists of up to 505 entries: 77 K (90 K), two lists per task: 17 K
-// (23 K).  512 threads instead of 1024: short lists 5 % faster, lists of 100 entries 5 % slower.
-__global__ void __launch_bounds__(REBUILD_THREADS)
-rebuild_kernel(DeviceCatalog c, int advance, uint32_t window_us) {
-  extern __shared__ __align__(16) unsigned char dyn[];
+__device__ __forceinline__ uint32_t build_list(const DeviceCatalog &c, uint32_t t, bool advance, uint32_t window_us,
+                                               unsigned char *dyn, IndexScratch &S, uint32_t &slo_seen) {
   constexpr uint32_t KEEP_WORDS = INFAAS_MAX_TASK_VARIANTS / 32;
   __shared__ uint32_t grid[GRID * GRID_PITCH];
-  __shared__ __align__(16) IndexScratch S;
   __shared__ uint32_t keep[KEEP_WORDS + 1], keep_pre[KEEP_WORDS + 1];   // bit sets: survivors, by local index ...
   __shared__ uint32_t passed_local[KEEP_WORDS], passed_acc[KEEP_WORDS];   // ... what the grid lets through, both orders
   __shared__ unsigned long long warp_min[REBUILD_WARPS];
@@ -479,7 +471,7 @@ rebuild_kernel(DeviceCatalog c, int advance, uint32_t window_us) {
   __shared__ uint32_t n_cand, n_inactive;
   constexpr uint32_t B = REBUILD_THREADS;
 
-  const uint32_t t = blockIdx.x, tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+  const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
   const uint32_t base = c.task_off[t], V = c.task_off[t + 1] - base;
   // shared memory per variant (REBUILD_ROW_SMEM bytes)
   uint2 *by_local = reinterpret_cast<uint2 *>(dyn);               // (pred, accuracy position); position 0xFFFF: not listed
@@ -516,7 +508,7 @@ rebuild_kernel(DeviceCatalog c, int advance, uint32_t window_us) {
   __syncthreads();
   chain_wait();
   chain_next();
-  const uint32_t slo_seen = *c.slo_seen;
+  slo_seen = *c.slo_seen;                                          // wanted by the index, requested early
   Row r = r0;
 #pragma unroll 1
   for (uint32_t i = tid; i < V;) {
@@ -537,8 +529,6 @@ rebuild_kernel(DeviceCatalog c, int advance, uint32_t window_us) {
     i += B;
     if (i < V) r = load_fixed(c, base + i, window_us);
   }
-  uint32_t bmin, Sh;                                               // SLO buckets
-  bucket_scale(c, slo_seen, Sh, bmin);
   __syncthreads();
   // 2. running minimum along the rows, then down the columns (GRID = two values per lane)
 #pragma unroll 1
@@ -737,6 +727,43 @@ rebuild_kernel(DeviceCatalog c, int advance, uint32_t window_us) {
     F += n_inactive;
   }
   __syncthreads();
+  return F;
+}
+
+// c.rebuild_ctas CTAs per task, a cluster: the first one makes the list, then each takes its share of
+// the list's segments.
+//
+// Bound by the latency of its chain of barriers and shared-memory round trips, and by fetching its
+// code: every line of it runs about once per launch, and with the compiler's unrolling (116 KB of
+// code) 40 % of the stalls were for instructions.  So the loops are not unrolled (47 KB) except the
+// few that run long.  Measured on one B200, in GPU clock cycles after the previous kernel's end: 64
+// tasks x 256 variants, lists of up to 100 entries: 16 K (18 K unrolled), 128 x 512: 19 K (22 K), 4 x
+// 4096 on a trade-off surface, lists of up to 505 entries: 77 K (90 K), two lists per task: 17 K
+// (23 K).  512 threads instead of 1024: short lists 5 % faster, lists of 100 entries 5 % slower.
+// The segments of a list of several hundred entries take as long as the list itself, so tasks of more
+// than 1024 variants have 4 CTAs: 47 us a window instead of 62 on the trade-off surface.
+__global__ void __launch_bounds__(REBUILD_THREADS)
+rebuild_kernel(DeviceCatalog c, int advance, uint32_t window_us) {
+  extern __shared__ __align__(16) unsigned char dyn[];
+  __shared__ __align__(16) IndexScratch S;
+  const uint32_t K = c.rebuild_ctas, t = blockIdx.x >> (K >> 1), share = blockIdx.x & (K - 1u), tid = threadIdx.x;   // K = 1 or 4
+  constexpr uint32_t B = REBUILD_THREADS;
+  uint32_t F = 0, slo_seen;
+  if (share == 0u) {
+    F = build_list(c, t, advance, window_us, dyn, S, slo_seen);
+    if (tid == 0u) c.f_len[t] = F;
+  } else {
+    chain_wait();
+    chain_next();
+    slo_seen = *c.slo_seen;
+  }
+  uint32_t bmin, Sh;                                               // SLO buckets
+  bucket_scale(c, slo_seen, Sh, bmin);
+  if (K > 1u) {                                                    // the list is in the region
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    F = *reinterpret_cast<volatile uint32_t *>(c.f_len + t);
+  }
   bool indexed = F > 0;
   bool counted = false;                       // has this CTA made its last allocation?
   // index the list -- the two lists of a state-aware catalog count as one, the Inactive entries
@@ -746,9 +773,12 @@ rebuild_kernel(DeviceCatalog c, int advance, uint32_t window_us) {
   if (indexed) {
     const uint32_t nseg = (F + INDEX_MAX_F - 1u) / INDEX_MAX_F, x0 = c.seg_base[t];
 #pragma unroll 1
-    for (uint32_t sg = 0; sg < nseg && indexed; ++sg) {
+    for (uint32_t sg = share; sg < nseg && indexed; sg += K) {
       const uint32_t off = sg * INDEX_MAX_F, Fseg = min(INDEX_MAX_F, F - off);
       if (sg) {                                   // later segments: back from the task's region
+        const unsigned char *region = c.regions + c.reg_off[t];
+        const unsigned long long *keys_g = reinterpret_cast<const unsigned long long *>(region);
+        const uint32_t *ids_g = reinterpret_cast<const uint32_t *>(region + 8u * (c.task_off[t + 1] - c.task_off[t]));
         __syncthreads();
         clear_scratch(S, c.n_buckets);
         __syncthreads();
@@ -759,11 +789,12 @@ rebuild_kernel(DeviceCatalog c, int advance, uint32_t window_us) {
         }
         __syncthreads();
       }
-      indexed = build_index(c, t, Fseg, S, sg ? x0 + sg - 1u : NONE, sg + 1u < nseg ? x0 + sg + 1u : 0u, Sh, bmin);
-      counted = sg + 1u == nseg;
+      indexed = build_index(c, t, Fseg, S, sg ? x0 + sg - 1u : NONE, sg + 1u < nseg ? x0 + sg + 1u : 0u, sg + K >= nseg, Sh, bmin);
+      counted = sg + K >= nseg;
     }
   }
   if (!counted && tid == 0u) place_block_finish(c, place_block_issue(c, 0u, true), 0u, true);   // nothing (more) to place
+  if (share) return;
   if (!indexed) {
     // no index: every query of this task reads "none"
     write_dummy_task(c, t);
@@ -781,7 +812,6 @@ rebuild_kernel(DeviceCatalog c, int advance, uint32_t window_us) {
       if (tid < IMAGE_DUMMY_BYTES / 4u) reinterpret_cast<uint32_t *>(c.image)[tid] = tid == 3u ? PENDING : 0u;
     }
   }
-  if (tid == 0u) c.f_len[t] = F;
 }
 
 // The block sizes the thread ranges above rely on.
@@ -797,7 +827,8 @@ cudaError_t prepare_rebuild_kernel() {
 cudaError_t launch_rebuild(const DeviceCatalog &c, bool advance_queues, uint32_t window_us,
                            cudaStream_t stream) {
   const size_t smem = (size_t)c.max_task_variants * REBUILD_ROW_SMEM;
-  return launch_chained(rebuild_kernel, c.n_tasks, REBUILD_THREADS, smem, stream, c, advance_queues ? 1 : 0, window_us);
+  return launch_chained_cluster(rebuild_kernel, c.n_tasks * c.rebuild_ctas, c.rebuild_ctas, REBUILD_THREADS, smem, stream, c,
+                                advance_queues ? 1 : 0, window_us);
 }
 
 }  // namespace infaas
