@@ -254,8 +254,8 @@ cudaError_t prepare_rebuild_kernel();
 // with launch_chained may start while its predecessor still runs.  Before chain_wait() it touches
 // only what no kernel writes (the layout made at load time); chain_wait() returns when everything
 // before the kernel in the stream is complete and visible.  A kernel lets its successor start
-// (chain_next) only after its own chain_wait, so at most two overlap.  Measured: the gap between
-// two kernels of a window goes from 2.0 to 0.9 us.
+// (chain_next) only after its own chain_wait, so at most two overlap.  Measured: a window of 65,536
+// queries (two kernels) 24.1 -> 19.6 us, a step of 2^24 queries (three) 77 -> 70 us.
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 template <class... P, class... A>
