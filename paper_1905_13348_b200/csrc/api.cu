@@ -284,9 +284,7 @@ int infaas_catalog_load(const infaas_variant *rows, uint32_t n_variants, uint32_
     if (e__ != cudaSuccess) { infaas_catalog_free(c); return cuda_fail(e__); } \
   } while (0)
 
-  cudaDeviceProp prop;
-  LOAD_TRY(cudaGetDeviceProperties(&prop, cuda_device));
-  c->sm_count = prop.multiProcessorCount;
+  LOAD_TRY(cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, cuda_device));
   LOAD_TRY(cudaMalloc(&c->arena, total));
   unsigned char *base = static_cast<unsigned char *>(c->arena);
   LOAD_TRY(cudaMemset(base, 0, total));
