@@ -372,6 +372,8 @@ int infaas_catalog_load(const infaas_variant *rows, uint32_t n_variants, uint32_
   LOAD_TRY(infaas::prepare_select_kernel());
   LOAD_TRY(infaas::prepare_tally_kernel());
   LOAD_TRY(infaas::prepare_rebuild_kernel());
+  // every kernel from here on reads the layout before it waits for its predecessor
+  LOAD_TRY(cudaStreamSynchronize(nullptr));
   LOAD_TRY(infaas::launch_rebuild(d, /*advance_queues=*/false, 0, nullptr));
   LOAD_TRY(cudaDeviceSynchronize());
   int rc = refresh_select_plan(c, nullptr);

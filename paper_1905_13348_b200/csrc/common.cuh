@@ -252,7 +252,8 @@ cudaError_t prepare_rebuild_kernel();
 
 // Kernels of one stream overlap at their seams (programmatic dependent launch): a kernel launched
 // with launch_chained may start while its predecessor still runs.  Before chain_wait() it touches
-// only what no kernel writes (the layout made at load time); chain_wait() returns when everything
+// only what no kernel writes once the catalog is loaded (the layout: infaas_catalog_load waits for
+// the layout kernel before it launches the first chained one); chain_wait() returns when everything
 // before the kernel in the stream is complete and visible.  A kernel lets its successor start
 // (chain_next) only after its own chain_wait, so at most two overlap.  Measured: a window of 65,536
 // queries (two kernels) 24.1 -> 19.6 us, a step of 2^24 queries (three) 77 -> 70 us.
