@@ -82,7 +82,7 @@ __device__ __forceinline__ bool stage_wait(unsigned long long *mbar, uint32_t pa
 }
 
 // The image, read either from shared memory (32-bit addresses, ld.shared) or from global
-// memory (read-only path).  Offsets are bytes from the start of the image.
+// memory.  Offsets are bytes from the start of the image.
 struct SharedImage {
   static constexpr bool FAR = false;         // short round trips: what counts is instructions
   uint32_t base;
@@ -100,12 +100,12 @@ struct SharedImage {
 struct GlobalImage {
   static constexpr bool FAR = true;          // long round trips: what counts is dependent loads
   const unsigned char *base;
-  __device__ __forceinline__ uint32_t u8(uint32_t off) const { return __ldg(base + off); }
+  __device__ __forceinline__ uint32_t u8(uint32_t off) const { return base[off]; }
   __device__ __forceinline__ uint32_t u32(uint32_t off) const {
-    return __ldg(reinterpret_cast<const uint32_t *>(base + off));
+    return *reinterpret_cast<const uint32_t *>(base + off);
   }
   __device__ __forceinline__ uint2 v2(uint32_t off) const {
-    return __ldg(reinterpret_cast<const uint2 *>(base + off));
+    return *reinterpret_cast<const uint2 *>(base + off);
   }
 };
 
@@ -277,7 +277,7 @@ template <class Img>
 __device__ __forceinline__ uint32_t decide_slow(const Img &img, const DeviceCatalog &c, const Fixed &fx, uint32_t task,
                                                 uint32_t slo, uint32_t min_acc) {
   if (task >= c.n_tasks) return INFAAS_INVALID;
-  uint4 sl = __ldg(c.slow + task);
+  uint4 sl = c.slow[task];
   // the list's segments in order: the first has its header word, records and bitmap in the fixed part
   // of the image, the others (lists longer than INDEX_MAX_F) a header in global memory
   const uint32_t h = img.u32(IMAGE_HDR_OFFSET + (task << 2));
@@ -299,39 +299,39 @@ __device__ __forceinline__ uint32_t decide_slow(const Img &img, const DeviceCata
       if (d != PENDING) return d;
       const uint32_t next = sl.w >> 8;                       // 1 + index of the next segment
       if (next == 0u) break;
-      sl = __ldg(c.slow + c.n_tasks + next - 1u);
-      const uint4 xh = __ldg(c.xhdr + next - 1u);
+      sl = c.slow[c.n_tasks + next - 1u];
+      const uint4 xh = c.xhdr[next - 1u];
       t2 = xh.x; width = xh.y; bm0 = xh.z - 4u * (fx.acc_lo / ACC_WORD_BITS);
       lo = 0u; n = (sl.y >> 8) & 0xFFu;
     }
     return INFAAS_NO_FEASIBLE | best_p;
   }
-  const uint32_t F = __ldg(c.f_len + task);
+  const uint32_t F = c.f_len[task];
   const uint32_t V = __ldg(c.task_off + task + 1) - __ldg(c.task_off + task);
   const unsigned char *region = c.regions + __ldg(c.reg_off + task);
   const unsigned long long *keys = reinterpret_cast<const unsigned long long *>(region);
   const uint32_t *ids = reinterpret_cast<const uint32_t *>(region + 8u * V);
 #pragma unroll 1
   for (uint32_t i = 0; i < F; ++i) {
-    const unsigned long long e = __ldg(keys + i);
-    if ((uint32_t)e <= slo && (uint32_t)(e >> 32) >= min_acc) return __ldg(ids + i);
+    const unsigned long long e = keys[i];
+    if ((uint32_t)e <= slo && (uint32_t)(e >> 32) >= min_acc) return ids[i];
   }
 #pragma unroll 1
   for (uint32_t i = 0; i < F; ++i) {
-    const unsigned long long e = __ldg(keys + i);
+    const unsigned long long e = keys[i];
     const uint32_t pred = (uint32_t)e, acc = (uint32_t)(e >> 32);
     const unsigned long long d = (unsigned long long)(pred > slo ? pred - slo : 0u) * 10000ull +
                                  (unsigned long long)slo * (min_acc > acc ? min_acc - acc : 0u);
     if (d < best) { best = d; best_p = i; }
   }
-  return INFAAS_NO_FEASIBLE | __ldg(ids + best_p);
+  return INFAAS_NO_FEASIBLE | ids[best_p];
 }
 
 struct Queries {
-  const uint16_t *__restrict__ task;
-  const uint32_t *__restrict__ slo;
-  const uint16_t *__restrict__ min_acc;
-  uint32_t *__restrict__ decision;
+  const uint16_t *task;
+  const uint32_t *slo;
+  const uint16_t *min_acc;
+  uint32_t *decision;
 };
 
 // A warp's park list in shared memory, three words per parked query, each in an array of its own:
@@ -435,9 +435,9 @@ __device__ __forceinline__ void select_body(const Img &img, const DeviceCatalog 
     const uint32_t next = tile + SELECT_WARPS;
     if (next < full_tiles) {
       const uint64_t i4 = (q0 + (uint64_t)next * WARP_TILE) / 4 + lane;
-      t4 = __ldcs(reinterpret_cast<const uint2 *>(q.task) + i4);
-      s4 = __ldcs(reinterpret_cast<const uint4 *>(q.slo) + i4);
-      a4 = __ldcs(reinterpret_cast<const uint2 *>(q.min_acc) + i4);
+      t4 = load_once(reinterpret_cast<const uint2 *>(q.task) + i4);
+      s4 = load_once(reinterpret_cast<const uint4 *>(q.slo) + i4);
+      a4 = load_once(reinterpret_cast<const uint2 *>(q.min_acc) + i4);
     }
     const uint32_t tq[4] = {t.x & 0xFFFFu, t.x >> 16, t.y & 0xFFFFu, t.y >> 16};
     const uint32_t aq[4] = {a.x & 0xFFFFu, a.x >> 16, a.y & 0xFFFFu, a.y >> 16};
@@ -519,16 +519,16 @@ select_kernel(DeviceCatalog c, uint32_t stage_bytes, uint32_t first, Queries q, 
   // Everything the kernel has to wait for before its first decision starts at once: the staging of the
   // image's first part, the words the last rebuild published, the SLO mask, and every warp's first tile.
   if (stage_bytes) stage_begin(staged, c.image, first, &mbar);
-  const uint4 hdr = __ldg(reinterpret_cast<const uint4 *>(c.image_hdr));
-  const uint32_t slo_seen = __ldg(c.slo_seen);
+  const uint4 hdr = *reinterpret_cast<const uint4 *>(c.image_hdr);
+  const uint32_t slo_seen = *c.slo_seen;
   uint2 t4 = make_uint2(0, 0), a4 = make_uint2(0, 0);
   uint4 s4 = make_uint4(0, 0, 0, 0);
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (warp < span / WARP_TILE) {
     const uint64_t i4 = (q0 + (uint64_t)warp * WARP_TILE) / 4 + lane;
-    t4 = __ldcs(reinterpret_cast<const uint2 *>(q.task) + i4);
-    s4 = __ldcs(reinterpret_cast<const uint4 *>(q.slo) + i4);
-    a4 = __ldcs(reinterpret_cast<const uint2 *>(q.min_acc) + i4);
+    t4 = load_once(reinterpret_cast<const uint2 *>(q.task) + i4);
+    s4 = load_once(reinterpret_cast<const uint4 *>(q.slo) + i4);
+    a4 = load_once(reinterpret_cast<const uint2 *>(q.min_acc) + i4);
   }
   // the copy is waited for in any case: the CTA must not end with it in flight
   bool staged_ok = !stage_bytes || stage_wait(&mbar, 0u);
@@ -576,9 +576,9 @@ select_direct_kernel(DeviceCatalog c, Queries q, uint32_t n) {
   chain_next();
   const bool live = i < n;
   uint32_t task = 0, slo = 0, min_acc = 0, d = 0;
-  if (live) { task = __ldg(q.task + i); slo = __ldg(q.slo + i); min_acc = __ldg(q.min_acc + i); }
-  const Fixed fx = make_fixed(c, __ldg(reinterpret_cast<const uint4 *>(c.image_hdr)));
-  const uint32_t slo_seen = __ldg(c.slo_seen);
+  if (live) { task = q.task[i]; slo = q.slo[i]; min_acc = q.min_acc[i]; }
+  const Fixed fx = make_fixed(c, *reinterpret_cast<const uint4 *>(c.image_hdr));
+  const uint32_t slo_seen = *c.slo_seen;
   const GlobalImage img{c.image};
   if (live) {
     d = decide_fast<false>(img, fx, task, slo, min_acc);

@@ -29,8 +29,8 @@ __device__ __forceinline__ void tally_one(uint32_t d, bool live, uint32_t n_vari
 }
 
 __global__ void __launch_bounds__(256)
-tally_kernel(const uint32_t *__restrict__ decision, uint64_t n, uint32_t n_variants,
-             uint32_t *__restrict__ count_by_id, unsigned long long *__restrict__ counters) {
+tally_kernel(const uint32_t *decision, uint64_t n, uint32_t n_variants,
+             uint32_t *count_by_id, unsigned long long *counters) {
   __shared__ uint32_t blk[3];
   if (threadIdx.x < 3) blk[threadIdx.x] = 0;
   __syncthreads();
@@ -44,7 +44,7 @@ tally_kernel(const uint32_t *__restrict__ decision, uint64_t n, uint32_t n_varia
   const uint64_t n4_warp = (n4 + 31) & ~(uint64_t)31;
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4_warp; i += stride) {
     bool live = i < n4;
-    uint4 d = live ? __ldg(dec4 + i) : make_uint4(0, 0, 0, 0);
+    uint4 d = live ? dec4[i] : make_uint4(0, 0, 0, 0);
     tally_one(d.x, live, n_variants, count_by_id, n_feas, n_nofeas, n_inval);
     tally_one(d.y, live, n_variants, count_by_id, n_feas, n_nofeas, n_inval);
     tally_one(d.z, live, n_variants, count_by_id, n_feas, n_nofeas, n_inval);
@@ -77,9 +77,9 @@ tally_kernel(const uint32_t *__restrict__ decision, uint64_t n, uint32_t n_varia
 constexpr int TALLY_SMEM_THREADS = 1024;
 
 __global__ void __launch_bounds__(TALLY_SMEM_THREADS)
-tally_smem_kernel(const uint32_t *__restrict__ decision, uint64_t n, uint32_t n_variants, uint32_t bins,
-                  uint32_t parts, uint32_t *__restrict__ count_by_id,
-                  unsigned long long *__restrict__ counters) {
+tally_smem_kernel(const uint32_t *decision, uint64_t n, uint32_t n_variants, uint32_t bins,
+                  uint32_t parts, uint32_t *count_by_id,
+                  unsigned long long *counters) {
   extern __shared__ uint32_t hist[];
   __shared__ uint32_t blk[3];
   const uint32_t part = blockIdx.x % parts, lo = part * bins, share = blockIdx.x / parts;
@@ -106,8 +106,8 @@ tally_smem_kernel(const uint32_t *__restrict__ decision, uint64_t n, uint32_t n_
   // four 128-bit loads in flight per thread
   uint32_t i = share * blockDim.x + threadIdx.x;
   for (; n4 >= 3 * stride && i < n4 - 3 * stride; i += 4 * stride) {
-    const uint4 d0 = __ldcs(dec4 + i), d1 = __ldcs(dec4 + i + stride);
-    const uint4 d2 = __ldcs(dec4 + i + 2 * stride), d3 = __ldcs(dec4 + i + 3 * stride);
+    const uint4 d0 = load_once(dec4 + i), d1 = load_once(dec4 + i + stride);
+    const uint4 d2 = load_once(dec4 + i + 2 * stride), d3 = load_once(dec4 + i + 3 * stride);
     one(d0.x); one(d0.y); one(d0.z); one(d0.w);
     one(d1.x); one(d1.y); one(d1.z); one(d1.w);
     one(d2.x); one(d2.y); one(d2.z); one(d2.w);
@@ -115,7 +115,7 @@ tally_smem_kernel(const uint32_t *__restrict__ decision, uint64_t n, uint32_t n_
     n_seen += 16;
   }
   for (; i < n4; i += stride) {
-    const uint4 d = __ldcs(dec4 + i);
+    const uint4 d = load_once(dec4 + i);
     one(d.x); one(d.y); one(d.z); one(d.w);
     n_seen += 4;
   }

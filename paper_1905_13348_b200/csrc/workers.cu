@@ -50,18 +50,18 @@ __global__ void workers_final_kernel(uint32_t n_variants, const unsigned char *h
 }
 
 __device__ __forceinline__ uint32_t worker_for(uint32_t d, uint32_t n_variants, const uint32_t *worker_of) {
-  return d < n_variants ? __ldg(worker_of + d) : INFAAS_INVALID;     // bit 31 set is >= n_variants too
+  return d < n_variants ? worker_of[d] : INFAAS_INVALID;     // bit 31 set is >= n_variants too
 }
 
 // 8 B per query: four decisions in, four workers out per thread and trip.
 __global__ void __launch_bounds__(256)
-assign_workers_kernel(const uint32_t *__restrict__ decision, uint64_t n, uint32_t n_variants,
-                      const uint32_t *__restrict__ worker_of, uint32_t *__restrict__ worker) {
+assign_workers_kernel(const uint32_t *decision, uint64_t n, uint32_t n_variants,
+                      const uint32_t *worker_of, uint32_t *worker) {
   chain_wait();
   chain_next();
   const uint64_t n4 = n >> 2, stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += stride) {
-    const uint4 d = __ldcs(reinterpret_cast<const uint4 *>(decision) + i);
+    const uint4 d = load_once(reinterpret_cast<const uint4 *>(decision) + i);
     uint4 w;
     w.x = worker_for(d.x, n_variants, worker_of);
     w.y = worker_for(d.y, n_variants, worker_of);

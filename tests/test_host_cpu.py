@@ -2,6 +2,7 @@
 the CUDA runtime and the kernel launchers (host_runtime.cpp) that writes down what is called."""
 import ctypes
 import os
+import re
 import subprocess
 
 import numpy as np
@@ -46,3 +47,20 @@ def test_load_waits_for_the_layout_before_the_first_rebuild(host):
     assert log.count("layout") == 1 and log.count("rebuild") == 1
     assert "wait" in log[log.index("layout"):log.index("rebuild")], log
     host.infaas_catalog_free(c)
+
+
+def test_overlapping_kernels_do_not_read_through_the_read_only_path():
+    """A kernel launched as a programmatic dependent runs while its predecessor still writes: loads that
+    promise constant data (__ldg, const __restrict__) or that the compiler may move over the wait are
+    allowed for the layout's arrays alone, which no kernel writes once the catalog is loaded."""
+    fixed = ("c.task_off", "c.reg_off")
+    seen = 0
+    for name in sorted(os.listdir(CSRC)):
+        text = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, name)).read())
+        if not name.endswith(".cu") or "chain_wait()" not in text:
+            continue
+        seen += 1
+        assert not re.search(r"const[^;,()]*\*\s*__restrict__", text), name
+        bad = [m.group(0) for m in re.finditer(r"__ld[a-z]+\(([^\n]{0,20})", text) if not m.group(1).startswith(fixed)]
+        assert not bad, (name, bad)
+    assert seen >= 5
