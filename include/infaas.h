@@ -238,8 +238,11 @@ int infaas_autoscale_step(infaas_catalog *c, uint32_t window_us, uint32_t slack_
  *     h_inst_worker / h_inst_load (n_inst entries each; rows whose variant or worker is out of
  *     range are ignored; may be NULL if n_inst == 0) and the worker table h_worker_hw (u8) /
  *     h_worker_util (n_workers entries; worker ids are the indices).  Replaces the previous
- *     tables (the paper's monitoring daemons refresh them every 2 s).  Allocates and frees a
- *     temporary device buffer; synchronises cuda_stream.  Errors: E_NULL, E_CUDA.
+ *     tables (the paper's monitoring daemons refresh them every 2 s).  Allocates nothing on the
+ *     device while the tables fit a buffer made with the catalog (32 bytes per variant and a
+ *     little more: about two instances per variant); larger ones get a device buffer of their
+ *     own, which is kept until infaas_catalog_free or until still larger tables replace it.
+ *     Synchronises cuda_stream.  Errors: E_NULL, E_CUDA.
  *   infaas_assign_workers: d_decision DEVICE n u32 (read), d_worker DEVICE n u32 (written),
  *     both 16-byte aligned; asynchronous, stream-ordered, allocates nothing.  Errors: E_NULL,
  *     E_ALIGN, E_BAD_ARG (infaas_workers_config never called), E_CUDA. */

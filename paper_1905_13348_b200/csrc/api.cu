@@ -1,6 +1,7 @@
 // C ABI of the library (declared in include/infaas.h): handle management, validation,
 // the host side of the catalog packer, and the calls that launch the kernels.
 #include <cstring>
+#include <memory>
 #include <mutex>
 #include <new>
 #include <string>
@@ -35,7 +36,8 @@ struct infaas_catalog {
   unsigned char *table = nullptr;        // in the arena, or table_grown
   size_t table_bytes = 0;
   void *table_grown = nullptr;
-  std::vector<unsigned char> h_table;
+  std::unique_ptr<unsigned char[]> h_table;   // from the first such call on
+  size_t h_table_bytes = 0;              // what it holds: the tables of the catalog's own size
 };
 
 namespace {
@@ -124,23 +126,38 @@ int reserve_table(infaas_catalog *c, size_t bytes) {
   return INFAAS_OK;
 }
 
-// Host tables put side by side and sent to the device in one copy.
+// The host side of the table buffer, `bytes` of it (table_lock held); null where they are more than the
+// catalog's own tables take, or memory is short: the tables are then copied one by one.
+unsigned char *host_table(infaas_catalog *c, size_t bytes) {
+  if (bytes > c->h_table_bytes) return nullptr;
+  if (!c->h_table) c->h_table.reset(new (std::nothrow) unsigned char[c->h_table_bytes]);
+  return c->h_table.get();
+}
+
+// Host tables sent to the device's table buffer: side by side in one copy while they fit the host
+// buffer, else each straight to its place.
 struct Upload {
   infaas_catalog *c;
+  struct { const void *src; size_t off, n; } part[5];
+  int n_parts = 0;
   size_t bytes = 0;
   explicit Upload(infaas_catalog *cat) : c(cat) {}
-  // Appends a table; returns its offset in the device's buffer.
+  // Adds a table (at most five); returns its offset in the device's buffer.
   size_t add(const void *src, size_t n) {
     const size_t off = bytes;
     bytes = round_up(off + n, 16);
-    if (c->h_table.size() < bytes) c->h_table.resize(bytes);
-    if (n) memcpy(c->h_table.data() + off, src, n);
+    if (n) part[n_parts++] = {src, off, n};
     return off;
   }
   int send(cudaStream_t s) {
     const int rc = reserve_table(c, bytes);
     if (rc != INFAAS_OK) return rc;
-    CUDA_TRY(cudaMemcpyAsync(c->table, c->h_table.data(), bytes, cudaMemcpyHostToDevice, s));
+    unsigned char *h = host_table(c, bytes);
+    for (int i = 0; i < n_parts; ++i) {
+      if (h) memcpy(h + part[i].off, part[i].src, part[i].n);
+      else CUDA_TRY(cudaMemcpyAsync(c->table + part[i].off, part[i].src, part[i].n, cudaMemcpyHostToDevice, s));
+    }
+    if (h && bytes) CUDA_TRY(cudaMemcpyAsync(c->table, h, bytes, cudaMemcpyHostToDevice, s));
     return INFAAS_OK;
   }
   const uint32_t *u32(size_t off) const { return reinterpret_cast<const uint32_t *>(c->table + off); }
@@ -296,7 +313,7 @@ int infaas_catalog_load(const infaas_variant *rows, uint32_t n_variants, uint32_
   c->hw_by_id = base + o_hw;
   c->slot_of_id = reinterpret_cast<uint32_t *>(base + o_slot_of_id);
   c->table = base + o_table;
-  c->table_bytes = table_bytes;
+  c->table_bytes = c->h_table_bytes = table_bytes;
   c->worker_of = reinterpret_cast<uint32_t *>(base + o_worker_of);
   c->best_inst = reinterpret_cast<unsigned long long *>(base + o_best_inst);
   c->best_hw = reinterpret_cast<unsigned long long *>(base + o_best_hw);
@@ -534,7 +551,7 @@ int infaas_workers_config(infaas_catalog *c, const uint32_t *h_inst_variant, con
   const size_t o_iv = up.add(h_inst_variant, (size_t)n_inst * 4), o_iw = up.add(h_inst_worker, (size_t)n_inst * 4),
                o_il = up.add(h_inst_load, (size_t)n_inst * 4), o_wu = up.add(h_worker_util, (size_t)n_workers * 4),
                o_wh = up.add(h_worker_hw, (size_t)n_workers);
-  const int rc = up.bytes ? up.send(s) : INFAAS_OK;
+  const int rc = up.send(s);
   if (rc != INFAAS_OK) return rc;
   CUDA_TRY(infaas::launch_workers_build(c->d.n_variants, c->hw_by_id, up.u32(o_iv), up.u32(o_iw), up.u32(o_il), n_inst,
                                         c->table + o_wh, up.u32(o_wu), n_workers, c->best_inst, c->best_hw, c->worker_of, s));
@@ -572,15 +589,23 @@ int infaas_catalog_get_state(infaas_catalog *c, uint32_t *h_queued, uint32_t *h_
                                      reinterpret_cast<unsigned long long *>(c->table + o_served),
                                      reinterpret_cast<uint32_t *>(c->table + o_queued),
                                      reinterpret_cast<uint32_t *>(c->table + o_pred), s));
-  if (c->h_table.size() < bytes) c->h_table.resize(bytes);
-  CUDA_TRY(cudaMemcpyAsync(c->h_table.data(), c->table, bytes, cudaMemcpyDeviceToHost, s));
-  CUDA_TRY(cudaStreamSynchronize(s));
-  const unsigned char *h = c->h_table.data();
+  unsigned char *h = host_table(c, bytes);
   infaas::LoadStateTail tail;
-  memcpy(&tail, h, sizeof(tail));
-  if (h_served_total) memcpy(h_served_total, h + o_served, nv * 8);
-  if (h_queued) memcpy(h_queued, h + o_queued, nv * 4);
-  if (h_pred_lat_us) memcpy(h_pred_lat_us, h + o_pred, nv * 4);
+  if (h) CUDA_TRY(cudaMemcpyAsync(h, c->table, bytes, cudaMemcpyDeviceToHost, s));
+  else CUDA_TRY(cudaMemcpyAsync(&tail, c->table, sizeof(tail), cudaMemcpyDeviceToHost, s));
+  auto fetch = [&](void *dst, size_t off, size_t n) {
+    return dst && !h ? cudaMemcpyAsync(dst, c->table + off, n, cudaMemcpyDeviceToHost, s) : cudaSuccess;
+  };
+  CUDA_TRY(fetch(h_served_total, o_served, nv * 8));
+  CUDA_TRY(fetch(h_queued, o_queued, nv * 4));
+  CUDA_TRY(fetch(h_pred_lat_us, o_pred, nv * 4));
+  CUDA_TRY(cudaStreamSynchronize(s));
+  if (h) {
+    memcpy(&tail, h, sizeof(tail));
+    if (h_served_total) memcpy(h_served_total, h + o_served, nv * 8);
+    if (h_queued) memcpy(h_queued, h + o_queued, nv * 4);
+    if (h_pred_lat_us) memcpy(h_pred_lat_us, h + o_pred, nv * 4);
+  }
   if (h_counters)
     for (int i = 0; i < 3; ++i) h_counters[i] = tail.counters[i];
   plan_select(c, tail.image_bytes);

@@ -10,13 +10,30 @@
 #include "common.cuh"
 
 namespace {
+size_t g_limit = SIZE_MAX;                 // C++ allocations above this many bytes fail
 std::string g_log;
 void note(const char *what) { g_log += what; g_log += ' '; }
+struct { const void *p[5]; } g_workers;    // what launch_workers_build was last given
 }  // namespace
+
+void *operator new(size_t n) {
+  void *p = n > g_limit ? nullptr : malloc(n);
+  if (!p) throw std::bad_alloc();
+  return p;
+}
+void *operator new[](size_t n) { return operator new(n); }
+void *operator new(size_t n, const std::nothrow_t &) noexcept { return n > g_limit ? nullptr : malloc(n); }
+void *operator new[](size_t n, const std::nothrow_t &) noexcept { return n > g_limit ? nullptr : malloc(n); }
+void operator delete(void *p) noexcept { free(p); }
+void operator delete[](void *p) noexcept { free(p); }
+void operator delete(void *p, size_t) noexcept { free(p); }
+void operator delete[](void *p, size_t) noexcept { free(p); }
 
 extern "C" {
 const char *host_log() { return g_log.c_str(); }
 void host_log_clear() { g_log.clear(); }
+void host_allocation_limit(size_t n) { g_limit = n; }
+const void *host_workers_table(int i) { return g_workers.p[i]; }
 
 cudaError_t cudaGetDevice(int *d) { *d = 0; return cudaSuccess; }
 cudaError_t cudaSetDevice(int) { return cudaSuccess; }
@@ -62,9 +79,13 @@ cudaError_t launch_load_state(const DeviceCatalog &, const uint32_t *, LoadState
 cudaError_t launch_states(const DeviceCatalog &, const uint32_t *, unsigned char *, cudaStream_t) { note("states"); return cudaSuccess; }
 cudaError_t launch_scatter(const DeviceCatalog &, const uint32_t *, uint32_t *, const unsigned char *, const uint32_t *, uint32_t *,
                            cudaStream_t) { note("scatter"); return cudaSuccess; }
-cudaError_t launch_workers_build(uint32_t, const unsigned char *, const uint32_t *, const uint32_t *, const uint32_t *, uint32_t,
-                                 const unsigned char *, const uint32_t *, uint32_t, unsigned long long *, unsigned long long *,
-                                 uint32_t *, cudaStream_t) { note("workers_build"); return cudaSuccess; }
+cudaError_t launch_workers_build(uint32_t, const unsigned char *, const uint32_t *iv, const uint32_t *iw, const uint32_t *il, uint32_t,
+                                 const unsigned char *wh, const uint32_t *wu, uint32_t, unsigned long long *, unsigned long long *,
+                                 uint32_t *, cudaStream_t) {
+  note("workers_build");
+  g_workers = {iv, iw, il, wh, wu};
+  return cudaSuccess;
+}
 cudaError_t launch_assign_workers(const uint32_t *, uint64_t, uint32_t, const uint32_t *, uint32_t *, int, cudaStream_t) {
   note("assign");
   return cudaSuccess;

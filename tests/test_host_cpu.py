@@ -23,6 +23,7 @@ def host(tmp_path_factory):
                            os.path.join(CSRC, "api.cu"), os.path.join(HERE, "host_runtime.cpp"), "-o", so])
     lib = ctypes.CDLL(so)
     lib.host_log.restype = ctypes.c_char_p
+    lib.host_allocation_limit.argtypes = [ctypes.c_size_t]
     return lib
 
 
@@ -64,3 +65,50 @@ def test_overlapping_kernels_do_not_read_through_the_read_only_path():
         bad = [m.group(0) for m in re.finditer(r"__ld[a-z]+\(([^\n]{0,20})", text) if not m.group(1).startswith(fixed)]
         assert not bad, (name, bad)
     assert seen >= 5
+
+
+def _workers_config(host, c, tables):
+    host.infaas_workers_config.argtypes = [ctypes.c_void_p] * 4 + [ctypes.c_uint32] + [ctypes.c_void_p] * 2 + [ctypes.c_uint32,
+                                                                                                          ctypes.c_void_p]
+    iv, iw, il, hw, ut = tables
+    host.host_log_clear()
+    rc = host.infaas_workers_config(c, iv.ctypes.data, iw.ctypes.data, il.ctypes.data, iv.size, hw.ctypes.data, ut.ctypes.data,
+                                    hw.size, None)
+    host.host_workers_table.restype = ctypes.c_void_p
+    got = [np.ctypeslib.as_array(ctypes.cast(host.host_workers_table(i), ctypes.POINTER(ctypes.c_uint8)), (a.nbytes,))
+           for i, a in enumerate(tables)]
+    return rc, all(np.array_equal(g, a.view(np.uint8)) for g, a in zip(got, tables))
+
+
+@pytest.mark.parametrize("n_inst,n_workers", [(1, 1), (1000, 17), (40_001, 5_003)])
+def test_host_tables_without_host_memory(host, n_inst, n_workers):
+    """The header promises that no function throws and asks for no host memory: a table call goes on
+    without the buffer it would pass its tables through, and no table is copied on the host that is
+    larger than the catalog's own."""
+    w = W.make("C1", n_queries=16)
+    rng = np.random.default_rng(n_inst)
+    tables = [rng.integers(0, 2**31, n, np.uint32) for n in (n_inst, n_inst, n_inst)] + \
+        [rng.integers(0, 256, n_workers, np.uint8), rng.integers(0, 2**31, n_workers, np.uint32)]
+    # a catalog's own buffers: 32 bytes per variant, 4 per task and 32 KB
+    own = 32 * w.n_variants + 4 * w.n_tasks + 32768
+    for limit, grown in ((64, False), (own, False), (2**62, False), (64, True)):
+        c = _load(host, w.rows, w.n_tasks)
+        if grown:                                     # buffers as an earlier, larger call leaves them
+            big = [np.repeat(a, 3) for a in tables]
+            assert _workers_config(host, c, big) == (0, True)
+        host.host_allocation_limit(limit)
+        try:
+            rc, same = _workers_config(host, c, tables)
+            log = _log(host)
+            state = np.ones(w.n_variants, np.uint8)
+            queued, served = np.empty(w.n_variants, np.uint32), np.empty(w.n_variants, np.uint64)
+            host.infaas_catalog_set_states.argtypes = host.infaas_autoscale_config.argtypes = [ctypes.c_void_p] * 4
+            host.infaas_catalog_get_state.argtypes = [ctypes.c_void_p] * 6
+            rcs = [host.infaas_catalog_set_states(c, state.ctypes.data, queued.ctypes.data, None),
+                   host.infaas_autoscale_config(c, queued.ctypes.data, np.zeros(w.n_tasks, np.uint32).ctypes.data, None),
+                   host.infaas_catalog_get_state(c, queued.ctypes.data, None, served.ctypes.data, None, None)]
+        finally:
+            host.host_allocation_limit(2**64 - 1)
+        assert rc == 0 and same and rcs == [0, 0, 0]
+        assert log.count("malloc") == (12 * n_inst + 5 * n_workers > own and not grown)
+        host.infaas_catalog_free(c)
