@@ -53,7 +53,8 @@ typedef struct {
 #define INFAAS_E_BAD_BATCH (-3) /* a row's batch == 0                                     */
 #define INFAAS_E_BAD_LAT (-4)   /* a row's lat_us == 0                                    */
 #define INFAAS_E_BAD_ACC (-5)   /* a row's acc_bp > 10000 or reserved != 0                */
-#define INFAAS_E_TOO_LARGE (-6) /* a size limit is exceeded (see each function)           */
+#define INFAAS_E_TOO_LARGE (-6) /* a size limit is exceeded (see each function), or host
+                                   memory has run out                                     */
 #define INFAAS_E_CUDA (-7)      /* a CUDA call failed; infaas_last_cuda_error() has text  */
 #define INFAAS_E_ALIGN (-8)     /* a device array is not 16-byte aligned                  */
 #define INFAAS_E_DEVICE (-9)    /* a kernel reported an internal error (a bounded wait ran

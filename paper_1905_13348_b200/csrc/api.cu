@@ -45,7 +45,11 @@ namespace {
 thread_local std::string g_cuda_error;
 
 int cuda_fail(cudaError_t e) {
-  g_cuda_error = std::string(cudaGetErrorName(e)) + ": " + cudaGetErrorString(e);
+  try {
+    g_cuda_error = std::string(cudaGetErrorName(e)) + ": " + cudaGetErrorString(e);
+  } catch (...) {             // no memory for the text
+    g_cuda_error.clear();
+  }
   (void)cudaGetLastError();   // clear the sticky-free error state
   return INFAAS_E_CUDA;
 }
@@ -191,7 +195,7 @@ const char *infaas_strerror(int code) {
     case INFAAS_E_BAD_BATCH: return "row batch size is 0";
     case INFAAS_E_BAD_LAT: return "row latency is 0";
     case INFAAS_E_BAD_ACC: return "row accuracy above 10000 basis points, or reserved field not 0";
-    case INFAAS_E_TOO_LARGE: return "size limit exceeded";
+    case INFAAS_E_TOO_LARGE: return "size limit exceeded, or out of host memory";
     case INFAAS_E_CUDA: return "CUDA call failed (see infaas_last_cuda_error)";
     case INFAAS_E_ALIGN: return "device array is not 16-byte aligned";
     case INFAAS_E_DEVICE: return "a kernel reported an internal error";
@@ -204,7 +208,7 @@ const char *infaas_strerror(int code) {
 const char *infaas_last_cuda_error(void) { return g_cuda_error.c_str(); }
 
 int infaas_catalog_load(const infaas_variant *rows, uint32_t n_variants, uint32_t n_tasks,
-                        int cuda_device, infaas_catalog **out) {
+                        int cuda_device, infaas_catalog **out) try {
   if (out) *out = nullptr;
   if (!rows || !out) return INFAAS_E_NULL;
   if (n_tasks == 0 || n_tasks > 65535u) return INFAAS_E_BAD_TASK;
@@ -247,13 +251,6 @@ int infaas_catalog_load(const infaas_variant *rows, uint32_t n_variants, uint32_
     for (uint32_t v = 0; v < n_variants; ++v) members[cursor[rows[v].task]++] = v;
   }
 
-  infaas_catalog *c = new (std::nothrow) infaas_catalog();
-  if (!c) return INFAAS_E_TOO_LARGE;
-  c->device = cuda_device;
-  DeviceScope scope(cuda_device);
-  if (scope.status != cudaSuccess) { delete c; return cuda_fail(scope.status); }
-
-  // ---- one arena, carved into 256-byte aligned arrays ----
   // lists longer than the index supports are cut into segments; every segment but a task's
   // first needs a header and parameters outside the image
   uint64_t worst_image = infaas::image_var_offset(n_tasks, infaas::buckets_for(n_tasks, max_task), nbw);
@@ -266,7 +263,15 @@ int infaas_catalog_load(const infaas_variant *rows, uint32_t n_variants, uint32_
     worst_image += (uint64_t)segs * infaas::block_capacity(V, nbw);
   }
   const uint32_t n_extra = seg_base[n_tasks];
-  if (worst_image > 0xFFFFFFF0ull) { delete c; return INFAAS_E_TOO_LARGE; }
+  if (worst_image > 0xFFFFFFF0ull) return INFAAS_E_TOO_LARGE;
+
+  infaas_catalog *c = new (std::nothrow) infaas_catalog();
+  if (!c) return INFAAS_E_TOO_LARGE;
+  c->device = cuda_device;
+  DeviceScope scope(cuda_device);
+  if (scope.status != cudaSuccess) { delete c; return cuda_fail(scope.status); }
+
+  // ---- one arena, carved into 256-byte aligned arrays ----
   size_t total = 0;
   auto carve = [&total](size_t bytes) { size_t off = total; total += round_up(bytes, 256); return off; };
   const size_t o_task_off = carve((n_tasks + 1) * 4), o_reg_off = carve((n_tasks + 1) * 4);
@@ -398,6 +403,8 @@ int infaas_catalog_load(const infaas_variant *rows, uint32_t n_variants, uint32_
 #undef LOAD_TRY
   *out = c;
   return INFAAS_OK;
+} catch (const std::bad_alloc &) {          // (no handle exists yet where host memory is allocated)
+  return INFAAS_E_TOO_LARGE;
 }
 
 int infaas_select_batch(infaas_catalog *c, const uint16_t *d_task, const uint32_t *d_slo_us,
@@ -638,7 +645,7 @@ int infaas_catalog_get_frontier(infaas_catalog *c, uint32_t task, uint32_t *h_id
   return INFAAS_OK;
 }
 
-int infaas_catalog_get_info(infaas_catalog *c, uint32_t h_info[8], void *cuda_stream) {
+int infaas_catalog_get_info(infaas_catalog *c, uint32_t h_info[8], void *cuda_stream) try {
   if (!c || !h_info) return INFAAS_E_NULL;
   DeviceScope scope(c->device);
   if (scope.status != cudaSuccess) return cuda_fail(scope.status);
@@ -663,6 +670,8 @@ int infaas_catalog_get_info(infaas_catalog *c, uint32_t h_info[8], void *cuda_st
   h_info[4] = infaas::select_image_smem(c->select_smem);
   h_info[5] = h_info[6] = h_info[7] = 0;
   return INFAAS_OK;
+} catch (const std::bad_alloc &) {
+  return INFAAS_E_TOO_LARGE;
 }
 
 void infaas_catalog_free(infaas_catalog *c) {

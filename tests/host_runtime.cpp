@@ -10,6 +10,7 @@
 #include "common.cuh"
 
 namespace {
+cudaError_t g_error = cudaSuccess;         // what cudaGetDevice returns
 size_t g_limit = SIZE_MAX;                 // C++ allocations above this many bytes fail
 std::string g_log;
 void note(const char *what) { g_log += what; g_log += ' '; }
@@ -33,13 +34,14 @@ extern "C" {
 const char *host_log() { return g_log.c_str(); }
 void host_log_clear() { g_log.clear(); }
 void host_allocation_limit(size_t n) { g_limit = n; }
+void host_device_error(int on) { g_error = on ? cudaErrorNoDevice : cudaSuccess; }
 const void *host_workers_table(int i) { return g_workers.p[i]; }
 
-cudaError_t cudaGetDevice(int *d) { *d = 0; return cudaSuccess; }
+cudaError_t cudaGetDevice(int *d) { *d = 0; return g_error; }
 cudaError_t cudaSetDevice(int) { return cudaSuccess; }
 cudaError_t cudaDeviceGetAttribute(int *v, cudaDeviceAttr, int) { *v = 148; return cudaSuccess; }
 cudaError_t cudaGetLastError() { return cudaSuccess; }
-const char *cudaGetErrorName(cudaError_t) { return "error"; }
+const char *cudaGetErrorName(cudaError_t) { return "an error name that does not fit into a short string"; }
 const char *cudaGetErrorString(cudaError_t) { return "of the stand-in"; }
 cudaError_t cudaMalloc(void **p, size_t n) {
   note("malloc");

@@ -112,3 +112,26 @@ def test_host_tables_without_host_memory(host, n_inst, n_workers):
         assert rc == 0 and same and rcs == [0, 0, 0]
         assert log.count("malloc") == (12 * n_inst + 5 * n_workers > own and not grown)
         host.infaas_catalog_free(c)
+
+
+def test_no_exception_leaves_the_c_entries(host):
+    """Host memory that runs out inside a call is an error code, not a C++ exception."""
+    w = W.make("C2", n_queries=16)
+    c = _load(host, w.rows, w.n_tasks)
+    out, info = ctypes.c_void_p(None), np.zeros(8, np.uint32)
+    host.infaas_catalog_get_info.argtypes = [ctypes.c_void_p] * 3
+    rcs = []
+    for limit in (0, 64, 200, 4 * w.n_tasks, 4 * w.n_variants - 1):
+        host.host_allocation_limit(limit)
+        rcs.append(host.infaas_catalog_load(w.rows.ctypes.data, w.rows.shape[0], w.n_tasks, 0, ctypes.byref(out)))
+        assert out.value is None
+        if limit < 4 * w.n_tasks:
+            rcs.append(host.infaas_catalog_get_info(c, info.ctypes.data, None))
+    host.host_device_error(1)
+    host.host_allocation_limit(0)                        # (no room for the error's text either)
+    failed = host.infaas_catalog_get_info(c, info.ctypes.data, None)
+    host.host_device_error(0)
+    host.host_allocation_limit(2**64 - 1)
+    assert set(rcs) == {-6} and failed == -7
+    assert host.infaas_catalog_get_info(c, info.ctypes.data, None) == 0
+    host.infaas_catalog_free(c)
