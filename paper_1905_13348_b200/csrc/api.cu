@@ -358,10 +358,7 @@ int infaas_catalog_load(const infaas_variant *rows, uint32_t n_variants, uint32_
   d.image_capacity = (uint32_t)worst_image;
   d.image_hdr = reinterpret_cast<uint32_t *>(base + o_hdr);
   d.n_buckets = infaas::buckets_for(n_tasks, max_task);
-  // several CTAs per task where lists can span several segments, the SMs are idle, and no block can lie
-  // out of reach of the task word (the CTAs of a task could not agree on an index then)
-  const bool spread = max_task > 1024 && worst_image < infaas::IMAGE_T2_LIMIT && 4ull * n_tasks <= (uint64_t)c->sm_count;
-  d.rebuild_ctas = spread ? 4 : 1;
+  d.rebuild_ctas = 1;
   d.acc_lo = acc_lo;
   d.nbw = nbw;
   d.lat_code_lo = float_bits_rz(lat_min) >> 16;
@@ -394,6 +391,17 @@ int infaas_catalog_load(const infaas_variant *rows, uint32_t n_variants, uint32_
   LOAD_TRY(infaas::prepare_select_kernel());
   LOAD_TRY(infaas::prepare_tally_kernel());
   LOAD_TRY(infaas::prepare_rebuild_kernel());
+  // Several CTAs per task where lists can span several segments, no block can lie out of reach of the task
+  // word (the CTAs of a task could not agree on an index then), and the clusters of all tasks run at
+  // once (33 of them on a B200).  A window of 20,000 queries with four CTAs / with one, us, tasks of
+  // 1100 variants, structured and trade-off: 4 tasks 28.7 / 33.0 and 33.2 / 36.9, 20 tasks 26.2 / 28.2
+  // and 32.3 / 35.5, 33 tasks 25.1 / 23.4 and 34.4 / 35.1; in a second wave, 34 tasks 32.2 / 23.3 and
+  // 43.0 / 34.9.  Where every list is one segment the clusters cost 1 us.
+  if (max_task > 1024 && worst_image < infaas::IMAGE_T2_LIMIT) {
+    uint32_t at_once = 0;
+    LOAD_TRY(infaas::rebuild_clusters_at_once(max_task, &at_once));
+    if (n_tasks <= at_once) d.rebuild_ctas = infaas::REBUILD_CLUSTER;
+  }
   // every kernel from here on reads the layout before it waits for its predecessor
   LOAD_TRY(cudaStreamSynchronize(nullptr));
   LOAD_TRY(infaas::launch_rebuild(d, /*advance_queues=*/false, 0, nullptr));

@@ -210,7 +210,7 @@ struct DeviceCatalog {
   uint32_t *image_hdr;       // published by the rebuild kernel: [0] bytes of the image, [1] the bucket
                              // scale 2^-S and [2] -bmin, both as float patterns
   uint32_t n_buckets;        // SLO buckets per task
-  uint32_t rebuild_ctas;     // CTAs per task of the rebuild kernel (1 or 4)
+  uint32_t rebuild_ctas;     // CTAs per task of the rebuild kernel (1 or REBUILD_CLUSTER)
   uint32_t acc_lo, nbw;      // accuracy window of every bitmap: acc_lo (multiple of 24) .. acc_lo + 24 nbw - 1
   uint32_t lat_code_lo;      // bits(smallest profiled latency) >> 16: where the SLO buckets start
 
@@ -244,11 +244,14 @@ enum : uint32_t {
 constexpr uint32_t SELECT_MAX_SMEM = 227u * 1024u - 256u;
 // Shared memory of the rebuild kernel per variant of the largest task.
 constexpr uint32_t REBUILD_ROW_SMEM = 22u;
+constexpr uint32_t REBUILD_CLUSTER = 4u;   // CTAs per large task
 
 // Once per device, with that device current: raise the kernels' shared-memory limits.
 cudaError_t prepare_select_kernel();
 cudaError_t prepare_tally_kernel();
 cudaError_t prepare_rebuild_kernel();
+// How many clusters of REBUILD_CLUSTER CTAs of the rebuild kernel the current device runs at once.
+cudaError_t rebuild_clusters_at_once(uint32_t max_task_variants, uint32_t *n);
 
 // Kernels of one stream overlap at their seams (programmatic dependent launch): a kernel launched
 // with launch_chained may start while its predecessor still runs.  Before chain_wait() it touches

@@ -816,12 +816,30 @@ rebuild_kernel(DeviceCatalog c, int advance, uint32_t window_us) {
 
 // The block sizes the thread ranges above rely on.
 static_assert(REBUILD_THREADS >= 512 && INDEX_MAX_F < 254, "thread ranges of build_index");
+static_assert(REBUILD_CLUSTER == 4, "task and share from the CTA's index in rebuild_kernel");
 
 }  // namespace
 
 cudaError_t prepare_rebuild_kernel() {
   return cudaFuncSetAttribute(rebuild_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               (int)(INFAAS_MAX_TASK_VARIANTS * REBUILD_ROW_SMEM));
+}
+
+cudaError_t rebuild_clusters_at_once(uint32_t max_task_variants, uint32_t *n) {
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = REBUILD_CLUSTER;
+  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(REBUILD_CLUSTER);
+  cfg.blockDim = dim3(REBUILD_THREADS);
+  cfg.dynamicSmemBytes = (size_t)max_task_variants * REBUILD_ROW_SMEM;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  int clusters = 0;
+  const cudaError_t e = cudaOccupancyMaxActiveClusters(&clusters, rebuild_kernel, &cfg);
+  *n = clusters > 0 ? (uint32_t)clusters : 0u;
+  return e;
 }
 
 cudaError_t launch_rebuild(const DeviceCatalog &c, bool advance_queues, uint32_t window_us,

@@ -63,7 +63,11 @@ cudaError_t prepare_tally_kernel() { return cudaSuccess; }
 cudaError_t prepare_rebuild_kernel() { return cudaSuccess; }
 uint32_t select_image_smem(uint32_t n) { return n; }
 cudaError_t launch_layout(const CatalogLayout &, uint32_t, uint32_t, cudaStream_t) { note("layout"); return cudaSuccess; }
-cudaError_t launch_rebuild(const DeviceCatalog &, bool, uint32_t, cudaStream_t) { note("rebuild"); return cudaSuccess; }
+cudaError_t rebuild_clusters_at_once(uint32_t, uint32_t *n) { *n = 33; return cudaSuccess; }
+cudaError_t launch_rebuild(const DeviceCatalog &c, bool, uint32_t, cudaStream_t) {
+  note(c.rebuild_ctas == 1 ? "rebuild" : "rebuild_by_clusters");
+  return cudaSuccess;
+}
 cudaError_t launch_tally(const DeviceCatalog &, const uint32_t *, uint64_t, int, cudaStream_t) { note("tally"); return cudaSuccess; }
 cudaError_t launch_select(const DeviceCatalog &, const uint16_t *, const uint32_t *, const uint16_t *, uint64_t, uint32_t *, int,
                           uint32_t, uint32_t, bool, cudaStream_t) { note("select"); return cudaSuccess; }

@@ -135,3 +135,16 @@ def test_no_exception_leaves_the_c_entries(host):
     assert set(rcs) == {-6} and failed == -7
     assert host.infaas_catalog_get_info(c, info.ctypes.data, None) == 0
     host.infaas_catalog_free(c)
+
+
+@pytest.mark.parametrize("n_tasks,per_task,clusters", [(1, 1024, False), (1, 1025, True), (33, 1025, True), (34, 1025, False),
+                                                       (37, 1025, False), (5, 8192, True), (7, 8192, False)])
+def test_clusters_only_where_all_run_at_once(host, n_tasks, per_task, clusters):
+    """Four CTAs per large task only while a second wave is not needed (the stand-in's device runs 33
+    clusters at once), and while every block is in reach of the task word (7 x 8192 variants are not)."""
+    rows = np.zeros(n_tasks * per_task, W.VARIANT_DTYPE)
+    rows["task"] = np.arange(rows.size) % n_tasks
+    rows["batch"] = rows["lat_us"] = rows["cost"] = 1
+    c = _load(host, rows, n_tasks)
+    assert [x for x in _log(host) if x.startswith("rebuild")] == ["rebuild_by_clusters" if clusters else "rebuild"]
+    host.infaas_catalog_free(c)
