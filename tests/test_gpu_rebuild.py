@@ -69,3 +69,36 @@ def test_two_lists_at_the_edges(V, kind):
     rng = np.random.default_rng(V)
     load = rng.choice(np.array([0, 1, 5000, 2**32 - 1], np.uint32), w.n_variants)
     run_stateful(w, _states(rng, w.n_variants, (0.45, 0.45, 0.05, 0.05)), load)
+
+
+# Lists of every variant: 7 and 34 segments, so that with four CTAs per task (3 tasks; 33 is the last
+# number of tasks for which all clusters run at once) a CTA indexes several of them, and with one (34) all
+@pytest.mark.parametrize("states", [False, True])
+@pytest.mark.parametrize("V,n_tasks", [(1500, 3), (1500, 33), (1500, 34), (8192, 3)])
+def test_lists_of_many_segments(V, n_tasks, states):
+    import paper_1905_13348_b200 as P
+    rng = np.random.default_rng([V, n_tasks])
+    i = np.concatenate([np.arange(V), np.arange(V)] + [np.arange(3)] * (n_tasks - 2))
+    task = np.concatenate([np.zeros(V), np.ones(V), np.repeat(np.arange(2, n_tasks), 3)]).astype(np.int64)
+    # slower is cheaper and more accurate: nothing is dominated
+    rows = rows_from(task, np.full(i.size, 64), 1000 + 37 * i, 1 + i * 9998 // V, 5 + 11 * (V - i), None)
+    rows = rows[rng.permutation(rows.size)].copy()
+    n = 4000
+    q_task = rng.choice([0, 0, 1, 1, 2, n_tasks], n).astype(np.uint16)
+    q_slo = np.exp(rng.uniform(np.log(500.0), np.log(80.0 * V), n)).astype(np.uint32)
+    q_acc = rng.integers(0, 10_001, n).astype(np.uint16)
+    w = W.Workload(f"segments{V}", n_tasks, rows, q_task, q_slo, q_acc, 1333, 3_000, "lists of many segments")
+    cat = P.infaas_catalog_load(rows, n_tasks)
+    try:
+        assert P.infaas_catalog_get_info(cat)["longest_list"] == V
+        if states:
+            state = _states(rng, rows.size, (0.45, 0.45, 0.05, 0.05))
+            load = np.zeros(rows.size, np.uint32)
+            P.infaas_catalog_set_states(cat, state, load)
+            assert P.infaas_catalog_get_info(cat)["longest_list"] > 0.85 * V > 1000
+    finally:
+        cat.free()
+    if states:
+        run_stateful(w, state, load)
+    else:
+        run_both(w)
