@@ -104,7 +104,11 @@ def _init_torch() -> None:
     global _raw_stream, _current_device
     import torch
     torch.cuda.init()                       # the raw getters below assume it (and it refuses a forked child)
-    _raw_stream, _current_device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+    try:
+        raw, device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+    except AttributeError:                  # they are torch's own; the public call costs some 2 us more
+        raw, device = (lambda d: torch.cuda.current_stream(d).cuda_stream), torch.cuda.current_device
+    _raw_stream, _current_device = raw, device
 
 
 def _forget_torch() -> None:

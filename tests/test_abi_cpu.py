@@ -87,3 +87,20 @@ def test_binding_constants_match_the_header():
     assert sorted(b.EXPORTS) == sorted(n for n in declared_functions())
     codes = sorted(v for k, v in defs.items() if k.startswith("INFAAS_E_"))
     assert codes == list(range(-11, 0))
+
+
+@pytest.mark.parametrize("missing", ["_cuda_getCurrentRawStream", "_cuda_getDevice"])
+def test_current_stream_without_torchs_private_getters(monkeypatch, missing):
+    import types
+
+    import torch
+
+    from paper_1905_13348_b200 import binding as b
+    monkeypatch.delattr(torch._C, missing)
+    monkeypatch.setattr(torch.cuda, "init", lambda: None)
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 3)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda device=None: types.SimpleNamespace(cuda_stream=4000 + device))
+    monkeypatch.setattr(b, "_raw_stream", None)
+    monkeypatch.setattr(b, "_current_device", None)
+    assert b._stream_ptr(None) == 4003
+    assert b._stream_ptr(types.SimpleNamespace(cuda_stream=5)) == 5
