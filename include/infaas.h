@@ -277,7 +277,8 @@ int infaas_catalog_get_frontier(infaas_catalog *c, uint32_t task, uint32_t *h_id
  *   h_info[3] tasks whose list has no rank index (longer than the index supports)
  *   h_info[4] shared memory (bytes) the next infaas_select_batch reserves for the image;
  *             if h_info[0] is larger the kernel reads the image from global memory
- *   h_info[5..7] reserved (0).
+ *   h_info[5] SLO buckets per task (fixed when the catalog is loaded)
+ *   h_info[6..7] reserved (0).
  * Synchronises cuda_stream. */
 int infaas_catalog_get_info(infaas_catalog *c, uint32_t h_info[8], void *cuda_stream);
 

@@ -106,7 +106,7 @@ def _init_torch() -> None:
     torch.cuda.init()                       # the raw getters below assume it (and it refuses a forked child)
     try:
         raw, device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
-    except AttributeError:                  # they are torch's own; the public call costs some 2 us more
+    except AttributeError:                  # they are torch's own; the public calls do the same
         raw, device = (lambda d: torch.cuda.current_stream(d).cuda_stream), torch.cuda.current_device
     _raw_stream, _current_device = raw, device
 
@@ -287,7 +287,7 @@ def infaas_catalog_get_info(cat: Catalog, stream=None) -> dict:
     _check(_load().infaas_catalog_get_info(cat.handle, info.ctypes.data, _stream_ptr(stream)),
            "infaas_catalog_get_info")
     return {"image_bytes": int(info[0]), "longest_list": int(info[1]), "list_entries": int(info[2]),
-            "tasks_not_indexed": int(info[3]), "image_smem": int(info[4])}
+            "tasks_not_indexed": int(info[3]), "image_smem": int(info[4]), "slo_buckets": int(info[5])}
 
 
 def infaas_catalog_get_frontier(cat: Catalog, task: int, stream=None) -> np.ndarray:

@@ -676,7 +676,8 @@ int infaas_catalog_get_info(infaas_catalog *c, uint32_t h_info[8], void *cuda_st
     if (f_len[t] > 0 && (slow[t].z & infaas::TASK_FLAG_NOT_INDEXED)) ++h_info[3];
   }
   h_info[4] = infaas::select_image_smem(c->select_smem);
-  h_info[5] = h_info[6] = h_info[7] = 0;
+  h_info[5] = c->d.n_buckets;
+  h_info[6] = h_info[7] = 0;
   return INFAAS_OK;
 } catch (const std::bad_alloc &) {
   return INFAAS_E_TOO_LARGE;

@@ -88,10 +88,11 @@ inline __host__ __device__ uint32_t round_up_u32(uint32_t x, uint32_t a) { retur
 // shared-memory banks.
 inline __host__ __device__ uint32_t rec_stride(uint32_t nb) { return 4u * (nb + 1u); }   // bytes from one task's records to the next's
 // SLO buckets per task: 256, more for tasks of more than 256 variants while all records together stay
-// within 48 KB (up to 23 tasks).  Long lists have several latencies per bucket, and every query of
-// such a bucket takes the slow path: 2^22 queries on 4 x 4096 variants (lists of up to 320 entries)
-// take 84 us with 256 buckets and 51 us with 2048; with 2048 for lists of 40 entries the rebuild only
-// takes 1 us longer.
+// within 48 KB (up to 22 tasks).  Long lists have several latencies per bucket, and every query of
+// such a bucket takes the slow path: 2^22 queries on trade-off catalogs with 256 buckets / with more,
+// us: 4 x 4096 variants (lists of up to 315 entries) 96.2 / 74.6, 8 x 1000 60.0 / 55.4, 2 x 1000 45.4 /
+// 39.8; the rebuild takes up to 1.7 us longer.  The records can push an image out of shared memory that
+// would fit with 256 buckets; both ways are as fast then: 4 x 1100 48.9 / 48.0, 5 x 1100 46.7 / 48.6.
 inline __host__ __device__ uint32_t buckets_for(uint32_t n_tasks, uint32_t max_task_variants) {
   uint32_t nb = MIN_BUCKETS;
   while (nb < MAX_BUCKETS && nb < max_task_variants && rec_stride(2u * nb) * (n_tasks + 1u) <= 48u * 1024u) nb *= 2u;

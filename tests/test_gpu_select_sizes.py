@@ -36,14 +36,18 @@ def test_batch_sizes_around_the_kernels_limits(name, kw, n):
         cat.free()
 
 
-# 2048, 2048, 1024, 512, 512, 512, 256, 256 buckets per task
-@pytest.mark.parametrize("n_tasks,per_task", [(1, 1100), (4, 1100), (10, 600), (11, 600), (23, 300), (2, 300), (24, 300), (2, 256)])
-def test_slos_at_every_latency_and_bucket_edge(n_tasks, per_task):
+# both sides of every line where the bucket count changes: 48 KB of records at 4 / 5, 10 / 11 and 22 / 23
+# tasks, 256 variants per task
+@pytest.mark.parametrize("n_tasks,per_task,buckets", [
+    (1, 1100, 2048), (4, 1100, 2048), (5, 1100, 1024), (10, 600, 1024), (11, 600, 512), (22, 300, 512), (23, 300, 256),
+    (2, 300, 512), (24, 300, 256), (2, 257, 512), (2, 256, 256)])
+def test_slos_at_every_latency_and_bucket_edge(n_tasks, per_task, buckets):
     import paper_1905_13348_b200 as P
     rng = np.random.default_rng(n_tasks)
     rows = W.tradeoff_catalog(rng, n_tasks, per_task)
     cat, o = P.infaas_catalog_load(rows, n_tasks), OracleCatalog(rows, n_tasks)
     try:
+        assert P.infaas_catalog_get_info(cat)["slo_buckets"] == buckets
         edges = np.arange(0x3F800000 >> 16, 0x4F80, dtype=np.uint32) << 16     # every possible bucket's start
         edge = np.floor(edges.view(np.float32).astype(np.float64)).astype(np.uint64)
         v = np.unique(np.concatenate([edge, rows["lat_us"].astype(np.uint64), np.array([0, 1, 2**24, 2**32 - 1], np.uint64)]))
