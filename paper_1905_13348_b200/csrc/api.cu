@@ -20,7 +20,6 @@ struct infaas_catalog {
   std::vector<uint32_t> task_off, reg_off;
   uint32_t select_smem = 0;              // shared memory reserved for the staged image
   uint32_t image_seen = 0;               // size of the image when the host last looked
-  uint32_t worst_image_bytes = 0;        // image size if every block had its largest size
   uint32_t *s_inst = nullptr;            // running instances per slot (Model-Autoscaler)
   uint16_t *s_arch = nullptr;            // architecture code per slot
   unsigned long long *s_qps = nullptr;   // profiled saturation throughput per slot, milli-queries/s
@@ -52,18 +51,6 @@ int cuda_fail(cudaError_t e) {
   }
   (void)cudaGetLastError();   // clear the sticky-free error state
   return INFAAS_E_CUDA;
-}
-
-// Multiprocessors of a device, asked once per device.
-int sm_count_of(int device) {
-  static int cached[64] = {};
-  if (device < 0 || device >= 64) return 0;
-  if (!cached[device]) {
-    int n = 0;
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return 0;
-    cached[device] = n;
-  }
-  return cached[device];
 }
 
 #define CUDA_TRY(expr)                         \
@@ -179,8 +166,8 @@ int infaas_intpipe_probe(uint32_t iters, uint32_t *d_sink, int cuda_device, uint
   if (iters == 0 || iters > (1u << 24)) return INFAAS_E_BAD_ARG;
   DeviceScope scope(cuda_device);
   if (scope.status != cudaSuccess) return cuda_fail(scope.status);
-  const int sms = sm_count_of(cuda_device);
-  if (sms <= 0) return cuda_fail(cudaErrorInvalidDevice);
+  int sms = 0;
+  CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, cuda_device));
   unsigned long long ops = 0;
   CUDA_TRY(infaas::launch_intpipe_probe(iters, 0x9E3779B1u, d_sink, sms, &ops, static_cast<cudaStream_t>(cuda_stream)));
   *h_lane_ops = ops;
@@ -368,7 +355,6 @@ int infaas_catalog_load(const infaas_variant *rows, uint32_t n_variants, uint32_
   d.slo_seen = reinterpret_cast<uint32_t *>(base + o_seen);
   c->task_off.swap(task_off);
   c->reg_off.swap(reg_off);
-  c->worst_image_bytes = (uint32_t)worst_image;
 
   {
     LOAD_TRY(cudaMemcpy(d.image, rows, (size_t)n_variants * sizeof(infaas_variant), cudaMemcpyHostToDevice));
