@@ -322,8 +322,8 @@ cudaError_t launch_select(const DeviceCatalog &c, const uint16_t *d_task, const 
                           int sm_count, uint32_t image_smem, uint32_t image_seen, bool tally, cudaStream_t stream);
 // Batches below this size are tallied by the selection kernel itself in infaas_select_update.  A window
 // (select, tally, rebuild) with the fused / the separate tally, us: 64 tasks x 256 variants, 131,072
-// queries 16.9 / 20.0, 200,000: 19.4 / 21.2, 262,143: 21.6 / 22.1; 4 x 132 (few, hot variants), 131,072:
-// 20.3 / 20.1, 262,143: 27.0 / 20.6; 128 x 512, 160,000: 18.1 / 22.2, 262,143: 22.4 / 24.1.
+// queries 18.5 / 26.2, 200,000: 17.8 / 19.2, 262,143: 19.3 / 19.4; 4 x 132 (few, hot variants), 131,072:
+// 19.4 / 19.4, 262,143: 26.8 / 19.0; 128 x 512, 160,000: 16.8 / 20.8, 262,143: 21.3 / 22.7.
 constexpr uint64_t FUSED_TALLY_MAX_N = 192 * 1024;
 
 // Scaling-up step of the Model-Autoscaler for every task, from the pending per-variant

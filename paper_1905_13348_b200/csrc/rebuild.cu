@@ -735,13 +735,14 @@ __device__ __forceinline__ uint32_t build_list(const DeviceCatalog &c, uint32_t 
 //
 // Bound by the latency of its chain of barriers and shared-memory round trips, and by fetching its
 // code: every line of it runs about once per launch, and with the compiler's unrolling (116 KB of
-// code) 40 % of the stalls were for instructions.  So the loops are not unrolled (47 KB) except the
+// code) 40 % of the stalls were for instructions.  So the loops are not unrolled (50 KB) except the
 // few that run long.  Measured on one B200, in GPU clock cycles after the previous kernel's end: 64
 // tasks x 256 variants, lists of up to 100 entries: 16 K (18 K unrolled), 128 x 512: 19 K (22 K), 4 x
-// 4096 on a trade-off surface, lists of up to 505 entries: 77 K (90 K), two lists per task: 17 K
+// 4096 on a trade-off surface, lists of up to 505 entries, with one CTA per task: 77 K (90 K), two lists: 17 K
 // (23 K).  512 threads instead of 1024: short lists 5 % faster, lists of 100 entries 5 % slower.
 // The segments of a list of several hundred entries take as long as the list itself, so tasks of more
-// than 1024 variants have 4 CTAs: 47 us a window instead of 62 on the trade-off surface.
+// than 1024 variants have 4 CTAs (rule in infaas_catalog_load): 48 us a window instead of 63 on the
+// trade-off surface, 4 x 4096.
 __global__ void __launch_bounds__(REBUILD_THREADS)
 rebuild_kernel(DeviceCatalog c, int advance, uint32_t window_us) {
   extern __shared__ __align__(16) unsigned char dyn[];

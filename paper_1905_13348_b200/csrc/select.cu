@@ -556,10 +556,12 @@ select_kernel(DeviceCatalog c, uint32_t stage_bytes, uint32_t first, Queries q, 
 // own query to the end.  Nothing is staged or parked: with a few hundred queries per SM the copy of
 // the image costs more than the lookups, and the latency of the slow path is hidden by the other
 // warps' queries rather than by filling a warp with parked ones.
-// Up to 96 K queries, 192 K where the image would not be staged anyway.  Measured, us per launch back
-// to back, this kernel / the staging one: 64 tasks x 256 variants, 37 queries 2.9 / 3.7, 65,536: 4.1 /
-// 4.5, 131,072: 5.0 / 4.6; 128 x 512 (image in global memory), 131,072: 4.6 / 5.6, 262,144: 6.3 / 6.1;
-// 4 x 4096 on a trade-off surface, 20,011: 6.6 / 10.5, 262,144: 12.1 / 11.6.
+// Up to 96 K queries, 192 K where the image would not be staged anyway.  Measured, us per launch in a
+// graph of launches, this kernel / the staging one: 64 tasks x 256 variants, 37 queries 1.7 / 3.1, 32,768:
+// 4.0 / 4.1, 98,304: 4.4 / 4.2, 131,072: 4.6 / 4.3; a window of them (tallies and load update with it),
+// 16,384: 15.9 / 19.0, 65,536: 15.2 / 17.9, 98,304: 15.4 / 17.9; 128 x 512 (image in global memory),
+// 131,072: 4.7 / 5.2, 262,144: 5.8 / 5.3; 4 x 4096 on a trade-off surface, 20,011: 6.3 / 7.8, 262,144:
+// 11.7 / 9.8.
 constexpr uint32_t DIRECT_THREADS = 256;
 constexpr uint64_t DIRECT_MAX_N_STAGED = 96 * 1024, DIRECT_MAX_N_GLOBAL = 192 * 1024;
 
