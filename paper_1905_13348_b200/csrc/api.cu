@@ -267,7 +267,7 @@ int infaas_catalog_load(const infaas_variant *rows, uint32_t n_variants, uint32_
   const size_t o_id = carve((size_t)n_variants * 4), o_queued = carve((size_t)n_variants * 4);
   const size_t o_order = carve((size_t)n_variants * 4), o_cost_run = carve((size_t)n_variants * 4);
   const size_t o_class = carve((size_t)n_variants * 2), o_class_acc = carve((size_t)n_variants * 2);
-  const size_t o_n_class = carve((size_t)n_tasks * 4);
+  const size_t o_n_class = carve((size_t)n_tasks * 4), o_by_acc = carve((size_t)n_variants * 8);
   const size_t o_pred = carve((size_t)n_variants * 4), o_served = carve((size_t)n_variants * 8);
   const size_t o_count = carve((size_t)n_variants * 4);
   const size_t o_state = carve((size_t)n_variants), o_load_lat = carve((size_t)n_variants * 4);
@@ -329,6 +329,7 @@ int infaas_catalog_load(const infaas_variant *rows, uint32_t n_variants, uint32_
   d.s_class = reinterpret_cast<const uint16_t *>(base + o_class);
   d.class_acc = reinterpret_cast<const uint16_t *>(base + o_class_acc);
   d.n_class = reinterpret_cast<const uint32_t *>(base + o_n_class);
+  d.by_acc = reinterpret_cast<const uint2 *>(base + o_by_acc);
   d.s_queued = reinterpret_cast<uint32_t *>(base + o_queued);
   d.s_pred = reinterpret_cast<uint32_t *>(base + o_pred);
   d.s_served = reinterpret_cast<unsigned long long *>(base + o_served);
@@ -371,6 +372,7 @@ int infaas_catalog_load(const infaas_variant *rows, uint32_t n_variants, uint32_
     o.s_batch = const_cast<uint16_t *>(d.s_batch); o.s_acc = const_cast<uint16_t *>(d.s_acc);
     o.s_arch = c->s_arch; o.s_class = const_cast<uint16_t *>(d.s_class);
     o.class_acc = const_cast<uint16_t *>(d.class_acc);
+    o.by_acc = const_cast<uint2 *>(d.by_acc);
     o.s_qps = c->s_qps; o.hw_by_id = c->hw_by_id;
     LOAD_TRY(infaas::launch_layout(o, n_tasks, max_task, nullptr));
   }

@@ -172,7 +172,7 @@ inline __host__ __device__ uint32_t region_capacity(uint32_t V) { return round_u
 // id); task t owns slots task_off[t] .. task_off[t+1]-1 and all s_* arrays are indexed by slot.
 // A variant's local index is its slot less the task's first.  Cost and accuracy never change, so
 // everything about the list order that does not hang on the predicted latency is laid down here
-// once: s_order, s_cost_run, s_class and class_acc below.
+// once: s_order, s_cost_run, s_class, class_acc and by_acc below.
 // ---------------------------------------------------------------------------------------
 struct DeviceCatalog {
   uint32_t n_variants;
@@ -192,6 +192,8 @@ struct DeviceCatalog {
   const uint16_t *s_class;     // rank of the accuracy among the task's distinct ones, 0 = highest
   const uint16_t *class_acc;   // accuracy of class k of task t at [task_off[t] + k]
   const uint32_t *n_class;     // [n_tasks] distinct accuracies
+  const uint2 *by_acc;         // task t's variant at accuracy position p, at [task_off[t] + p]: x = its local index, y = bit
+                               // m (m < p % 32): the variant m places into p's 32 comes before it in local order too
   uint32_t *s_queued;
   uint32_t *s_pred;
   unsigned long long *s_served;
@@ -230,6 +232,7 @@ struct CatalogLayout {
   const uint32_t *members, *task_off;
   uint32_t *s_lat, *s_cost, *s_id, *s_queued, *s_order, *s_cost_run, *n_class, *slot_of_id;
   uint16_t *s_batch, *s_acc, *s_arch, *s_class, *class_acc;
+  uint2 *by_acc;
   unsigned long long *s_qps;
   unsigned char *hw_by_id;
 };
@@ -279,22 +282,36 @@ __device__ __forceinline__ uint4 load_once(const uint4 *p) {
                : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
   return v;
 }
+// Kernels without dynamic shared memory ask for the same split of an SM's L1 / shared memory, 32 KB of the
+// 228: a CTA only starts beside those of the previous kernel where the split suits it.  With the driver's own
+// choice the rebuild's CTAs (19 or 27 KB each) had to share the few SMs the selection's did not occupy: 64 CTAs on
+// 14 SMs, a window of 65,536 queries 17.6 us; with 64 KB or 100 KB the same, with 32 KB one CTA on each of 64
+// SMs, 13.4 us.
+constexpr uint32_t CARVEOUT_PCT = 14;
 template <class... P, class... A>
 inline cudaError_t launch_chained_cluster(void (*kernel)(P...), uint32_t grid, uint32_t cluster, uint32_t block, size_t smem,
                                           cudaStream_t stream, A... args) {
-  cudaLaunchAttribute attr[2] = {};
+  cudaLaunchAttribute attr[3] = {};
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
-  attr[1].id = cudaLaunchAttributeClusterDimension;
-  attr[1].val.clusterDim.x = cluster;
-  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+  uint32_t n = 1;
+  if (smem == 0) {
+    attr[n].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    attr[n++].val.sharedMemCarveout = CARVEOUT_PCT;
+  }
+  if (cluster > 1) {
+    attr[n].id = cudaLaunchAttributeClusterDimension;
+    attr[n].val.clusterDim.x = cluster;
+    attr[n].val.clusterDim.y = attr[n].val.clusterDim.z = 1;
+    ++n;
+  }
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(block);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
   cfg.attrs = attr;
-  cfg.numAttrs = cluster > 1 ? 2 : 1;
+  cfg.numAttrs = n;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 template <class... P, class... A>

@@ -89,6 +89,9 @@ layout_kernel(CatalogLayout o) {
       o.s_order[base + local] = p | head[local];
       o.s_class[base + local] = (uint16_t)k;
       if (fresh) o.class_acc[base + k] = (uint16_t)(10000u - (e >> 13));
+      uint32_t before_too = 0;
+      for (uint32_t q = p & ~31u; q < p; ++q) before_too |= (uint32_t)((by_acc[q] & 0x1FFFu) < local) << (q & 31u);
+      o.by_acc[base + p] = make_uint2(local, before_too);
     }
   }
   if (tid == 0u) o.n_class[t] = classes;

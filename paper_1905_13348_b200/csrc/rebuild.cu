@@ -29,23 +29,40 @@ constexpr uint32_t BITS_OF_2_POW_32 = 0x4F800000u;
 // of positions in accuracy order), one word of padding per row.
 constexpr uint32_t GRID = 64, GRID_PITCH = GRID + 1;
 
-// Shared memory used while building the index of one list segment.
+// Shared memory of a CTA of B threads while it builds the index of one list segment; NB: SLO buckets.
+template <uint32_t B, uint32_t NB>
 struct IndexScratch {
   uint32_t pred[256], ids[256];     // the segment in scan order; latencies behind its end are NONE
   uint32_t sorted[256];             // its latencies ascending (equal ones in scan order)
-  uint32_t ent[256];                // same order: accuracy rank << 16 | last of its latency << 8 | position
+  uint32_t ent[256];                // same order: accuracy rank << 24 | latency rank << 16 | last of its latency << 8 | position
   uint32_t Pd[256];                 // distinct latencies
-  uint32_t bcnt[MAX_BUCKETS];       // how many of them per SLO bucket
+  uint32_t bcnt[NB];                // how many of them per SLO bucket
   uint32_t wbits[MAX_ACC_WORDS];    // per bitmap word: the accuracies present
   // per latency rank: the most accurate entry (acc << 16 | 0xFFFF - position, 0 = none); per
   // accuracy rank: the fastest entry (its index in latency order, NONE = none)
   uint32_t rankA[256], rankB[256];
   uint16_t acc[256];
   unsigned char wpre[MAX_ACC_WORDS];         // accuracies present in the words before
-  unsigned char at[256], rank[256];          // sorted order: position, latency rank
+  unsigned char at[256];                     // sorted order: position
   unsigned char stair[256];                  // latency rank holds a stair entry
-  unsigned char part[REBUILD_WARPS * 32];    // rank table: first position per column of a run of entries
+  unsigned char part[B];                     // rank table: first position per column of a run of entries
   uint32_t ks, ka, base;
+
+  // Entry `pos` of the segment (its accuracy's bit too).
+  __device__ __forceinline__ void put(uint32_t pos, uint32_t latency, uint32_t accuracy, uint32_t id, uint32_t acc_lo) {
+    ids[pos] = id; pred[pos] = latency; acc[pos] = (uint16_t)accuracy;
+    const uint32_t x = accuracy - acc_lo, xw = x / ACC_WORD_BITS;
+    atomicOr(&wbits[xw], 1u << (x - xw * ACC_WORD_BITS));
+  }
+  // Clears what is accumulated into (all threads; a barrier must follow).
+  __device__ __forceinline__ void clear(uint32_t n_buckets, uint32_t nbw) {
+#pragma unroll 1
+    for (uint32_t i = threadIdx.x; i < 256u; i += B) { pred[i] = NONE; rankA[i] = 0u; rankB[i] = NONE; }
+#pragma unroll 1
+    for (uint32_t i = threadIdx.x; i < n_buckets; i += B) bcnt[i] = 0u;
+#pragma unroll 1
+    for (uint32_t i = threadIdx.x; i < nbw; i += B) wbits[i] = 0u;
+  }
 };
 
 // Fixed part of the image for a task without index (also entry n_tasks): a header word,
@@ -69,19 +86,13 @@ __device__ __forceinline__ void bucket_scale(const DeviceCatalog &c, uint32_t sl
   cap |= cap >> 1; cap |= cap >> 2; cap |= cap >> 4; cap |= cap >> 8; cap |= cap >> 16;
   const uint32_t clo = c.lat_code_lo;
   const uint32_t chi = max(clo, __float_as_uint(__uint2float_rz(cap)) >> 16);
-  uint32_t sh = 0;
+  // (a distance of 2^k spans at least 2^(k - sh) buckets: more than n_buckets below this start)
+  const int start = 31 - (int)__clz((chi - clo) | 1u) - (31 - (int)__clz(c.n_buckets));
+  uint32_t sh = (uint32_t)max(start, 0);
 #pragma unroll 1
   while ((chi >> sh) - (clo >> sh) > c.n_buckets - 2u) ++sh;
   bmin = clo >> sh;
   Sh = 16u + sh;
-}
-
-// Sum over the aligned group of 8 lanes this lane belongs to.
-__device__ __forceinline__ uint32_t group8_add(uint32_t v) {
-  v += __shfl_xor_sync(0xFFFFFFFFu, v, 1);
-  v += __shfl_xor_sync(0xFFFFFFFFu, v, 2);
-  v += __shfl_xor_sync(0xFFFFFFFFu, v, 4);
-  return v;
 }
 
 // Inclusive scans over the lanes of a warp.
@@ -130,182 +141,176 @@ __device__ __forceinline__ uint32_t place_block_finish(const DeviceCatalog &c, u
   return (uint32_t)old;
 }
 
-// Clears what build_index accumulates into (all threads; a barrier must follow).
-__device__ __forceinline__ void clear_scratch(IndexScratch &S, uint32_t n_buckets) {
-#pragma unroll 1
-  for (uint32_t i = threadIdx.x; i < 256u; i += REBUILD_THREADS) {
-    S.pred[i] = NONE; S.rankA[i] = 0u; S.rankB[i] = NONE; S.stair[i] = 0;
-  }
-#pragma unroll 1
-  for (uint32_t i = threadIdx.x; i < n_buckets; i += REBUILD_THREADS) S.bcnt[i] = 0u;
-#pragma unroll 1
-  for (uint32_t i = threadIdx.x; i < MAX_ACC_WORDS; i += REBUILD_THREADS) S.wbits[i] = 0u;
-}
-
 // Builds the exact index of a list segment of F <= INDEX_MAX_F entries (layout in common.cuh) into
-// a block of the image obtained from the block cursor.  S.pred / S.acc / S.ids hold the segment
-// in scan order, the accumulators are clear.  Returns false (all threads) if it cannot be
-// indexed: its block lies beyond the image's capacity or beyond what the header's offset field
-// addresses.
+// a block of the image obtained from the block cursor.  S holds the segment in scan order (S.put), the
+// other accumulators are clear.  Returns false (all threads) if it cannot be indexed: its block lies
+// beyond the image's capacity or beyond what the header's offset field addresses.
 // `xi`: NONE for the task's first segment (header word, SLO records and bitmap go into the
 // fixed part of the image), else the index of this further segment (header to xhdr[xi], bitmap
 // into the block, no records: only the slow path comes here).  `next`: 1 + index of the task's
 // next segment, 0 if this is the last.  `done`: the CTA's last allocation.
 //
-// The chain is bound by latency (barriers and shared-memory round trips), so it has few steps:
-// one pair loop (latency order), accuracy ranks straight from the bitmap, and the rank table as a
-// running minimum down its columns -- F steps per column, cut into runs of entries so that all
-// warps work, instead of F bits per cell.
-__device__ bool build_index(const DeviceCatalog &c, uint32_t t, uint32_t F, IndexScratch &S, uint32_t xi,
-                            uint32_t next, bool done, uint32_t Sh, uint32_t bmin) {
+// The chain is bound by latency (barriers and shared-memory round trips) and by the instructions of
+// the warps that have nothing to do in a step, so it has few steps (three barriers inside), no
+// division, and the block's place is asked for as early as its size is known (one atomic that all
+// CTAs send to the same word: 0.4 us): one pair loop (latency order), accuracy ranks straight from the
+// bitmap, and the rank table as a running minimum down its columns -- F steps per column, cut into
+// runs of entries so that all warps work, instead of F bits per cell.
+template <uint32_t B, uint32_t NB>
+__device__ __forceinline__ bool build_index(const DeviceCatalog &c, uint32_t t, uint32_t F, IndexScratch<B, NB> &S,
+                                            uint32_t xi, uint32_t next, bool done, uint32_t Sh, uint32_t bmin) {
+  constexpr uint32_t WARPS = B / 32u;
+  static_assert(B >= 256u && INDEX_MAX_F < 254u, "one thread per entry");
   const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
-  constexpr uint32_t B = REBUILD_THREADS;
   const bool first = xi == NONE;
   const uint32_t acc_lo = c.acc_lo, nbw = c.nbw;      // the catalog's accuracy window
 
   // 1. latency order: entry p comes behind the entries before it in the list that are not slower and
-  // those after it that are faster (latencies are at least 1).  8 lanes per entry, 4 entries per
-  // load; the accuracies' bits
-#pragma unroll 1
-  for (uint32_t p0 = 0; p0 < F; p0 += B / 8u) {        // uniform trip count
-    const uint32_t p = p0 + (tid >> 3), sub = tid & 7u, own = p & ~3u;
-    uint32_t cnt = 0, pp = 0;
-    if (p < F) {
-      pp = S.pred[p];
-#pragma unroll 2
-      for (uint32_t q = 4u * sub; q < F; q += 32u) {
-        const uint4 v = *reinterpret_cast<const uint4 *>(&S.pred[q]);
-        const uint32_t lim = pp - (uint32_t)(q >= own);
-        cnt += (uint32_t)(v.x <= lim) + (uint32_t)(v.y <= lim) + (uint32_t)(v.z <= lim) + (uint32_t)(v.w <= lim);
-      }
-      // equal latencies in front of p inside its own four
-      if (sub < (p & 3u)) cnt += S.pred[own + sub] == pp;
+  // those after it that are faster (latencies are at least 1).  1 << ls lanes per entry, 4 entries per load
+  uint32_t ls = 3;
+  while (ls && (F << ls) > B) --ls;
+  if ((32u * warp) >> ls < F) {
+    const uint32_t p = tid >> ls, sub = tid & ((1u << ls) - 1u), mine = min(p, F - 1u), own = mine & ~3u;
+    const uint32_t pp = S.pred[mine];
+    uint32_t cnt = 0;
+#pragma unroll 4
+    for (uint32_t q = 4u * sub; q < F; q += 4u << ls) {
+      const uint4 v = *reinterpret_cast<const uint4 *>(&S.pred[q]);
+      const uint32_t lim = pp - (uint32_t)(q >= own);
+      cnt += (uint32_t)(v.x <= lim) + (uint32_t)(v.y <= lim) + (uint32_t)(v.z <= lim) + (uint32_t)(v.w <= lim);
     }
-    cnt = group8_add(cnt);
+    if (sub == 0u) {                                   // equal latencies in front of p inside its own four
+      const uint4 v = *reinterpret_cast<const uint4 *>(&S.pred[own]);
+      const uint32_t e = mine & 3u;
+      cnt += (uint32_t)(e > 0u && v.x == pp) + (uint32_t)(e > 1u && v.y == pp) + (uint32_t)(e > 2u && v.z == pp);
+    }
+    __syncwarp();
+#pragma unroll 1
+    for (uint32_t o = 1u; o < (1u << ls); o <<= 1) cnt += __shfl_xor_sync(0xFFFFFFFFu, cnt, o);
     if (p < F && sub == 0u) {
       S.sorted[cnt] = pp;
       S.at[cnt] = (unsigned char)p;
-      const uint32_t x = S.acc[p] - acc_lo, xw = x / ACC_WORD_BITS;
-      atomicOr(&S.wbits[xw], 1u << (x - xw * ACC_WORD_BITS));
     }
+  }
+  // running popcounts of the accuracy bitmap, one word per thread (the last warps first: they have no
+  // entries); the bitmap itself, where its place is fixed
+  uint32_t *bitmap = reinterpret_cast<uint32_t *>(c.image + image_bitmap_offset(c.n_tasks, c.n_buckets) + t * bitmap_stride(nbw));
+#pragma unroll 1
+  for (uint32_t w0 = 32u * (WARPS - 1u - warp); w0 < nbw; w0 += B) {           // uniform per warp
+    uint32_t below = 0;
+#pragma unroll 4
+    for (uint32_t x = lane; x < w0; x += 32u) below += __popc(S.wbits[x]);
+    below = __reduce_add_sync(0xFFFFFFFFu, below);
+    const uint32_t w = w0 + lane, bits = w < nbw ? S.wbits[w] : 0u, pc = __popc(bits);
+    const uint32_t incl = below + warp_scan_add(pc);
+    if (w < nbw) {
+      S.wpre[w] = (unsigned char)(incl - pc);
+      if (first) bitmap[w] = ((incl - pc) << 24) | bits;
+    }
+    if (w == nbw - 1u) S.ka = incl;
   }
   __syncthreads();
 
-  // 2. dense latency ranks (warps 0-7, one sorted entry per thread), running popcounts of the
-  // accuracy bitmap (warps 8 and up, one word per thread)
-  if (warp < 8u) {
+  // 2. the block's place in the image (the atomic is in flight until step 3 ends; sized as if all
+  // latencies were distinct, which they nearly always are); dense latency ranks, accuracy ranks and the
+  // best entry per rank, one sorted entry per thread
+  const uint32_t Ka = S.ka, width = Ka + 1u, bytes = block_layout(F, F, Ka, first ? 0u : nbw).bytes;
+  unsigned long long placed = 0;
+  if (tid == B - 1u) placed = place_block_issue(c, bytes, done);
+  if (32u * warp < F) {
     const uint32_t i = tid;
     uint32_t before = 0;
 #pragma unroll 1
-    for (uint32_t w = 0; w < warp && 32u * w < F; ++w) {
-      const uint32_t x = 32u * w + lane;
-      before += __popc(__ballot_sync(0xFFFFFFFFu, x < F && (x == 0u || S.sorted[x] != S.sorted[x - 1u])));
-    }
-    const bool fresh = i < F && (i == 0u || S.sorted[i] != S.sorted[i - 1u]);
+    for (uint32_t x = lane; x < 32u * warp; x += 32u)
+      before += __popc(__ballot_sync(0xFFFFFFFFu, x == 0u || S.sorted[x] != S.sorted[x - 1u]));
+    const uint32_t v = S.sorted[i];                                                 // (behind F: not used)
+    const bool fresh = i < F && (i == 0u || v != S.sorted[i - 1u]);
     const unsigned m = __ballot_sync(0xFFFFFFFFu, fresh);
     if (i < F) {
       const uint32_t r = before + __popc(m & ((2u << lane) - 1u)) - 1u;
-      S.rank[i] = (unsigned char)r;
+      const uint32_t last = i == F - 1u || v != S.sorted[i + 1u];
       if (fresh) {
-        const uint32_t v = S.sorted[i];
         S.Pd[r] = v;
         // larger latencies than the largest SLO asked for so far share the last bucket
         atomicAdd(&S.bcnt[min(max(float_bits(v) >> Sh, bmin) - bmin, c.n_buckets - 1u)], 1u);
       }
+      const uint32_t p = S.at[i], acc = S.acc[p], x = acc - acc_lo, xw = x / ACC_WORD_BITS;
+      const uint32_t ra = S.wpre[xw] + __popc(S.wbits[xw] & ((1u << (x - xw * ACC_WORD_BITS)) - 1u));
+      S.ent[i] = (ra << 24) | (r << 16) | (last << 8) | p;
+      atomicMax(&S.rankA[r], (acc << 16) | (0xFFFFu - p));                          // most accurate, first position
+      atomicMin(&S.rankB[ra], i);                                                   // fastest, first position
       if (i == F - 1u) S.ks = r + 1u;
-    }
-  } else {
-#pragma unroll 1
-    for (uint32_t w0 = 32u * (warp - 8u); w0 < nbw; w0 += B - 256u) {     // uniform per warp
-      uint32_t below = 0;
-#pragma unroll 1
-      for (uint32_t x = lane; x < w0; x += 32u) below += __popc(S.wbits[x]);
-      below = __reduce_add_sync(0xFFFFFFFFu, below);
-      const uint32_t w = w0 + lane, pc = w < nbw ? __popc(S.wbits[w]) : 0u;
-      const uint32_t incl = below + warp_scan_add(pc);
-      if (w < nbw) S.wpre[w] = (unsigned char)(incl - pc);
-      if (w == nbw - 1u) S.ka = incl;
     }
   }
   __syncthreads();
-  const uint32_t Ks = S.ks, Ka = S.ka, width = Ka + 1u;
+  const uint32_t Ks = S.ks;
   const BlockLayout BL = block_layout(F, Ks, Ka, first ? 0u : nbw);
   const SlowLayout SL = slow_layout(F, Ks, Ka);
 
-  // 3. the block's place in the image (the atomic is in flight until step 4 ends); the sorted
-  // entries with their accuracy ranks, and the best entry per rank; SLO records
-  unsigned long long placed = 0;
-  if (tid == B - 1u) placed = place_block_issue(c, BL.bytes, done);
-  if (tid < F) {
-    const uint32_t p = S.at[tid], r = S.rank[tid], acc = S.acc[p];
-    const uint32_t x = acc - acc_lo, xw = x / ACC_WORD_BITS;
-    const uint32_t ra = S.wpre[xw] + __popc(S.wbits[xw] & ((1u << (x - xw * ACC_WORD_BITS)) - 1u));
-    const uint32_t last = tid == F - 1u || S.rank[tid + 1u] != r;
-    S.ent[tid] = (ra << 16) | (last << 8) | p;
-    atomicMax(&S.rankA[r], (acc << 16) | (0xFFFFu - p));                            // most accurate, first position
-    atomicMin(&S.rankB[ra], tid);                                                   // fastest, first position
-  }
-  if (first) {
-    // SLO records, 32 neighbouring buckets per warp and trip; below = latencies in lower buckets
-    const uint32_t nb = c.n_buckets;
-    uint32_t *rec = reinterpret_cast<uint32_t *>(c.image + image_rec_offset(c.n_tasks) + t * rec_stride(nb));
-#pragma unroll 1
-    for (uint32_t j = (tid + B / 2u) % B; j < nb; j += B) {        // (not the first warps: they are busy above)
-      uint32_t below = 0;
-#pragma unroll 4
-      for (uint32_t i = lane; i < (j & ~31u); i += 32u) below += S.bcnt[i];
-      below = __reduce_add_sync(0xFFFFFFFFu, below);
-      const uint32_t cnt = S.bcnt[j];
-      below += warp_scan_add(cnt) - cnt;
-      const uint32_t lo = j ? float_bits_floor((bmin + j) << Sh) : 0u;
-      const uint32_t nxt = (bmin + j + 1u) << Sh;
-      const uint32_t hi = (j == nb - 1u || nxt >= BITS_OF_2_POW_32) ? NONE : float_bits_floor(nxt) - 1u;
-      uint32_t r = ((Ks + 1u) << 24) | (cnt << 8) | below;          // exact slow path
-      if (cnt == 0u) {
-        r = below << 24;
-      } else if (cnt == 1u && (lo >> 24) == (hi >> 24)) {
-        const uint32_t thr = S.Pd[below];
-        r = thr <= lo ? (below + 1u) << 24 : (below << 24) | (0x00FFFFFFu - ((thr - 1u) & 0x00FFFFFFu));
-      }
-      rec[j] = r;
-      if (j == nb - 1u) rec[nb] = r;                               // what an SLO beyond the last bucket reads
-    }
-  }
-  __syncthreads();
-
-  // 4. rank table, first half.  T2[r][k] = smallest position among the entries whose latency rank
+  // 3. rank table, first half.  T2[r][k] = smallest position among the entries whose latency rank
   // is < r and whose accuracy rank is >= k: a running minimum over the entries in latency order.
   // A thread takes one column and one run of entries: here the run's minimum.
-  const uint32_t cols = (width + 31u) >> 5, runs = REBUILD_WARPS / cols;      // warps side by side; at least 4 runs
-  const uint32_t run_len = max(8u, ((F + runs - 1u) / runs + 3u) & ~3u);
-  const uint32_t run = warp / cols, col = (warp - run * cols) * 32u + lane;
-  const uint32_t i0 = min(F, run * run_len), i1 = run < runs ? min(F, i0 + run_len) : i0;
-  const uint32_t col_key = col << 16;
-  if (i0 < i1) {
+  const uint32_t cols = (width + 31u) >> 5, lc = cols > 1u ? 32u - __clz(cols - 1u) : 0u;   // warps side by side: 1 << lc
+  constexpr uint32_t LOG_WARPS = B == 256u ? 3u : B == 512u ? 4u : 5u;
+  static_assert(WARPS == 1u << LOG_WARPS, "log2 of the warps");
+  const uint32_t runs = WARPS >> lc, run_len = max(8u, (((F + runs - 1u) >> (LOG_WARPS - lc)) + 3u) & ~3u);
+  const uint32_t run = warp >> lc, colw = warp & ((1u << lc) - 1u), col = colw * 32u + lane;
+  const uint32_t i0 = min(F, run * run_len), i1 = colw < cols ? min(F, i0 + run_len) : i0;
+  const uint32_t col_key = col << 24;
+  if (i0 < i1 && i1 < F) {
     uint32_t v = 0xFFu;
 #pragma unroll 4
     for (uint32_t i = i0; i < i1; ++i) {
       const uint32_t e = S.ent[i];
       if (e >= col_key) v = min(v, e & 0xFFu);
     }
-    S.part[run * cols * 32u + col] = (unsigned char)v;
+    S.part[tid] = (unsigned char)v;
   }
   // stair entries: those more accurate than everything faster (one per latency at most); 32 latency
   // ranks per warp
+  const uint32_t ws = (warp + WARPS / 2u + 2u) & (WARPS - 1u);    // (not the warps with a run, nor the last)
   uint32_t best_a = 0;                                            // latency ranks < this thread's
-  if (32u * warp <= Ks) {
-    const uint32_t r = tid;
+  if (32u * ws <= Ks) {
+    const uint32_t r = 32u * ws + lane;
     uint32_t below = 0;
 #pragma unroll 1
-    for (uint32_t i = lane; i < 32u * warp; i += 32u) below = max(below, S.rankA[i]);
+    for (uint32_t i = lane; i < 32u * ws; i += 32u) below = max(below, S.rankA[i]);
     below = __reduce_max_sync(0xFFFFFFFFu, below);
     const uint32_t x = r < Ks ? S.rankA[r] : 0u;
     best_a = max(below, lanes_before(warp_scan_max(x), 0u));
     if (r < Ks) S.stair[r] = best_a == 0u || (x >> 16) > (best_a >> 16);
   }
+  if (first) {
+    // SLO records, 32 neighbouring buckets per warp and trip (the last warps first); below = latencies in
+    // lower buckets
+    const uint32_t nb = c.n_buckets;
+    uint32_t *rec = reinterpret_cast<uint32_t *>(c.image + image_rec_offset(c.n_tasks) + t * rec_stride(nb));
+#pragma unroll 1
+    for (uint32_t j0 = 32u * (WARPS - 1u - warp); j0 < nb; j0 += B) {
+      uint32_t below = 0;
+#pragma unroll 4
+      for (uint32_t i = lane; i < j0; i += 32u) below += S.bcnt[i];
+      below = __reduce_add_sync(0xFFFFFFFFu, below);
+      const uint32_t j = j0 + lane, cnt = S.bcnt[j];
+      below += warp_scan_add(cnt) - cnt;
+      uint32_t r = ((Ks + 1u) << 24) | (cnt << 8) | below;          // exact slow path
+      if (cnt == 0u) {
+        r = below << 24;
+      } else if (cnt == 1u) {
+        const uint32_t lo = j ? float_bits_floor((bmin + j) << Sh) : 0u;
+        const uint32_t nxt = (bmin + j + 1u) << Sh;
+        const uint32_t hi = (j == nb - 1u || nxt >= BITS_OF_2_POW_32) ? NONE : float_bits_floor(nxt) - 1u;
+        const uint32_t thr = S.Pd[below];
+        if ((lo >> 24) == (hi >> 24))
+          r = thr <= lo ? (below + 1u) << 24 : (below << 24) | (0x00FFFFFFu - ((thr - 1u) & 0x00FFFFFFu));
+      }
+      rec[j] = r;
+      if (j == nb - 1u) rec[nb] = r;                               // what an SLO beyond the last bucket reads
+    }
+  }
   if (tid == B - 1u) {
-    uint32_t base = image_var_offset(c.n_tasks, c.n_buckets, nbw) + place_block_finish(c, placed, BL.bytes, done);
-    if (base + BL.bytes > c.image_capacity || base + BL.t2 >= IMAGE_T2_LIMIT) base = NONE;
+    uint32_t base = image_var_offset(c.n_tasks, c.n_buckets, nbw) + place_block_finish(c, placed, bytes, done);
+    if (base + bytes > c.image_capacity || base + BL.t2 >= IMAGE_T2_LIMIT) base = NONE;
     S.base = base;
   }
   __syncthreads();
@@ -314,15 +319,15 @@ __device__ bool build_index(const DeviceCatalog &c, uint32_t t, uint32_t F, Inde
   unsigned char *blk = c.image + base;
   unsigned char *slow = blk + BL.slow;
 
-  // 5. rank table, second half: each run starts from the minimum of the runs before it and writes a
+  // 4. rank table, second half: each run starts from the minimum of the runs before it and writes a
   // row after the last entry of every latency
   unsigned char *T2 = blk + BL.t2;
   if (i0 < i1 && col < width) {
     uint32_t v = F;
 #pragma unroll 4
-    for (uint32_t w = 0; w < run; ++w) v = min(v, (uint32_t)S.part[w * cols * 32u + col]);
+    for (uint32_t w = 0; w < run; ++w) v = min(v, (uint32_t)S.part[(((w << lc) + colw) << 5) + lane]);
     if (run == 0u) T2[col] = (unsigned char)F;                   // nothing is fast enough
-    unsigned char *row = T2 + (S.rank[i0] + 1u) * width + col;
+    unsigned char *row = T2 + (((S.ent[i0] >> 16) & 0xFFu) + 1u) * width + col;
 #pragma unroll 4
     for (uint32_t i = i0; i < i1; ++i) {
       const uint32_t e = S.ent[i];
@@ -332,24 +337,14 @@ __device__ bool build_index(const DeviceCatalog &c, uint32_t t, uint32_t F, Inde
     if (i1 == F) { row[0] = (unsigned char)F; row[width] = (unsigned char)F; }   // rows Ks + 1, Ks + 2: the slow path's
   }
 
-  // the small tables, each by a range of warps of its own: [lo, lo + n) of the CTA's threads run
-  // `body(x)` for x = 0 .. count - 1
-  auto share = [&](uint32_t lo, uint32_t n, uint32_t count, auto body) {
-    if (tid >= lo && tid < lo + n)
-#pragma unroll 1
-      for (uint32_t x = tid - lo; x < count; x += n) body(x);
-  };
-  uint32_t *bitmap = first ? reinterpret_cast<uint32_t *>(c.image + image_bitmap_offset(c.n_tasks, c.n_buckets) + t * bitmap_stride(nbw))
-                           : reinterpret_cast<uint32_t *>(blk + BL.bitmap);
-  share(0, B / 4u, nbw, [&](uint32_t w) { bitmap[w] = ((uint32_t)S.wpre[w] << 24) | S.wbits[w]; });
-  // what the nearest-miss search reads: bestA[r] over latency ranks < r, the stair entries in
-  // ascending latency, ordStart[r] = stair entries with latency rank < r (the warps of step 4);
-  // position 0xFF stands for "none"
-  if (32u * warp <= Ks) {
-    const uint32_t r = tid;
+  // the small tables.  What the nearest-miss search reads: bestA[r] over latency ranks < r, the stair
+  // entries in ascending latency, ordStart[r] = stair entries with latency rank < r (the warps of step
+  // 3); position 0xFF stands for "none"
+  if (32u * ws <= Ks) {
+    const uint32_t r = 32u * ws + lane;
     uint32_t before = 0;
 #pragma unroll 1
-    for (uint32_t i = lane; i < 32u * warp; i += 32u) before += __popc(__ballot_sync(0xFFFFFFFFu, S.stair[i]));
+    for (uint32_t i = lane; i < 32u * ws; i += 32u) before += __popc(__ballot_sync(0xFFFFFFFFu, S.stair[i]));
     const bool st = r < Ks && S.stair[r];
     const uint32_t o = before + __popc(__ballot_sync(0xFFFFFFFFu, st) & ((1u << lane) - 1u));
     if (r <= Ks) {
@@ -365,8 +360,9 @@ __device__ bool build_index(const DeviceCatalog &c, uint32_t t, uint32_t F, Inde
       c.slow[first ? t : c.n_tasks + xi] = make_uint4(base + BL.slow, F | (Ks << 8) | (Ka << 16), 0u, o | (next << 8));
   }
   // bestB[k] over accuracy ranks >= k, 32 ranks from the top down per warp
-  if (warp >= 8u && warp < 16u && 32u * (warp - 8u) <= Ka) {
-    const uint32_t q0 = 32u * (warp - 8u), q = q0 + lane;        // q-th value of bestB from the top; bestB[Ka] is none
+  const uint32_t wb = (warp + WARPS / 2u) & (WARPS - 1u);
+  if (32u * wb <= Ka) {
+    const uint32_t q0 = 32u * wb, q = q0 + lane;                  // q-th value of bestB from the top; bestB[Ka] is none
     uint32_t above = NONE;
 #pragma unroll 1
     for (uint32_t i = lane; i < q0; i += 32u) above = min(above, S.rankB[Ka - 1u - i]);
@@ -376,11 +372,12 @@ __device__ bool build_index(const DeviceCatalog &c, uint32_t t, uint32_t F, Inde
       reinterpret_cast<uint2 *>(slow + SL.bestB)[Ka - q] = i == NONE ? make_uint2(0u, 0xFFu) : make_uint2(S.sorted[i], S.at[i]);
   }
   uint32_t *ids_end = reinterpret_cast<uint32_t *>(blk + BL.t2);   // ids, reversed; slot F holds PENDING
-  uint32_t *Pd_g = reinterpret_cast<uint32_t *>(slow + SL.Pd);
-  share(3u * B / 4u, B / 4u, F + 1u, [&](uint32_t p) {
-    ids_end[-1 - (int)p] = p < F ? S.ids[p] : PENDING;
-    if (p < Ks) Pd_g[p] = S.Pd[p];
-  });
+  const uint32_t p = (tid + 256u) & (B - 1u);                      // (the last 256 threads)
+  if (p <= F) ids_end[-1 - (int)p] = p < F ? S.ids[p] : PENDING;
+  if (p < Ks) reinterpret_cast<uint32_t *>(slow + SL.Pd)[p] = S.Pd[p];
+  if (!first)
+#pragma unroll 1
+    for (uint32_t w = tid; w < nbw; w += B) reinterpret_cast<uint32_t *>(blk + BL.bitmap)[w] = ((uint32_t)S.wpre[w] << 24) | S.wbits[w];
   if (tid == 0u) {
     if (first) reinterpret_cast<uint32_t *>(c.image + IMAGE_HDR_OFFSET)[t] = (base + BL.t2) | (width << 24);
     else c.xhdr[xi] = make_uint4(base + BL.t2, width, base + BL.bitmap, 0u);
@@ -461,7 +458,8 @@ __device__ __forceinline__ uint32_t advance_row(const DeviceCatalog &c, uint32_t
 // pred; at most the fastest variant (lowest id) of every distinct accuracy is on it, if it is
 // faster than everything more accurate, and the list runs from the lowest accuracy up.
 __device__ __forceinline__ uint32_t build_list(const DeviceCatalog &c, uint32_t t, bool advance, uint32_t window_us,
-                                               unsigned char *dyn, IndexScratch &S, uint32_t &slo_seen) {
+                                               unsigned char *dyn,
+                                               IndexScratch<REBUILD_THREADS, MAX_BUCKETS> &S, uint32_t &slo_seen) {
   constexpr uint32_t KEEP_WORDS = INFAAS_MAX_TASK_VARIANTS / 32;
   __shared__ uint32_t grid[GRID * GRID_PITCH];
   __shared__ uint32_t keep[KEEP_WORDS + 1], keep_pre[KEEP_WORDS + 1];   // bit sets: survivors, by local index ...
@@ -486,6 +484,7 @@ __device__ __forceinline__ uint32_t build_list(const DeviceCatalog &c, uint32_t 
   // 1. queue recursion, states, predicted latencies; coarse grid.  Each thread's first variant
   // stays in registers.  Before chain_wait: only what no kernel writes, and clearing.
   Row r0;
+  r0.drain = 0;
   uint32_t acc0 = 0, run0 = 0, class0 = 0, pred0 = 0;
   if (tid < V) {
     r0 = load_fixed(c, base + tid, window_us);
@@ -503,9 +502,10 @@ __device__ __forceinline__ uint32_t build_list(const DeviceCatalog &c, uint32_t 
   for (uint32_t i = tid; i < V; i += B) run_min[i] = NONE;
 #pragma unroll 1
   for (uint32_t i = tid; i <= KEEP_WORDS; i += B) { keep[i] = 0u; if (i < KEEP_WORDS) passed_acc[i] = 0u; }
-  clear_scratch(S, c.n_buckets);
+  S.clear(c.n_buckets, c.nbw);
   if (tid == 0u) { n_cand = 0u; n_inactive = 0u; }
   __syncthreads();
+  asm volatile("" : "+r"(r0.drain));                               // (else the compiler moves the division behind the wait)
   chain_wait();
   chain_next();
   slo_seen = *c.slo_seen;                                          // wanted by the index, requested early
@@ -637,7 +637,7 @@ __device__ __forceinline__ uint32_t build_list(const DeviceCatalog &c, uint32_t 
   auto emit = [&](uint32_t pos, uint32_t pred, uint32_t acc, uint32_t id) {
     keys_g[pos] = ((unsigned long long)acc << 32) | pred;
     ids_g[pos] = id;
-    if (pos < INDEX_MAX_F) { S.ids[pos] = id; S.pred[pos] = pred; S.acc[pos] = (uint16_t)acc; }
+    if (pos < INDEX_MAX_F) S.put(pos, pred, acc, id, c.acc_lo);
   };
   auto before = [&](uint32_t i) { return keep_pre[i >> 5] + __popc(keep[i >> 5] & ((1u << (i & 31u)) - 1u)); };
 #pragma unroll 1
@@ -730,63 +730,31 @@ __device__ __forceinline__ uint32_t build_list(const DeviceCatalog &c, uint32_t 
   return F;
 }
 
-// c.rebuild_ctas CTAs per task, a cluster: the first one makes the list, then each takes its share of
-// the list's segments.
-//
-// Bound by the latency of its chain of barriers and shared-memory round trips, and by fetching its
-// code: every line of it runs about once per launch, and with the compiler's unrolling (116 KB of
-// code) 40 % of the stalls were for instructions.  So the loops are not unrolled (50 KB) except the
-// few that run long.  Measured on one B200, in GPU clock cycles after the previous kernel's end: 64
-// tasks x 256 variants, lists of up to 100 entries: 16 K (18 K unrolled), 128 x 512: 19 K (22 K), 4 x
-// 4096 on a trade-off surface, lists of up to 505 entries, with one CTA per task: 77 K (90 K), two lists: 17 K
-// (23 K).  512 threads instead of 1024: short lists 5 % faster, lists of 100 entries 5 % slower.
-// The segments of a list of several hundred entries take as long as the list itself, so tasks of more
-// than 1024 variants have 4 CTAs (rule in infaas_catalog_load): 48 us a window instead of 63 on the
-// trade-off surface, 4 x 4096.
-__global__ void __launch_bounds__(REBUILD_THREADS)
-rebuild_kernel(DeviceCatalog c, int advance, uint32_t window_us) {
-  extern __shared__ __align__(16) unsigned char dyn[];
-  __shared__ __align__(16) IndexScratch S;
-  const uint32_t K = c.rebuild_ctas, t = blockIdx.x >> (K >> 1), share = blockIdx.x & (K - 1u), tid = threadIdx.x;   // K = 1 or 4
-  constexpr uint32_t B = REBUILD_THREADS;
-  uint32_t F = 0, slo_seen;
-  if (share == 0u) {
-    F = build_list(c, t, advance, window_us, dyn, S, slo_seen);
-    if (tid == 0u) c.f_len[t] = F;
-  } else {
-    chain_wait();
-    chain_next();
-    slo_seen = *c.slo_seen;
-  }
-  uint32_t bmin, Sh;                                               // SLO buckets
-  bucket_scale(c, slo_seen, Sh, bmin);
-  if (K > 1u) {                                                    // the list is in the region
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-    F = *reinterpret_cast<volatile uint32_t *>(c.f_len + t);
-  }
+// Index of a task's list, segment by segment (INDEX_MAX_F positions each; almost always one); of K CTAs
+// the one numbered `share` takes every K-th.  The two lists of a state-aware catalog count as one, the
+// Inactive entries behind the Active ones: "first position that meets both requirements, else the
+// smallest distance at the lowest position" is all the index knows about order.  Returns false if
+// there is no index (empty list, or no room).
+template <uint32_t B, uint32_t NB>
+__device__ __forceinline__ bool index_list(const DeviceCatalog &c, uint32_t t, uint32_t F, IndexScratch<B, NB> &S, uint32_t share,
+                                           uint32_t K, uint32_t Sh, uint32_t bmin) {
   bool indexed = F > 0;
   bool counted = false;                       // has this CTA made its last allocation?
-  // index the list -- the two lists of a state-aware catalog count as one, the Inactive entries
-  // behind the Active ones: "first position that meets both requirements, else the smallest
-  // distance at the lowest position" is all the index knows about order -- segment by segment
-  // (INDEX_MAX_F positions each; almost always one)
   if (indexed) {
-    const uint32_t nseg = (F + INDEX_MAX_F - 1u) / INDEX_MAX_F, x0 = c.seg_base[t];
+    const uint32_t nseg = (F + INDEX_MAX_F - 1u) / INDEX_MAX_F;
 #pragma unroll 1
     for (uint32_t sg = share; sg < nseg && indexed; sg += K) {
-      const uint32_t off = sg * INDEX_MAX_F, Fseg = min(INDEX_MAX_F, F - off);
+      const uint32_t off = sg * INDEX_MAX_F, Fseg = min(INDEX_MAX_F, F - off), x0 = nseg > 1u ? c.seg_base[t] : 0u;
       if (sg) {                                   // later segments: back from the task's region
         const unsigned char *region = c.regions + c.reg_off[t];
         const unsigned long long *keys_g = reinterpret_cast<const unsigned long long *>(region);
         const uint32_t *ids_g = reinterpret_cast<const uint32_t *>(region + 8u * (c.task_off[t + 1] - c.task_off[t]));
         __syncthreads();
-        clear_scratch(S, c.n_buckets);
+        S.clear(c.n_buckets, c.nbw);
         __syncthreads();
-#pragma unroll 1
-        for (uint32_t i = tid; i < Fseg; i += B) {
-          const unsigned long long e = keys_g[off + i];
-          S.ids[i] = ids_g[off + i]; S.pred[i] = (uint32_t)e; S.acc[i] = (uint16_t)(e >> 32);
+        if (threadIdx.x < Fseg) {
+          const unsigned long long e = keys_g[off + threadIdx.x];
+          S.put(threadIdx.x, (uint32_t)e, (uint32_t)(e >> 32), ids_g[off + threadIdx.x], c.acc_lo);
         }
         __syncthreads();
       }
@@ -794,8 +762,14 @@ rebuild_kernel(DeviceCatalog c, int advance, uint32_t window_us) {
       counted = sg + K >= nseg;
     }
   }
-  if (!counted && tid == 0u) place_block_finish(c, place_block_issue(c, 0u, true), 0u, true);   // nothing (more) to place
-  if (share) return;
+  if (!counted && threadIdx.x == 0u) place_block_finish(c, place_block_issue(c, 0u, true), 0u, true);   // nothing (more) to place
+  return indexed;
+}
+
+// What is left to write once a task's list is indexed, or is not (one CTA per task).
+__device__ __forceinline__ void finish_task(const DeviceCatalog &c, uint32_t t, uint32_t F, bool indexed, bool advance, uint32_t Sh,
+                                            uint32_t bmin) {
+  const uint32_t tid = threadIdx.x;
   if (!indexed) {
     // no index: every query of this task reads "none"
     write_dummy_task(c, t);
@@ -815,8 +789,253 @@ rebuild_kernel(DeviceCatalog c, int advance, uint32_t window_us) {
   }
 }
 
-// The block sizes the thread ranges above rely on.
-static_assert(REBUILD_THREADS >= 512 && INDEX_MAX_F < 254, "thread ranges of build_index");
+// Tasks of more than 512 variants: c.rebuild_ctas CTAs per task, a cluster; the first one makes the list, then
+// each takes its share of the list's segments.
+//
+// Bound by the latency of its chain of barriers and shared-memory round trips, and by fetching its
+// code: every line of it runs about once per launch, and with the compiler's unrolling (116 KB of
+// code) 40 % of the stalls were for instructions.  So the loops are not unrolled (50 KB) except the
+// few that run long.  The segments of a list of several hundred entries take as long as the list
+// itself, so tasks of more than 1024 variants have 4 CTAs (rule in infaas_catalog_load): 48 us a window
+// instead of 63 on the trade-off surface, 4 x 4096.
+__global__ void __launch_bounds__(REBUILD_THREADS)
+rebuild_kernel(DeviceCatalog c, int advance, uint32_t window_us) {
+  extern __shared__ __align__(16) unsigned char dyn[];
+  __shared__ __align__(16) IndexScratch<REBUILD_THREADS, MAX_BUCKETS> S;
+  const uint32_t K = c.rebuild_ctas, t = blockIdx.x >> (K >> 1), share = blockIdx.x & (K - 1u);   // K = 1 or 4
+  uint32_t F = 0, slo_seen;
+  if (share == 0u) {
+    F = build_list(c, t, advance, window_us, dyn, S, slo_seen);
+    if (threadIdx.x == 0u) c.f_len[t] = F;
+  } else {
+    chain_wait();
+    chain_next();
+    slo_seen = *c.slo_seen;
+  }
+  uint32_t bmin, Sh;                                               // SLO buckets
+  bucket_scale(c, slo_seen, Sh, bmin);
+  if (K > 1u) {                                                    // the list is in the region
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    F = *reinterpret_cast<volatile uint32_t *>(c.f_len + t);
+  }
+  const bool indexed = index_list(c, t, F, S, share, K, Sh, bmin);
+  if (share == 0u) finish_task(c, t, F, indexed, advance, Sh, bmin);
+}
+
+// Queue recursion, prune and list of one task of at most B variants, one per thread; otherwise as
+// build_list.  Contains chain_wait.  Returns the list's length.
+//
+// List of the Active variants: p is dominated by a faster variant of the same cost and accuracy, or by
+// a variant q before it in both orders (local, accuracy) with pred_q <= pred_p.  Both orders are fixed, so
+// everything about them is known before the wait.  Warp g owns the 32 variants at accuracy positions
+// 32 g .. 32 g + 31.  Those q in lower groups come before all of its own in accuracy order: a running
+// minimum over their latencies in local order (B / 32 consecutive variants per lane, then one warp
+// scan) answers for them.  Those inside the group are compared directly, against a bit mask of which
+// of them come before in both orders (laid down with the catalog).  No list of candidates, one barrier.
+//
+// List of the Inactive variants: the fastest (lowest id) of every accuracy class, if it is faster than
+// everything more accurate, from the lowest accuracy up; one warp goes through the classes while the
+// others place the Active ones.
+template <uint32_t B>
+__device__ __forceinline__ uint32_t build_list_small(const DeviceCatalog &c, uint32_t t, bool advance, uint32_t window_us,
+                                                     IndexScratch<B, B> &S, uint32_t &Sh, uint32_t &bmin) {
+  constexpr uint32_t GROUPS = B / 32u, E = B / 32u;                // E: consecutive variants (or classes) per lane
+  static_assert(GROUPS < 32u, "a lane per word of a bit set, and one behind them");
+  // Where element i is in an array of which each lane reads E consecutive elements: lane l's j-th at j * PITCH + l,
+  // without bank conflicts for readers (j fixed) and for writers (32 consecutive i).
+  constexpr uint32_t PITCH = 32u + 32u / E;
+  auto at = [](uint32_t i) { return (i % E) * PITCH + i / E; };
+  // latencies as the prune compares them: NONE = not listed, so a saturated one counts as one less
+  __shared__ uint32_t by_lane[E * PITCH];                          // by local index (laid out by `at`)
+  __shared__ __align__(16) uint32_t by_pos[B];                  // ... by accuracy position
+  __shared__ uint32_t run_min[B];                               // at the first of each (cost, accuracy): smallest pred
+  __shared__ uint16_t pos_of[B];                                // accuracy position of each local index
+  __shared__ uint32_t listed[GROUPS], dominated[GROUPS], spared[GROUPS];   // bit sets by local index
+  __shared__ uint32_t class_eff[E * PITCH], class_id[E * PITCH];   // per accuracy class: smallest latency, lowest id with it
+  __shared__ uint16_t class_acc[E * PITCH];
+  __shared__ uint32_t n_inactive;
+  const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+  const uint32_t base = c.task_off[t], V = c.task_off[t + 1] - base;
+  const bool live = tid < V;
+  unsigned char *region = c.regions + c.reg_off[t];
+  unsigned long long *keys_g = reinterpret_cast<unsigned long long *>(region);
+  uint32_t *ids_g = reinterpret_cast<uint32_t *>(region + 8u * V);
+
+  // 1. before the wait: what no kernel writes, and clearing
+  Row r;
+  r.drain = 0;
+  uint32_t acc = 0, run = 0, cls = 0, pos = 0xFFFFu;
+  uint2 own = make_uint2(0u, 0u);                                  // local index at accuracy position tid, mask of its group
+  if (live) {
+    r = load_fixed(c, base + tid, window_us);
+    acc = c.s_acc[base + tid];
+    run = c.s_cost_run[base + tid];
+    own = c.by_acc[base + tid];
+    pos = r.order & 0x1FFFu;
+    if (c.stateful) cls = c.s_class[base + tid];
+  }
+  pos_of[tid] = (uint16_t)pos;
+  by_lane[at(tid)] = NONE;
+  by_pos[tid] = NONE;
+  run_min[tid] = NONE;
+  if (tid < GROUPS) { dominated[tid] = 0u; spared[tid] = 0u; }
+  if (c.stateful) {
+    class_eff[at(tid)] = NONE; class_id[at(tid)] = NONE;
+    if (live) class_acc[at(cls)] = (uint16_t)acc;
+  }
+  if (tid == 0u) n_inactive = 0u;
+  S.clear(c.n_buckets, c.nbw);
+  __syncthreads();
+  // this lane's E variants: which belong to lower groups, which to this warp's
+  uint32_t lower = 0, same = 0;
+#pragma unroll
+  for (uint32_t j = 0; j < E; ++j) {
+    const uint32_t g = pos_of[lane * E + j] >> 5;
+    lower |= (uint32_t)(g < warp) << j;
+    same |= (uint32_t)(g == warp) << j;
+  }
+  // (the compiler would move the division and the masks behind the wait, to their use: 1000 cycles)
+  asm volatile("" : "+r"(r.drain), "+r"(lower), "+r"(same));
+  chain_wait();
+  chain_next();
+  const uint32_t slo_seen = *c.slo_seen;
+  // 2. queue recursion, states, predicted latencies
+  uint32_t pred = NONE, eff = NONE;
+  bool active = false, inactive = false;
+  if (live) {
+    load_load(c, base + tid, advance, r);
+    pred = advance_row(c, base + tid, r, advance);
+    active = r.state == INFAAS_STATE_ACTIVE;
+    inactive = r.state == INFAAS_STATE_INACTIVE;
+    if (active) {
+      by_lane[at(tid)] = by_pos[pos] = min(pred, NONE - 1u);
+      if (r.order >> 31) atomicMin(&run_min[(r.order >> 13) & 0x1FFFu], pred);
+    }
+    if (inactive) {
+      const unsigned long long e = (unsigned long long)pred + r.load_lat;
+      eff = e > NONE ? NONE : (uint32_t)e;
+      atomicMin(&class_eff[at(cls)], eff);
+    }
+  }
+  const unsigned m = __ballot_sync(0xFFFFFFFFu, active);
+  if (lane == 0u) listed[warp] = m;
+  bucket_scale(c, slo_seen, Sh, bmin);
+  __syncthreads();
+  // 3. prune
+  if (32u * warp < V) {
+    uint32_t x[E], least = NONE;
+#pragma unroll
+    for (uint32_t j = 0; j < E; ++j) {
+      x[j] = by_lane[j * PITCH + lane];
+      least = min(least, (lower >> j) & 1u ? x[j] : NONE);
+    }
+    least = lanes_before(warp_scan_min(least), NONE);
+    uint32_t dom = 0;
+#pragma unroll
+    for (uint32_t j = 0; j < E; ++j) {
+      dom |= (uint32_t)(((same >> j) & 1u) && least <= x[j]) << j;
+      least = min(least, (lower >> j) & 1u ? x[j] : NONE);
+    }
+    if (dom) atomicOr(&dominated[(lane * E) >> 5], dom << ((lane * E) & 31u));
+  }
+  if (live) {                                                      // the variant at accuracy position tid
+    const uint32_t p = by_pos[tid], o = own.x;
+    uint32_t le = 0;
+#pragma unroll
+    for (uint32_t j = 0; j < 8u; ++j) {
+      const uint4 v = *reinterpret_cast<const uint4 *>(&by_pos[32u * warp + 4u * j]);
+      le |= (uint32_t)(v.x <= p) << (4u * j) | (uint32_t)(v.y <= p) << (4u * j + 1u) | (uint32_t)(v.z <= p) << (4u * j + 2u) |
+            (uint32_t)(v.w <= p) << (4u * j + 3u);
+    }
+    if (le & own.y) atomicOr(&dominated[o >> 5], 1u << (o & 31u));   // (one that is not listed: no harm)
+  }
+  const bool slower_twin = active && (r.order >> 31) && pred > run_min[(r.order >> 13) & 0x1FFFu];
+  if (slower_twin) atomicOr(&dominated[warp], 1u << lane);
+  if (active && pred == NONE - 1u && !slower_twin) {               // saturated ones looked as fast: look again
+    bool dom = false;
+#pragma unroll 1
+    for (uint32_t q = 0; q < tid && !dom; ++q)
+      dom = ((listed[q >> 5] >> (q & 31u)) & 1u) && pos_of[q] < pos && c.s_pred[base + q] <= pred;
+    if (!dom) atomicOr(&spared[warp], 1u << lane);
+  }
+  if (inactive && class_eff[at(cls)] == eff) atomicMin(&class_id[at(cls)], r.id);
+  __syncthreads();
+  // 4. the list into the task's region, its first segment also into the index scratch.  Positions:
+  // survivors before the run of equal cost, then the run backwards
+  const uint32_t kept = lane < GROUPS ? listed[lane] & (~dominated[lane] | spared[lane]) : 0u, n_kept = __popc(kept);
+  const uint32_t before_word = warp_scan_add(n_kept) - n_kept;
+  const uint32_t n_active = __shfl_sync(0xFFFFFFFFu, before_word + n_kept, 31);
+  auto before = [&](uint32_t i) {                                  // survivors before local index i <= B (all lanes)
+    const int w = (int)(i >> 5);                                   // (word GROUPS is empty)
+    return __shfl_sync(0xFFFFFFFFu, before_word, w) + __popc(__shfl_sync(0xFFFFFFFFu, kept, w) & ((1u << (i & 31u)) - 1u));
+  };
+  auto emit = [&](uint32_t at_pos, uint32_t latency, uint32_t accuracy, uint32_t id) {
+    keys_g[at_pos] = ((unsigned long long)accuracy << 32) | latency;
+    ids_g[at_pos] = id;
+    if (at_pos < INDEX_MAX_F) S.put(at_pos, latency, accuracy, id, c.acc_lo);
+  };
+  const uint32_t list_pos = before(run & 0xFFFFu) + before(run >> 16) - 1u - before(tid);
+  const uint32_t own_word = __shfl_sync(0xFFFFFFFFu, kept, (int)warp);
+  if ((own_word >> lane) & 1u) emit(list_pos, pred, acc, r.id);
+  // the counts are cleared here, far behind their loads: a store to a line whose load is still in flight
+  // holds up everything behind it
+  if (advance && live) c.count_by_id[r.id] = 0u;
+  if (c.stateful && warp == GROUPS - 1u) {
+    // E classes per lane, from the highest accuracy down: those with an entry, their running minimum,
+    // survivors, their number
+    uint32_t x[E], some = 0, least = NONE;
+#pragma unroll
+    for (uint32_t j = 0; j < E; ++j) {
+      x[j] = class_eff[j * PITCH + lane];
+      some |= (uint32_t)(class_id[j * PITCH + lane] != NONE) << j;
+      least = min(least, x[j]);                                    // (NONE in a class without entry)
+    }
+    least = lanes_before(warp_scan_min(least), NONE);
+    bool first = !(__ballot_sync(0xFFFFFFFFu, some != 0u) & ((1u << lane) - 1u));   // none before this lane's
+    // on the list: faster than every more accurate variant (equally fast ones are dominated)
+    uint32_t on = 0;
+#pragma unroll
+    for (uint32_t j = 0; j < E; ++j) {
+      const bool here = (some >> j) & 1u;
+      on |= (uint32_t)(here && (first || x[j] < least)) << j;
+      least = min(least, x[j]);
+      first = first && !here;
+    }
+    const uint32_t n = __popc(on), incl = warp_scan_add(n), total = __shfl_sync(0xFFFFFFFFu, incl, 31);
+    uint32_t slot = n_active + total - 1u - (incl - n);
+#pragma unroll 1
+    for (; on; on &= on - 1u) {
+      const uint32_t k = ((uint32_t)__ffs(on) - 1u) * PITCH + lane;
+      emit(slot--, class_eff[k], class_acc[k], class_id[k]);
+    }
+    if (lane == 0u) n_inactive = total;
+  }
+  __syncthreads();
+  return n_active + n_inactive;
+}
+
+// Tasks of at most B variants: one CTA of B threads per task, a thread per variant (B = 256 or 512).
+//
+// Bound by the latency of its chain: the loads after the wait (1.7 K cycles, of which the gather of
+// counts that other SMs' atomics have just written is half), seven barriers with a few shared-memory round trips each,
+// and the instructions of every warp.  Cycles after the wait, 64 tasks x 256 variants with lists of up to 100
+// entries, this kernel / rebuild_kernel with its 1024 threads: 11.2 K / 16.6 K; lists of up to 50: 9.7 K /
+// 16.4 K; 128 x 512, up to 134: 14.3 K / 19.6 K; two lists per task: 10.5 K / 16.7 K.  A window of 65,536
+// queries: 15.3 -> 13.4 us (64 x 256), 16.2 -> 15.2 (128 x 512).  512 threads for tasks of up to 256: the
+// steps with work for few warps 30 % faster, the rank table slower, the sum the same.
+template <uint32_t B>
+__global__ void __launch_bounds__(B)
+rebuild_small_kernel(DeviceCatalog c, int advance, uint32_t window_us) {
+  __shared__ __align__(16) IndexScratch<B, B> S;
+  const uint32_t t = blockIdx.x;
+  uint32_t Sh, bmin;
+  const uint32_t F = build_list_small<B>(c, t, advance, window_us, S, Sh, bmin);
+  if (threadIdx.x == 0u) c.f_len[t] = F;
+  const bool indexed = index_list(c, t, F, S, 0u, 1u, Sh, bmin);
+  finish_task(c, t, F, indexed, advance, Sh, bmin);
+}
+
 static_assert(REBUILD_CLUSTER == 4, "task and share from the CTA's index in rebuild_kernel");
 
 }  // namespace
@@ -845,6 +1064,10 @@ cudaError_t rebuild_clusters_at_once(uint32_t max_task_variants, uint32_t *n) {
 
 cudaError_t launch_rebuild(const DeviceCatalog &c, bool advance_queues, uint32_t window_us,
                            cudaStream_t stream) {
+  // a thread per variant up to 512 (as fast as it gets with registers and bit masks), beyond that in rounds
+  if (c.max_task_variants <= 512u)
+    return launch_chained(c.max_task_variants <= 256u ? rebuild_small_kernel<256> : rebuild_small_kernel<512>, c.n_tasks,
+                          c.max_task_variants <= 256u ? 256u : 512u, 0, stream, c, advance_queues ? 1 : 0, window_us);
   const size_t smem = (size_t)c.max_task_variants * REBUILD_ROW_SMEM;
   return launch_chained_cluster(rebuild_kernel, c.n_tasks * c.rebuild_ctas, c.rebuild_ctas, REBUILD_THREADS, smem, stream, c,
                                 advance_queues ? 1 : 0, window_us);

@@ -71,6 +71,18 @@ def test_two_lists_at_the_edges(V, kind):
     run_stateful(w, _states(rng, w.n_variants, (0.45, 0.45, 0.05, 0.05)), load)
 
 
+# A thread per variant up to 256 and up to 512 variants per task: the sizes on either side, lists of one and of
+# two segments (248 entries), equal costs and accuracies across the groups of 32, both kinds of catalog
+@pytest.mark.parametrize("kind", ["ties", "saturated", "tradeoff"])
+@pytest.mark.parametrize("V", [32, 248, 249, 256, 511, 513])
+def test_a_thread_per_variant(V, kind):
+    w = _workload(V, kind)
+    run_both(w)
+    rng = np.random.default_rng(V)
+    load = rng.choice(np.array([0, 1, 5000, 2**32 - 1], np.uint32), w.n_variants)
+    run_stateful(w, _states(rng, w.n_variants, (0.45, 0.45, 0.05, 0.05)), load)
+
+
 # Lists of every variant: 7 and 34 segments, so that with four CTAs per task (3 tasks; 33 is the last
 # number of tasks for which all clusters run at once) a CTA indexes several of them, and with one (34) all
 @pytest.mark.parametrize("states", [False, True])
