@@ -1,4 +1,5 @@
-"""Thin ctypes binding of the C ABI in include/infaas.h (argument marshalling only).
+"""Thin binding of the C ABI in include/infaas.h (argument marshalling only): ctypes, and for the calls
+of every window the extension module built from csrc/calls.cpp.
 
 Every step of the path runs inside the CUDA library; this module passes pointers and
 sizes.  Device arrays are torch CUDA tensors (torch is used for device memory and streams
@@ -98,6 +99,27 @@ def _check(code: int, where: str) -> None:
 # current stream's pointer (a call that issues one kernel took 11 us on the host, 5 of them here).
 _widths: dict = {}
 _raw_stream = _current_device = None
+_calls = None                               # the extension module, from the first such call on
+
+
+def _load_calls():
+    """The calls of every window: tensors looked at in C++ (5.0 -> 2.9 us for a call that issues one kernel)."""
+    global _calls
+    if _calls is None:
+        _load()
+        import torch  # noqa: F401          (its libraries, which the module needs)
+        try:
+            from . import _calls as module
+        except ImportError as e:
+            raise RuntimeError("the binding's extension module is not built or does not suit this torch "
+                               "(run `python -m paper_1905_13348_b200.build`); there is no fallback") from e
+        module.setup(_dev_ptr, _length)
+        _calls = module
+    return _calls
+
+
+def _length(t) -> int:
+    return int(t.shape[0])
 
 
 def _init_torch() -> None:
@@ -171,31 +193,30 @@ def infaas_catalog_load(rows: np.ndarray, n_tasks: int, cuda_device: int = 0) ->
 
 def infaas_select_batch(cat: Catalog, d_task, d_slo_us, d_min_acc_bp, d_decision, n=None,
                         stream=None) -> None:
-    n = int(d_task.shape[0]) if n is None else int(n)
-    _check(_load().infaas_select_batch(cat.handle, _dev_ptr(d_task, "u16"), _dev_ptr(d_slo_us, "u32"),
-                                       _dev_ptr(d_min_acc_bp, "u16"), n, _dev_ptr(d_decision, "u32"),
-                                       _stream_ptr(stream)), "infaas_select_batch")
+    code = (_calls or _load_calls()).select_batch(cat, d_task, d_slo_us, d_min_acc_bp, d_decision, n, _stream_ptr(stream))
+    if code:
+        raise InfaasError(code, "infaas_select_batch")
 
 
 def infaas_load_update(cat: Catalog, d_decision, window_us: int, n=None, stream=None) -> None:
-    n = int(d_decision.shape[0]) if n is None else int(n)
-    _check(_load().infaas_load_update(cat.handle, _dev_ptr(d_decision, "u32"), n, int(window_us),
-                                      _stream_ptr(stream)), "infaas_load_update")
+    code = (_calls or _load_calls()).load_update(cat, d_decision, n, window_us, _stream_ptr(stream))
+    if code:
+        raise InfaasError(code, "infaas_load_update")
 
 
 def infaas_select_update(cat: Catalog, d_task, d_slo_us, d_min_acc_bp, d_decision, window_us: int, n=None,
                          stream=None) -> None:
     """One window: decide its queries, then fold the decisions into the load (one call)."""
-    n = int(d_task.shape[0]) if n is None else int(n)
-    _check(_load().infaas_select_update(cat.handle, _dev_ptr(d_task, "u16"), _dev_ptr(d_slo_us, "u32"),
-                                        _dev_ptr(d_min_acc_bp, "u16"), n, _dev_ptr(d_decision, "u32"),
-                                        int(window_us), _stream_ptr(stream)), "infaas_select_update")
+    code = (_calls or _load_calls()).select_update(cat, d_task, d_slo_us, d_min_acc_bp, d_decision, n, window_us,
+                                                   _stream_ptr(stream))
+    if code:
+        raise InfaasError(code, "infaas_select_update")
 
 
 def infaas_tally(cat: Catalog, d_decision, n=None, stream=None) -> None:
-    n = int(d_decision.shape[0]) if n is None else int(n)
-    _check(_load().infaas_tally(cat.handle, _dev_ptr(d_decision, "u32"), n, _stream_ptr(stream)),
-           "infaas_tally")
+    code = (_calls or _load_calls()).tally(cat, d_decision, n, _stream_ptr(stream))
+    if code:
+        raise InfaasError(code, "infaas_tally")
 
 
 def infaas_pending_counts(cat: Catalog, d_counts, set: bool, stream=None) -> None:
@@ -207,7 +228,9 @@ def infaas_pending_counts(cat: Catalog, d_counts, set: bool, stream=None) -> Non
 
 
 def infaas_advance(cat: Catalog, window_us: int, stream=None) -> None:
-    _check(_load().infaas_advance(cat.handle, int(window_us), _stream_ptr(stream)), "infaas_advance")
+    code = (_calls or _load_calls()).advance(cat, window_us, _stream_ptr(stream))
+    if code:
+        raise InfaasError(code, "infaas_advance")
 
 
 def infaas_catalog_set_states(cat: Catalog, state, load_lat_us=None, stream=None) -> None:
@@ -246,9 +269,10 @@ def infaas_autoscale_step(cat: Catalog, window_us: int, slack_pct: int, lambda_m
     """d_variant, d_delta: int32/uint32 CUDA tensors of n_tasks, overwritten."""
     if d_variant.numel() < cat.n_tasks or d_delta.numel() < cat.n_tasks:
         raise ValueError("outputs are shorter than n_tasks")
-    _check(_load().infaas_autoscale_step(cat.handle, int(window_us), int(slack_pct), int(lambda_milli),
-                                         _dev_ptr(d_variant, "u32"), _dev_ptr(d_delta, "u32"),
-                                         _stream_ptr(stream)), "infaas_autoscale_step")
+    code = (_calls or _load_calls()).autoscale_step(cat, window_us, slack_pct, lambda_milli, d_variant, d_delta,
+                                                    _stream_ptr(stream))
+    if code:
+        raise InfaasError(code, "infaas_autoscale_step")
 
 
 def infaas_workers_config(cat: Catalog, inst_variant, inst_worker, inst_load, worker_hw, worker_util,
@@ -266,9 +290,9 @@ def infaas_workers_config(cat: Catalog, inst_variant, inst_worker, inst_load, wo
 
 
 def infaas_assign_workers(cat: Catalog, d_decision, d_worker, n=None, stream=None) -> None:
-    n = int(d_decision.shape[0]) if n is None else int(n)
-    _check(_load().infaas_assign_workers(cat.handle, _dev_ptr(d_decision, "u32"), n, _dev_ptr(d_worker, "u32"),
-                                         _stream_ptr(stream)), "infaas_assign_workers")
+    code = (_calls or _load_calls()).assign_workers(cat, d_decision, n, d_worker, _stream_ptr(stream))
+    if code:
+        raise InfaasError(code, "infaas_assign_workers")
 
 
 def infaas_catalog_get_state(cat: Catalog, stream=None) -> dict:

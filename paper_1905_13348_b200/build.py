@@ -1,13 +1,16 @@
-"""Builds the CUDA library in-tree with nvcc for sm_100a (no GPU needed to compile)."""
+"""Builds the CUDA library in-tree with nvcc for sm_100a (no GPU needed to compile), and the extension
+module with the binding's per-window calls against it."""
 from __future__ import annotations
 
 import glob
 import os
 import subprocess
+import sysconfig
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 _ROOT = os.path.dirname(_HERE)
 LIB_PATH = os.path.join(_HERE, "libinfaas_b200.so")
+CALLS_PATH = os.path.join(_HERE, "_calls.so")
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 
 
@@ -16,11 +19,27 @@ def sources() -> list[str]:
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB_PATH):
+    if not (os.path.exists(LIB_PATH) and os.path.exists(CALLS_PATH)):
         return True
-    deps = sources() + glob.glob(os.path.join(_HERE, "csrc", "*.cuh")) + \
+    deps = sources() + [os.path.join(_HERE, "csrc", "calls.cpp")] + glob.glob(os.path.join(_HERE, "csrc", "*.cuh")) + \
         glob.glob(os.path.join(_ROOT, "include", "*.h"))
-    return any(os.path.getmtime(d) > os.path.getmtime(LIB_PATH) for d in deps)
+    built = min(os.path.getmtime(LIB_PATH), os.path.getmtime(CALLS_PATH))
+    return any(os.path.getmtime(d) > built for d in deps)
+
+
+def _build_calls() -> None:
+    import torch
+    top = os.path.dirname(torch.__file__)
+    tmp = CALLS_PATH + f".tmp{os.getpid()}"
+    subprocess.check_call(
+        ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden",
+         f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+         "-I", os.path.join(_ROOT, "include"), "-I", sysconfig.get_paths()["include"],
+         "-isystem", os.path.join(top, "include"),
+         os.path.join(_HERE, "csrc", "calls.cpp"), "-o", tmp,
+         "-L", _HERE, "-l:libinfaas_b200.so", "-Wl,-rpath,$ORIGIN",
+         "-L", os.path.join(top, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10"])
+    os.replace(tmp, CALLS_PATH)
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -35,6 +54,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     cmd += sources() + ["-o", tmp]
     subprocess.check_call(cmd)
     os.replace(tmp, LIB_PATH)
+    _build_calls()
     return LIB_PATH
 
 

@@ -104,3 +104,49 @@ def test_current_stream_without_torchs_private_getters(monkeypatch, missing):
     monkeypatch.setattr(b, "_current_device", None)
     assert b._stream_ptr(None) == 4003
     assert b._stream_ptr(types.SimpleNamespace(cuda_stream=5)) == 5
+
+
+def test_per_window_calls_convert_arguments_as_before():
+    """The extension module's calls: errors and conversions of the Python they stand for."""
+    import types
+
+    import torch
+
+    import paper_1905_13348_b200 as P
+    s = types.SimpleNamespace(cuda_stream=0)
+    cat = types.SimpleNamespace(handle=ctypes.c_void_p(None), n_tasks=1, n_variants=1)
+    t32 = torch.zeros(4, dtype=torch.int32)
+
+    class Like:                              # not a tensor, but it answers what is asked of one
+        is_cuda, dtype, device, shape = True, torch.int32, "cuda", (4,)
+        numel = staticmethod(lambda: 4)
+        is_contiguous = staticmethod(lambda: True)
+        data_ptr = staticmethod(lambda: 4096)
+
+    calls = [lambda d, **k: P.infaas_tally(cat, d, stream=s, **k),
+             lambda d, **k: P.infaas_load_update(cat, d, 1000, stream=s, **k),
+             lambda d, **k: P.infaas_assign_workers(cat, d, d, stream=s, **k),
+             lambda d, **k: P.infaas_select_batch(cat, None, d, None, d, stream=s, **{"n": 4, **k}),
+             lambda d, **k: P.infaas_select_update(cat, None, d, None, d, 1000, stream=s, **{"n": 4, **k})]
+    for call in calls:
+        with pytest.raises(TypeError, match="expected a contiguous CUDA tensor of u32, got torch.int32 on cpu"):
+            call(t32)
+        for d, n in ((Like(), 3), (Like(), 3.7), (Like(), True), (None, 0)):
+            with pytest.raises(P.InfaasError, match="NULL"):             # the catalog's handle
+                call(d, n=n)
+        with pytest.raises((TypeError, ValueError)):
+            call(Like(), n="many")
+    with pytest.raises(TypeError, match="u16, got torch.int32"):
+        P.infaas_select_batch(cat, t32, None, None, None, stream=s)
+    with pytest.raises(AttributeError):
+        P.infaas_select_batch(cat, None, None, None, None, stream=s)     # no length to be had
+    with pytest.raises(IndexError):
+        P.infaas_tally(cat, torch.zeros((), dtype=torch.int32), stream=s)
+    with pytest.raises(P.InfaasError, match="NULL"):
+        P.infaas_advance(cat, 1000, stream=s)
+    with pytest.raises(P.InfaasError, match="NULL"):
+        P.infaas_autoscale_step(cat, 1000, 105, 100, Like(), Like(), stream=s)
+    with pytest.raises((TypeError, ValueError)):
+        P.infaas_advance(cat, None, stream=s)
+    with pytest.raises(AttributeError):
+        P.infaas_advance(object(), 1000, stream=s)
