@@ -2,9 +2,8 @@
 //
 // What bounds such a call is the host.  Through ctypes infaas_select_batch took 5.0 us, of which the launch
 // itself is 2.5: 1.0 went into asking four tensors for their device, layout, type and address one attribute
-// at a time and 0.7 into ctypes.  Here a tensor is looked at in C++:
-// 2.9 us a call here.  Anything but a plain contiguous CUDA
-// tensor of the wanted width goes through the binding's own `_dev_ptr` (subclasses, objects that only look
+// at a time and 0.7 into ctypes.  Here a tensor is looked at in C++: 2.9 us.  Anything but a plain contiguous
+// CUDA tensor of the wanted width goes through the binding's own `_dev_ptr` (subclasses, objects that only look
 // like tensors, None) or gets its error from there.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>

@@ -46,6 +46,7 @@ struct IndexScratch {
   unsigned char at[256];                     // sorted order: position
   unsigned char stair[256];                  // latency rank holds a stair entry
   unsigned char part[B];                     // rank table: first position per column of a run of entries
+  uint32_t warp_bcnt[B / 32u];               // latencies in the SLO buckets of a warp
   uint32_t ks, ka, base;
 
   // Entry `pos` of the segment (its accuracy's bit too).
@@ -268,7 +269,7 @@ __device__ __forceinline__ bool build_index(const DeviceCatalog &c, uint32_t t, 
   }
   // stair entries: those more accurate than everything faster (one per latency at most); 32 latency
   // ranks per warp
-  const uint32_t ws = (warp + WARPS / 2u + 2u) & (WARPS - 1u);    // (not the warps with a run, nor the last)
+  const uint32_t ws = (warp + WARPS / 2u) & (WARPS - 1u);         // (not the warps with a run)
   uint32_t best_a = 0;                                            // latency ranks < this thread's
   if (32u * ws <= Ks) {
     const uint32_t r = 32u * ws + lane;
@@ -280,19 +281,39 @@ __device__ __forceinline__ bool build_index(const DeviceCatalog &c, uint32_t t, 
     best_a = max(below, lanes_before(warp_scan_max(x), 0u));
     if (r < Ks) S.stair[r] = best_a == 0u || (x >> 16) > (best_a >> 16);
   }
-  if (first) {
-    // SLO records, 32 neighbouring buckets per warp and trip (the last warps first); below = latencies in
-    // lower buckets
-    const uint32_t nb = c.n_buckets;
+  // SLO records, first half: latencies in the buckets before this thread's (`per` consecutive ones) in its warp;
+  // the warps' sums are added behind the barrier (each warp adding up all buckets before its own took 10 us of
+  // the 16 windows of 128 x 512, more with 2048 buckets)
+  constexpr uint32_t PER = NB > B ? NB / B : 1u;
+  const uint32_t nb = c.n_buckets, per = nb > B ? PER : 1u, j0 = tid * per;
+  uint32_t below = 0;
+  if (first && 32u * warp * per < nb) {
+    uint32_t n = S.bcnt[j0];
+    if (PER > 1u && per > 1u)
+#pragma unroll
+      for (uint32_t k = 1; k < PER; ++k) n += S.bcnt[j0 + k];
+    const uint32_t incl = warp_scan_add(n);
+    below = incl - n;
+    if (lane == 31u) S.warp_bcnt[warp] = incl;
+  }
+  if (tid == B - 1u) {
+    uint32_t base = image_var_offset(c.n_tasks, c.n_buckets, nbw) + place_block_finish(c, placed, bytes, done);
+    if (base + bytes > c.image_capacity || base + BL.t2 >= IMAGE_T2_LIMIT) base = NONE;
+    S.base = base;
+  }
+  __syncthreads();
+  const uint32_t base = S.base;
+  if (base == NONE) return false;
+  unsigned char *blk = c.image + base;
+  unsigned char *slow = blk + BL.slow;
+
+  // 4. SLO records, second half
+  if (first && 32u * warp * per < nb) {
+    below += __reduce_add_sync(0xFFFFFFFFu, lane < warp ? S.warp_bcnt[lane] : 0u);
     uint32_t *rec = reinterpret_cast<uint32_t *>(c.image + image_rec_offset(c.n_tasks) + t * rec_stride(nb));
 #pragma unroll 1
-    for (uint32_t j0 = 32u * (WARPS - 1u - warp); j0 < nb; j0 += B) {
-      uint32_t below = 0;
-#pragma unroll 4
-      for (uint32_t i = lane; i < j0; i += 32u) below += S.bcnt[i];
-      below = __reduce_add_sync(0xFFFFFFFFu, below);
-      const uint32_t j = j0 + lane, cnt = S.bcnt[j];
-      below += warp_scan_add(cnt) - cnt;
+    for (uint32_t j = j0; j < j0 + per; ++j) {
+      const uint32_t cnt = S.bcnt[j];
       uint32_t r = ((Ks + 1u) << 24) | (cnt << 8) | below;          // exact slow path
       if (cnt == 0u) {
         r = below << 24;
@@ -306,20 +327,10 @@ __device__ __forceinline__ bool build_index(const DeviceCatalog &c, uint32_t t, 
       }
       rec[j] = r;
       if (j == nb - 1u) rec[nb] = r;                               // what an SLO beyond the last bucket reads
+      below += cnt;
     }
   }
-  if (tid == B - 1u) {
-    uint32_t base = image_var_offset(c.n_tasks, c.n_buckets, nbw) + place_block_finish(c, placed, bytes, done);
-    if (base + bytes > c.image_capacity || base + BL.t2 >= IMAGE_T2_LIMIT) base = NONE;
-    S.base = base;
-  }
-  __syncthreads();
-  const uint32_t base = S.base;
-  if (base == NONE) return false;
-  unsigned char *blk = c.image + base;
-  unsigned char *slow = blk + BL.slow;
-
-  // 4. rank table, second half: each run starts from the minimum of the runs before it and writes a
+  // rank table, second half: each run starts from the minimum of the runs before it and writes a
   // row after the last entry of every latency
   unsigned char *T2 = blk + BL.t2;
   if (i0 < i1 && col < width) {
@@ -438,9 +449,26 @@ __device__ __forceinline__ uint32_t advance_row(const DeviceCatalog &c, uint32_t
   return pred;
 }
 
-// Queue recursion, prune and list of one task (all threads of one CTA): the list goes into the
-// task's region, its first segment also into S, which is cleared here.  Contains chain_wait.  Returns
-// the list's length.
+// The same variable of CTA `rank` of this CTA's cluster.
+template <class T>
+__device__ __forceinline__ T *peer(T *p, uint32_t rank) {
+  unsigned long long a;
+  asm("mapa.u64 %0, %1, %2;" : "=l"(a) : "l"(p), "r"(rank));
+  return reinterpret_cast<T *>(a);
+}
+// Barrier over the K CTAs of a task's cluster (all their threads), for shared and global memory.
+__device__ __forceinline__ void task_sync(uint32_t K) {
+  if (K > 1u) {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  } else {
+    __syncthreads();
+  }
+}
+
+// Queue recursion, prune and list of one task, by the K CTAs of its cluster: the list goes into the
+// task's region, segment s < K of it also into CTA s's S, which is cleared here.  Contains chain_wait.
+// Returns the list's length.
 //
 // List of the Active variants (all variants of a catalog without states).  Slots are in (cost,
 // 10000-acc, id) order, so with `order` = position in (10000-acc, local) order a variant q before
@@ -454,14 +482,20 @@ __device__ __forceinline__ uint32_t advance_row(const DeviceCatalog &c, uint32_t
 // positions follow from counting survivors: those before the run of equal cost, then the run
 // backwards.
 //
+// Each CTA has a share of the grid's rows, with their variants: the running minimum down the columns
+// goes on from the last rows of the CTAs before it, what passes is made known to the CTAs behind it (by
+// accuracy position), survivors to all.  4 x 4096 variants on a trade-off surface, lists of up to 505 entries: a window of
+// 20,011 queries 46.8 us with the list made by the first CTA alone, 38.4 so.
+//
 // List of the Inactive variants: ordered by (eff, 10000-acc, id) with eff in place of cost and
 // pred; at most the fastest variant (lowest id) of every distinct accuracy is on it, if it is
-// faster than everything more accurate, and the list runs from the lowest accuracy up.
-__device__ __forceinline__ uint32_t build_list(const DeviceCatalog &c, uint32_t t, bool advance, uint32_t window_us,
-                                               unsigned char *dyn,
+// faster than everything more accurate, and the list runs from the lowest accuracy up.  CTA 0 makes it.
+__device__ __forceinline__ uint32_t build_list(const DeviceCatalog &c, uint32_t t, uint32_t share, uint32_t K, bool advance,
+                                               uint32_t window_us, unsigned char *dyn,
                                                IndexScratch<REBUILD_THREADS, MAX_BUCKETS> &S, uint32_t &slo_seen) {
   constexpr uint32_t KEEP_WORDS = INFAAS_MAX_TASK_VARIANTS / 32;
-  __shared__ uint32_t grid[GRID * GRID_PITCH];
+  __shared__ uint32_t grid[GRID * GRID_PITCH];                    // this CTA's rows
+  __shared__ uint32_t carry[GRID];                                // per column: smallest of the rows of the CTAs before
   __shared__ uint32_t keep[KEEP_WORDS + 1], keep_pre[KEEP_WORDS + 1];   // bit sets: survivors, by local index ...
   __shared__ uint32_t passed_local[KEEP_WORDS], passed_acc[KEEP_WORDS];   // ... what the grid lets through, both orders
   __shared__ unsigned long long warp_min[REBUILD_WARPS];
@@ -471,11 +505,23 @@ __device__ __forceinline__ uint32_t build_list(const DeviceCatalog &c, uint32_t 
 
   const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
   const uint32_t base = c.task_off[t], V = c.task_off[t + 1] - base;
-  // shared memory per variant (REBUILD_ROW_SMEM bytes)
-  uint2 *by_local = reinterpret_cast<uint2 *>(dyn);               // (pred, accuracy position); position 0xFFFF: not listed
-  uint2 *by_acc = by_local + V;                                    // accuracy order: (pred, local); local 0xFFFF: not listed
-  uint32_t *run_min = reinterpret_cast<uint32_t *>(by_acc + V);   // at the first of each (cost, accuracy): smallest pred
+  uint32_t cs = 4;                                                 // log2 of the rows' and columns' run length
+#pragma unroll 1
+  while (V > (GRID << cs)) ++cs;
+  // rows of a CTA: an even number, so that its variants [lo, hi) are whole words of the bit sets
+  const uint32_t ng = (V + (1u << cs) - 1u) >> cs, rows = K > 1u ? ((ng + K - 1u) / K + 1u) & ~1u : ng, y0 = share * rows;
+  const uint32_t lo = min(V, y0 << cs), hi = min(V, (y0 + rows) << cs), own = hi - lo, own_rows = (own + (1u << cs) - 1u) >> cs;
+  // shared memory per variant (REBUILD_ROW_SMEM bytes); those by local index: of this CTA's, from lo
+  uint2 *by_acc = reinterpret_cast<uint2 *>(dyn);                 // accuracy order: (pred, local), of what passed
+  uint2 *by_local = by_acc + V;                                    // (pred, accuracy position); position 0xFFFF: not listed
+  uint32_t *run_min = reinterpret_cast<uint32_t *>(by_local + V); // at the first of each (cost, accuracy): smallest pred
   uint16_t *cand = reinterpret_cast<uint16_t *>(run_min + V);     // entries the grid lets through
+  auto run_min_of = [&](uint32_t order) {                         // (a run can begin in an earlier CTA's share)
+    const uint32_t f = (order >> 13) & 0x1FFFu;
+    if (f >= lo) return run_min + (f - lo);
+    const uint32_t o = (f >> cs) / rows;
+    return peer(run_min + (f - ((o * rows) << cs)), o);
+  };
 
   unsigned char *region = c.regions + c.reg_off[t];
   unsigned long long *keys_g = reinterpret_cast<unsigned long long *>(region);
@@ -483,62 +529,57 @@ __device__ __forceinline__ uint32_t build_list(const DeviceCatalog &c, uint32_t 
 
   // 1. queue recursion, states, predicted latencies; coarse grid.  Each thread's first variant
   // stays in registers.  Before chain_wait: only what no kernel writes, and clearing.
+  const uint32_t own0 = lo + tid;
   Row r0;
   r0.drain = 0;
   uint32_t acc0 = 0, run0 = 0, class0 = 0, pred0 = 0;
-  if (tid < V) {
-    r0 = load_fixed(c, base + tid, window_us);
-    acc0 = c.s_acc[base + tid];
-    run0 = c.s_cost_run[base + tid];
-    if (c.stateful) class0 = c.s_class[base + tid];
+  if (own0 < hi) {
+    r0 = load_fixed(c, base + own0, window_us);
+    acc0 = c.s_acc[base + own0];
+    run0 = c.s_cost_run[base + own0];
+    if (c.stateful) class0 = c.s_class[base + own0];
   }
-  uint32_t cs = 4;                                                 // log2 of the rows' and columns' run length
 #pragma unroll 1
-  while (V > (GRID << cs)) ++cs;
-  const uint32_t ng = (V + (1u << cs) - 1u) >> cs;
+  for (uint32_t i = tid; i < rows * GRID_PITCH; i += B) grid[i] = NONE;
 #pragma unroll 1
-  for (uint32_t i = tid; i < ng * GRID_PITCH; i += B) grid[i] = NONE;
-#pragma unroll 1
-  for (uint32_t i = tid; i < V; i += B) run_min[i] = NONE;
+  for (uint32_t i = tid; i < own; i += B) run_min[i] = NONE;
 #pragma unroll 1
   for (uint32_t i = tid; i <= KEEP_WORDS; i += B) { keep[i] = 0u; if (i < KEEP_WORDS) passed_acc[i] = 0u; }
   S.clear(c.n_buckets, c.nbw);
+  if (tid < GRID) carry[tid] = NONE;
   if (tid == 0u) { n_cand = 0u; n_inactive = 0u; }
-  __syncthreads();
+  task_sync(K);
   asm volatile("" : "+r"(r0.drain));                               // (else the compiler moves the division behind the wait)
   chain_wait();
   chain_next();
   slo_seen = *c.slo_seen;                                          // wanted by the index, requested early
   Row r = r0;
 #pragma unroll 1
-  for (uint32_t i = tid; i < V;) {
+  for (uint32_t i = own0; i < hi;) {
     load_load(c, base + i, advance, r);
     const uint32_t pred = advance_row(c, base + i, r, advance);
     const uint32_t pos = r.order & 0x1FFFu;
-    if (r.state == INFAAS_STATE_ACTIVE) {
-      by_local[i] = make_uint2(pred, pos);
-      by_acc[pos] = make_uint2(pred, i);
+    const bool listed = r.state == INFAAS_STATE_ACTIVE;
+    by_local[i - lo] = listed ? make_uint2(pred, pos) : make_uint2(NONE, 0xFFFFu);
+    if (listed) {
       // NONE stands for "no entry" in the grid: a saturated latency counts as one less there
-      atomicMin(&grid[(i >> cs) * GRID_PITCH + (pos >> cs)], min(pred, NONE - 1u));
-      if (r.order >> 31) atomicMin(&run_min[(r.order >> 13) & 0x1FFFu], pred);
-    } else {
-      by_local[i] = make_uint2(NONE, 0xFFFFu);
-      by_acc[pos] = make_uint2(NONE, 0xFFFFu);
+      atomicMin(&grid[((i >> cs) - y0) * GRID_PITCH + (pos >> cs)], min(pred, NONE - 1u));
+      if (r.order >> 31) atomicMin(run_min_of(r.order), pred);
     }
-    if (i == tid) { pred0 = pred; r0.state = r.state; r0.load_lat = r.load_lat; }
+    if (i == own0) { pred0 = pred; r0.state = r.state; r0.load_lat = r.load_lat; }
     i += B;
-    if (i < V) r = load_fixed(c, base + i, window_us);
+    if (i < hi) r = load_fixed(c, base + i, window_us);
   }
   __syncthreads();
   // 2. running minimum along the rows, then down the columns (GRID = two values per lane)
 #pragma unroll 1
-  for (uint32_t y = warp; y < ng; y += REBUILD_WARPS) {
+  for (uint32_t y = warp; y < own_rows; y += REBUILD_WARPS) {
     uint32_t *row = grid + y * GRID_PITCH;
     const uint32_t x0 = warp_scan_min(lane < ng ? row[lane] : NONE);
     if (lane < ng) row[lane] = x0;
     if (ng > 32u) {
-      const uint32_t carry = __shfl_sync(0xFFFFFFFFu, x0, 31);
-      const uint32_t x1 = min(warp_scan_min(lane + 32u < ng ? row[lane + 32u] : NONE), carry);
+      const uint32_t before = __shfl_sync(0xFFFFFFFFu, x0, 31);
+      const uint32_t x1 = min(warp_scan_min(lane + 32u < ng ? row[lane + 32u] : NONE), before);
       if (lane + 32u < ng) row[lane + 32u] = x1;
     }
   }
@@ -546,89 +587,110 @@ __device__ __forceinline__ uint32_t build_list(const DeviceCatalog &c, uint32_t 
 #pragma unroll 1
   for (uint32_t x = warp; x < ng; x += REBUILD_WARPS) {
     uint32_t *col = grid + x;
-    const uint32_t x0 = warp_scan_min(lane < ng ? col[lane * GRID_PITCH] : NONE);
-    if (lane < ng) col[lane * GRID_PITCH] = x0;
-    if (ng > 32u) {
-      const uint32_t carry = __shfl_sync(0xFFFFFFFFu, x0, 31);
-      const uint32_t x1 = min(warp_scan_min(lane + 32u < ng ? col[(lane + 32u) * GRID_PITCH] : NONE), carry);
-      if (lane + 32u < ng) col[(lane + 32u) * GRID_PITCH] = x1;
+    const uint32_t x0 = warp_scan_min(lane < own_rows ? col[lane * GRID_PITCH] : NONE);
+    if (lane < own_rows) col[lane * GRID_PITCH] = x0;
+    if (own_rows > 32u) {
+      const uint32_t before = __shfl_sync(0xFFFFFFFFu, x0, 31);
+      const uint32_t x1 = min(warp_scan_min(lane + 32u < own_rows ? col[(lane + 32u) * GRID_PITCH] : NONE), before);
+      if (lane + 32u < own_rows) col[(lane + 32u) * GRID_PITCH] = x1;
     }
+  }
+  task_sync(K);
+  // (a CTA with variants comes behind full ones only)
+  if (share && own && tid < ng) {
+    uint32_t v = NONE;
+#pragma unroll 1
+    for (uint32_t o = 0; o < share; ++o) v = min(v, *peer(&grid[(rows - 1u) * GRID_PITCH + tid], o));
+    carry[tid] = v;
   }
   __syncthreads();
   // 3. what the grid lets through ...
 #pragma unroll 1
-  for (uint32_t i0 = 0; i0 < V; i0 += B) {
-    const uint32_t i = i0 + tid;
+  for (uint32_t b = lo; b < hi; b += B) {
+    const uint32_t i = b + tid;
     bool pass = false;
-    if (i < V) {
-      const uint2 a = by_local[i];
+    uint2 a = make_uint2(0u, 0u);
+    if (i < hi) {
+      a = by_local[i - lo];
       if (a.y != 0xFFFFu) {
-        const uint32_t y = i >> cs, x = a.y >> cs;
-        const uint32_t g = y && x ? grid[(y - 1u) * GRID_PITCH + x - 1u] : NONE;
-        const uint32_t order = i0 ? c.s_order[base + i] : r0.order;
+        const uint32_t y = (i >> cs) - y0, x = a.y >> cs;
+        const uint32_t g = x ? min(carry[x - 1u], y ? grid[(y - 1u) * GRID_PITCH + x - 1u] : NONE) : NONE;
+        const uint32_t order = i == own0 ? r0.order : c.s_order[base + i];
         // (a latency of NONE - 1 cannot be told from a saturated one in the grid: step 4 looks at all)
         pass = g > min(a.x, NONE - 1u) || (a.x == NONE - 1u && g == NONE - 1u);
-        if (order >> 31) pass = pass && a.x <= run_min[(order >> 13) & 0x1FFFu];
+        if (order >> 31) pass = pass && a.x <= *run_min_of(order);
       }
     }
     const unsigned m = __ballot_sync(0xFFFFFFFFu, pass);
     uint32_t at = 0;
     if (m && lane == 0u) at = atomicAdd(&n_cand, (uint32_t)__popc(m));
     at = __shfl_sync(0xFFFFFFFFu, at, 0);
-    if (lane == 0u && i < V) passed_local[i >> 5] = m;
+    if (lane == 0u && i < hi) passed_local[(i - lo) >> 5] = m;
     if (pass) {
-      cand[at + __popc(m & ((1u << lane) - 1u))] = (uint16_t)i;
-      const uint32_t pos = by_local[i].y;
-      atomicOr(&passed_acc[pos >> 5], 1u << (pos & 31u));
+      cand[at + __popc(m & ((1u << lane) - 1u))] = (uint16_t)(i - lo);
+#pragma unroll 1
+      for (uint32_t o = share; o < K; ++o) {
+        *peer(&by_acc[a.y], o) = make_uint2(a.x, i);
+        atomicOr(peer(&passed_acc[a.y >> 5], o), 1u << (a.y & 31u));
+      }
     }
   }
-  __syncthreads();
+  task_sync(K);
   // 4. ... against the entries before it in its own row and column of the grid that were let through
-  // too (dominance is transitive and what is dominated by nothing is let through): one lane for
-  // the row, one for the column
+  // too (dominance is transitive and what is dominated by nothing is let through): four lanes for
+  // the row, four for the column
   const uint32_t nc = n_cand;
 #pragma unroll 1
-  for (uint32_t x0 = 0; x0 < nc; x0 += B / 2u) {
-    const uint32_t x = x0 + (tid >> 1);
+  for (uint32_t x0 = 0; x0 < nc; x0 += B / 8u) {
+    const uint32_t x = x0 + (tid >> 3);
     uint32_t dom = 0, p = 0;
     if (x < nc) {
       p = cand[x];
       const uint2 a = by_local[p];
-      const bool row = !(tid & 1u);
+      const bool row = !(tid & 4u);
       const uint2 *v = row ? by_local : by_acc;
       const uint32_t *bits = row ? passed_local : passed_acc;
-      const uint32_t hi = row ? p : a.y, limit = row ? a.y : p;
-      const uint32_t lo = row && a.x == NONE - 1u ? 0u : (hi >> cs) << cs;
+      const uint32_t end = row ? p : a.y, limit = row ? a.y : lo + p;
+      const uint32_t from = !row && a.x == NONE - 1u ? 0u : (end >> cs) << cs;
 #pragma unroll 1
-      for (uint32_t w = lo >> 5; w <= hi >> 5 && !dom; ++w) {
-        uint32_t m = bits[w];
-        if (w == lo >> 5) m &= ~0u << (lo & 31u);
-        if (w == hi >> 5) m &= (1u << (hi & 31u)) - 1u;
+      for (uint32_t w = from >> 5; w <= end >> 5 && !dom; ++w) {
+        uint32_t m = bits[w] & (0x11111111u << (tid & 3u));
+        if (w == from >> 5) m &= ~0u << (from & 31u);
+        if (w == end >> 5) m &= (1u << (end & 31u)) - 1u;
 #pragma unroll 1
         while (m && !dom) {
-          const uint2 b = v[32u * w + (uint32_t)__ffs(m) - 1u];
+          const uint2 e = v[32u * w + (uint32_t)__ffs(m) - 1u];
           m &= m - 1u;
-          dom = (uint32_t)(b.x <= a.x) & (uint32_t)(b.y < limit);
+          dom = (uint32_t)(e.x <= a.x) & (uint32_t)(e.y < limit);
         }
       }
     }
-    dom |= __shfl_xor_sync(0xFFFFFFFFu, dom, 1);
-    if (x < nc && !(tid & 1u) && !dom) atomicOr(&keep[p >> 5], 1u << (p & 31u));
+    dom = __ballot_sync(0xFFFFFFFFu, dom != 0u) >> (lane & 24u) & 0xFFu;
+    if (x < nc && !(tid & 7u) && !dom) atomicOr(&keep[(lo + p) >> 5], 1u << (p & 31u));
   }
-  __syncthreads();
-  // 5. survivors before each word of the bit set (warp 0)
-  const uint32_t n_words = (V + 31u) >> 5;
-  if (warp == 0u) {
-    uint32_t carry = 0;
+  if (K > 1u) {                                                    // survivors to all
+    __syncthreads();
+    const uint32_t w = (lo >> 5) + tid;
+    if (w < (hi + 31u) >> 5) {
+      const uint32_t bits = keep[w];
 #pragma unroll 1
-    for (uint32_t w0 = 0; w0 <= n_words; w0 += 32u) {
-      const uint32_t w = w0 + lane, pc = w < n_words ? __popc(keep[w]) : 0u;
-      const uint32_t incl = carry + warp_scan_add(pc);
-      if (w <= n_words) keep_pre[w] = incl - pc;
-      carry = __shfl_sync(0xFFFFFFFFu, incl, 31);
+      for (uint32_t o = 0; o < K; ++o)
+        if (o != share) *peer(&keep[w], o) = bits;
     }
   }
-  const uint32_t n_class = c.stateful ? c.n_class[t] : 0u;
+  task_sync(K);
+  // 5. survivors before each word of the bit set
+  const uint32_t n_words = (V + 31u) >> 5;
+  if (32u * warp <= n_words) {
+    uint32_t below = 0;
+#pragma unroll 4
+    for (uint32_t x = lane; x < 32u * warp; x += 32u) below += __popc(keep[x]);
+    below = __reduce_add_sync(0xFFFFFFFFu, below);
+    const uint32_t pc = tid < n_words ? __popc(keep[tid]) : 0u;
+    const uint32_t incl = below + warp_scan_add(pc);
+    if (tid <= n_words) keep_pre[tid] = incl - pc;
+  }
+  const uint32_t n_class = c.stateful && share == 0u ? c.n_class[t] : 0u;
   uint32_t *class_eff = reinterpret_cast<uint32_t *>(by_acc), *class_id = class_eff + n_class;   // by_acc is not needed any more
 #pragma unroll 1
   for (uint32_t k = tid; k < n_class; k += B) { class_eff[k] = NONE; class_id[k] = NONE; }
@@ -637,39 +699,40 @@ __device__ __forceinline__ uint32_t build_list(const DeviceCatalog &c, uint32_t 
   auto emit = [&](uint32_t pos, uint32_t pred, uint32_t acc, uint32_t id) {
     keys_g[pos] = ((unsigned long long)acc << 32) | pred;
     ids_g[pos] = id;
-    if (pos < INDEX_MAX_F) S.put(pos, pred, acc, id, c.acc_lo);
+    const uint32_t seg = pos / INDEX_MAX_F;
+    if (seg < K) peer(&S, seg)->put(pos - seg * INDEX_MAX_F, pred, acc, id, c.acc_lo);
   };
   auto before = [&](uint32_t i) { return keep_pre[i >> 5] + __popc(keep[i >> 5] & ((1u << (i & 31u)) - 1u)); };
 #pragma unroll 1
-  for (uint32_t i = tid; i < V; i += B) {
+  for (uint32_t i = own0; i < hi; i += B) {
     if (!((keep[i >> 5] >> (i & 31u)) & 1u)) continue;
-    const bool reg = i == tid;
+    const bool reg = i == own0;
     const uint32_t run = reg ? run0 : c.s_cost_run[base + i];
     const uint32_t pos = before(run & 0xFFFFu) + before(run >> 16) - 1u - before(i);
-    emit(pos, reg ? pred0 : by_local[i].x, reg ? acc0 : c.s_acc[base + i], reg ? r0.id : c.s_id[base + i]);
+    emit(pos, reg ? pred0 : by_local[i - lo].x, reg ? acc0 : c.s_acc[base + i], reg ? r0.id : c.s_id[base + i]);
   }
   // the counts are cleared here, far behind their loads: a store to a line whose load is still in flight
   // holds up everything behind it (4 us a launch when the store came right behind)
   if (advance)
 #pragma unroll 1
-    for (uint32_t i = tid; i < V; i += B) c.count_by_id[i == tid ? r0.id : c.s_id[base + i]] = 0u;
+    for (uint32_t i = own0; i < hi; i += B) c.count_by_id[i == own0 ? r0.id : c.s_id[base + i]] = 0u;
   uint32_t F = keep_pre[n_words];
-  if (c.stateful) {
+  if (c.stateful && share == 0u) {                                 // (lo = 0)
     // the fastest Inactive variant of every accuracy class: its latency, then the lowest id with it
     auto eff_of = [&](uint32_t i) {
-      const unsigned long long e = (unsigned long long)(i == tid ? pred0 : c.s_pred[base + i]) +
-                                   (i == tid ? r0.load_lat : c.s_load_lat[base + i]);
+      const unsigned long long e = (unsigned long long)(i == own0 && i < hi ? pred0 : c.s_pred[base + i]) +
+                                   (i == own0 && i < hi ? r0.load_lat : c.s_load_lat[base + i]);
       return e > NONE ? NONE : (uint32_t)e;
     };
-    auto inactive = [&](uint32_t i) { return (i == tid ? r0.state : c.s_state[base + i]) == INFAAS_STATE_INACTIVE; };
-    auto class_of = [&](uint32_t i) { return i == tid ? class0 : c.s_class[base + i]; };
+    auto inactive = [&](uint32_t i) { return (i == own0 && i < hi ? r0.state : c.s_state[base + i]) == INFAAS_STATE_INACTIVE; };
+    auto class_of = [&](uint32_t i) { return i == own0 && i < hi ? class0 : c.s_class[base + i]; };
 #pragma unroll 1
     for (uint32_t i = tid; i < V; i += B)
       if (inactive(i)) atomicMin(&class_eff[class_of(i)], eff_of(i));
     __syncthreads();
 #pragma unroll 1
     for (uint32_t i = tid; i < V; i += B)
-      if (inactive(i) && class_eff[class_of(i)] == eff_of(i)) atomicMin(&class_id[class_of(i)], i == tid ? r0.id : c.s_id[base + i]);
+      if (inactive(i) && class_eff[class_of(i)] == eff_of(i)) atomicMin(&class_id[class_of(i)], i == own0 && i < hi ? r0.id : c.s_id[base + i]);
     __syncthreads();
     // each thread takes consecutive classes (one, up to 1024 of them): running minimum from the
     // highest accuracy down, survivors, their number.  A class without entry counts as 2^32.
@@ -726,7 +789,9 @@ __device__ __forceinline__ uint32_t build_list(const DeviceCatalog &c, uint32_t 
     __syncthreads();
     F += n_inactive;
   }
-  __syncthreads();
+  if (share == 0u && tid == 0u) c.f_len[t] = F;
+  task_sync(K);
+  if (K > 1u) F = *reinterpret_cast<volatile uint32_t *>(c.f_len + t);   // (with the Inactive list's, which CTA 0 made)
   return F;
 }
 
@@ -745,7 +810,7 @@ __device__ __forceinline__ bool index_list(const DeviceCatalog &c, uint32_t t, u
 #pragma unroll 1
     for (uint32_t sg = share; sg < nseg && indexed; sg += K) {
       const uint32_t off = sg * INDEX_MAX_F, Fseg = min(INDEX_MAX_F, F - off), x0 = nseg > 1u ? c.seg_base[t] : 0u;
-      if (sg) {                                   // later segments: back from the task's region
+      if (sg >= K) {                              // not there yet: back from the task's region
         const unsigned char *region = c.regions + c.reg_off[t];
         const unsigned long long *keys_g = reinterpret_cast<const unsigned long long *>(region);
         const uint32_t *ids_g = reinterpret_cast<const uint32_t *>(region + 8u * (c.task_off[t + 1] - c.task_off[t]));
@@ -789,36 +854,22 @@ __device__ __forceinline__ void finish_task(const DeviceCatalog &c, uint32_t t, 
   }
 }
 
-// Tasks of more than 512 variants: c.rebuild_ctas CTAs per task, a cluster; the first one makes the list, then
-// each takes its share of the list's segments.
+// Tasks of more than 512 variants: c.rebuild_ctas CTAs per task, a cluster, which share the list's variants and
+// then its segments.
 //
 // Bound by the latency of its chain of barriers and shared-memory round trips, and by fetching its
 // code: every line of it runs about once per launch, and with the compiler's unrolling (116 KB of
 // code) 40 % of the stalls were for instructions.  So the loops are not unrolled (50 KB) except the
-// few that run long.  The segments of a list of several hundred entries take as long as the list
-// itself, so tasks of more than 1024 variants have 4 CTAs (rule in infaas_catalog_load): 48 us a window
-// instead of 63 on the trade-off surface, 4 x 4096.
+// few that run long.  4 CTAs for tasks of more than 1024 variants (rule in infaas_catalog_load): 38 us a window
+// on the trade-off surface, 4 x 4096; 63 us with one.
 __global__ void __launch_bounds__(REBUILD_THREADS)
 rebuild_kernel(DeviceCatalog c, int advance, uint32_t window_us) {
   extern __shared__ __align__(16) unsigned char dyn[];
   __shared__ __align__(16) IndexScratch<REBUILD_THREADS, MAX_BUCKETS> S;
   const uint32_t K = c.rebuild_ctas, t = blockIdx.x >> (K >> 1), share = blockIdx.x & (K - 1u);   // K = 1 or 4
-  uint32_t F = 0, slo_seen;
-  if (share == 0u) {
-    F = build_list(c, t, advance, window_us, dyn, S, slo_seen);
-    if (threadIdx.x == 0u) c.f_len[t] = F;
-  } else {
-    chain_wait();
-    chain_next();
-    slo_seen = *c.slo_seen;
-  }
-  uint32_t bmin, Sh;                                               // SLO buckets
+  uint32_t slo_seen, bmin, Sh;                                     // SLO buckets
+  const uint32_t F = build_list(c, t, share, K, advance, window_us, dyn, S, slo_seen);
   bucket_scale(c, slo_seen, Sh, bmin);
-  if (K > 1u) {                                                    // the list is in the region
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-    F = *reinterpret_cast<volatile uint32_t *>(c.f_len + t);
-  }
   const bool indexed = index_list(c, t, F, S, share, K, Sh, bmin);
   if (share == 0u) finish_task(c, t, F, indexed, advance, Sh, bmin);
 }
