@@ -201,18 +201,20 @@ __device__ __forceinline__ uint32_t decide_fast(const Img &img, const Fixed &fx,
 //   first segment with a feasible entry answers; otherwise the closest of the segments' misses.
 //   List without index: walk it in global memory, for a feasible entry, then for the distance.
 //
-// From global memory it is bound by the latency of dependent loads: the walk requests four entries at
-// once there.
+// From global memory it is bound by the latency of dependent loads, about 0.4 us each: everything that the
+// ranks lead to is requested at once there, whether it will be wanted or not, the walk requests four entries
+// at a time, and a query whose rank the record gave is not looked up in T2 again (the fast path found
+// nothing there).
 //
 // One segment of a task's list (at most INDEX_MAX_F consecutive positions with their own
-// tables), whose latencies of rank lo .. lo + n - 1 are still to be compared with the SLO: returns
-// the id of its first feasible entry, or PENDING after folding the segment's nearest miss into
+// tables), whose latencies of rank lo .. lo + n - 1 are still to be compared with the SLO (`none`: it is known to
+// have no feasible entry): returns the id of its first feasible entry, or PENDING after folding the segment's nearest miss into
 // (best, best_id); a later segment wins only with a strictly smaller distance, since its positions
 // are all higher.
 template <class Img>
 __device__ __forceinline__ uint32_t slow_segment(const Img &img, const Fixed &fx, const uint4 sl, uint32_t t2,
-                                                 uint32_t width, uint32_t bm0, uint32_t lo, uint32_t n, uint32_t slo,
-                                                 uint32_t min_acc, unsigned long long &best, uint32_t &best_id) {
+                                                 uint32_t width, uint32_t bm0, uint32_t lo, uint32_t n, bool none,
+                                                 uint32_t slo, uint32_t min_acc, unsigned long long &best, uint32_t &best_id) {
   const uint32_t F = sl.y & 0xFFu, Ks = (sl.y >> 8) & 0xFFu, Ka = sl.y >> 16, Fs = sl.w & 0xFFu;
   const SlowLayout SL = slow_layout(F, Ks, Ka);
   const uint32_t so = sl.x;
@@ -232,28 +234,35 @@ __device__ __forceinline__ uint32_t slow_segment(const Img &img, const Fixed &fx
       if (probe <= Ks && img.u32(so + SL.Pd + ((probe - 1u) << 2)) <= slo) r = probe;
     }
   }
-  const uint32_t pos = img.u8(t2 + r * width + k);
+  uint32_t far_A = 0, far_o = 0;
+  uint2 far_B = make_uint2(0u, 0u);
+  if (Img::FAR) {
+    far_A = img.u32(so + SL.bestA + (r << 2));
+    far_B = img.v2(so + SL.bestB + (slo ? k << 3 : 0u));
+    far_o = img.u8(so + SL.ordStart + r);
+  }
+  const uint32_t pos = Img::FAR && none ? F : img.u8(t2 + r * width + k);
   if (pos < F) return img.u32(t2 - 4u - (pos << 2));
   unsigned long long mine = ~0ull;        // this segment's nearest miss
   uint32_t mine_p = 0;
   if (slo == 0u) {                        // the accuracy term vanishes: the fastest entry
-    const uint2 Bv = img.v2(so + SL.bestB);
+    const uint2 Bv = Img::FAR ? far_B : img.v2(so + SL.bestB);
     mine = (unsigned long long)Bv.x * 10000ull;
     mine_p = Bv.y;
   } else {
     if (r > 0) {                          // some entry meets the SLO (and misses the accuracy)
-      const uint32_t A = img.u32(so + SL.bestA + (r << 2));
+      const uint32_t A = Img::FAR ? far_A : img.u32(so + SL.bestA + (r << 2));
       mine = (unsigned long long)slo * (min_acc - (A & 0xFFFFu));
       mine_p = A >> 16;
     }
     if (k < Ka) {                         // some entry meets the accuracy (and misses the SLO)
-      const uint2 Bv = img.v2(so + SL.bestB + (k << 3));
+      const uint2 Bv = Img::FAR ? far_B : img.v2(so + SL.bestB + (k << 3));
       const unsigned long long d = (unsigned long long)(Bv.x - slo) * 10000ull;
       if (d < mine || (d == mine && Bv.y < mine_p)) { mine = d; mine_p = Bv.y; }
     }
     constexpr uint32_t W = Img::FAR ? 4u : 1u;               // entries requested at once
 #pragma unroll 1
-    for (uint32_t o = img.u8(so + SL.ordStart + r); o < Fs; o += W) {   // stair entries above the SLO, ascending
+    for (uint32_t o = Img::FAR ? far_o : img.u8(so + SL.ordStart + r); o < Fs; o += W) {   // stair entries above the SLO, ascending
       uint2 e[W];
 #pragma unroll
       for (uint32_t i = 0; i < W; ++i) e[i] = img.v2(so + SL.walk + ((W > 1u ? min(o + i, Fs - 1u) : o) << 3));   // (the last again: no harm)
@@ -273,11 +282,11 @@ __device__ __forceinline__ uint32_t slow_segment(const Img &img, const Fixed &fx
   return PENDING;
 }
 
+// `sl`: slow-path parameters of the task's first segment (anything if the task is out of range).
 template <class Img>
-__device__ __forceinline__ uint32_t decide_slow(const Img &img, const DeviceCatalog &c, const Fixed &fx, uint32_t task,
+__device__ __forceinline__ uint32_t decide_slow(const Img &img, const DeviceCatalog &c, const Fixed &fx, uint4 sl, uint32_t task,
                                                 uint32_t slo, uint32_t min_acc) {
   if (task >= c.n_tasks) return INFAAS_INVALID;
-  uint4 sl = c.slow[task];
   // the list's segments in order: the first has its header word, records and bitmap in the fixed part
   // of the image, the others (lists longer than INDEX_MAX_F) a header in global memory
   const uint32_t h = img.u32(IMAGE_HDR_OFFSET + (task << 2));
@@ -288,21 +297,22 @@ __device__ __forceinline__ uint32_t decide_slow(const Img &img, const DeviceCata
   if (!(sl.z & TASK_FLAG_NOT_INDEXED)) {
     uint32_t t2 = h & 0x00FFFFFFu, width = h >> 24, bm0 = fx.bm_off + task * fx.bm_stride;
     uint32_t lo = 0u, n = 0u;
+    bool several = true;
     if (Img::FAR) {
-      const bool several = rec >> 24 == ((sl.y >> 8) & 0xFFu) + 1u;
+      several = rec >> 24 == ((sl.y >> 8) & 0xFFu) + 1u;
       lo = several ? rec & 0xFFu : __umulhi(rec + (slo & 0x00FFFFFFu), 1u << 8);
       n = several ? (rec >> 8) & 0xFFu : 0u;
     }
 #pragma unroll 1
     for (;;) {
-      const uint32_t d = slow_segment(img, fx, sl, t2, width, bm0, lo, n, slo, min_acc, best, best_p);
+      const uint32_t d = slow_segment(img, fx, sl, t2, width, bm0, lo, n, !several, slo, min_acc, best, best_p);
       if (d != PENDING) return d;
       const uint32_t next = sl.w >> 8;                       // 1 + index of the next segment
       if (next == 0u) break;
       sl = c.slow[c.n_tasks + next - 1u];
       const uint4 xh = c.xhdr[next - 1u];
       t2 = xh.x; width = xh.y; bm0 = xh.z - 4u * (fx.acc_lo / ACC_WORD_BITS);
-      lo = 0u; n = (sl.y >> 8) & 0xFFu;
+      lo = 0u; n = (sl.y >> 8) & 0xFFu; several = true;
     }
     return INFAAS_NO_FEASIBLE | best_p;
   }
@@ -372,7 +382,7 @@ __device__ __forceinline__ void resolve_parked(const Img &img, const DeviceCatal
   if (lane < count) {
     const uint32_t *e = pk.e + first + lane;
     const uint32_t ta = e[2u * PARK_CAP];
-    d = decide_slow(img, c, fx, ta & 0xFFFFu, e[PARK_CAP], ta >> 16);
+    d = decide_slow(img, c, fx, c.slow[min(ta & 0xFFFFu, c.n_tasks - 1u)], ta & 0xFFFFu, e[PARK_CAP], ta >> 16);
     out[e[0]] = d;
   }
   if (Tally) {
@@ -566,7 +576,7 @@ constexpr uint32_t DIRECT_THREADS = 256;
 constexpr uint64_t DIRECT_MAX_N_STAGED = 96 * 1024, DIRECT_MAX_N_GLOBAL = 192 * 1024;
 
 template <bool Tally>
-__global__ void __launch_bounds__(DIRECT_THREADS)
+__global__ void __launch_bounds__(DIRECT_THREADS, 4)
 select_direct_kernel(DeviceCatalog c, Queries q, uint32_t n) {
   __shared__ uint32_t sums[3];
   const uint32_t i = blockIdx.x * DIRECT_THREADS + threadIdx.x, lane = threadIdx.x & 31u;
@@ -583,8 +593,9 @@ select_direct_kernel(DeviceCatalog c, Queries q, uint32_t n) {
   const uint32_t slo_seen = *c.slo_seen;
   const GlobalImage img{c.image};
   if (live) {
+    const uint4 sl = c.slow[min(task, c.n_tasks - 1u)];      // in case: with the first lookups instead of behind the last
     d = decide_fast<false>(img, fx, task, slo, min_acc);
-    if (d == PENDING) d = decide_slow(img, c, fx, task, slo, min_acc);
+    if (d == PENDING) d = decide_slow(img, c, fx, sl, task, slo, min_acc);
     q.decision[i] = d;
   }
   __syncwarp();
