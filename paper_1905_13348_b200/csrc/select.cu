@@ -85,6 +85,7 @@ __device__ __forceinline__ bool stage_wait(unsigned long long *mbar, uint32_t pa
 // memory.  Offsets are bytes from the start of the image.
 struct SharedImage {
   static constexpr bool FAR = false;         // short round trips: what counts is instructions
+  static constexpr uint32_t PROBES = 1;      // latencies a search requests at once
   uint32_t base;
   __device__ __forceinline__ uint32_t u8(uint32_t off) const {
     uint32_t v; asm("ld.shared.u8 %0, [%1];" : "=r"(v) : "r"(base + off)); return v;
@@ -99,6 +100,7 @@ struct SharedImage {
 
 struct GlobalImage {
   static constexpr bool FAR = true;          // long round trips: what counts is dependent loads
+  static constexpr uint32_t PROBES = 1;
   const unsigned char *base;
   __device__ __forceinline__ uint32_t u8(uint32_t off) const { return base[off]; }
   __device__ __forceinline__ uint32_t u32(uint32_t off) const {
@@ -107,6 +109,11 @@ struct GlobalImage {
   __device__ __forceinline__ uint2 v2(uint32_t off) const {
     return *reinterpret_cast<const uint2 *>(base + off);
   }
+};
+
+// The same for small batches, where nothing else hides the round trips: more loads, fewer of them in sequence.
+struct DirectImage : GlobalImage {
+  static constexpr uint32_t PROBES = 7;
 };
 
 // floor(a / 24) for a < 2^16 as the high half of a product (multiply pipe).
@@ -220,7 +227,20 @@ __device__ __forceinline__ uint32_t slow_segment(const Img &img, const Fixed &fx
   const uint32_t so = sl.x;
   const uint32_t k = acc_rank<false>(img, fx, bm0, min_acc);
   uint32_t r = lo;                                           // r = #{Pd <= slo}
-  if (Img::FAR) {
+  if (Img::PROBES > 1u) {                                    // 248 latencies in three rounds instead of eight
+#pragma unroll 1
+    while (n) {
+      constexpr uint32_t P = Img::PROBES;
+      const uint32_t step = (n + 1u + P) / (P + 1u);             // what is left behind any probe is shorter
+      uint32_t v[P], passed = 0;
+#pragma unroll
+      for (uint32_t i = 0; i < P; ++i) v[i] = img.u32(so + SL.Pd + ((r + min(step * (i + 1u), n) - 1u) << 2));
+#pragma unroll
+      for (uint32_t i = 0; i < P; ++i) passed += (uint32_t)(step * (i + 1u) <= n && v[i] <= slo);
+      r += passed * step;
+      n = min(step - 1u, n - passed * step);
+    }
+  } else if (Img::FAR) {
 #pragma unroll 1
     while (n) {
       const uint32_t half = n >> 1;
@@ -591,7 +611,8 @@ select_direct_kernel(DeviceCatalog c, Queries q, uint32_t n) {
   if (live) { task = q.task[i]; slo = q.slo[i]; min_acc = q.min_acc[i]; }
   const Fixed fx = make_fixed(c, *reinterpret_cast<const uint4 *>(c.image_hdr));
   const uint32_t slo_seen = *c.slo_seen;
-  const GlobalImage img{c.image};
+  DirectImage img;
+  img.base = c.image;
   if (live) {
     const uint4 sl = c.slow[min(task, c.n_tasks - 1u)];      // in case: with the first lookups instead of behind the last
     d = decide_fast<false>(img, fx, task, slo, min_acc);
