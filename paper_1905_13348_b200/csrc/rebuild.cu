@@ -886,8 +886,7 @@ rebuild_kernel(DeviceCatalog c, int advance, uint32_t window_us) {
 // of them come before in both orders (laid down with the catalog).  No list of candidates, one barrier.
 //
 // List of the Inactive variants: the fastest (lowest id) of every accuracy class, if it is faster than
-// everything more accurate, from the lowest accuracy up; one warp goes through the classes while the
-// others place the Active ones.
+// everything more accurate, from the lowest accuracy up.
 template <uint32_t B>
 __device__ __forceinline__ uint32_t build_list_small(const DeviceCatalog &c, uint32_t t, bool advance, uint32_t window_us,
                                                      IndexScratch<B, B> &S, uint32_t &Sh, uint32_t &bmin) {
@@ -905,7 +904,6 @@ __device__ __forceinline__ uint32_t build_list_small(const DeviceCatalog &c, uin
   __shared__ uint32_t listed[GROUPS], dominated[GROUPS], spared[GROUPS];   // bit sets by local index
   __shared__ uint32_t class_eff[E * PITCH], class_id[E * PITCH];   // per accuracy class: smallest latency, lowest id with it
   __shared__ uint16_t class_acc[E * PITCH];
-  __shared__ uint32_t n_inactive;
   const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
   const uint32_t base = c.task_off[t], V = c.task_off[t + 1] - base;
   const bool live = tid < V;
@@ -935,7 +933,6 @@ __device__ __forceinline__ uint32_t build_list_small(const DeviceCatalog &c, uin
     class_eff[at(tid)] = NONE; class_id[at(tid)] = NONE;
     if (live) class_acc[at(cls)] = (uint16_t)acc;
   }
-  if (tid == 0u) n_inactive = 0u;
   S.clear(c.n_buckets, c.nbw);
   __syncthreads();
   // this lane's E variants: which belong to lower groups, which to this warp's
@@ -1032,8 +1029,9 @@ __device__ __forceinline__ uint32_t build_list_small(const DeviceCatalog &c, uin
   // the counts are cleared here, far behind their loads: a store to a line whose load is still in flight
   // holds up everything behind it
   if (advance && live) c.count_by_id[r.id] = 0u;
-  if (c.stateful && warp == GROUPS - 1u) {
-    // E classes per lane, from the highest accuracy down: those with an entry, their running minimum,
+  uint32_t n_inactive = 0;
+  if (c.stateful) {
+    // (every warp goes through all classes.)  E classes per lane, from the highest accuracy down: those with an entry, their running minimum,
     // survivors, their number
     uint32_t x[E], some = 0, least = NONE;
 #pragma unroll
@@ -1053,14 +1051,12 @@ __device__ __forceinline__ uint32_t build_list_small(const DeviceCatalog &c, uin
       least = min(least, x[j]);
       first = first && !here;
     }
-    const uint32_t n = __popc(on), incl = warp_scan_add(n), total = __shfl_sync(0xFFFFFFFFu, incl, 31);
-    uint32_t slot = n_active + total - 1u - (incl - n);
-#pragma unroll 1
-    for (; on; on &= on - 1u) {
-      const uint32_t k = ((uint32_t)__ffs(on) - 1u) * PITCH + lane;
-      emit(slot--, class_eff[k], class_acc[k], class_id[k]);
-    }
-    if (lane == 0u) n_inactive = total;
+    const uint32_t n = __popc(on), incl = warp_scan_add(n);
+    n_inactive = __shfl_sync(0xFFFFFFFFu, incl, 31);
+    // one class per thread: the list runs from the lowest accuracy up
+    const uint32_t top = n_active + n_inactive - 1u - (incl - n), its_top = __shfl_sync(0xFFFFFFFFu, top, (int)(tid / E)),
+                   its_on = __shfl_sync(0xFFFFFFFFu, on, (int)(tid / E)), j = tid % E, k = at(tid);
+    if ((its_on >> j) & 1u) emit(its_top - __popc(its_on & ((1u << j) - 1u)), class_eff[k], class_acc[k], class_id[k]);
   }
   __syncthreads();
   return n_active + n_inactive;
