@@ -190,10 +190,11 @@ __device__ __forceinline__ uint32_t decide_fast(const Img &img, const Fixed &fx,
 }
 
 // Slow path for a query the fast path could not answer.
-//   Indexed list: exact ranks, then T2.  The latency rank comes from a search, which, where the tables
-//   come from global memory, starts from what the bucket's record says: nothing to search unless the
-//   bucket holds several latencies (or, for the further segments of a long list, always).  (From
-//   shared memory the record costs more instructions than the search: +1.2 us on 2^24 queries.)  If
+//   Indexed list: exact ranks, then T2.  The latency rank starts from what the bucket's record says: nothing to
+//   search, and T2 not to be looked up again, unless the bucket holds several latencies (or, for the further
+//   segments of a long list, always).  (A branchless search over all latencies instead, from shared memory, us:
+//   14.2 M queries, 67 % of them without a feasible variant 135 / 122 with the record; 2^24, 14 %: 76.5 / 74.4;
+//   2^24, 1 %: 45.6 / 45.7.)  If
 //   nothing is feasible the nearest miss is the entry smallest in (d, position), with
 //   d = 10^4 * max(0, pred - slo) + slo * max(0, min_acc - acc) in 64 bits -- position
 //   order is (cost, pred_lat, -acc, id) order.  Entries that meet the SLO all miss the
@@ -213,6 +214,11 @@ __device__ __forceinline__ uint32_t decide_fast(const Img &img, const Fixed &fx,
 // at a time, and a query whose rank the record gave is not looked up in T2 again (the fast path found
 // nothing there).
 //
+constexpr uint32_t DIST_OVER = 10000u << 8;
+__device__ __forceinline__ unsigned long long mul_add(uint32_t a, uint32_t b, uint32_t c) {
+  return (unsigned long long)a * b + c;
+}
+
 // One segment of a task's list (at most INDEX_MAX_F consecutive positions with their own
 // tables), whose latencies of rank lo .. lo + n - 1 are still to be compared with the SLO (`none`: it is known to
 // have no feasible entry): returns the id of its first feasible entry, or PENDING after folding the segment's nearest miss into
@@ -240,18 +246,12 @@ __device__ __forceinline__ uint32_t slow_segment(const Img &img, const Fixed &fx
       r += passed * step;
       n = min(step - 1u, n - passed * step);
     }
-  } else if (Img::FAR) {
+  } else {
 #pragma unroll 1
     while (n) {
       const uint32_t half = n >> 1;
       if (img.u32(so + SL.Pd + ((r + half) << 2)) <= slo) { r += half + 1u; n -= half + 1u; }
       else n = half;
-    }
-  } else {                                                   // all latencies, without branches
-#pragma unroll
-    for (uint32_t step = 128; step; step >>= 1) {
-      const uint32_t probe = r + step;
-      if (probe <= Ks && img.u32(so + SL.Pd + ((probe - 1u) << 2)) <= slo) r = probe;
     }
   }
   uint32_t far_A = 0, far_o = 0;
@@ -261,24 +261,23 @@ __device__ __forceinline__ uint32_t slow_segment(const Img &img, const Fixed &fx
     far_B = img.v2(so + SL.bestB + (slo ? k << 3 : 0u));
     far_o = img.u8(so + SL.ordStart + r);
   }
-  const uint32_t pos = Img::FAR && none ? F : img.u8(t2 + r * width + k);
+  const uint32_t pos = none ? F : img.u8(t2 + r * width + k);
   if (pos < F) return img.u32(t2 - 4u - (pos << 2));
-  unsigned long long mine = ~0ull;        // this segment's nearest miss
-  uint32_t mine_p = 0;
+  // this segment's nearest miss, as one number to compare (distance and position apart: 145 / 135 us and 78 / 76.5
+  // on the first two of the cases above): distance << 8 | position.  Positions are below
+  // 256, and a distance is below 2^49 (10^4 * 2^32 + 2^32 * 2^16).
+  unsigned long long mine = ~0ull;
   if (slo == 0u) {                        // the accuracy term vanishes: the fastest entry
     const uint2 Bv = Img::FAR ? far_B : img.v2(so + SL.bestB);
-    mine = (unsigned long long)Bv.x * 10000ull;
-    mine_p = Bv.y;
+    mine = mul_add(Bv.x, DIST_OVER, Bv.y);
   } else {
     if (r > 0) {                          // some entry meets the SLO (and misses the accuracy)
       const uint32_t A = Img::FAR ? far_A : img.u32(so + SL.bestA + (r << 2));
-      mine = (unsigned long long)slo * (min_acc - (A & 0xFFFFu));
-      mine_p = A >> 16;
+      mine = mul_add(slo, (min_acc - (A & 0xFFFFu)) << 8, A >> 16);
     }
     if (k < Ka) {                         // some entry meets the accuracy (and misses the SLO)
       const uint2 Bv = Img::FAR ? far_B : img.v2(so + SL.bestB + (k << 3));
-      const unsigned long long d = (unsigned long long)(Bv.x - slo) * 10000ull;
-      if (d < mine || (d == mine && Bv.y < mine_p)) { mine = d; mine_p = Bv.y; }
+      mine = min(mine, mul_add(Bv.x - slo, DIST_OVER, Bv.y));
     }
     constexpr uint32_t W = Img::FAR ? 4u : 1u;               // entries requested at once
 #pragma unroll 1
@@ -289,20 +288,18 @@ __device__ __forceinline__ uint32_t slow_segment(const Img &img, const Fixed &fx
       bool done = false;
 #pragma unroll
       for (uint32_t i = 0; i < W; ++i) {
-        const uint32_t acc = e[i].y & 0xFFFFu, p = e[i].y >> 16;
-        const unsigned long long over = (unsigned long long)(e[i].x - slo) * 10000ull;
-        if (acc >= min_acc || over > mine) { done = true; break; }
-        const unsigned long long d = over + (unsigned long long)slo * (min_acc - acc);
-        if (d < mine || (d == mine && p < mine_p)) { mine = d; mine_p = p; }
+        const uint32_t acc = e[i].y & 0xFFFFu;
+        const unsigned long long over = mul_add(e[i].x - slo, DIST_OVER, e[i].y >> 16);
+        if (acc >= min_acc || over > mine) { done = true; break; }   // (from here on nothing is closer)
+        mine = min(mine, over + (unsigned long long)slo * ((min_acc - acc) << 8));
       }
       if (done) break;
     }
   }
-  if (mine < best) { best = mine; best_id = img.u32(t2 - 4u - (mine_p << 2)); }
+  if (mine >> 8 < best) { best = mine >> 8; best_id = img.u32(t2 - 4u - (((uint32_t)mine & 0xFFu) << 2)); }
   return PENDING;
 }
 
-// `sl`: slow-path parameters of the task's first segment (anything if the task is out of range).
 template <class Img>
 __device__ __forceinline__ uint32_t decide_slow(const Img &img, const DeviceCatalog &c, const Fixed &fx, uint4 sl, uint32_t task,
                                                 uint32_t slo, uint32_t min_acc) {
@@ -310,19 +307,15 @@ __device__ __forceinline__ uint32_t decide_slow(const Img &img, const DeviceCata
   // the list's segments in order: the first has its header word, records and bitmap in the fixed part
   // of the image, the others (lists longer than INDEX_MAX_F) a header in global memory
   const uint32_t h = img.u32(IMAGE_HDR_OFFSET + (task << 2));
-  const uint32_t rec = Img::FAR ? slo_record(img, fx, task, slo) : 0u;
+  const uint32_t rec = slo_record(img, fx, task, slo);
   if (sl.z & TASK_FLAG_INVALID) return INFAAS_INVALID;
   unsigned long long best = ~0ull;
   uint32_t best_p = 0;
   if (!(sl.z & TASK_FLAG_NOT_INDEXED)) {
     uint32_t t2 = h & 0x00FFFFFFu, width = h >> 24, bm0 = fx.bm_off + task * fx.bm_stride;
-    uint32_t lo = 0u, n = 0u;
-    bool several = true;
-    if (Img::FAR) {
-      several = rec >> 24 == ((sl.y >> 8) & 0xFFu) + 1u;
-      lo = several ? rec & 0xFFu : __umulhi(rec + (slo & 0x00FFFFFFu), 1u << 8);
-      n = several ? (rec >> 8) & 0xFFu : 0u;
-    }
+    bool several = rec >> 24 == ((sl.y >> 8) & 0xFFu) + 1u;
+    uint32_t lo = several ? rec & 0xFFu : __umulhi(rec + (slo & 0x00FFFFFFu), 1u << 8);
+    uint32_t n = several ? (rec >> 8) & 0xFFu : 0u;
 #pragma unroll 1
     for (;;) {
       const uint32_t d = slow_segment(img, fx, sl, t2, width, bm0, lo, n, !several, slo, min_acc, best, best_p);
