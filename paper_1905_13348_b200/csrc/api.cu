@@ -381,10 +381,11 @@ int infaas_catalog_load(const infaas_variant *rows, uint32_t n_variants, uint32_
   LOAD_TRY(infaas::prepare_rebuild_kernel());
   // Several CTAs per task where lists can span several segments, no block can lie out of reach of the task
   // word (the CTAs of a task could not agree on an index then), and the clusters of all tasks run at
-  // once (33 of them on a B200).  A window of 20,000 queries with four CTAs / with one, us, tasks of
-  // 1100 variants, structured and trade-off: 4 tasks 28.7 / 33.0 and 33.2 / 36.9, 20 tasks 26.2 / 28.2
-  // and 32.3 / 35.5, 33 tasks 25.1 / 23.4 and 34.4 / 35.1; in a second wave, 34 tasks 32.2 / 23.3 and
-  // 43.0 / 34.9.  Where every list is one segment the clusters cost 1 us.
+  // once (33 of them on a B200).  A window of 20,000 queries with four CTAs / with one, us, structured and
+  // trade-off catalogs: 4 tasks of 4096 variants 32.4 / 49.7 and 31.2 / 50.3; of 1100 variants 4 tasks
+  // 22.6 / 26.6 and 26.4 / 31.7, 20 tasks 21.0 / 22.1 and 28.8 / 32.8, 33 tasks 23.8 / 21.3 and 35.2 / 33.2; of 1000
+  // variants 20 tasks 20.6 / 20.2 and 27.1 / 29.6; of 600 variants 18.6 / 18.3 and 22.1 / 22.2 with 4 tasks,
+  // 20.9 / 17.1 and 28.9 / 23.0 with 33.  A second wave of clusters takes 10 us more.
   if (max_task > 1024 && worst_image < infaas::IMAGE_T2_LIMIT) {
     uint32_t at_once = 0;
     LOAD_TRY(infaas::rebuild_clusters_at_once(max_task, &at_once));
