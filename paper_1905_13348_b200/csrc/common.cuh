@@ -250,6 +250,31 @@ constexpr uint32_t SELECT_MAX_SMEM = 227u * 1024u - 256u;
 constexpr uint32_t REBUILD_ROW_SMEM = 22u;
 constexpr uint32_t REBUILD_CLUSTER = 4u;   // CTAs per large task
 
+// The rebuild kernel's coarse grid over a task of V variants (at most GRID x GRID cells; row = run of 2^cs
+// local indices, column = run of as many positions in accuracy order) and what CTA `share` of the task's K has
+// of it: rows from y0, local indices lo .. hi - 1, and words w0 .. w1 - 1 of the bit sets by local index.  The
+// rows of a CTA are an even number, so its variants are whole words; behind the last variant a CTA has nothing
+// at all, no part of the last word either: every word has one CTA that writes it.
+constexpr uint32_t GRID = 64;
+struct TaskShare {
+  uint32_t cs, ng, rows, y0, lo, hi, w0, w1;
+};
+inline __host__ __device__ TaskShare task_share(uint32_t V, uint32_t K, uint32_t share) {
+  TaskShare s;
+  s.cs = 4;
+#pragma unroll 1
+  while (V > (GRID << s.cs)) ++s.cs;
+  s.ng = (V + (1u << s.cs) - 1u) >> s.cs;
+  s.rows = K > 1u ? ((s.ng + K - 1u) / K + 1u) & ~1u : s.ng;
+  s.y0 = share * s.rows;
+  const uint32_t lo = s.y0 << s.cs, hi = (s.y0 + s.rows) << s.cs;
+  s.lo = lo < V ? lo : V;
+  s.hi = hi < V ? hi : V;
+  s.w0 = s.lo >> 5;
+  s.w1 = s.lo < s.hi ? (s.hi + 31u) >> 5 : s.w0;
+  return s;
+}
+
 // Once per device, with that device current: raise the kernels' shared-memory limits.
 cudaError_t prepare_select_kernel();
 cudaError_t prepare_tally_kernel();

@@ -25,9 +25,7 @@ __device__ __forceinline__ uint32_t float_bits_floor(uint32_t pattern) {
 }
 constexpr uint32_t BITS_OF_2_POW_32 = 0x4F800000u;
 
-// Coarse grid of the prune: at most GRID x GRID cells (row = run of local indices, column = run
-// of positions in accuracy order), one word of padding per row.
-constexpr uint32_t GRID = 64, GRID_PITCH = GRID + 1;
+constexpr uint32_t GRID_PITCH = GRID + 1;   // one word of padding per row of the prune's grid
 
 // Shared memory of a CTA of B threads while it builds the index of one list segment; NB: SLO buckets.
 template <uint32_t B, uint32_t NB>
@@ -505,12 +503,9 @@ __device__ __forceinline__ uint32_t build_list(const DeviceCatalog &c, uint32_t 
 
   const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
   const uint32_t base = c.task_off[t], V = c.task_off[t + 1] - base;
-  uint32_t cs = 4;                                                 // log2 of the rows' and columns' run length
-#pragma unroll 1
-  while (V > (GRID << cs)) ++cs;
-  // rows of a CTA: an even number, so that its variants [lo, hi) are whole words of the bit sets
-  const uint32_t ng = (V + (1u << cs) - 1u) >> cs, rows = K > 1u ? ((ng + K - 1u) / K + 1u) & ~1u : ng, y0 = share * rows;
-  const uint32_t lo = min(V, y0 << cs), hi = min(V, (y0 + rows) << cs), own = hi - lo, own_rows = (own + (1u << cs) - 1u) >> cs;
+  const TaskShare sh = task_share(V, K, share);
+  const uint32_t cs = sh.cs, ng = sh.ng, rows = sh.rows, y0 = sh.y0, lo = sh.lo, hi = sh.hi;
+  const uint32_t own = hi - lo, own_rows = (own + (1u << cs) - 1u) >> cs;
   // shared memory per variant (REBUILD_ROW_SMEM bytes); those by local index: of this CTA's, from lo
   uint2 *by_acc = reinterpret_cast<uint2 *>(dyn);                 // accuracy order: (pred, local), of what passed
   uint2 *by_local = by_acc + V;                                    // (pred, accuracy position); position 0xFFFF: not listed
@@ -668,10 +663,10 @@ __device__ __forceinline__ uint32_t build_list(const DeviceCatalog &c, uint32_t 
     dom = __ballot_sync(0xFFFFFFFFu, dom != 0u) >> (lane & 24u) & 0xFFu;
     if (x < nc && !(tid & 7u) && !dom) atomicOr(&keep[(lo + p) >> 5], 1u << (p & 31u));
   }
-  if (K > 1u) {                                                    // survivors to all
+  if (K > 1u) {                                                    // survivors to all, each word by the CTA that has it
     __syncthreads();
-    const uint32_t w = (lo >> 5) + tid;
-    if (w < (hi + 31u) >> 5) {
+    const uint32_t w = sh.w0 + tid;
+    if (w < sh.w1) {
       const uint32_t bits = keep[w];
 #pragma unroll 1
       for (uint32_t o = 0; o < K; ++o)

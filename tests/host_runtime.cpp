@@ -36,6 +36,11 @@ void host_log_clear() { g_log.clear(); }
 void host_allocation_limit(size_t n) { g_limit = n; }
 void host_device_error(int on) { g_error = on ? cudaErrorNoDevice : cudaSuccess; }
 const void *host_workers_table(int i) { return g_workers.p[i]; }
+void host_task_share(uint32_t V, uint32_t K, uint32_t share, uint32_t *out) {
+  const infaas::TaskShare s = infaas::task_share(V, K, share);
+  const uint32_t v[8] = {s.cs, s.ng, s.rows, s.y0, s.lo, s.hi, s.w0, s.w1};
+  memcpy(out, v, sizeof(v));
+}
 
 cudaError_t cudaGetDevice(int *d) { *d = 0; return g_error; }
 cudaError_t cudaSetDevice(int) { return cudaSuccess; }

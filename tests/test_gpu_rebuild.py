@@ -114,3 +114,72 @@ def test_lists_of_many_segments(V, n_tasks, states):
         run_stateful(w, state, load)
     else:
         run_both(w)
+
+
+# Beside a task of more than 1024 variants, which brings four CTAs for every task, tasks so small that some of
+# the four have no variants: every list after every window, with and without states.
+SMALL = [1, 3, 10, 31, 33, 37, 63, 70, 95, 100, 130, 255, 260, 287]
+
+
+def _lists(o, state, load):
+    """Every task's list at the oracle's present load: Active variants, then (with states) Inactive ones."""
+    if state is None:
+        return [o.frontier(t) for t in range(o.n_tasks)]
+    active = np.flatnonzero(state == 1)
+    a = OracleCatalog(o.rows[active], o.n_tasks)
+    a.queued = o.queued[active].copy()
+    eff = np.minimum(o.pred_lat().astype(np.int64) + load, 2**32 - 1)
+    out = []
+    for t in range(o.n_tasks):
+        ids, best = list(active[a.frontier(t)]) if active.size else [], -1
+        rest = np.flatnonzero((o.rows["task"] == t) & (state == 0))
+        for v in rest[np.lexsort((rest, -o.rows["acc_bp"][rest].astype(np.int64), eff[rest]))]:
+            if int(o.rows["acc_bp"][v]) > best:
+                best = int(o.rows["acc_bp"][v])
+                ids.append(v)
+        out.append(np.array(ids, np.uint32))
+    return out
+
+
+@pytest.mark.parametrize("states", [False, True])
+@pytest.mark.parametrize("kind", ["ties", "tradeoff"])
+@pytest.mark.parametrize("V", [1025, 1999])
+def test_small_tasks_beside_large_ones(V, kind, states):
+    import torch
+
+    import paper_1905_13348_b200 as P
+    from oracle import StatefulOracleCatalog
+    from tests.test_gpu_parity import _to_dev, _to_host_u32
+    rng = np.random.default_rng([V, len(kind), states])
+    sizes = [V] + SMALL
+    T, task = len(sizes), np.repeat(np.arange(len(sizes)), sizes)
+    N, windows, n = task.size, 120, 1500
+    lat = np.exp(rng.uniform(np.log(500.0), np.log(2e6), N)).astype(np.int64)
+    if kind == "ties":
+        cost, acc, lat = rng.integers(1, 4, N), 7000 + 30 * rng.integers(0, 5, N), rng.choice([1000, 4000, 20_000, 20_001], N)
+    else:
+        cost = (4e7 / lat**0.6 * np.exp(0.2 * rng.standard_normal(N))).astype(np.int64) + 1
+        acc = np.clip(3000 + 900 * np.log10(lat) + 150 * rng.standard_normal(N), 0, 10000).astype(np.int64)
+    rows = rows_from(task, rng.choice([1, 2, 7, 64], N), lat, acc, cost, None)
+    rows = rows[rng.permutation(N)].copy()
+    load = rng.choice(np.array([0, 1, 5000, 2**32 - 1], np.uint32), N)
+    state = _states(rng, N, (0.45, 0.45, 0.05, 0.05)) if states else None
+    cat = P.infaas_catalog_load(rows, T)
+    o = StatefulOracleCatalog(rows, T, state, load) if states else OracleCatalog(rows, T)
+    if states:
+        P.infaas_catalog_set_states(cat, state, load)
+    d = torch.empty(n, dtype=torch.int32, device="cuda")
+    try:
+        for w in range(windows):
+            for t, want in enumerate(_lists(o, o.state if states else None, load)):
+                got = P.infaas_catalog_get_frontier(cat, t)
+                assert np.array_equal(got, want), (w, t, sizes[t], got[:5], want[:5])
+            q = (rng.integers(0, T, n).astype(np.uint16),
+                 np.exp(rng.uniform(np.log(300.0), np.log(4e6), n)).astype(np.uint32),
+                 rng.choice(rows["acc_bp"], n).astype(np.uint16))
+            P.infaas_select_update(cat, *map(_to_dev, q), d, 3000)
+            want = o.select(*q, 8)
+            assert np.array_equal(_to_host_u32(d), want), w
+            o.load_update(want, 3000)
+    finally:
+        cat.free()

@@ -148,3 +148,24 @@ def test_clusters_only_where_all_run_at_once(host, n_tasks, per_task, clusters):
     c = _load(host, rows, n_tasks)
     assert [x for x in _log(host) if x.startswith("rebuild")] == ["rebuild_by_clusters" if clusters else "rebuild"]
     host.infaas_catalog_free(c)
+
+
+@pytest.mark.parametrize("K", [1, 4])
+def test_every_word_of_a_tasks_bit_sets_has_one_writer(host, K):
+    """The CTAs of a task share its variants out, and the words of the bit sets over them: a CTA behind the
+    last variant has no word either (it would overwrite another's)."""
+    out = (ctypes.c_uint32 * 8)()
+    empty = 0
+    for V in range(8193):
+        writers, at = [0] * ((V + 31) // 32), 0
+        for share in range(K):
+            host.host_task_share(V, K, share, out)
+            cs, ng, rows, y0, lo, hi, w0, w1 = out
+            assert ng <= 64 and y0 == share * rows and at == lo <= hi <= V, (V, share)
+            assert lo == hi or (lo % 32 == 0 and lo == y0 << cs and w0 == lo // 32 and w1 == (hi + 31) // 32), (V, share)
+            at = hi
+            empty += lo == hi and V > 0
+            for w in range(w0, w1):
+                writers[w] += 1
+        assert at == V and writers == [1] * len(writers), (V, writers)
+    assert empty > 100 or K == 1
