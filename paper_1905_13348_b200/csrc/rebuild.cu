@@ -210,12 +210,23 @@ __device__ __forceinline__ bool build_index(const DeviceCatalog &c, uint32_t t, 
   }
   __syncthreads();
 
-  // 2. the block's place in the image (the atomic is in flight until step 3 ends; sized as if all
-  // latencies were distinct, which they nearly always are); dense latency ranks, accuracy ranks and the
-  // best entry per rank, one sorted entry per thread
-  const uint32_t Ka = S.ka, width = Ka + 1u, bytes = block_layout(F, F, Ka, first ? 0u : nbw).bytes;
+  // 2. the block's place in the image (the atomic is in flight until step 3 ends): its size needs the number of
+  // distinct latencies, which the last warp counts for itself, a barrier before the others know; dense
+  // latency ranks, accuracy ranks and the best entry per rank, one sorted entry per thread
+  const uint32_t Ka = S.ka, width = Ka + 1u;
   unsigned long long placed = 0;
-  if (tid == B - 1u) placed = place_block_issue(c, bytes, done);
+  uint32_t bytes = 0;
+  if (warp == WARPS - 1u) {
+    uint32_t distinct = 0;
+#pragma unroll 4
+    for (uint32_t x = lane; x < F; x += 32u) distinct += (uint32_t)(x == 0u || S.sorted[x] != S.sorted[x - 1u]);
+    distinct = __reduce_add_sync(0xFFFFFFFFu, distinct);
+    bytes = block_layout(F, distinct, Ka, first ? 0u : nbw).bytes;
+    if (lane == 31u) {
+      placed = place_block_issue(c, bytes, done);
+      S.ks = distinct;
+    }
+  }
   if (32u * warp < F) {
     const uint32_t i = tid;
     uint32_t before = 0;
@@ -238,7 +249,6 @@ __device__ __forceinline__ bool build_index(const DeviceCatalog &c, uint32_t t, 
       S.ent[i] = (ra << 24) | (r << 16) | (last << 8) | p;
       atomicMax(&S.rankA[r], (acc << 16) | (0xFFFFu - p));                          // most accurate, first position
       atomicMin(&S.rankB[ra], i);                                                   // fastest, first position
-      if (i == F - 1u) S.ks = r + 1u;
     }
   }
   __syncthreads();

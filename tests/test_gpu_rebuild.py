@@ -183,3 +183,37 @@ def test_small_tasks_beside_large_ones(V, kind, states):
             o.load_update(want, 3000)
     finally:
         cat.free()
+
+
+def _image_bytes(rows, lists, lat, n_buckets):
+    """Size of the image for these lists (layout in common.cuh): no block is larger than its tables."""
+    T, up = len(lists), lambda x, a: -(-x // a) * a
+    lo, hi = int(rows["acc_bp"].min()) // 24 * 24, int(rows["acc_bp"].max())
+    nbw = (hi + 1 - lo) // 24 + 1
+    size = up(up(64 + 4 * (T + 1), 128) + 4 * (n_buckets + 1) * (T + 1) + 4 * (nbw | 1) * (T + 1), 64)
+    for ids in lists:
+        for at in range(0, len(ids), 248):
+            seg = ids[at:at + 248]
+            F, Ks, Ka = len(seg), len(set(lat[seg].tolist())), len(set(rows["acc_bp"][seg].tolist()))
+            slow = up(8 * F + 8 * (Ka + 1) + 4 * Ks + 4 * (Ks + 1) + Ks + 1, 8)
+            block = up(4 * (F + 1) + (Ks + 3) * (Ka + 1), 4) + (4 * nbw if at else 0)
+            size += up(up(block, 8) + slow, 16)
+    return size
+
+
+# Few distinct latencies, as a profile in whole milliseconds has them, and nothing dominated (cheaper is less
+# accurate): lists of 2, 3, 5 and 9 segments.  One CTA of 256, 512 and 1024 threads per task, and four
+@pytest.mark.parametrize("n_tasks,V", [(40, 256), (20, 512), (8, 1000), (3, 1999)])
+def test_blocks_of_the_image_are_as_large_as_their_tables(n_tasks, V):
+    import paper_1905_13348_b200 as P
+    rng = np.random.default_rng(V)
+    i, task = np.tile(np.arange(V), n_tasks), np.repeat(np.arange(n_tasks), V)
+    rows = rows_from(task, np.full(i.size, 8), 1000 * rng.integers(1, 40, i.size), 7000 + i, 5 + 11 * i, None)
+    cat, o = P.infaas_catalog_load(rows, n_tasks), OracleCatalog(rows, n_tasks)
+    try:
+        lists = [o.frontier(t) for t in range(n_tasks)]
+        assert [len(x) for x in lists] == [V] * n_tasks
+        info = P.infaas_catalog_get_info(cat)
+        assert info["image_bytes"] == _image_bytes(rows, lists, o.pred_lat(), info["slo_buckets"])
+    finally:
+        cat.free()
