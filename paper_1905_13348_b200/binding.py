@@ -9,11 +9,12 @@ raises.
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 
 import numpy as np
 
-from .build import LIB_PATH
+from .build import LIB_PATH, calls_path
 
 NO_FEASIBLE = 0x80000000
 INVALID = 0xFFFFFFFF
@@ -107,12 +108,14 @@ def _load_calls():
     global _calls
     if _calls is None:
         _load()
-        import torch  # noqa: F401          (its libraries, which the module needs)
+        path = calls_path()                 # (imports torch, whose libraries the module needs)
         try:
-            from . import _calls as module
+            spec = importlib.util.spec_from_file_location(f"{__package__}._calls", path)
+            module = importlib.util.module_from_spec(spec)
+            spec.loader.exec_module(module)
         except ImportError as e:
-            raise RuntimeError("the binding's extension module is not built or does not suit this torch "
-                               "(run `python -m paper_1905_13348_b200.build`); there is no fallback") from e
+            raise RuntimeError(f"the binding's extension module is not built for this torch and Python ({path}; "
+                               "run `python -m paper_1905_13348_b200.build`); there is no fallback") from e
         module.setup(_dev_ptr, _length)
         _calls = module
     return _calls

@@ -10,7 +10,6 @@ import sysconfig
 _HERE = os.path.dirname(os.path.abspath(__file__))
 _ROOT = os.path.dirname(_HERE)
 LIB_PATH = os.path.join(_HERE, "libinfaas_b200.so")
-CALLS_PATH = os.path.join(_HERE, "_calls.so")
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 
 
@@ -18,19 +17,27 @@ def sources() -> list[str]:
     return sorted(glob.glob(os.path.join(_HERE, "csrc", "*.cu")))
 
 
+def calls_path() -> str:
+    """The extension module for the torch and the Python that run: it looks into tensors through torch's C++
+    headers, so one that was built for others is not even found."""
+    import torch
+    return os.path.join(_HERE, f"_calls.{sysconfig.get_config_var('SOABI')}-torch-{torch.__version__}.so")
+
+
 def _stale() -> bool:
-    if not (os.path.exists(LIB_PATH) and os.path.exists(CALLS_PATH)):
+    calls = calls_path()
+    if not (os.path.exists(LIB_PATH) and os.path.exists(calls)):
         return True
     deps = sources() + [os.path.join(_HERE, "csrc", "calls.cpp")] + glob.glob(os.path.join(_HERE, "csrc", "*.cuh")) + \
         glob.glob(os.path.join(_ROOT, "include", "*.h"))
-    built = min(os.path.getmtime(LIB_PATH), os.path.getmtime(CALLS_PATH))
+    built = min(os.path.getmtime(LIB_PATH), os.path.getmtime(calls))
     return any(os.path.getmtime(d) > built for d in deps)
 
 
 def _build_calls() -> None:
     import torch
-    top = os.path.dirname(torch.__file__)
-    tmp = CALLS_PATH + f".tmp{os.getpid()}"
+    top, path = os.path.dirname(torch.__file__), calls_path()
+    tmp = path + f".tmp{os.getpid()}"
     subprocess.check_call(
         ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden",
          f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
@@ -39,7 +46,7 @@ def _build_calls() -> None:
          os.path.join(_HERE, "csrc", "calls.cpp"), "-o", tmp,
          "-L", _HERE, "-l:libinfaas_b200.so", "-Wl,-rpath,$ORIGIN",
          "-L", os.path.join(top, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10"])
-    os.replace(tmp, CALLS_PATH)
+    os.replace(tmp, path)
 
 
 def build(force: bool = False, verbose: bool = False) -> str:

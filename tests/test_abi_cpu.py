@@ -150,3 +150,21 @@ def test_per_window_calls_convert_arguments_as_before():
         P.infaas_advance(cat, None, stream=s)
     with pytest.raises(AttributeError):
         P.infaas_advance(object(), 1000, stream=s)
+
+
+def test_extension_module_of_another_torch_is_not_used(monkeypatch):
+    """The module reads tensors by the layout of the torch it was built against: after an upgrade it has to be
+    built again, not loaded."""
+    import torch
+
+    import paper_1905_13348_b200 as P
+    from paper_1905_13348_b200 import binding as b, build
+    build.build()
+    monkeypatch.setattr(b, "_calls", None)
+    assert not build._stale() and b._load_calls() is not None
+    monkeypatch.setattr(torch, "__version__", "99.0.0+other")
+    monkeypatch.setattr(b, "_calls", None)
+    assert build._stale()
+    with pytest.raises(RuntimeError, match="not built for this torch"):
+        P.infaas_advance(object(), 1000)
+    assert b._calls is None
