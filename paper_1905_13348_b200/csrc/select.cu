@@ -86,6 +86,7 @@ __device__ __forceinline__ bool stage_wait(unsigned long long *mbar, uint32_t pa
 struct SharedImage {
   static constexpr bool FAR = false;         // short round trips: what counts is instructions
   static constexpr uint32_t PROBES = 1;      // latencies a search requests at once
+  static constexpr bool AHEAD = false;       // read everything the ranks lead to at once, wanted or not
   uint32_t base;
   __device__ __forceinline__ uint32_t u8(uint32_t off) const {
     uint32_t v; asm("ld.shared.u8 %0, [%1];" : "=r"(v) : "r"(base + off)); return v;
@@ -101,6 +102,7 @@ struct SharedImage {
 struct GlobalImage {
   static constexpr bool FAR = true;          // long round trips: what counts is dependent loads
   static constexpr uint32_t PROBES = 1;
+  static constexpr bool AHEAD = false;
   const unsigned char *base;
   __device__ __forceinline__ uint32_t u8(uint32_t off) const { return base[off]; }
   __device__ __forceinline__ uint32_t u32(uint32_t off) const {
@@ -114,6 +116,7 @@ struct GlobalImage {
 // The same for small batches, where nothing else hides the round trips: more loads, fewer of them in sequence.
 struct DirectImage : GlobalImage {
   static constexpr uint32_t PROBES = 7;
+  static constexpr bool AHEAD = true;
 };
 
 // floor(a / 24) for a < 2^16 as the high half of a product (multiply pipe).
@@ -191,11 +194,10 @@ __device__ __forceinline__ uint32_t decide_fast(const Img &img, const Fixed &fx,
 
 // Slow path for a query the fast path could not answer.
 //   Indexed list: exact ranks, then T2.  The latency rank starts from what the bucket's record says: nothing to
-//   search, and T2 not to be looked up again, unless the bucket holds several latencies (or, for the further
-//   segments of a long list, always).  (A branchless search over all latencies instead, from shared memory, us:
-//   14.2 M queries, 67 % of them without a feasible variant 135 / 122 with the record; 2^24, 14 %: 76.5 / 74.4;
-//   2^24, 1 %: 45.6 / 45.7.)  If
-//   nothing is feasible the nearest miss is the entry smallest in (d, position), with
+//   search unless the bucket holds several latencies (or, for the further segments of a long list, always).  (A
+//   branchless search over all latencies instead, from shared memory, us: four windows of 1.5 M queries, 48 x 192
+//   variants, 92.9 / 91.5 with the record; two batches of 2^24 with their updates 141.1 / 141.1; 2^22 queries, 4 x
+//   1000 variants under a load that leaves 88 % without a feasible one, 86.1 / 89.7.)  If nothing is feasible the nearest miss is the entry smallest in (d, position), with
 //   d = 10^4 * max(0, pred - slo) + slo * max(0, min_acc - acc) in 64 bits -- position
 //   order is (cost, pred_lat, -acc, id) order.  Entries that meet the SLO all miss the
 //   accuracy, the best of them is the one with the highest accuracy (bestA); entries that
@@ -209,10 +211,12 @@ __device__ __forceinline__ uint32_t decide_fast(const Img &img, const Fixed &fx,
 //   first segment with a feasible entry answers; otherwise the closest of the segments' misses.
 //   List without index: walk it in global memory, for a feasible entry, then for the distance.
 //
-// From global memory it is bound by the latency of dependent loads, about 0.4 us each: everything that the
-// ranks lead to is requested at once there, whether it will be wanted or not, the walk requests four entries
-// at a time, and a query whose rank the record gave is not looked up in T2 again (the fast path found
-// nothing there).
+// From global memory it is bound by the latency of dependent loads, about 0.4 us each: the walk requests four
+// entries at a time there, and small batches read everything that the ranks lead to at once and do not look up T2
+// again where the record gave the rank (the fast path found nothing there).  Large batches do neither: three more
+// lines of L1 and L2 for each query cost more than they hide, and without T2 for some of them the lanes of a warp
+// go separate ways and each runs the rest by itself.  2^22 queries, us, both / neither: 4 x 1000 variants 98 / 90, 33
+// x 1100 on a trade-off surface 125 / 112, 26 x 4096 290 / 254, 64 x 600 261 / 250.
 //
 constexpr uint32_t DIST_OVER = 10000u << 8;
 __device__ __forceinline__ unsigned long long mul_add(uint32_t a, uint32_t b, uint32_t c) {
@@ -222,8 +226,7 @@ __device__ __forceinline__ unsigned long long mul_add(uint32_t a, uint32_t b, ui
 // One segment of a task's list (at most INDEX_MAX_F consecutive positions with their own
 // tables), whose latencies of rank lo .. lo + n - 1 are still to be compared with the SLO (`none`: it is known to
 // have no feasible entry): returns the id of its first feasible entry, or PENDING after folding the segment's nearest miss into
-// (best, best_id); a later segment wins only with a strictly smaller distance, since its positions
-// are all higher.
+// (best, best_id); a later segment wins only with a strictly smaller distance, since its positions are all higher.
 template <class Img>
 __device__ __forceinline__ uint32_t slow_segment(const Img &img, const Fixed &fx, const uint4 sl, uint32_t t2,
                                                  uint32_t width, uint32_t bm0, uint32_t lo, uint32_t n, bool none,
@@ -256,32 +259,31 @@ __device__ __forceinline__ uint32_t slow_segment(const Img &img, const Fixed &fx
   }
   uint32_t far_A = 0, far_o = 0;
   uint2 far_B = make_uint2(0u, 0u);
-  if (Img::FAR) {
+  if (Img::AHEAD) {
     far_A = img.u32(so + SL.bestA + (r << 2));
     far_B = img.v2(so + SL.bestB + (slo ? k << 3 : 0u));
     far_o = img.u8(so + SL.ordStart + r);
   }
-  const uint32_t pos = none ? F : img.u8(t2 + r * width + k);
+  const uint32_t pos = Img::AHEAD && none ? F : img.u8(t2 + r * width + k);
   if (pos < F) return img.u32(t2 - 4u - (pos << 2));
-  // this segment's nearest miss, as one number to compare (distance and position apart: 145 / 135 us and 78 / 76.5
-  // on the first two of the cases above): distance << 8 | position.  Positions are below
-  // 256, and a distance is below 2^49 (10^4 * 2^32 + 2^32 * 2^16).
+  // this segment's nearest miss, as one number to compare: distance << 8 | position.  Positions are below 256, and
+  // a distance is below 2^49 (10^4 * 2^32 + 2^32 * 2^16).
   unsigned long long mine = ~0ull;
   if (slo == 0u) {                        // the accuracy term vanishes: the fastest entry
-    const uint2 Bv = Img::FAR ? far_B : img.v2(so + SL.bestB);
+    const uint2 Bv = Img::AHEAD ? far_B : img.v2(so + SL.bestB);
     mine = mul_add(Bv.x, DIST_OVER, Bv.y);
   } else {
     if (r > 0) {                          // some entry meets the SLO (and misses the accuracy)
-      const uint32_t A = Img::FAR ? far_A : img.u32(so + SL.bestA + (r << 2));
+      const uint32_t A = Img::AHEAD ? far_A : img.u32(so + SL.bestA + (r << 2));
       mine = mul_add(slo, (min_acc - (A & 0xFFFFu)) << 8, A >> 16);
     }
     if (k < Ka) {                         // some entry meets the accuracy (and misses the SLO)
-      const uint2 Bv = Img::FAR ? far_B : img.v2(so + SL.bestB + (k << 3));
+      const uint2 Bv = Img::AHEAD ? far_B : img.v2(so + SL.bestB + (k << 3));
       mine = min(mine, mul_add(Bv.x - slo, DIST_OVER, Bv.y));
     }
     constexpr uint32_t W = Img::FAR ? 4u : 1u;               // entries requested at once
 #pragma unroll 1
-    for (uint32_t o = Img::FAR ? far_o : img.u8(so + SL.ordStart + r); o < Fs; o += W) {   // stair entries above the SLO, ascending
+    for (uint32_t o = Img::AHEAD ? far_o : img.u8(so + SL.ordStart + r); o < Fs; o += W) {   // stair entries above the SLO, ascending
       uint2 e[W];
 #pragma unroll
       for (uint32_t i = 0; i < W; ++i) e[i] = img.v2(so + SL.walk + ((W > 1u ? min(o + i, Fs - 1u) : o) << 3));   // (the last again: no harm)
