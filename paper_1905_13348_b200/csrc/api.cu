@@ -574,7 +574,7 @@ int infaas_assign_workers(infaas_catalog *c, const uint32_t *d_decision, uint64_
   DeviceScope scope(c->device);
   if (scope.status != cudaSuccess) return cuda_fail(scope.status);
   CUDA_TRY(infaas::launch_assign_workers(d_decision, n, c->d.n_variants, c->worker_of, d_worker, c->sm_count,
-                                         static_cast<cudaStream_t>(cuda_stream)));
+                                         infaas::split_for(c->d), static_cast<cudaStream_t>(cuda_stream)));
   return INFAAS_OK;
 }
 

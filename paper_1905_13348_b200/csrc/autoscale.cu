@@ -180,7 +180,7 @@ cudaError_t launch_autoscale(const DeviceCatalog &c, const uint32_t *s_inst, con
                              const unsigned long long *s_qps, const uint32_t *task_slo, uint32_t window_us, uint32_t slack_pct,
                              uint32_t lambda_milli, uint32_t *d_variant, uint32_t *d_delta,
                              cudaStream_t stream) {
-  return launch_chained(autoscale_kernel, c.n_tasks, AUTOSCALE_THREADS, 0, stream, c, s_inst, s_arch, s_qps, task_slo,
+  return launch_chained(autoscale_kernel, c.n_tasks, AUTOSCALE_THREADS, 0, split_for(c), stream, c, s_inst, s_arch, s_qps, task_slo,
                         window_us, slack_pct, lambda_milli, d_variant, d_delta);
 }
 

@@ -307,22 +307,29 @@ __device__ __forceinline__ uint4 load_once(const uint4 *p) {
                : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
   return v;
 }
-// Kernels without dynamic shared memory ask for the same split of an SM's L1 / shared memory, 32 KB of the
-// 228: a CTA only starts beside those of the previous kernel where the split suits it.  With the driver's own
-// choice the rebuild's CTAs (19 or 27 KB each) had to share the few SMs the selection's did not occupy: 64 CTAs on
-// 14 SMs, a window of 65,536 queries 17.6 us; with 64 KB or 100 KB the same, with 32 KB one CTA on each of 64
-// SMs, 13.4 us.
-constexpr uint32_t CARVEOUT_PCT = 14;
+// How an SM's 228 KB are split between L1 and shared memory: a CTA only starts beside those of the previous
+// kernel where the split suits both.  Catalogs whose rebuild has a thread per variant (19 or 27 KB a CTA) ask for 32 KB
+// with every kernel around it, else the driver's choice.  Of 64 x 256 variants the rebuild's CTAs shared the few
+// SMs that the selection's did not occupy with the driver's choice, 64 KB or 100 KB (64 CTAs on 14 SMs, a window of
+// 65,536 queries 17.6 us), and have an SM each with 32 KB (13.4 us).  The rebuild of larger tasks (41 KB and 22 bytes
+// per variant) does not fit into 32 KB: it would wait until the selection's SMs are empty and split anew, a window
+// of 20,000 queries, 32 KB / driver's choice, us: 64 x 600 variants 19.0 / 18.3, 64 x 1000 on a trade-off surface 26.6 /
+// 25.7, 33 x 1100 32.3 / 27.6 and 36.3 / 30.7.
+// 32 KB also hold one CTA of the rebuild at a time, so more than 148 tasks run in waves of one CTA per SM.
+constexpr uint32_t REBUILD_THREAD_MAX = 512u;   // largest task whose rebuild has a thread per variant
+constexpr int SPLIT_32K = 14;                   // per cent
+constexpr int SPLIT_DRIVER = cudaSharedmemCarveoutDefault;
+inline int split_for(const DeviceCatalog &c) { return c.max_task_variants <= REBUILD_THREAD_MAX ? SPLIT_32K : SPLIT_DRIVER; }
 template <class... P, class... A>
 inline cudaError_t launch_chained_cluster(void (*kernel)(P...), uint32_t grid, uint32_t cluster, uint32_t block, size_t smem,
-                                          cudaStream_t stream, A... args) {
+                                          int split, cudaStream_t stream, A... args) {
   cudaLaunchAttribute attr[3] = {};
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   uint32_t n = 1;
-  if (smem == 0) {
+  if (split != SPLIT_DRIVER) {
     attr[n].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
-    attr[n++].val.sharedMemCarveout = CARVEOUT_PCT;
+    attr[n++].val.sharedMemCarveout = (unsigned)split;
   }
   if (cluster > 1) {
     attr[n].id = cudaLaunchAttributeClusterDimension;
@@ -340,9 +347,9 @@ inline cudaError_t launch_chained_cluster(void (*kernel)(P...), uint32_t grid, u
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 template <class... P, class... A>
-inline cudaError_t launch_chained(void (*kernel)(P...), uint32_t grid, uint32_t block, size_t smem, cudaStream_t stream,
-                                  A... args) {
-  return launch_chained_cluster(kernel, grid, 1, block, smem, stream, args...);
+inline cudaError_t launch_chained(void (*kernel)(P...), uint32_t grid, uint32_t block, size_t smem, int split,
+                                  cudaStream_t stream, A... args) {
+  return launch_chained_cluster(kernel, grid, 1, block, smem, split, stream, args...);
 }
 
 // Launchers (host).  All are asynchronous on `stream` and allocate nothing.
@@ -401,7 +408,7 @@ cudaError_t launch_workers_build(uint32_t n_variants, const unsigned char *hw_by
                                  unsigned long long *best_inst, unsigned long long *best_hw,
                                  uint32_t *worker_of, cudaStream_t stream);
 cudaError_t launch_assign_workers(const uint32_t *d_decision, uint64_t n, uint32_t n_variants,
-                                  const uint32_t *worker_of, uint32_t *d_worker, int sm_count,
+                                  const uint32_t *worker_of, uint32_t *d_worker, int sm_count, int split,
                                   cudaStream_t stream);
 
 // Integer-pipe probe: two CTAs per SM run `iters` steps of independent add / xor / compare /

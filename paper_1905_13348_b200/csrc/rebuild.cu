@@ -1117,11 +1117,11 @@ cudaError_t rebuild_clusters_at_once(uint32_t max_task_variants, uint32_t *n) {
 cudaError_t launch_rebuild(const DeviceCatalog &c, bool advance_queues, uint32_t window_us,
                            cudaStream_t stream) {
   // a thread per variant up to 512 (as fast as it gets with registers and bit masks), beyond that in rounds
-  if (c.max_task_variants <= 512u)
+  if (c.max_task_variants <= REBUILD_THREAD_MAX)
     return launch_chained(c.max_task_variants <= 256u ? rebuild_small_kernel<256> : rebuild_small_kernel<512>, c.n_tasks,
-                          c.max_task_variants <= 256u ? 256u : 512u, 0, stream, c, advance_queues ? 1 : 0, window_us);
+                          c.max_task_variants <= 256u ? 256u : 512u, 0, split_for(c), stream, c, advance_queues ? 1 : 0, window_us);
   const size_t smem = (size_t)c.max_task_variants * REBUILD_ROW_SMEM;
-  return launch_chained_cluster(rebuild_kernel, c.n_tasks * c.rebuild_ctas, c.rebuild_ctas, REBUILD_THREADS, smem, stream, c,
+  return launch_chained_cluster(rebuild_kernel, c.n_tasks * c.rebuild_ctas, c.rebuild_ctas, REBUILD_THREADS, smem, split_for(c), stream, c,
                                 advance_queues ? 1 : 0, window_us);
 }
 

@@ -653,7 +653,7 @@ cudaError_t launch_select(const DeviceCatalog &c, const uint16_t *d_task, const 
   if (n == 0) return cudaSuccess;
   if (n <= (image_smem ? DIRECT_MAX_N_STAGED : DIRECT_MAX_N_GLOBAL))
     return launch_chained(tally ? select_direct_kernel<true> : select_direct_kernel<false>,
-                          (uint32_t)((n + DIRECT_THREADS - 1) / DIRECT_THREADS), DIRECT_THREADS, 0, stream, c,
+                          (uint32_t)((n + DIRECT_THREADS - 1) / DIRECT_THREADS), DIRECT_THREADS, 0, split_for(c), stream, c,
                           Queries{d_task, d_slo, d_min_acc, d_decision}, (uint32_t)n);
   image_smem = select_image_smem(image_smem);
   // the image grows and shrinks with the load: a quarter more than the host last saw
@@ -670,7 +670,7 @@ cudaError_t launch_select(const DeviceCatalog &c, const uint16_t *d_task, const 
   const uint32_t stage_bytes = (image_smem < c.image_capacity ? image_smem : c.image_capacity) & ~15u;
   const uint32_t first = expected < stage_bytes ? (uint32_t)expected & ~15u : stage_bytes;
   return launch_chained(tally ? select_kernel<true> : select_kernel<false>, (uint32_t)grid, SELECT_THREADS,
-                        image_smem + PARK_BYTES, stream, c, stage_bytes, first, q, n, per_cta);
+                        image_smem + PARK_BYTES, SPLIT_DRIVER, stream, c, stage_bytes, first, q, n, per_cta);
 }
 
 }  // namespace infaas

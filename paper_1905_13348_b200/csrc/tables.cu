@@ -56,19 +56,19 @@ scatter_kernel(DeviceCatalog c, const uint32_t *value_by_id, uint32_t *s_value, 
 
 cudaError_t launch_load_state(const DeviceCatalog &c, const uint32_t *slot_of_id, LoadStateTail *tail,
                               unsigned long long *served, uint32_t *queued, uint32_t *pred, cudaStream_t stream) {
-  return launch_chained(load_state_kernel, blocks_for(c.n_variants), TABLE_THREADS, 0, stream, c, slot_of_id, tail, served,
+  return launch_chained(load_state_kernel, blocks_for(c.n_variants), TABLE_THREADS, 0, split_for(c), stream, c, slot_of_id, tail, served,
                         queued, pred);
 }
 
 cudaError_t launch_states(const DeviceCatalog &c, const uint32_t *slot_of_id, unsigned char *state, cudaStream_t stream) {
-  return launch_chained(states_kernel, blocks_for(c.n_variants), TABLE_THREADS, 0, stream, c, slot_of_id, state);
+  return launch_chained(states_kernel, blocks_for(c.n_variants), TABLE_THREADS, 0, split_for(c), stream, c, slot_of_id, state);
 }
 
 cudaError_t launch_scatter(const DeviceCatalog &c, const uint32_t *value_by_id, uint32_t *s_value,
                            const unsigned char *state_by_id, const uint32_t *by_task, uint32_t *task_value,
                            cudaStream_t stream) {
   const uint32_t n = c.n_variants > c.n_tasks ? c.n_variants : c.n_tasks;
-  return launch_chained(scatter_kernel, blocks_for(n), TABLE_THREADS, 0, stream, c, value_by_id, s_value, state_by_id,
+  return launch_chained(scatter_kernel, blocks_for(n), TABLE_THREADS, 0, split_for(c), stream, c, value_by_id, s_value, state_by_id,
                         by_task, task_value);
 }
 

@@ -166,13 +166,13 @@ cudaError_t launch_tally(const DeviceCatalog &c, const uint32_t *d_decision, uin
     uint64_t shares = (uint64_t)sm_count / parts;              // CTAs per id range
     if (shares > want) shares = want;
     if (shares < 1) shares = 1;
-    return launch_chained(tally_smem_kernel, (uint32_t)(shares * parts), TALLY_SMEM_THREADS, smem, stream, d_decision, n,
+    return launch_chained(tally_smem_kernel, (uint32_t)(shares * parts), TALLY_SMEM_THREADS, smem, SPLIT_DRIVER, stream, d_decision, n,
                           c.n_variants, bins, parts, c.count_by_id, c.counters);
   }
   uint64_t want = ((n >> 2) + 255) / 256;
   const uint64_t most = (uint64_t)sm_count * 8;
   uint32_t grid = (uint32_t)(want < 1 ? 1 : (want > most ? most : want));
-  return launch_chained(tally_kernel, grid, 256, 0, stream, d_decision, n, c.n_variants, c.count_by_id, c.counters);
+  return launch_chained(tally_kernel, grid, 256, 0, split_for(c), stream, d_decision, n, c.n_variants, c.count_by_id, c.counters);
 }
 
 cudaError_t prepare_tally_kernel() {

@@ -85,25 +85,25 @@ cudaError_t launch_workers_build(uint32_t n_variants, const unsigned char *hw_by
                                  uint32_t *worker_of, cudaStream_t stream) {
   const uint32_t B = 256;
   const uint32_t m = n_variants > 256u ? n_variants : 256u;
-  cudaError_t e = launch_chained(workers_reset_kernel, (m + B - 1) / B, B, 0, stream, best_inst, n_variants, best_hw);
+  cudaError_t e = launch_chained(workers_reset_kernel, (m + B - 1) / B, B, 0, SPLIT_32K, stream, best_inst, n_variants, best_hw);
   const uint32_t k = n_inst > n_workers ? n_inst : n_workers;
   if (e == cudaSuccess && k)
-    e = launch_chained(workers_scan_kernel, (k + B - 1) / B, B, 0, stream, inst_variant, inst_worker, inst_load, n_inst,
+    e = launch_chained(workers_scan_kernel, (k + B - 1) / B, B, 0, SPLIT_32K, stream, inst_variant, inst_worker, inst_load, n_inst,
                        n_variants, worker_hw, worker_util, n_workers, best_inst, best_hw);
   if (e == cudaSuccess)
-    e = launch_chained(workers_final_kernel, (n_variants + B - 1) / B, B, 0, stream, n_variants, hw_by_id, best_inst,
+    e = launch_chained(workers_final_kernel, (n_variants + B - 1) / B, B, 0, SPLIT_32K, stream, n_variants, hw_by_id, best_inst,
                        best_hw, worker_of);
   return e;
 }
 
 cudaError_t launch_assign_workers(const uint32_t *d_decision, uint64_t n, uint32_t n_variants,
-                                  const uint32_t *worker_of, uint32_t *d_worker, int sm_count,
+                                  const uint32_t *worker_of, uint32_t *d_worker, int sm_count, int split,
                                   cudaStream_t stream) {
   if (n == 0) return cudaSuccess;
   uint64_t want = ((n >> 2) + 255) / 256;
   const uint64_t cap = (uint64_t)sm_count * 8;
   const uint32_t grid = (uint32_t)(want < 1 ? 1 : (want > cap ? cap : want));
-  return launch_chained(assign_workers_kernel, grid, 256, 0, stream, d_decision, n, n_variants, worker_of, d_worker);
+  return launch_chained(assign_workers_kernel, grid, 256, 0, split, stream, d_decision, n, n_variants, worker_of, d_worker);
 }
 
 }  // namespace infaas

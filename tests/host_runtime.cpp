@@ -36,6 +36,11 @@ void host_log_clear() { g_log.clear(); }
 void host_allocation_limit(size_t n) { g_limit = n; }
 void host_device_error(int on) { g_error = on ? cudaErrorNoDevice : cudaSuccess; }
 const void *host_workers_table(int i) { return g_workers.p[i]; }
+int host_split(uint32_t max_task_variants) {
+  infaas::DeviceCatalog c{};
+  c.max_task_variants = max_task_variants;
+  return infaas::split_for(c);
+}
 void host_task_share(uint32_t V, uint32_t K, uint32_t share, uint32_t *out) {
   const infaas::TaskShare s = infaas::task_share(V, K, share);
   const uint32_t v[8] = {s.cs, s.ng, s.rows, s.y0, s.lo, s.hi, s.w0, s.w1};
@@ -97,7 +102,7 @@ cudaError_t launch_workers_build(uint32_t, const unsigned char *, const uint32_t
   g_workers = {iv, iw, il, wh, wu};
   return cudaSuccess;
 }
-cudaError_t launch_assign_workers(const uint32_t *, uint64_t, uint32_t, const uint32_t *, uint32_t *, int, cudaStream_t) {
+cudaError_t launch_assign_workers(const uint32_t *, uint64_t, uint32_t, const uint32_t *, uint32_t *, int, int, cudaStream_t) {
   note("assign");
   return cudaSuccess;
 }

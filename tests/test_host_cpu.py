@@ -169,3 +169,11 @@ def test_every_word_of_a_tasks_bit_sets_has_one_writer(host, K):
                 writers[w] += 1
         assert at == V and writers == [1] * len(writers), (V, writers)
     assert empty > 100 or K == 1
+
+
+def test_small_split_only_where_the_rebuild_fits_into_it(host):
+    """Kernels ask for 32 KB of shared memory per SM only around a rebuild whose CTA fits into that; -1 = the
+    driver's choice."""
+    src = open(os.path.join(CSRC, "rebuild.cu")).read()
+    assert "c.max_task_variants <= REBUILD_THREAD_MAX" in src
+    assert [host.host_split(n) for n in (0, 1, 256, 257, 512, 513, 1024, 8192)] == [14] * 5 + [-1] * 3
