@@ -85,8 +85,7 @@ __device__ __forceinline__ bool stage_wait(unsigned long long *mbar, uint32_t pa
 // memory.  Offsets are bytes from the start of the image.
 struct SharedImage {
   static constexpr bool FAR = false;         // short round trips: what counts is instructions
-  static constexpr uint32_t PROBES = 1;      // latencies a search requests at once
-  static constexpr bool AHEAD = false;       // read everything the ranks lead to at once, wanted or not
+  static constexpr bool ALONE = false;       // nothing else hides a search's round trips
   uint32_t base;
   __device__ __forceinline__ uint32_t u8(uint32_t off) const {
     uint32_t v; asm("ld.shared.u8 %0, [%1];" : "=r"(v) : "r"(base + off)); return v;
@@ -101,8 +100,7 @@ struct SharedImage {
 
 struct GlobalImage {
   static constexpr bool FAR = true;          // long round trips: what counts is dependent loads
-  static constexpr uint32_t PROBES = 1;
-  static constexpr bool AHEAD = false;
+  static constexpr bool ALONE = false;
   const unsigned char *base;
   __device__ __forceinline__ uint32_t u8(uint32_t off) const { return base[off]; }
   __device__ __forceinline__ uint32_t u32(uint32_t off) const {
@@ -113,10 +111,9 @@ struct GlobalImage {
   }
 };
 
-// The same for small batches, where nothing else hides the round trips: more loads, fewer of them in sequence.
+// The same for small batches.
 struct DirectImage : GlobalImage {
-  static constexpr uint32_t PROBES = 7;
-  static constexpr bool AHEAD = true;
+  static constexpr bool ALONE = true;
 };
 
 // floor(a / 24) for a < 2^16 as the high half of a product (multiply pipe).
@@ -211,12 +208,13 @@ __device__ __forceinline__ uint32_t decide_fast(const Img &img, const Fixed &fx,
 //   first segment with a feasible entry answers; otherwise the closest of the segments' misses.
 //   List without index: walk it in global memory, for a feasible entry, then for the distance.
 //
-// From global memory it is bound by the latency of dependent loads, about 0.4 us each: the walk requests four
-// entries at a time there, and small batches read everything that the ranks lead to at once and do not look up T2
-// again where the record gave the rank (the fast path found nothing there).  Large batches do neither: three more
-// lines of L1 and L2 for each query cost more than they hide, and without T2 for some of them the lanes of a warp
-// go separate ways and each runs the rest by itself.  2^22 queries, us, both / neither: 4 x 1000 variants 98 / 90, 33
-// x 1100 on a trade-off surface 125 / 112, 26 x 4096 290 / 254, 64 x 600 261 / 250.
+// From global memory it is bound by the latency of dependent loads: the walk requests four entries at a time
+// there, and in small batches a search seven latencies.  Two ways to save more of them lost: T2 is looked up
+// also for queries whose rank the record gave, although the fast path found nothing there (without that the lanes
+// of a warp go separate ways and each runs the rest by itself), and bestA, bestB and ordStart are read as they
+// are wanted, not all at once with T2's position (three more lines of L1 and L2 for each query).  2^22 queries, us,
+// both / neither: 4 x 1000 variants 98 / 90, 33 x 1100 on a trade-off surface 125 / 112, 26 x 4096 290 / 254; 20,000
+// queries, 64 x 256 on a trade-off surface, a window 17.3 / 16.6.
 //
 constexpr uint32_t DIST_OVER = 10000u << 8;
 __device__ __forceinline__ unsigned long long mul_add(uint32_t a, uint32_t b, uint32_t c) {
@@ -224,22 +222,22 @@ __device__ __forceinline__ unsigned long long mul_add(uint32_t a, uint32_t b, ui
 }
 
 // One segment of a task's list (at most INDEX_MAX_F consecutive positions with their own
-// tables), whose latencies of rank lo .. lo + n - 1 are still to be compared with the SLO (`none`: it is known to
-// have no feasible entry): returns the id of its first feasible entry, or PENDING after folding the segment's nearest miss into
-// (best, best_id); a later segment wins only with a strictly smaller distance, since its positions are all higher.
+// tables), whose latencies of rank lo .. lo + n - 1 are still to be compared with the SLO: returns the id of its
+// first feasible entry, or PENDING after folding the segment's nearest miss into (best, best_id); a later segment
+// wins only with a strictly smaller distance, since its positions are all higher.
 template <class Img>
 __device__ __forceinline__ uint32_t slow_segment(const Img &img, const Fixed &fx, const uint4 sl, uint32_t t2,
-                                                 uint32_t width, uint32_t bm0, uint32_t lo, uint32_t n, bool none,
-                                                 uint32_t slo, uint32_t min_acc, unsigned long long &best, uint32_t &best_id) {
+                                                 uint32_t width, uint32_t bm0, uint32_t lo, uint32_t n, uint32_t slo,
+                                                 uint32_t min_acc, unsigned long long &best, uint32_t &best_id) {
   const uint32_t F = sl.y & 0xFFu, Ks = (sl.y >> 8) & 0xFFu, Ka = sl.y >> 16, Fs = sl.w & 0xFFu;
   const SlowLayout SL = slow_layout(F, Ks, Ka);
   const uint32_t so = sl.x;
   const uint32_t k = acc_rank<false>(img, fx, bm0, min_acc);
   uint32_t r = lo;                                           // r = #{Pd <= slo}
-  if (Img::PROBES > 1u) {                                    // 248 latencies in three rounds instead of eight
+  if (Img::ALONE) {                                          // 248 latencies in three rounds instead of eight
 #pragma unroll 1
     while (n) {
-      constexpr uint32_t P = Img::PROBES;
+      constexpr uint32_t P = 7;
       const uint32_t step = (n + 1u + P) / (P + 1u);             // what is left behind any probe is shorter
       uint32_t v[P], passed = 0;
 #pragma unroll
@@ -257,33 +255,26 @@ __device__ __forceinline__ uint32_t slow_segment(const Img &img, const Fixed &fx
       else n = half;
     }
   }
-  uint32_t far_A = 0, far_o = 0;
-  uint2 far_B = make_uint2(0u, 0u);
-  if (Img::AHEAD) {
-    far_A = img.u32(so + SL.bestA + (r << 2));
-    far_B = img.v2(so + SL.bestB + (slo ? k << 3 : 0u));
-    far_o = img.u8(so + SL.ordStart + r);
-  }
-  const uint32_t pos = Img::AHEAD && none ? F : img.u8(t2 + r * width + k);
+  const uint32_t pos = img.u8(t2 + r * width + k);
   if (pos < F) return img.u32(t2 - 4u - (pos << 2));
   // this segment's nearest miss, as one number to compare: distance << 8 | position.  Positions are below 256, and
   // a distance is below 2^49 (10^4 * 2^32 + 2^32 * 2^16).
   unsigned long long mine = ~0ull;
   if (slo == 0u) {                        // the accuracy term vanishes: the fastest entry
-    const uint2 Bv = Img::AHEAD ? far_B : img.v2(so + SL.bestB);
+    const uint2 Bv = img.v2(so + SL.bestB);
     mine = mul_add(Bv.x, DIST_OVER, Bv.y);
   } else {
     if (r > 0) {                          // some entry meets the SLO (and misses the accuracy)
-      const uint32_t A = Img::AHEAD ? far_A : img.u32(so + SL.bestA + (r << 2));
+      const uint32_t A = img.u32(so + SL.bestA + (r << 2));
       mine = mul_add(slo, (min_acc - (A & 0xFFFFu)) << 8, A >> 16);
     }
     if (k < Ka) {                         // some entry meets the accuracy (and misses the SLO)
-      const uint2 Bv = Img::AHEAD ? far_B : img.v2(so + SL.bestB + (k << 3));
+      const uint2 Bv = img.v2(so + SL.bestB + (k << 3));
       mine = min(mine, mul_add(Bv.x - slo, DIST_OVER, Bv.y));
     }
     constexpr uint32_t W = Img::FAR ? 4u : 1u;               // entries requested at once
 #pragma unroll 1
-    for (uint32_t o = Img::AHEAD ? far_o : img.u8(so + SL.ordStart + r); o < Fs; o += W) {   // stair entries above the SLO, ascending
+    for (uint32_t o = img.u8(so + SL.ordStart + r); o < Fs; o += W) {   // stair entries above the SLO, ascending
       uint2 e[W];
 #pragma unroll
       for (uint32_t i = 0; i < W; ++i) e[i] = img.v2(so + SL.walk + ((W > 1u ? min(o + i, Fs - 1u) : o) << 3));   // (the last again: no harm)
@@ -315,19 +306,19 @@ __device__ __forceinline__ uint32_t decide_slow(const Img &img, const DeviceCata
   uint32_t best_p = 0;
   if (!(sl.z & TASK_FLAG_NOT_INDEXED)) {
     uint32_t t2 = h & 0x00FFFFFFu, width = h >> 24, bm0 = fx.bm_off + task * fx.bm_stride;
-    bool several = rec >> 24 == ((sl.y >> 8) & 0xFFu) + 1u;
+    const bool several = rec >> 24 == ((sl.y >> 8) & 0xFFu) + 1u;
     uint32_t lo = several ? rec & 0xFFu : __umulhi(rec + (slo & 0x00FFFFFFu), 1u << 8);
     uint32_t n = several ? (rec >> 8) & 0xFFu : 0u;
 #pragma unroll 1
     for (;;) {
-      const uint32_t d = slow_segment(img, fx, sl, t2, width, bm0, lo, n, !several, slo, min_acc, best, best_p);
+      const uint32_t d = slow_segment(img, fx, sl, t2, width, bm0, lo, n, slo, min_acc, best, best_p);
       if (d != PENDING) return d;
       const uint32_t next = sl.w >> 8;                       // 1 + index of the next segment
       if (next == 0u) break;
       sl = c.slow[c.n_tasks + next - 1u];
       const uint4 xh = c.xhdr[next - 1u];
       t2 = xh.x; width = xh.y; bm0 = xh.z - 4u * (fx.acc_lo / ACC_WORD_BITS);
-      lo = 0u; n = (sl.y >> 8) & 0xFFu; several = true;
+      lo = 0u; n = (sl.y >> 8) & 0xFFu;
     }
     return INFAAS_NO_FEASIBLE | best_p;
   }
@@ -590,8 +581,19 @@ select_kernel(DeviceCatalog c, uint32_t stage_bytes, uint32_t first, Queries q, 
 constexpr uint32_t DIRECT_THREADS = 256;
 constexpr uint64_t DIRECT_MAX_N_STAGED = 96 * 1024, DIRECT_MAX_N_GLOBAL = 192 * 1024;
 
-template <bool Tally>
-__global__ void __launch_bounds__(DIRECT_THREADS, 4)
+// Two builds, for 5 and for 6 CTAs per SM (48 and 40 registers), so that all of a batch's CTAs run at once: 196,608
+// queries in one wave / two, us: 64 x 256 variants 5.5 / 7.1, 4 x 4096 10.6 / 11.6; the second build below its
+// range: 4 x 4096, 180,000 queries 10.8 / 9.2.
+// In windows (with the tally, around the rebuild whose CTAs take 19 or 27 KB of the 32) it asks for more shared
+// memory than it uses, as much as leaves room for that many CTAs: next to a CTA of the rebuild there is then
+// room for none or one of them.  Without, the next window's CTAs gather beside the rebuild's and the rebuild's
+// wait for them to leave.  A window with / without, us: 20,000 queries, 128 x 512 13.4 / 16.2, 64 x 256 on a trade-off
+// surface 15.2 / 15.6; 140,000: 14.2 / 16.8 and 15.5 / 19.9.
+constexpr uint32_t DIRECT_CTAS = 5, DIRECT_CTAS_MANY = 6;
+constexpr uint32_t direct_pad(uint32_t ctas) { return (32u * 1024u / ctas - 1280u) & ~15u; }
+
+template <bool Tally, bool Many>
+__global__ void __launch_bounds__(DIRECT_THREADS, Many ? DIRECT_CTAS_MANY : 4)
 select_direct_kernel(DeviceCatalog c, Queries q, uint32_t n) {
   __shared__ uint32_t sums[3];
   const uint32_t i = blockIdx.x * DIRECT_THREADS + threadIdx.x, lane = threadIdx.x & 31u;
@@ -651,10 +653,14 @@ cudaError_t launch_select(const DeviceCatalog &c, const uint16_t *d_task, const 
                           const uint16_t *d_min_acc, uint64_t n, uint32_t *d_decision,
                           int sm_count, uint32_t image_smem, uint32_t image_seen, bool tally, cudaStream_t stream) {
   if (n == 0) return cudaSuccess;
-  if (n <= (image_smem ? DIRECT_MAX_N_STAGED : DIRECT_MAX_N_GLOBAL))
-    return launch_chained(tally ? select_direct_kernel<true> : select_direct_kernel<false>,
-                          (uint32_t)((n + DIRECT_THREADS - 1) / DIRECT_THREADS), DIRECT_THREADS, 0, split_for(c), stream, c,
-                          Queries{d_task, d_slo, d_min_acc, d_decision}, (uint32_t)n);
+  if (n <= (image_smem ? DIRECT_MAX_N_STAGED : DIRECT_MAX_N_GLOBAL)) {
+    const uint32_t grid = (uint32_t)((n + DIRECT_THREADS - 1) / DIRECT_THREADS);
+    const bool many = grid > (uint32_t)sm_count * DIRECT_CTAS;
+    const uint32_t pad = tally && split_for(c) == SPLIT_32K ? direct_pad(many ? DIRECT_CTAS_MANY : DIRECT_CTAS) : 0u;
+    return launch_chained(many ? (tally ? select_direct_kernel<true, true> : select_direct_kernel<false, true>)
+                               : (tally ? select_direct_kernel<true, false> : select_direct_kernel<false, false>),
+                          grid, DIRECT_THREADS, pad, split_for(c), stream, c, Queries{d_task, d_slo, d_min_acc, d_decision}, (uint32_t)n);
+  }
   image_smem = select_image_smem(image_smem);
   // the image grows and shrinks with the load: a quarter more than the host last saw
   const uint64_t expected = (uint64_t)image_seen + image_seen / 4 + 4096;

@@ -90,3 +90,12 @@ def test_image_that_outgrows_what_the_host_last_saw():
         assert grown > 0, (first, info)
     finally:
         cat.free()
+
+
+# the small-batch kernel's two builds: 5 of its CTAs of 256 queries per SM, and one query more
+@pytest.mark.parametrize("name,kw", [("C4", {}), ("C5", {"n_windows": 5})])
+@pytest.mark.parametrize("over", [0, 1])
+def test_small_batches_that_fill_the_chip(name, kw, over):
+    import torch
+    n = torch.cuda.get_device_properties(0).multi_processor_count * 5 * 256 + over
+    test_batch_sizes_around_the_kernels_limits(name, kw, n)
