@@ -382,10 +382,10 @@ int infaas_catalog_load(const infaas_variant *rows, uint32_t n_variants, uint32_
   // Several CTAs per task where lists can span several segments, no block can lie out of reach of the task
   // word (the CTAs of a task could not agree on an index then), and the clusters of all tasks run at
   // once (33 of them on a B200).  A window of 20,000 queries with four CTAs / with one, us, structured and
-  // trade-off catalogs: 4 tasks of 4096 variants 32.4 / 49.7 and 31.2 / 50.3; of 1100 variants 4 tasks
-  // 22.6 / 26.6 and 26.4 / 31.7, 20 tasks 21.0 / 22.1 and 28.8 / 32.8, 33 tasks 23.8 / 21.3 and 35.2 / 33.2; of 1000
-  // variants 20 tasks 20.6 / 20.2 and 27.1 / 29.6; of 600 variants 18.6 / 18.3 and 22.1 / 22.2 with 4 tasks,
-  // 20.9 / 17.1 and 28.9 / 23.0 with 33.  A second wave of clusters takes 10 us more.
+  // trade-off catalogs: 4 tasks of 4096 variants 29.6 / 41.2 and 34.4 / 56.7; of 1100 variants 4 tasks
+  // 19.9 / 21.3 and 26.8 / 33.0, 20 tasks 18.9 / 20.1 and 27.4 / 33.4, 33 tasks 21.5 / 21.6 and 30.0 / 32.9, in two waves
+  // of clusters 34 tasks 26.7 / 21.4 and 36.6 / 33.1; of 1000 variants 20 tasks 18.1 / 18.1 and 26.9 / 30.2; of 600
+  // variants 17.9 / 17.8 and 23.0 / 22.5 with 4 tasks, 19.4 / 17.3 and 25.6 / 22.6 with 33.
   if (max_task > 1024 && worst_image < infaas::IMAGE_T2_LIMIT) {
     uint32_t at_once = 0;
     LOAD_TRY(infaas::rebuild_clusters_at_once(max_task, &at_once));

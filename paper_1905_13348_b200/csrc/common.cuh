@@ -371,8 +371,9 @@ cudaError_t launch_select(const DeviceCatalog &c, const uint16_t *d_task, const 
                           int sm_count, uint32_t image_smem, uint32_t image_seen, bool tally, cudaStream_t stream);
 // Batches below this size are tallied by the selection kernel itself in infaas_select_update.  A window
 // (select, tally, rebuild) with the fused / the separate tally, us: 64 tasks x 256 variants, 131,072
-// queries 18.5 / 26.2, 200,000: 17.8 / 19.2, 262,143: 19.3 / 19.4; 4 x 132 (few, hot variants), 131,072:
-// 19.4 / 19.4, 262,143: 26.8 / 19.0; 128 x 512, 160,000: 16.8 / 20.8, 262,143: 21.3 / 22.7.
+// queries 16.0 / 23.8, 196,000: 15.6 / 17.1, 262,143: 16.7 / 16.7; 128 x 512, 160,000: 14.4 / 19.6, 262,143:
+// 18.7 / 21.3.  Few, hot variants would be better off without below it too (4 x 132, 131,072: 20.4 / 13.6,
+// 262,143: 31.0 / 13.7): their counts are a few words that all atomics go to.
 constexpr uint64_t FUSED_TALLY_MAX_N = 192 * 1024;
 
 // Scaling-up step of the Model-Autoscaler for every task, from the pending per-variant

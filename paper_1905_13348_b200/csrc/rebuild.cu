@@ -493,7 +493,7 @@ __device__ __forceinline__ void task_sync(uint32_t K) {
 // Each CTA has a share of the grid's rows, with their variants: the running minimum down the columns
 // goes on from the last rows of the CTAs before it, what passes is made known to the CTAs behind it (by
 // accuracy position), survivors to all.  4 x 4096 variants on a trade-off surface, lists of up to 505 entries: a window of
-// 20,011 queries 46.8 us with the list made by the first CTA alone, 38.4 so.
+// 20,011 queries took 8 us longer with the list made by the first CTA alone.
 //
 // List of the Inactive variants: ordered by (eff, 10000-acc, id) with eff in place of cost and
 // pred; at most the fastest variant (lowest id) of every distinct accuracy is on it, if it is
@@ -865,8 +865,8 @@ __device__ __forceinline__ void finish_task(const DeviceCatalog &c, uint32_t t, 
 // Bound by the latency of its chain of barriers and shared-memory round trips, and by fetching its
 // code: every line of it runs about once per launch, and with the compiler's unrolling (116 KB of
 // code) 40 % of the stalls were for instructions.  So the loops are not unrolled (50 KB) except the
-// few that run long.  4 CTAs for tasks of more than 1024 variants (rule in infaas_catalog_load): 38 us a window
-// on the trade-off surface, 4 x 4096; 63 us with one.
+// few that run long.  4 CTAs for tasks of more than 1024 variants (rule and figures in infaas_catalog_load).  With
+// them a twentieth of the stalls are for instructions, 27 % at barriers, 14 % for the cluster barriers' fences.
 __global__ void __launch_bounds__(REBUILD_THREADS)
 rebuild_kernel(DeviceCatalog c, int advance, uint32_t window_us) {
   extern __shared__ __align__(16) unsigned char dyn[];
@@ -1074,7 +1074,7 @@ __device__ __forceinline__ uint32_t build_list_small(const DeviceCatalog &c, uin
 // and the instructions of every warp.  Cycles after the wait, 64 tasks x 256 variants with lists of up to 100
 // entries, this kernel / rebuild_kernel with its 1024 threads: 11.2 K / 16.6 K; lists of up to 50: 9.7 K /
 // 16.4 K; 128 x 512, up to 134: 14.3 K / 19.6 K; two lists per task: 10.5 K / 16.7 K.  A window of 65,536
-// queries: 15.3 -> 13.4 us (64 x 256), 16.2 -> 15.2 (128 x 512).  512 threads for tasks of up to 256: the
+// queries: 15.3 -> 13.4 us (64 x 256), 16.2 -> 15.2 (128 x 512); 12.6 and 13.9 since the selection keeps off its SMs.  512 threads for tasks of up to 256: the
 // steps with work for few warps 30 % faster, the rank table slower, the sum the same.
 template <uint32_t B>
 __global__ void __launch_bounds__(B)

@@ -573,11 +573,11 @@ select_kernel(DeviceCatalog c, uint32_t stage_bytes, uint32_t first, Queries q, 
 // the image costs more than the lookups, and the latency of the slow path is hidden by the other
 // warps' queries rather than by filling a warp with parked ones.
 // Up to 96 K queries, 192 K where the image would not be staged anyway.  Measured, us per launch in a
-// graph of launches, this kernel / the staging one: 64 tasks x 256 variants, 37 queries 1.7 / 3.1, 32,768:
-// 4.0 / 4.1, 98,304: 4.4 / 4.2, 131,072: 4.6 / 4.3; a window of them (tallies and load update with it),
-// 16,384: 15.9 / 19.0, 65,536: 15.2 / 17.9, 98,304: 15.4 / 17.9; 128 x 512 (image in global memory),
-// 131,072: 4.7 / 5.2, 262,144: 5.8 / 5.3; 4 x 4096 on a trade-off surface, 20,011: 6.3 / 7.8, 262,144:
-// 11.7 / 9.8.
+// graph of four, this kernel / the staging one: 64 tasks x 256 variants, 37 queries 3.7 / 4.7, 32,768:
+// 4.8 / 5.1, 98,304: 5.4 / 5.4, 131,072: 5.6 / 5.3; a window of them (tallies and load update with it),
+// 16,384: 12.2 / 15.3, 65,536: 11.9 / 15.1, 98,304: 12.1 / 15.3 (131,072: 12.6 / 16.0: windows alone would have
+// the line higher); 128 x 512 (image in global memory), 131,072: 5.6 / 6.4, 196,608: 6.0 / 6.5, 262,144:
+// 7.5 / 6.9; 4 x 4096 on a trade-off surface, 20,011: 6.9 / 8.4, 196,608: 10.4 / 10.0, 262,144: 12.5 / 10.3.
 constexpr uint32_t DIRECT_THREADS = 256;
 constexpr uint64_t DIRECT_MAX_N_STAGED = 96 * 1024, DIRECT_MAX_N_GLOBAL = 192 * 1024;
 

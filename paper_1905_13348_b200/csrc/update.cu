@@ -143,9 +143,9 @@ constexpr uint32_t TALLY_SMEM_MAX_VARIANTS = 49152;   // 192 KB of bins
 constexpr uint32_t TALLY_SMEM_MAX_PARTS = 8;           // beyond this many id ranges: global atomics
 constexpr size_t TALLY_SMEM_ALONE = 116 * 1024;
 // Below this size the clear and flush passes over the bins cost more than the shared-memory atomics
-// save.  A window with the shared-memory / the global tally, us: 528 variants, 98,000 queries 18.0 /
-// 20.6; 6,000 variants, 65,536: 18.8 / 17.4, 131,072: 19.0 / 19.5; 16,384 variants, 98,000: 20.0 / 18.5,
-// 160,000: 20.0 / 20.6; 65,536 variants, 131,072: 22.7 / 21.0, 200,000: 23.5 / 27.1.
+// save.  Selection and load update with the shared-memory / the global tally, us: 528 variants, 65,536 queries
+// 13.9 / 17.6, 98,000: 13.9 / 20.2; 6,000 variants, 65,536: 16.2 / 15.3, 131,072: 17.2 / 21.2; 16,384 variants,
+// 98,000: 16.5 / 15.1, 160,000: 18.7 / 23.6; 65,536 variants, 131,072: 19.0 / 17.5, 200,000: 19.8 / 24.1.
 inline uint64_t tally_smem_min_n(uint32_t n_variants) {
   const uint64_t n = 65536 + 10ull * n_variants;
   return n < 163840 ? n : 163840;
